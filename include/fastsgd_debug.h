@@ -45,7 +45,7 @@ int fastsgd_debug_set_grid(uint32_t blocks);
 /* Byte offsets inside the registered workspace (all of them in its fixed first
  * part): [0] u32 bar_count[8], arrivals at each gradient's grid barrier;
  * [1] u32 ne_count[8], tiles the last encoder launch read a second time, per
- * gradient; [2] u32 error; [3] decoder trace; [4] encoder trace, [5] its size
+ * gradient; [2] u32 error; [3] unused; [4] encoder trace, [5] its size
  * in bytes; [6] u32 decoder queue slots; [7] u32 decoder queue counters[6]. */
 #define FASTSGD_DEBUG_LAYOUT_FIELDS 8
 int fastsgd_debug_layout(uint64_t* offsets, uint32_t count);

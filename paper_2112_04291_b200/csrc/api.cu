@@ -199,6 +199,19 @@ int ensure_device_setup() {
     return FASTSGD_OK;
 }
 
+// A launch whose blocks may move onto the GPU while the previous kernel of the stream drains (programmatic dependent launch): the
+// kernel itself waits (wait_for_previous_kernels) before it reads or writes memory.
+cudaError_t launch_overlapped(const void* fn, unsigned grid, unsigned threads, size_t smem, void** kargs, cudaStream_t st) {
+    cudaLaunchConfig_t c;
+    std::memset(&c, 0, sizeof(c));
+    c.gridDim = dim3(grid); c.blockDim = dim3(threads); c.dynamicSmemBytes = smem; c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at; c.numAttrs = 1;
+    return cudaLaunchKernelExC(&c, fn, kargs);
+}
+
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
 int launch_sum(const float* grad, uint64_t n, uint32_t groups, uint32_t tau, const PowTable& pw,
@@ -570,17 +583,11 @@ int decode_launches(const void* const* streams_in, const uint64_t* bytes, uint32
     rc = ensure_device_setup();
     if (rc) return rc;
     const uint64_t G = groups_of(n, params->group_log2);
-    // a warp per group at least; for few groups a block per group (up to two per SM), since groups
-    // with many keys are decoded by whole blocks taken from a shared queue
-    const int warps_per_block = kDecThreads / 32;
-    uint64_t grid = (G + warps_per_block - 1) / warps_per_block;
-    const uint64_t want = 2ull * (uint64_t)g_state.sm_count;
-    const uint64_t per_group = G < want ? G : want;
-    if (grid < per_group) grid = per_group;
+    // a block per group until the GPU is full
     const uint64_t cap = (uint64_t)g_state.sm_count * g_state.dec_blocks_per_sm;
-    if (grid > cap) grid = cap;
-    const uint64_t min_grid = (G + kDecListMax - 1) / kDecListMax;     // a block owns at most kDecListMax groups
-    if (grid < min_grid) grid = min_grid;
+    const uint64_t grid = G < cap ? G : cap;
+    PowTable inv;                         // 1 / b^k: the decoder's value table multiplies where that is exact
+    for (int k = 0; k <= kMaxTau; ++k) inv.P[k] = 1.0 / pw.P[k];
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (uint32_t first = 0; first < num_streams; first += kDecMaxStreams) {
         DecArgs da;
@@ -592,7 +599,6 @@ int decode_launches(const void* const* streams_in, const uint64_t* bytes, uint32
         }
         da.n = n; da.dense = dense_out;
         da.status = &view(g_state.ws, n).ctl->decode_status;
-        da.trace = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + kTraceOffset);
         da.q_ctl = view(g_state.ws, n).ctl->dq;
         da.q_list = reinterpret_cast<unsigned int*>(static_cast<unsigned char*>(g_state.ws) + kQueueOffset);
         da.base = params->base; da.G = (uint32_t)G; da.tau = params->tau; da.l = params->flag_bits;
@@ -604,22 +610,15 @@ int decode_launches(const void* const* streams_in, const uint64_t* bytes, uint32
         }
         {
             LaunchTimer lt(2, st);
-            if (packed) {
-                if (da.W == 1u) k_decode_accumulate<true, 3><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-                else k_decode_accumulate<false, 3><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-            } else if (fused) {
-                if (da.W == 1u) k_decode_accumulate<true, 2><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-                else k_decode_accumulate<false, 2><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-            } else if (adam) {
-                if (da.W == 1u) k_decode_accumulate<true, 1><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-                else k_decode_accumulate<false, 1><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-            } else {
-                if (da.W == 1u) k_decode_accumulate<true><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-                else k_decode_accumulate<false><<<(unsigned)grid, kDecThreads, sizeof(DecShared), st>>>(da, pw);
-            }
+            void* kargs[] = {&da, &pw, &inv};
+            const bool one = da.W == 1u;
+            const void* fn = packed ? (one ? (const void*)k_decode_accumulate<true, 3> : (const void*)k_decode_accumulate<false, 3>)
+                             : fused ? (one ? (const void*)k_decode_accumulate<true, 2> : (const void*)k_decode_accumulate<false, 2>)
+                             : adam ? (one ? (const void*)k_decode_accumulate<true, 1> : (const void*)k_decode_accumulate<false, 1>)
+                                    : (one ? (const void*)k_decode_accumulate<true> : (const void*)k_decode_accumulate<false>);
+            if (launch_overlapped(fn, (unsigned)grid, kDecThreads, sizeof(DecShared), kargs, st) != cudaSuccess) { cudaGetLastError(); return FASTSGD_E_CUDA; }
         }
         g_launches.fetch_add(1, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) return FASTSGD_E_CUDA;
     }
     return FASTSGD_OK;
 }

@@ -1,0 +1,101 @@
+"""The decoder at the key counts where it changes its way of working: groups for one warp or a whole block, the group's
+slice of dense_out in shared memory or its entries alone, all streams together or one after the other.  Decoded sums
+and the model update (three arrays, and packed) bit-equal to the oracle's."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import gpu_util as G
+from paper_2112_04291_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+TILE = 16384
+HYPER = (1e-3, 0.9, 0.999, 1e-8)
+
+
+def _streams(n, counts, workers, seed, tau=128):
+    """One stream per worker with exactly counts[g] kept keys in group g; half of the keys shared with the worker before."""
+    rng = np.random.default_rng(seed)
+    out, prev = [], None
+    po = oracle.params(1.3 if tau == 128 else 1.9, tau, 2, 14)
+    for w in range(workers):
+        v = np.zeros(n, np.float32)
+        keys = []
+        for g, c in enumerate(counts):
+            lo, span = g * TILE, min(TILE, n - g * TILE)
+            c = min(c, span)
+            if prev is None:
+                k = rng.choice(span, c, replace=False)
+            else:
+                old = rng.choice(prev[g], c // 2, replace=False)
+                k = np.concatenate([old, rng.choice(np.setdiff1d(np.arange(span), old), c - c // 2, replace=False)])
+            keys.append(k)
+            v[lo + k] = (rng.uniform(0.5, 2.0, c) * rng.choice([-1.0, 1.0], c)).astype(np.float32)
+        prev = keys
+        rc, s = oracle.compress(v, po)
+        assert rc == 0 and int(np.frombuffer(s[24:32].tobytes(), np.uint64)[0]) == sum(len(k) for k in keys)
+        out.append(s)
+    return out, po, binding.params(po.base, tau, 2, 14)
+
+
+def _check(n, counts, workers, seed, tau=128, update=True):
+    streams, po, pg = _streams(n, counts, workers, seed, tau)
+    rng = np.random.default_rng(seed + 1)
+    binding.ensure_workspace(n, pg)
+    dev = [G.to_dev(np.concatenate([s, np.zeros(-s.size % 16 + 16, np.uint8)])) for s in streams]
+    sizes = [s.size for s in streams]
+    want = rng.standard_normal(n).astype(np.float32)
+    buf = G.Guarded(4 * n)
+    dense = buf.view.view(torch.float32)
+    dense.copy_(torch.from_numpy(want))
+    for s in streams:
+        assert oracle.decompress_accumulate(s, n, po, want) == 0
+    assert binding.decompress_accumulate_batch(dev, sizes, n, pg, dense) == 0
+    assert binding.decode_status() == 0 and buf.intact()
+    assert np.array_equal(dense.cpu().numpy(), want)
+    if not update:
+        return
+    theta, m, v = (rng.standard_normal(n).astype(np.float32), (rng.standard_normal(n) * 1e-3).astype(np.float32),
+                   (rng.standard_normal(n) ** 2 * 1e-6).astype(np.float32))
+    arrays = [torch.from_numpy(x.copy()).to(G.dev()) for x in (theta, m, v)] + [torch.zeros(n, dtype=torch.float32, device=G.dev())]
+    packed = torch.stack(arrays, dim=1).reshape(-1)
+    assert oracle.sparse_adam_update(streams, n, po, *HYPER, theta, m, v) == 0
+    assert binding.sparse_adam_update_batch(dev, sizes, n, pg, binding.Adam(*HYPER), arrays[3], *arrays[:3]) == 0
+    assert binding.sparse_adam_update_packed_batch(dev, sizes, n, pg, binding.Adam(*HYPER), packed) == 0
+    assert binding.decode_status() == 0
+    packed = packed.reshape(n, 4)
+    for i, x in enumerate((theta, m, v, np.zeros(n, np.float32))):
+        assert np.array_equal(arrays[i].cpu().numpy(), x) and np.array_equal(packed[:, i].cpu().numpy(), x), i
+
+
+# one stream: warp / block (256), sweep of the update (768, packed 2048), slice of dense_out (1536), words of a blob that fit
+# the stage (4096 words at 8 + 2 + up to 8 bits a key), keys that fit the lists (8192); the last group is ragged
+@pytest.mark.parametrize("count", [1, 32, 33, 255, 256, 257, 767, 768, 1535, 1536, 2047, 2048, 2049, 4096, 4097, 8184, 8192, 8193, TILE])
+def test_one_stream(count):
+    _check(3 * TILE - 5, [count, 0, max(1, count - 1)], 1, 100 + count)
+
+
+# several streams: the same sizes for all streams of a group together (warp / block: 248)
+@pytest.mark.parametrize("workers,count", [(2, 1), (2, 124), (2, 125), (3, 83), (4, 62), (4, 63), (8, 31), (8, 32), (4, 192), (4, 383), (4, 384), (4, 512),
+                                           (3, 700), (2, 2048), (8, 256), (4, 2048), (4, 2049), (8, 1023), (8, 1025), (5, 2100), (3, 9000), (2, TILE)])
+def test_several_streams(workers, count):
+    _check(3 * TILE + 1, [count, 2, count + 1, 1], workers, 300 + 10 * workers + count)
+
+
+# codes are checked against tau only where tau leaves some out
+def test_tau_below_the_largest():
+    _check(2 * TILE + 3, [900, 40, 1], 1, 7, tau=33)
+    _check(2 * TILE + 3, [900, 40, 1], 4, 8, tau=33)
+
+
+# many groups per block: one warp takes up to 1024 keys of one stream; a few large groups among many small ones are shared
+@pytest.mark.parametrize("workers", [1, 3])
+def test_many_groups_per_block(workers):
+    groups = 2400
+    rng = np.random.default_rng(workers)
+    counts = rng.integers(0, 4, groups)
+    counts[300:330] = [1023, 1024, 1025] * 10
+    counts[1000:1012] = 300
+    _check(groups * TILE - 9, counts.tolist(), workers, 40 + workers, update=False)
