@@ -13,6 +13,7 @@
 #include "sum.cuh"
 #include "bits.cuh"
 #include "compress.cuh"
+#include "encode.cuh"
 #include "keys_paper.cuh"
 #include "kv.cuh"
 #include "decode.cuh"
@@ -29,6 +30,7 @@ struct State {
     int        sum_blocks_per_sm = 0;
     int        dec_blocks_per_sm = 0;
     int        cmp_blocks_per_sm = 0;
+    int        res_blocks_per_sm = 0;
     int        kv_blocks_per_sm = 0;
     bool       attrs_set = false;
     bool       timed_out = false;          // a status query saw FASTSGD_ST_TIMEOUT: the workspace's counters are not at rest
@@ -162,6 +164,8 @@ int ensure_device_setup() {
         g_state.kv_blocks_per_sm = b3b < b3c ? b3b : b3c;
     }
     g_state.cmp_blocks_per_sm = b3;
+    if (cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_state.res_blocks_per_sm, k_resident, kEncThreads, sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_abs_sum, kSumThreads, 0) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_decode_accumulate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecShared)) != cudaSuccess)
         return FASTSGD_E_CUDA;
@@ -213,6 +217,13 @@ cudaError_t launch_overlapped(const void* fn, unsigned grid, unsigned threads, s
 }
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
+
+// 1 / b^k (kernels multiply with it where that gives the quotient's rounding)
+PowTable inverse_of(const PowTable& pw) {
+    PowTable inv;
+    for (int k = 0; k <= kMaxTau; ++k) inv.P[k] = 1.0 / pw.P[k];
+    return inv;
+}
 
 int launch_sum(const float* grad, uint64_t n, uint32_t groups, uint32_t tau, const PowTable& pw,
                const WorkspaceView& w, double* sum_out, cudaStream_t st) {
@@ -274,7 +285,7 @@ int fastsgd_debug_layout(uint64_t* offsets, uint32_t count) {
     if (!offsets) return FASTSGD_E_NULL;
     const uint64_t v[FASTSGD_DEBUG_LAYOUT_FIELDS] = {
         offsetof(Control, bar_count), offsetof(Control, ne_count), offsetof(Control, error),
-        kTraceOffset, kJobTraceOffset, kJobTraceBytes, kQueueOffset, offsetof(Control, dq)};
+        0, kJobTraceOffset, kJobTraceBytes, kQueueOffset, offsetof(Control, dq)};
     for (uint32_t i = 0; i < count && i < (uint32_t)FASTSGD_DEBUG_LAYOUT_FIELDS; ++i) offsets[i] = v[i];
     return FASTSGD_OK;
 }
@@ -485,6 +496,28 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
             cb.grad[i] = grads[first + i];
             cb.out[i] = static_cast<uint8_t*>(outs[first + i]);
         }
+        // every tile on the GPU at once (a single block waits for nobody, so it need not be launched cooperatively)
+        const uint64_t tiles = (uint64_t)cb.jobs * G, resident = (uint64_t)g_state.sm_count * (uint64_t)(g_state.res_blocks_per_sm > 0 ? g_state.res_blocks_per_sm : 0);
+        if (tiles <= resident && tiles <= kMaxResident && (!g_tun.grid_override || tiles <= g_tun.grid_override)) {
+            EncArgs ea;
+            std::memset(&ea, 0, sizeof(ea));
+            for (uint32_t i = 0; i < cb.jobs; ++i) { ea.grad[i] = cb.grad[i]; ea.out[i] = cb.out[i]; }
+            ea.out_bytes = out_bytes; ea.n = n; ea.ctl = w.ctl;
+            ea.st = reinterpret_cast<EncState*>(static_cast<unsigned char*>(g_state.ws) + kEncStateOffset);
+            ea.base = params->base; ea.J = cb.jobs; ea.G = (uint32_t)G; ea.tau = params->tau; ea.l = params->flag_bits;
+            ea.wait_limit = g_tun.wait_limit; ea.try_limit = g_tun.try_limit;
+            PowTable inv = inverse_of(pw);
+            void* kargs[] = {&ea, &pw, &inv};
+            cudaError_t err;
+            {
+                LaunchTimer lt(1, st);
+                err = tiles == 1u ? launch_overlapped((const void*)k_resident, 1u, kEncThreads, sizeof(ResShared), kargs, st)
+                                  : cudaLaunchCooperativeKernel((const void*)k_resident, dim3((unsigned)tiles), dim3(kEncThreads), kargs, sizeof(ResShared), st);
+            }
+            if (err != cudaSuccess) { cudaGetLastError(); return FASTSGD_E_CUDA; }
+            g_launches.fetch_add(1, std::memory_order_relaxed);
+            continue;
+        }
         cb.out_bytes = out_bytes; cb.n = n; cb.ctl = w.ctl; cb.partials = w.partials; cb.desc = w.desc; cb.prefix = w.prefix; cb.tmax = w.tmax; cb.nelist = w.nelist; cb.nebits = w.nebits;
         cb.sm_slots = reinterpret_cast<unsigned int*>(static_cast<unsigned char*>(g_state.ws) + kSmSlotOffset);
         cb.dense_scratch = static_cast<unsigned char*>(g_state.ws) + ws_dense_offset(n, params->group_log2);
@@ -586,8 +619,7 @@ int decode_launches(const void* const* streams_in, const uint64_t* bytes, uint32
     // a block per group until the GPU is full
     const uint64_t cap = (uint64_t)g_state.sm_count * g_state.dec_blocks_per_sm;
     const uint64_t grid = G < cap ? G : cap;
-    PowTable inv;                         // 1 / b^k: the decoder's value table multiplies where that is exact
-    for (int k = 0; k <= kMaxTau; ++k) inv.P[k] = 1.0 / pw.P[k];
+    PowTable inv = inverse_of(pw);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (uint32_t first = 0; first < num_streams; first += kDecMaxStreams) {
         DecArgs da;

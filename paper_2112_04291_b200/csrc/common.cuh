@@ -49,7 +49,7 @@ static_assert(sizeof(Control) == 256, "control block is 256 bytes");
 
 constexpr uint64_t kThrOffset      = 256;    // float thr[132]: RU32(B_k)
 constexpr uint64_t kJobSumOffset   = 800;    // double S[8]: the sum of each gradient of a k_compress launch
-constexpr uint64_t kTraceOffset    = 1024;   // (unused)
+constexpr uint64_t kEncStateOffset = 1024;   // EncState (encode.cuh)
 constexpr uint64_t kQueueOffset    = 32768;  // u32 queue[2^17]: decoder's grid-wide queue of groups (zero between launches)
 constexpr uint64_t kQueueBytes     = 4ull << 17;
 constexpr uint64_t kJobTraceOffset = kQueueOffset + kQueueBytes;  // u64 [320 blocks][8 gradients][8]: k_compress stamps (profiling aid)

@@ -1,0 +1,59 @@
+"""The encoder at the sizes where it changes its way of working: gradients whose tiles are all on the GPU at once (up to
+two per SM) and beyond, tiles without, with few and with only kept entries.  Streams byte-equal to the oracle's."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import gpu_util as G
+from paper_2112_04291_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+TILE = 16384
+
+
+def _check(grads, base, tau=128, l=2):
+    n = grads[0].size
+    pg, po = binding.params(base, tau, l, 14), oracle.params(base, tau, l, 14)
+    binding.ensure_workspace(n, pg)
+    cap = min(binding.compress_bound(n, pg), (8 * n + 4096 + 255) & ~255)
+    bufs = [G.Guarded(cap, fill=0x5C) for _ in grads]
+    dev = [G.to_dev(v) for v in grads]
+    for rep in range(2):
+        assert binding.compress_batch(dev, pg, [b.view for b in bufs]) == 0
+        for v, b in zip(grads, bufs):
+            rc, want = oracle.compress(v, po)
+            total, d, status = binding.stream_info(b.view)
+            assert status == rc == 0 and total == want.size and b.intact()
+            assert np.array_equal(b.view[:total].cpu().numpy(), want)
+
+
+def _tiles(n, counts, seed, small=1e-9):
+    """A gradient whose tile t has counts[t % len(counts)] entries far above the threshold of base 1.2, the others far below it."""
+    rng = np.random.default_rng(seed)
+    v = (rng.standard_normal(n) * small).astype(np.float32)
+    for t in range(-(-n // TILE)):
+        lo, span = t * TILE, min(TILE, n - t * TILE)
+        c = min(span, counts[t % len(counts)])
+        k = rng.choice(span, c, replace=False)
+        v[lo + k] = (rng.uniform(0.5, 2.0, c) * rng.choice([-1.0, 1.0], c)).astype(np.float32)
+    return v
+
+
+# kept entries of a tile around what a lane, a warp, a block takes in one step, and whole tiles; the last tile ragged
+@pytest.mark.parametrize("l", [1, 2, 5])
+@pytest.mark.parametrize("counts", [(0, 1), (31, 32, 33), (511, 512, 513), (1023, 1024, 1025), (4095, 4096, 4097), (TILE, TILE - 1, 0)])
+def test_kept_entries_of_a_tile(counts, l):
+    _check([_tiles(7 * TILE - 11, counts, 10 * l + counts[0])], 1.2, l=l)
+
+
+# tiles of a launch around the number that is resident at once (two per SM of 148), by one gradient and by several
+@pytest.mark.parametrize("workers,tiles", [(1, 1), (1, 2), (1, 148), (1, 149), (1, 295), (1, 296), (1, 297), (2, 148), (2, 149), (8, 37), (8, 38)])
+def test_tiles_of_a_launch(workers, tiles):
+    _check([_tiles(tiles * TILE - 3, (5 * w, 3, 200), 70 + w) for w in range(workers)], 1.2)
+
+
+def test_tau_below_the_largest_and_no_entry_kept():
+    _check([_tiles(5 * TILE + 1, (700, 3), 5)], 1.5, tau=40)
+    _check([np.zeros(5 * TILE + 1, np.float32), _tiles(5 * TILE + 1, (0, 0, 1), 6)], 1.2)
