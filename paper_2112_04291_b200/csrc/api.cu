@@ -12,7 +12,7 @@
 #include "common.cuh"
 #include "sum.cuh"
 #include "bits.cuh"
-#include "compress.cuh"
+#include "prims.cuh"
 #include "encode.cuh"
 #include "keys_paper.cuh"
 #include "kv.cuh"
@@ -29,8 +29,9 @@ struct State {
     int        sm_count = 0;
     int        sum_blocks_per_sm = 0;
     int        dec_blocks_per_sm = 0;
-    int        cmp_blocks_per_sm = 0;
     int        res_blocks_per_sm = 0;
+    int        enc_blocks_per_sm = 0;
+    int        place_blocks_per_sm = 0;
     int        kv_blocks_per_sm = 0;
     bool       attrs_set = false;
     bool       timed_out = false;          // a status query saw FASTSGD_ST_TIMEOUT: the workspace's counters are not at rest
@@ -107,30 +108,55 @@ uint64_t bound_bytes(uint64_t n, const fastsgd_params* p) {
     return kHeaderBytes + 8ull * G + 4ull * G * per_group_words;
 }
 
-uint64_t ws_dense_offset(uint64_t n, uint32_t group_log2) {
-    // partials, descriptors, prefixes, tile maxima, the list of tiles to encode and its bitmap for every gradient one launch can take
-    const uint64_t G = groups_of(n, group_log2);
-    const uint64_t b = kPartialsOffset + (uint64_t)kCmpMaxJobs * (8ull * chunks_of(n) + 24ull * G + 4ull * ((G + 31ull) >> 5));
-    return (b + 255ull) & ~255ull;
+// Gradients one encoder launch takes: up to eight, as long as they are no more than 3 * 2^30 entries together (the workspace has to
+// hold all their lists).
+uint32_t jobs_per_launch(uint64_t n) {
+    const uint64_t j = (3ull << 30) / n;
+    return j < 1ull ? 1u : j > (uint64_t)kEncMaxJobs ? (uint32_t)kEncMaxJobs : (uint32_t)j;
 }
 
-uint64_t ws_bytes_for(uint64_t n, uint32_t group_log2) {
-    return ws_dense_offset(n, group_log2) + (uint64_t)kMaxCtas * kDenseScratchBytes;
+// The part of the workspace that depends on n, as byte offsets: per unit (a quarter of a tile of 2^14 entries) of the gradients one
+// launch can take its node of the sum tree, largest |v| and list; nodes of 512 units; per tile its descriptor and blob's place; per
+// segment of tiles its totals; the lists (a slot per unit and a pool for longer ones).  The list encoder's group entries use
+// the descriptors' place.
+struct Layout {
+    uint64_t partials, chunk, umax, info, desc, blob, seg, scratch, pool_begin, pool_bytes, end;
+    uint32_t J, tiles, chunks, seg_log2, segments;
+};
+Layout layout_of(uint64_t n, uint32_t group_log2) {
+    Layout y;
+    y.J = jobs_per_launch(n);
+    y.tiles = (uint32_t)chunks_of(n);
+    y.chunks = (4u * y.tiles + kChunkUnits - 1u) / kChunkUnits;
+    y.seg_log2 = 6u;
+    while ((uint64_t)y.J * ((y.tiles + (1ull << y.seg_log2) - 1ull) >> y.seg_log2) > kMaxSegments) ++y.seg_log2;
+    y.segments = (uint32_t)((y.tiles + (1ull << y.seg_log2) - 1ull) >> y.seg_log2);
+    const uint64_t T = (uint64_t)y.J * y.tiles, G = groups_of(n, group_log2), descs = T > G ? T : G;
+    uint64_t at = kPartialsOffset;
+    auto take = [&](uint64_t bytes) { const uint64_t here = at; at = (at + bytes + 255ull) & ~255ull; return here; };
+    y.partials = take(32ull * T);
+    y.chunk = take(16ull * y.J * y.chunks);
+    y.umax = take(16ull * T);
+    y.info = take(4ull * sizeof(UnitInfo) * T);
+    y.desc = take(8ull * descs);
+    y.blob = take(4ull * T);
+    y.seg = take(8ull * y.J * y.segments);
+    // the pool: a sixth of the entries, within 2^24 (or all of a smaller gradient) and 2^27
+    const uint64_t all = (uint64_t)y.J * n;
+    uint64_t pool = all / 6ull;
+    if (pool < (1ull << 24)) pool = 1ull << 24;
+    if (pool > (1ull << 27)) pool = 1ull << 27;
+    if (pool > all) pool = all;
+    y.pool_begin = (uint64_t)kSlotBytes * T;
+    y.pool_bytes = 6ull * pool + 65536ull;
+    y.scratch = take(y.pool_begin + y.pool_bytes);
+    y.end = at;
+    return y;
 }
 
-WorkspaceView view(void* ws, uint64_t n, uint32_t group_log2 = kGroupLog2) {
-    WorkspaceView v;
-    unsigned char* base = static_cast<unsigned char*>(ws);
-    v.ctl = reinterpret_cast<Control*>(base);
-    v.thr = reinterpret_cast<float*>(base + kThrOffset);
-    v.partials = reinterpret_cast<double*>(base + kPartialsOffset);
-    v.desc = reinterpret_cast<unsigned long long*>(base + kPartialsOffset + (uint64_t)kCmpMaxJobs * 8ull * chunks_of(n));
-    v.prefix = v.desc + (uint64_t)kCmpMaxJobs * groups_of(n, group_log2);
-    v.tmax = reinterpret_cast<float*>(v.prefix + (uint64_t)kCmpMaxJobs * groups_of(n, group_log2));
-    v.nelist = reinterpret_cast<uint32_t*>(v.tmax + (uint64_t)kCmpMaxJobs * groups_of(n, group_log2));
-    v.nebits = v.nelist + (uint64_t)kCmpMaxJobs * groups_of(n, group_log2);
-    return v;
-}
+uint64_t ws_bytes_for(uint64_t n, uint32_t group_log2) { return layout_of(n, group_log2).end; }
+
+Control* control_of(void* ws) { return static_cast<Control*>(ws); }
 
 int ensure_device_setup() {
     // caller holds g_mu; once per device
@@ -140,32 +166,26 @@ int ensure_device_setup() {
     if (cudaGetDevice(&dev) != cudaSuccess) return FASTSGD_E_CUDA;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return FASTSGD_E_CUDA;
-    if (cudaFuncSetAttribute(k_compress<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CmpSmem)) != cudaSuccess)
-        return FASTSGD_E_CUDA;
-    if (cudaFuncSetAttribute(k_compress<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CmpSmem)) != cudaSuccess)
-        return FASTSGD_E_CUDA;
-    if (cudaFuncSetAttribute(k_compress<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CmpSmem)) != cudaSuccess)
-        return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ScanShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_encode, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EncShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_compress_kv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess)
         return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_compress_kv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess)
         return FASTSGD_E_CUDA;
-    int b1 = 0, b2 = 0, b3 = 0;
+    int b1 = 0, b2 = 0;
     {
-        int b3b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3, k_compress<false>, kCmpThreads, sizeof(CmpSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3b, k_compress<true>, kCmpThreads, sizeof(CmpSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        if (b3b < b3) b3 = b3b;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3b, k_compress<false, true>, kCmpThreads, sizeof(CmpSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        if (b3b < b3) b3 = b3b;
-        int b3c = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3b, k_compress_kv<false>, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3c, k_compress_kv<true>, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        g_state.kv_blocks_per_sm = b3b < b3c ? b3b : b3c;
+        int x = 0, y = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_compress_kv<false>, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_compress_kv<true>, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
+        g_state.kv_blocks_per_sm = x < y ? x : y;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_state.res_blocks_per_sm, k_resident, kEncThreads, sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_encode, kEncThreads, sizeof(EncShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_place, kEncThreads, sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+        g_state.enc_blocks_per_sm = x > 0 ? x : 1;
+        g_state.place_blocks_per_sm = y > 0 ? y : 1;
     }
-    g_state.cmp_blocks_per_sm = b3;
-    if (cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_state.res_blocks_per_sm, k_resident, kEncThreads, sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_abs_sum, kSumThreads, 0) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_decode_accumulate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecShared)) != cudaSuccess)
         return FASTSGD_E_CUDA;
@@ -225,15 +245,14 @@ PowTable inverse_of(const PowTable& pw) {
     return inv;
 }
 
-int launch_sum(const float* grad, uint64_t n, uint32_t groups, uint32_t tau, const PowTable& pw,
-               const WorkspaceView& w, double* sum_out, cudaStream_t st) {
+int launch_sum(const float* grad, uint64_t n, Control* ctl, double* partials, double* sum_out, cudaStream_t st) {
     FSG_DEVICE_STATE();
     SumArgs sa;
-    sa.grad = grad; sa.n = n; sa.chunks = (uint32_t)chunks_of(n); sa.groups = groups; sa.tau = tau;
-    sa.ctl = w.ctl; sa.thr = w.thr; sa.partials = w.partials; sa.desc = w.desc; sa.sum_out = sum_out;
+    sa.grad = grad; sa.n = n; sa.chunks = (uint32_t)chunks_of(n);
+    sa.ctl = ctl; sa.partials = partials; sa.sum_out = sum_out;
     uint64_t grid = (uint64_t)g_state.sm_count * g_state.sum_blocks_per_sm;
     if (grid > sa.chunks) grid = sa.chunks;
-    { LaunchTimer lt(0, st); k_abs_sum<<<(unsigned)grid, kSumThreads, 0, st>>>(sa, pw); }
+    { LaunchTimer lt(0, st); k_abs_sum<<<(unsigned)grid, kSumThreads, 0, st>>>(sa); }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? FASTSGD_OK : FASTSGD_E_CUDA;
 }
@@ -285,18 +304,12 @@ int fastsgd_debug_layout(uint64_t* offsets, uint32_t count) {
     if (!offsets) return FASTSGD_E_NULL;
     const uint64_t v[FASTSGD_DEBUG_LAYOUT_FIELDS] = {
         offsetof(Control, bar_count), offsetof(Control, ne_count), offsetof(Control, error),
-        0, kJobTraceOffset, kJobTraceBytes, kQueueOffset, offsetof(Control, dq)};
+        0, 0, 0, kQueueOffset, offsetof(Control, dq)};
     for (uint32_t i = 0; i < count && i < (uint32_t)FASTSGD_DEBUG_LAYOUT_FIELDS; ++i) offsets[i] = v[i];
     return FASTSGD_OK;
 }
 
-int fastsgd_debug_trace_compiled(void) {
-#ifdef FASTSGD_TRACE
-    return 1;
-#else
-    return 0;
-#endif
-}
+int fastsgd_debug_trace_compiled(void) { return 0; }
 
 const char* fastsgd_strerror(int code) {
     switch (code) {
@@ -367,9 +380,8 @@ int fastsgd_abs_sum(const float* grad, uint64_t n, double* sum_out, void* stream
     if (!g_state.ws || g_state.ws_bytes < ws_bytes_for(n, kGroupLog2)) return FASTSGD_E_NO_WORKSPACE;
     rc = ensure_device_setup();
     if (rc) return rc;
-    PowTable pw;
-    for (int k = 0; k <= kMaxTau; ++k) pw.P[k] = 1.0;
-    return launch_sum(grad, n, 0u, 0u, pw, view(g_state.ws, n), sum_out, static_cast<cudaStream_t>(stream));
+    double* partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + layout_of(n, kGroupLog2).partials);
+    return launch_sum(grad, n, control_of(g_state.ws), partials, sum_out, static_cast<cudaStream_t>(stream));
 }
 
 namespace {
@@ -381,13 +393,13 @@ int launch_list_encoder(bool dense, const uint32_t* keys, const float* values, u
     FSG_DEVICE_STATE();
     if (g_state.kv_blocks_per_sm < 1) return FASTSGD_E_CUDA;
     const uint64_t G = groups_of(n, params->group_log2);
-    WorkspaceView w = view(g_state.ws, n, params->group_log2);
+    const Layout y = layout_of(n, params->group_log2);
     KvArgs ka;
     std::memset(&ka, 0, sizeof(ka));
     ka.keys = keys; ka.vals = values; ka.count = dense ? n : count; ka.n = n;
-    ka.out = static_cast<uint8_t*>(out); ka.out_bytes = out_bytes; ka.ctl = w.ctl;
+    ka.out = static_cast<uint8_t*>(out); ka.out_bytes = out_bytes; ka.ctl = control_of(g_state.ws);
     ka.partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + kKvPartialsOffset);
-    ka.meta = w.desc;
+    ka.meta = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + y.desc);
     ka.blk_agg = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + kKvAggOffset);
     ka.base = params->base; ka.G = (uint32_t)G; ka.chunks = (uint32_t)chunks_of(n);
     ka.tau = params->tau; ka.l = params->flag_bits; ka.group_log2 = params->group_log2;
@@ -446,16 +458,17 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
         // Any other group size: the sum kernel, then the list encoder over the dense gradient (the fused kernel's
         // tile is the group of 2^14).  Two launches per gradient, the gradient read three times.
         if (params->group_log2 < 8u) return FASTSGD_E_NOT_IMPLEMENTED;
-        // sum kernel; the kept entries selected into a list in the workspace (the fused kernel's scratch for dense tiles,
-        // 4.5 M pairs); the list encoder on that list -- or, should the list not fit, over the dense gradient itself
+        // sum kernel; the kept entries selected into a list in the workspace (where the default group size keeps its
+        // tiles' lists); the list encoder on that list -- or, should the list not fit, over the dense gradient itself
         // (a warp per group: slow for large groups).  Which of the two runs is decided on the device.
         unsigned char* wsb = static_cast<unsigned char*>(g_state.ws);
         double* S = reinterpret_cast<double*>(wsb + kJobSumOffset);
         unsigned long long* count_dev = reinterpret_cast<unsigned long long*>(wsb + kKvAggOffset + kKvAggBytes - 8);
-        unsigned char* list = wsb + ws_dense_offset(n, params->group_log2);
-        const uint64_t capacity = ((uint64_t)kMaxCtas * kDenseScratchBytes) / 8ull;
+        const Layout y = layout_of(n, params->group_log2);
+        unsigned char* list = wsb + y.scratch;
+        const uint64_t capacity = ((y.end - y.scratch) / 8ull) & ~63ull;
         for (uint32_t i = 0; i < num_grads; ++i) {
-            rc = launch_sum(grads[i], n, 0u, params->tau, pw, view(g_state.ws, n, params->group_log2), S, st);
+            rc = launch_sum(grads[i], n, control_of(g_state.ws), reinterpret_cast<double*>(wsb + y.partials), S, st);
             if (rc) return rc;
             SelArgs sa;
             std::memset(&sa, 0, sizeof(sa));
@@ -481,71 +494,62 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
         }
         return FASTSGD_OK;
     }
-    WorkspaceView w = view(g_state.ws, n);
-    if (g_state.cmp_blocks_per_sm < 1) return FASTSGD_E_CUDA;
-    uint64_t grid = (uint64_t)g_state.sm_count * g_state.cmp_blocks_per_sm;
-    if (grid > kMaxCtas) grid = kMaxCtas;
-    const uint64_t grid_full = grid;
-    if (g_tun.grid_override && g_tun.grid_override < grid) grid = g_tun.grid_override;      // (never two teams then)
-    if (grid > G) grid = G;
-    for (uint32_t first = 0; first < num_grads; first += kCmpMaxJobs) {
-        CmpBatch cb;
-        std::memset(&cb, 0, sizeof(cb));
-        cb.jobs = num_grads - first < (uint32_t)kCmpMaxJobs ? num_grads - first : (uint32_t)kCmpMaxJobs;
-        for (uint32_t i = 0; i < cb.jobs; ++i) {
-            cb.grad[i] = grads[first + i];
-            cb.out[i] = static_cast<uint8_t*>(outs[first + i]);
+    const Layout y = layout_of(n, params->group_log2);
+    unsigned char* wsb = static_cast<unsigned char*>(g_state.ws);
+    PowTable inv = inverse_of(pw);
+    for (uint32_t first = 0; first < num_grads; first += y.J) {
+        EncArgs ea;
+        std::memset(&ea, 0, sizeof(ea));
+        ea.J = num_grads - first < y.J ? num_grads - first : y.J;
+        for (uint32_t i = 0; i < ea.J; ++i) {
+            ea.grad[i] = grads[first + i];
+            ea.out[i] = static_cast<uint8_t*>(outs[first + i]);
         }
+        ea.out_bytes = out_bytes; ea.n = n; ea.ctl = control_of(wsb);
+        ea.st = reinterpret_cast<EncState*>(wsb + kEncStateOffset);
+        ea.partials = reinterpret_cast<double*>(wsb + y.partials);
+        ea.chunk = reinterpret_cast<unsigned long long*>(wsb + y.chunk); ea.chunks = y.chunks;
+        ea.umax = reinterpret_cast<float*>(wsb + y.umax);
+        ea.info = reinterpret_cast<UnitInfo*>(wsb + y.info);
+        ea.desc = reinterpret_cast<unsigned long long*>(wsb + y.desc);
+        ea.blob = reinterpret_cast<uint32_t*>(wsb + y.blob);
+        ea.seg = reinterpret_cast<unsigned long long*>(wsb + y.seg); ea.seg_log2 = y.seg_log2; ea.segments = y.segments;
+        ea.scratch = wsb + y.scratch; ea.pool_begin = y.pool_begin; ea.pool_bytes = y.pool_bytes;
+        ea.base = params->base; ea.inv_ptau = inv.P[params->tau]; ea.G = y.tiles;
+        ea.tau = params->tau; ea.l = params->flag_bits; ea.wait_limit = g_tun.wait_limit; ea.try_limit = g_tun.try_limit;
+        const uint64_t tiles = (uint64_t)ea.J * ea.G;
+        void* kargs[] = {&ea, &pw, &inv};
         // every tile on the GPU at once (a single block waits for nobody, so it need not be launched cooperatively)
-        const uint64_t tiles = (uint64_t)cb.jobs * G, resident = (uint64_t)g_state.sm_count * (uint64_t)(g_state.res_blocks_per_sm > 0 ? g_state.res_blocks_per_sm : 0);
+        const uint64_t resident = (uint64_t)g_state.sm_count * (uint64_t)(g_state.res_blocks_per_sm > 0 ? g_state.res_blocks_per_sm : 0);
         if (tiles <= resident && tiles <= kMaxResident && (!g_tun.grid_override || tiles <= g_tun.grid_override)) {
-            EncArgs ea;
-            std::memset(&ea, 0, sizeof(ea));
-            for (uint32_t i = 0; i < cb.jobs; ++i) { ea.grad[i] = cb.grad[i]; ea.out[i] = cb.out[i]; }
-            ea.out_bytes = out_bytes; ea.n = n; ea.ctl = w.ctl;
-            ea.st = reinterpret_cast<EncState*>(static_cast<unsigned char*>(g_state.ws) + kEncStateOffset);
-            ea.base = params->base; ea.J = cb.jobs; ea.G = (uint32_t)G; ea.tau = params->tau; ea.l = params->flag_bits;
-            ea.wait_limit = g_tun.wait_limit; ea.try_limit = g_tun.try_limit;
-            PowTable inv = inverse_of(pw);
-            void* kargs[] = {&ea, &pw, &inv};
-            cudaError_t err;
-            {
-                LaunchTimer lt(1, st);
-                err = tiles == 1u ? launch_overlapped((const void*)k_resident, 1u, kEncThreads, sizeof(ResShared), kargs, st)
-                                  : cudaLaunchCooperativeKernel((const void*)k_resident, dim3((unsigned)tiles), dim3(kEncThreads), kargs, sizeof(ResShared), st);
-            }
+            LaunchTimer lt(1, st);
+            const cudaError_t err = tiles == 1u ? launch_overlapped((const void*)k_resident, 1u, kEncThreads, sizeof(ResShared), kargs, st)
+                                                : cudaLaunchCooperativeKernel((const void*)k_resident, dim3((unsigned)tiles), dim3(kEncThreads), kargs, sizeof(ResShared), st);
             if (err != cudaSuccess) { cudaGetLastError(); return FASTSGD_E_CUDA; }
             g_launches.fetch_add(1, std::memory_order_relaxed);
             continue;
         }
-        cb.out_bytes = out_bytes; cb.n = n; cb.ctl = w.ctl; cb.partials = w.partials; cb.desc = w.desc; cb.prefix = w.prefix; cb.tmax = w.tmax; cb.nelist = w.nelist; cb.nebits = w.nebits;
-        cb.sm_slots = reinterpret_cast<unsigned int*>(static_cast<unsigned char*>(g_state.ws) + kSmSlotOffset);
-        cb.dense_scratch = static_cast<unsigned char*>(g_state.ws) + ws_dense_offset(n, params->group_log2);
-        cb.base = params->base; cb.G = (uint32_t)G; cb.tau = params->tau; cb.l = params->flag_bits;
-        cb.wait_limit = g_tun.wait_limit; cb.try_limit = g_tun.try_limit;
-        // Two or more gradients, two resident blocks per SM and enough tiles: the two blocks of an SM
-        // form two teams that work on different gradients.  One gradient: the tiles below the grid
-        // size are assigned statically, so every block gets an equal share.
-        uint64_t launch_grid = grid;
-        cb.teams = 1u;
-        if (cb.jobs >= 2u && g_state.cmp_blocks_per_sm >= 2 && grid_full == 2ull * (uint64_t)g_state.sm_count &&
-            g_state.sm_count <= 256 && G >= grid_full && !g_tun.grid_override) {
-            cb.teams = 2u;
-            launch_grid = grid_full;
-        } else if (cb.jobs == 1u) {
-            const uint64_t rounds = (G + grid - 1) / grid;
-            launch_grid = (G + rounds - 1) / rounds;
+        uint64_t g1 = (uint64_t)g_state.sm_count, g2 = (uint64_t)g_state.sm_count * g_state.enc_blocks_per_sm, g3 = (uint64_t)g_state.sm_count * g_state.place_blocks_per_sm;
+        if (g_tun.grid_override) {
+            if (g_tun.grid_override < g1) g1 = g_tun.grid_override;
+            if (g_tun.grid_override < g2) g2 = g_tun.grid_override;
+            if (g_tun.grid_override < g3) g3 = g_tun.grid_override;
         }
-        void* kargs[] = {&cb, &pw};
-        cudaError_t err;
+        if (g1 > tiles) g1 = tiles;
+        if (g2 > tiles) g2 = tiles;
+        if (g3 > tiles) g3 = tiles;
+        ea.scan_blocks = (uint32_t)g1;
+        ea.samplers = (uint32_t)g1 / ea.J < kSampleBlocks ? (uint32_t)g1 / ea.J : kSampleBlocks;      // (none: no estimate, every tile is read again)
         {
             LaunchTimer lt(1, st);
-            const void* fn = cb.jobs > 1u ? (const void*)k_compress<true>
-                                          : (cb.G > kCmpBigTiles ? (const void*)k_compress<false, true> : (const void*)k_compress<false>);
-            err = cudaLaunchCooperativeKernel(fn, dim3((unsigned)launch_grid), dim3(kCmpThreads), kargs, sizeof(CmpSmem), st);
+            if (launch_overlapped((const void*)k_scan, (unsigned)g1, kScanThreads, sizeof(ScanShared), kargs, st) != cudaSuccess ||
+                launch_overlapped((const void*)k_encode, (unsigned)g2, kEncThreads, sizeof(EncShared), kargs, st) != cudaSuccess ||
+                launch_overlapped((const void*)k_place, (unsigned)g3, kEncThreads, sizeof(PlaceShared), kargs, st) != cudaSuccess) {
+                cudaGetLastError();
+                return FASTSGD_E_CUDA;
+            }
         }
-        if (err != cudaSuccess) { cudaGetLastError(); return FASTSGD_E_CUDA; }
-        g_launches.fetch_add(1, std::memory_order_relaxed);
+        g_launches.fetch_add(3, std::memory_order_relaxed);
     }
     return FASTSGD_OK;
 }
@@ -630,8 +634,8 @@ int decode_launches(const void* const* streams_in, const uint64_t* bytes, uint32
             da.bytes[i] = bytes[first + i];
         }
         da.n = n; da.dense = dense_out;
-        da.status = &view(g_state.ws, n).ctl->decode_status;
-        da.q_ctl = view(g_state.ws, n).ctl->dq;
+        da.status = &control_of(g_state.ws)->decode_status;
+        da.q_ctl = control_of(g_state.ws)->dq;
         da.q_list = reinterpret_cast<unsigned int*>(static_cast<unsigned char*>(g_state.ws) + kQueueOffset);
         da.base = params->base; da.G = (uint32_t)G; da.tau = params->tau; da.l = params->flag_bits;
         da.group_log2 = params->group_log2;
@@ -929,17 +933,12 @@ extern "C" int fastsgd_abs_sum_noalloc(const float* grad, uint64_t n, double* su
     if (cudaMemsetAsync(d->scratch, 0, sizeof(fsg::Control), st) != cudaSuccess) return FASTSGD_E_CUDA;
     fsg::SumArgs sa;
     sa.grad = grad; sa.n = n; sa.chunks = (uint32_t)((n + fsg::kChunk - 1) >> fsg::kChunkLog2);
-    sa.groups = 0u; sa.tau = 0u;
     sa.ctl = reinterpret_cast<fsg::Control*>(d->scratch);
-    sa.thr = reinterpret_cast<float*>(d->scratch + fsg::kThrOffset);
     sa.partials = reinterpret_cast<double*>(d->scratch + kNoAllocCtlBytes);
-    sa.desc = nullptr;
     sa.sum_out = sum_out;
-    fsg::PowTable pw;
-    for (int k = 0; k <= fsg::kMaxTau; ++k) pw.P[k] = 1.0;
     unsigned grid = (unsigned)d->grid_cap;
     if (grid > sa.chunks) grid = sa.chunks;
-    fsg::k_abs_sum<<<grid, fsg::kSumThreads, 0, st>>>(sa, pw);
+    fsg::k_abs_sum<<<grid, fsg::kSumThreads, 0, st>>>(sa);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? FASTSGD_OK : FASTSGD_E_CUDA;
 }

@@ -33,7 +33,7 @@
 
 #include "common.cuh"
 #include "bits.cuh"
-#include "compress.cuh"     // mbarrier / bulk-copy primitives
+#include "prims.cuh"
 
 namespace fsg {
 

@@ -1,31 +1,69 @@
 // The encoder for dense gradients: Algorithm 1 and, per group of 2^14 entries (a tile), Algorithm 2, for up to eight
 // gradients of the same length.
 //
-// k_resident: gradients that fit the GPU's shared memory, a tile per block (up to two blocks per SM).  Every entry is read
-// from memory once; the blocks exchange their tiles' sums and, later, sizes through tagged words of the workspace, everyone
-// reading what it needs; one launch.
+// The threshold B_tau = sum / b^tau is known only when every entry has been read, so the definition reads a gradient twice.  Here
+// it comes from memory once.
+//
+// k_resident: gradients that fit the GPU's shared memory, a tile per block (up to two blocks per SM).  The blocks exchange
+// their tiles' sums and, later, sizes through tagged words of the workspace, everyone reading what it needs; one launch.
+//
+// Larger ones take three launches that overlap at their edges:
+//   k_scan    streams the gradient.  A sample gives an estimate of the sum; every unit (a quarter of a tile) leaves its node of the
+//             fixed fp64 tree, its largest |v|, and the list (key, value) of the entries that reach the estimated threshold,
+//             lowered by a margin for the sampling error.
+//   k_encode  the sum from the units' nodes (same tree), the exact boundaries.  A tile whose estimate was not above the threshold
+//             has all its kept entries in its units' lists: filter, quantisation, delta keys, M, bit-packing; the blob
+//             replaces the lists.  Where it was too high (or missing) the tile itself is read again, unless its largest |v| is
+//             below the threshold.
+//   k_place   the tiles' places in the stream by exclusive sums, directory, header, and the blobs copied there.
+// The estimate steers only what is read again: which entries are kept and every bit of the stream follow from the exact sum.
 #pragma once
 
 #include "common.cuh"
 #include "sum.cuh"
 #include "bits.cuh"
-#include "compress.cuh"     // copy and ordering primitives, table search, flag rule
+#include "prims.cuh"
 
 namespace fsg {
 
 constexpr int      kEncThreads   = 512;
 constexpr int      kEncWarps     = kEncThreads / 32;
+constexpr uint32_t kTile         = 1u << kGroupLog2;           // entries per tile = per group
 constexpr uint32_t kSlab         = kTile / kEncWarps;          // entries a warp takes at a time
 static_assert(kSlab == 1024u, "eight rows of 128 entries per slab");
 constexpr int      kEncMaxJobs   = 8;                          // gradients (simulated workers) one launch can take
 constexpr uint32_t kMaxResident  = 320;                        // tiles k_resident can take (its exchange words in the workspace)
 
-// Encoder state in the workspace's fixed part (the exchange words are told apart by their tags).
+constexpr uint32_t kUnit         = 4u * kSlab;                 // entries of a unit, the quarter of a tile: what a warp of k_scan leaves a list of
+constexpr uint32_t kSlotEntries  = 96;                         // candidates a unit may have in its own slot of the workspace; longer lists go on in the pool
+constexpr uint32_t kUnitSlotBytes = kSlotEntries * 6u;
+constexpr uint32_t kSlotBytes    = 4u * kUnitSlotBytes;        // of a tile
+constexpr uint32_t kSlotWords    = kSlotBytes / 4u;
+constexpr uint32_t kListMost     = 2048;                       // units that promise more candidates are not listed (a list costs 6 bytes an entry, reading again 4)
+constexpr uint32_t kNoPlace      = 0xFFFFFFFFu;                // no room in the pool
+constexpr uint32_t kSampleBlocks = 32;                         // blocks that sample one gradient, four entries at 768 places each
+constexpr uint32_t kSamplePolls  = 64;                         // looks (0.7 us each) a block takes for another block's sample
+constexpr uint32_t kTicketGroups = 8;
+constexpr uint32_t kChunkUnits   = 512;                        // units under one node of the upper part of the sum tree
+constexpr uint32_t kMaxChunks    = 1552;                       // such nodes in a launch
+constexpr uint32_t kMaxSegments  = 1600;                       // segments of tiles (64 or more) whose sizes k_place scans
+constexpr uint32_t kWarpListMax  = 4u * kSlotEntries, kQuadListMax = 4096;      // candidates of a tile that one warp (all in slots), four warps take
+
+// Encoder state in the workspace's fixed part (zero between launches, except S and the tables; k_resident's exchange words are told
+// apart by their tags).
 struct EncState {
     alignas(16) unsigned long long res_node[2 * kMaxResident]; // k_resident: a tile's node, tag
     unsigned long long res_size[kMaxResident];                 // tag << 32 | kept entries << 16 | words
+    unsigned long long sample[kEncMaxJobs][kSampleBlocks];     // a block's sum and sum of squares (two floats, the latter not 0); 0: not there yet
+    uint32_t ticket[kTicketGroups][32];                        // k_scan: units handed out beyond each warp's first
+    double   S[kEncMaxJobs];
+    double   pw[132], inv[132];                                // b^k, 1 / b^k
+    unsigned long long pool_used;                              // bytes of the pool in use
+    uint32_t noblob;                                           // tiles k_place has to pack
 };
 static_assert(kEncStateOffset + sizeof(EncState) <= kQueueOffset, "fits before the decoder's queue");
+
+struct alignas(16) UnitInfo { uint32_t count, piece, room; float sthr; };      // list: candidates, piece of the pool (16-byte units) and its entries, what it was made with (+inf: no list)
 
 struct EncArgs {
     const float*        grad[kEncMaxJobs];
@@ -34,28 +72,38 @@ struct EncArgs {
     uint64_t            n;
     Control*            ctl;
     EncState*           st;
+    double*             partials;        // [J][4 G] units' nodes
+    unsigned long long* chunk;           // [J][chunks] pairs: node of 512 units, 1 when it is there
+    float*              umax;            // [J][4 G] largest |v|
+    UnitInfo*           info;            // [J][4 G]
+    unsigned long long* desc;            // [J][G] words << 32 | M << 24 | count
+    uint32_t*           blob;            // [J][G] the packed blob's place in the scratch (16-byte units)
+    unsigned long long* seg;             // [J][segments] kept entries << 32 | words of the segment's tiles
+    unsigned char*      scratch;         // [J G] slots, then the pool
+    uint64_t            pool_begin, pool_bytes;
     double              base;
+    double              inv_ptau;        // 1 / b^tau (steers the estimate only)
     uint32_t            J, G;
+    uint32_t            chunks;          // of a gradient
+    uint32_t            seg_log2, segments;
+    uint32_t            scan_blocks, samplers;      // blocks of k_scan; blocks that sample each gradient
     uint32_t            tau, l;
     uint32_t            wait_limit, try_limit;      // polls before a wait on another block, tries before a wait on a bulk copy gives up
 };
 
-// a pair of words that travels as one
-__device__ __forceinline__ void ld_relaxed_pair(const unsigned long long* p, unsigned long long& lo, unsigned long long& hi) {
-    asm volatile("{\n .reg .b128 q;\n ld.relaxed.gpu.global.b128 q, [%2];\n mov.b128 {%0, %1}, q;\n}" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned long long tile_desc(uint32_t count, uint32_t M, uint32_t words) {
+    return ((unsigned long long)words << 32) | (M << 24) | count;
 }
-__device__ __forceinline__ void st_relaxed_pair(unsigned long long* p, unsigned long long lo, unsigned long long hi) {
-    asm volatile("{\n .reg .b128 q;\n mov.b128 q, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], q;\n}" ::"l"(p), "l"(lo), "l"(hi) : "memory");
+__device__ __forceinline__ UnitInfo load_info(const UnitInfo* p) {
+    const uint4 q = __ldcg(reinterpret_cast<const uint4*>(p));
+    UnitInfo in;
+    in.count = q.x; in.piece = q.y; in.room = q.z; in.sthr = __uint_as_float(q.w);
+    return in;
 }
-
-// log2 S and 1 / log2 b only steer the table search (its result does not depend on them): single precision, and the exponent of
-// S taken from its bits so that sums beyond the fp32 range still give a finite estimate.  hints: thr + 130.
-__device__ __forceinline__ void table_hints(double S, double base, float* hints) {
-    const unsigned long long sb = (unsigned long long)__double_as_longlong(S);
-    const int ex = (int)((sb >> 52) & 0x7FFull) - 1023;
-    const float mant = __uint_as_float(0x3F800000u | (uint32_t)((sb >> 29) & 0x7FFFFFull));      // [1, 2)
-    hints[0] = (float)ex + __log2f(mant);
-    hints[1] = 1.0f / __log2f((float)base);
+// a piece of the pool (16-byte units), or kNoPlace
+__device__ __forceinline__ uint32_t pool_take(const EncArgs& a, uint32_t bytes) {
+    const unsigned long long b = (bytes + 15u) & ~15u, at = atomicAdd(&a.st->pool_used, b);
+    return at + b <= a.pool_bytes ? (uint32_t)((a.pool_begin + at) >> 4) : kNoPlace;
 }
 
 // RU32(B_k) for one gradient: |v| >= B_k on an fp32 |v| equals |v| >= RU32(B_k); never below the smallest denormal, because an entry
@@ -188,6 +236,157 @@ __device__ __forceinline__ void enc_write_header(const EncArgs& a, uint32_t j, i
     outw[12] = (uint32_t)bb;            outw[13] = (uint32_t)(bb >> 32);
     outw[14] = a.l | ((uint32_t)kGroupLog2 << 8);
     outw[15] = a.G;
+}
+
+// A unit's list of candidates: the first kSlotEntries in its slot, the others in a piece of the pool.
+struct List {
+    const float *v1, *v2; const uint16_t *k1, *k2;
+    // batch b of 32: the slot holds three
+    __device__ __forceinline__ const float* values(uint32_t b) const { return b < kSlotEntries / 32u ? v1 + 32u * b : v2 + (32u * b - kSlotEntries); }
+    __device__ __forceinline__ const uint16_t* keys(uint32_t b) const { return b < kSlotEntries / 32u ? k1 + 32u * b : k2 + (32u * b - kSlotEntries); }
+};
+__device__ __forceinline__ List list_of(const EncArgs& a, uint32_t u, const UnitInfo& in) {
+    List x;
+    x.v1 = reinterpret_cast<const float*>(a.scratch + (uint64_t)u * kUnitSlotBytes);
+    x.k1 = reinterpret_cast<const uint16_t*>(x.v1 + kSlotEntries);
+    x.v2 = reinterpret_cast<const float*>(a.scratch + 16ull * in.piece);
+    x.k2 = reinterpret_cast<const uint16_t*>(x.v2 + in.room);
+    return x;
+}
+
+// Kept keys, codes and M of a tile from its units' lists, by four or sixteen warps: warp w takes its share of unit w / (W / 4); returns the
+// number of kept entries.
+template <int W>
+__device__ __forceinline__ uint32_t team_list(const EncArgs& a, uint32_t t, const float* thr, uint16_t* keys, uint32_t* blob, uint32_t& M,
+                                              TeamScratch& s, int w, int lane, int id) {
+    const float thr_e = thr[a.tau];
+    const uint32_t u = 4u * t + (uint32_t)w / (W / 4), part = (uint32_t)w % (W / 4);
+    const UnitInfo in = load_info(a.info + u);
+    const List x = list_of(a, u, in);
+    const uint32_t cnt = __ldcg(a.umax + u) >= thr_e ? in.count : 0u;
+    const uint32_t nb = (cnt + 31u) >> 5, b0 = nb * part / (W / 4), b1 = nb * (part + 1u) / (W / 4);
+    // how many are kept
+    uint32_t n = 0u;
+    for (uint32_t b = b0; b < b1; b += 4u) {
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = b + i < b1 && 32u * (b + i) + (uint32_t)lane < cnt ? __ldcg(x.values(b + i) + lane) : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) n += (uint32_t)__popc(__ballot_sync(kFullMask, fabsf(v[i]) >= thr_e));
+    }
+    if (lane == 0) s.cnt[w] = n;
+    team_sync<W>(id);
+    const uint32_t c = lane < W ? s.cnt[lane] : 0u, ci = warp_incl_scan(c, lane);
+    uint32_t rank = __shfl_sync(kFullMask, ci - c, w);
+    const uint32_t count = __shfl_sync(kFullMask, ci, 31);
+    uint32_t maxd = 0u, prev = 0u, first = 0u;
+    bool none = true;
+    auto value = [&](uint32_t b) -> float { return b < b1 && 32u * b + (uint32_t)lane < cnt ? __ldcg(x.values(b) + lane) : 0.0f; };
+    auto key = [&](uint32_t b) -> uint32_t { return b < b1 && 32u * b + (uint32_t)lane < cnt ? __ldcg(x.keys(b) + lane) : 0u; };
+    float v0 = value(b0), v1 = value(b0 + 1u);
+    uint32_t k0 = key(b0), k1 = key(b0 + 1u);
+    for (uint32_t b = b0; b < b1; ++b) {
+        const float v2 = value(b + 2u);
+        const uint32_t k2 = key(b + 2u);
+        const bool kept = fabsf(v0) >= thr_e;
+        const uint32_t km = __ballot_sync(kFullMask, kept);
+        if (km) {
+            const uint32_t lower = km & ((1u << lane) - 1u);
+            const uint32_t pk = __shfl_sync(kFullMask, k0, lower ? 31 - __clz((int)lower) : 0);
+            if (none) { prev = first = __shfl_sync(kFullMask, k0, __ffs((int)km) - 1); none = false; }      // (the delta before the share's first key: below)
+            if (kept) {
+                const uint32_t q = rank + (uint32_t)__popc(lower);
+                maxd = max(maxd, k0 - (lower ? pk : prev));
+                keys[q] = (uint16_t)k0;
+                put_code(blob, q, code_byte_of(thr, a.tau, v0));
+            }
+            prev = __shfl_sync(kFullMask, k0, 31 - __clz((int)km));
+            rank += (uint32_t)__popc(km);
+        }
+        v0 = v1; k0 = k1; v1 = v2; k1 = k2;
+    }
+    // the largest delta: within the shares, and from one share's last key to the next one's first (keys ascend)
+    maxd = __reduce_max_sync(kFullMask, maxd);
+    if (lane == 0) { s.maxd[w] = maxd; s.first[w] = first; s.last[w] = none ? 0u : prev; }
+    team_sync<W>(id);
+    uint32_t last = lane < W ? s.last[lane] : 0u;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) { const uint32_t y = __shfl_up_sync(kFullMask, last, o); if (lane >= o) last = max(last, y); }
+    uint32_t before = __shfl_up_sync(kFullMask, last, 1);
+    if (lane == 0) before = 0u;
+    maxd = 0u;
+    if (lane < W) maxd = c ? max(s.maxd[lane], s.first[lane] - before) : 0u;
+    maxd = __reduce_max_sync(kFullMask, maxd);
+    M = maxd ? 32u - (uint32_t)__clz((int)maxd) : 1u;
+    return count;
+}
+
+// The same by one warp, all candidates (off[q]: those of the units before unit q) in the units' slots; maxd instead of M.
+__device__ __forceinline__ uint32_t warp_list(const EncArgs& a, uint32_t t, const uint32_t (&off)[5], const float* thr, uint16_t* keys, uint32_t* blob,
+                                              uint32_t& maxd, int lane) {
+    const float thr_e = thr[a.tau];
+    const unsigned char* slots = a.scratch + (uint64_t)t * kSlotBytes;
+    auto load = [&](uint32_t e, float& v, uint32_t& k) {
+        v = 0.0f; k = 0u;
+        if (e >= off[4]) return;
+        const uint32_t q = (e >= off[1] ? 1u : 0u) + (e >= off[2] ? 1u : 0u) + (e >= off[3] ? 1u : 0u);
+        const uint32_t i = e - (q == 0u ? 0u : q == 1u ? off[1] : q == 2u ? off[2] : off[3]);
+        const unsigned char* slot = slots + q * kUnitSlotBytes;
+        v = __ldcg(reinterpret_cast<const float*>(slot) + i);
+        k = __ldcg(reinterpret_cast<const uint16_t*>(slot + 4u * kSlotEntries) + i);
+    };
+    uint32_t rank = 0u, prev = 0u, k0, k1, k2; float v0, v1, v2;
+    maxd = 0u;
+    load((uint32_t)lane, v0, k0);
+    load(32u + (uint32_t)lane, v1, k1);
+    for (uint32_t e = 0; e < off[4]; e += 32u) {
+        load(e + 64u + (uint32_t)lane, v2, k2);
+        const bool kept = fabsf(v0) >= thr_e;
+        const uint32_t km = __ballot_sync(kFullMask, kept), lower = km & ((1u << lane) - 1u);
+        const uint32_t pk = __shfl_sync(kFullMask, k0, lower ? 31 - __clz((int)lower) : 0);
+        if (kept) {
+            const uint32_t q = rank + (uint32_t)__popc(lower);
+            maxd = max(maxd, k0 - (lower ? pk : prev));
+            keys[q] = (uint16_t)k0;
+            put_code(blob, q, code_byte_of(thr, a.tau, v0));
+        }
+        if (km) prev = __shfl_sync(kFullMask, k0, 31 - __clz((int)km));
+        rank += (uint32_t)__popc(km);
+        v0 = v1; k0 = k1; v1 = v2; k1 = k2;
+    }
+    return rank;
+}
+
+// The same from the tile itself, by the whole block: the kept keys of warp w's slab, then codes and deltas.
+__device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uint32_t tile, const float* thr, uint16_t* keys, uint32_t* blob, uint32_t& maxd,
+                                               TeamScratch& s, int tid, int lane, int warp) {
+    const float* g = a.grad[j] + ((uint64_t)tile << kGroupLog2);
+    const uint64_t left = a.n - ((uint64_t)tile << kGroupLog2);
+    const float thr_e = thr[a.tau];
+    // (32 loads of consecutive entries: row i of the slab's 32 rows of 32)
+    uint32_t mine = 0u, mask = 0u;
+#pragma unroll 8
+    for (int i = 0; i < 32; ++i) {
+        const uint32_t e = (uint32_t)warp * kSlab + 32u * (uint32_t)i + (uint32_t)lane;
+        const uint32_t b = __ballot_sync(kFullMask, e < left && fabsf(__ldg(g + (e < left ? e : 0u))) >= thr_e);
+        if (lane == i) mask = b;                               // lane i: row i
+        mine += (uint32_t)__popc(b);
+    }
+    if (lane == 0) s.cnt[warp] = mine;
+    __syncthreads();
+    const uint32_t c = lane < kEncWarps ? s.cnt[lane] : 0u, ci = warp_incl_scan(c, lane);
+    const uint32_t count = __shfl_sync(kFullMask, ci, 31);
+    const uint32_t own = (uint32_t)__popc(mask), incl = warp_incl_scan(own, lane);
+    uint32_t pos = __shfl_sync(kFullMask, ci - c, warp) + incl - own;
+    for (; mask != 0u; mask &= mask - 1u, ++pos) keys[pos] = (uint16_t)((uint32_t)warp * kSlab + 32u * (uint32_t)lane + (uint32_t)__ffs((int)mask) - 1u);
+    __syncthreads();
+    maxd = 0u;
+    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) {
+        const uint32_t k = keys[q];
+        maxd = max(maxd, k - (q ? (uint32_t)keys[q - 1u] : 0u));
+        put_code(blob, q, code_byte_of(thr, a.tau, __ldg(g + k)));
+    }
+    return count;
 }
 
 // ---- k_resident ----------------------------------------------------------------------------------
@@ -348,6 +547,596 @@ k_resident(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_co
             for (uint32_t i = 0; i < a.J; ++i) { a.ctl->bar_count[i] = 0u; a.ctl->ne_count[i] = 0u; }
             a.ctl->exit_count = 0u;
             st_release_u32(&a.ctl->bar_gen, gen);
+        }
+    }
+}
+
+// ---- k_scan ------------------------------------------------------------------------------------
+// A warp takes whole units, slab after slab, through a ring of its own in shared memory: bulk copies of two slabs (8 KB a warp, 192 KB
+// an SM) are in flight, no warp waits for another, and a unit's list is written in order as it goes.
+//
+// What bounds it is instructions and the latency of their chains: at 7 TB/s an SM has 160 cycles per slab.  A lane takes 32 consecutive
+// entries (slab_read), so that five levels of the tree need no shuffles and the kept mask is in index order.  Measured on 1 GiB: rows of
+// 128 entries across the warp 209 us; 32 warps that load into registers, slabs asked for in L2 ahead of time, 300 us; a fence and an
+// atomic per tile 207 us; the rings alone, without arithmetic, 159 us.
+constexpr int kScanThreads = 768;
+constexpr int kScanWarps   = kScanThreads / 32;
+constexpr int kRing        = 2;                                // slabs in flight per warp
+struct ScanShared {
+    alignas(128) float ring[kScanWarps][kRing][kSlab];
+    unsigned long long mbar[kScanWarps][kRing];
+    float samp[2][kScanWarps];
+    float est[kEncMaxJobs];
+};
+static_assert(sizeof(ScanShared) <= 232448, "shared memory of one block");
+
+__global__ void __launch_bounds__(kScanThreads, 1)
+k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_constant__ PowTable inv) {
+    extern __shared__ __align__(128) unsigned char scan_smem_raw[];
+    ScanShared& s = *reinterpret_cast<ScanShared*>(scan_smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t units = 4u * a.G, T = a.J * units;
+    allow_next_kernel();
+    if (lane == 0) {
+        for (int i = 0; i < kRing; ++i) mbar_init(&s.mbar[warp][i], 1u);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    wait_for_previous_kernels();
+    // unit k: unit k / J of gradient k % J (gradients interleaved).  Lane 0 starts the copy of one of its slabs; one that reaches beyond n
+    // is read by its consumer instead.
+    struct Where { const float* g; uint64_t left; };           // the unit's first entry, entries from there to the gradient's end
+    auto where = [&](uint32_t k) -> Where {
+        const uint32_t i = k / a.J;
+        const uint64_t e = (uint64_t)i * kUnit;
+        Where w;
+        w.g = a.grad[k - i * a.J] + e; w.left = e < a.n ? a.n - e : 0ull;
+        return w;
+    };
+    auto issue = [&](const Where& w, uint32_t slab, uint32_t slot) {
+        if (w.left >= (slab + 1u) * kSlab) {
+            mbar_expect_tx(&s.mbar[warp][slot], kSlab * 4u);
+            bulk_load(s.ring[warp][slot], w.g + slab * kSlab, kSlab * 4u, &s.mbar[warp][slot]);
+        } else {
+            mbar_arrive(&s.mbar[warp][slot]);
+        }
+    };
+    // ---- sample: blocks j, j + J, ... of the first J * samplers take gradient j; their loads go first, the rings are only half filled until
+    // the estimate is there (behind full rings the sample took 20 us)
+    const uint32_t sj = blockIdx.x % a.J, si = blockIdx.x / a.J;
+    const bool sampler = si < a.samplers;
+    float sx = 0.0f, sy = 0.0f;
+    if (sampler) {
+        const uint32_t places = (uint32_t)(a.n >> 2), count = a.samplers * (uint32_t)kScanThreads, step = places / count, at = si * (uint32_t)kScanThreads + (uint32_t)tid;
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (places) q = __ldg(reinterpret_cast<const float4*>(a.grad[sj]) + (step ? at * step + (step >> 1) : at % places));
+        sx = fabsf(q.x) + fabsf(q.y) + fabsf(q.z) + fabsf(q.w);
+        sy = sx * sx;
+    }
+    uint32_t cur = (uint32_t)warp * gridDim.x + blockIdx.x;
+    Where here = where(min(cur, T - 1u));
+    if (lane == 0 && cur < T) issue(here, 0u, 0u);
+    if (sampler) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { sx += __shfl_xor_sync(kFullMask, sx, o); sy += __shfl_xor_sync(kFullMask, sy, o); }
+        if (lane == 0) { s.samp[0][warp] = sx; s.samp[1][warp] = sy; }
+        __syncthreads();
+        if (warp == 0) {
+            sx = lane < kScanWarps ? s.samp[0][lane] : 0.0f; sy = lane < kScanWarps ? s.samp[1][lane] : 0.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) { sx += __shfl_xor_sync(kFullMask, sx, o); sy += __shfl_xor_sync(kFullMask, sy, o); }
+            if (lane == 0) st_relaxed_u64(&a.st->sample[sj][si], ((unsigned long long)__float_as_uint(sx) << 32) | max(__float_as_uint(sy), 1u));
+        }
+    }
+    if (warp == 0) {
+        // every block forms the estimates by itself: lane <-> sampling block.  Margin: 2 % and three standard errors of the mean of k samples
+        static_assert(kSampleBlocks == 32u, "a lane per sampling block");
+        for (uint32_t j = 0; j < a.J; ++j) {
+            unsigned long long v = 1ull;
+            if ((uint32_t)lane < a.samplers)
+                for (uint32_t p = 0; p < kSamplePolls; ++p) if ((v = ld_relaxed_u64(&a.st->sample[j][lane])) != 0ull) break;
+            const bool all = __all_sync(kFullMask, v != 0ull);
+            float x = __uint_as_float((uint32_t)(v >> 32)), y = __uint_as_float((uint32_t)v);
+            if ((uint32_t)lane >= a.samplers) x = y = 0.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) { x += __shfl_xor_sync(kFullMask, x, o); y += __shfl_xor_sync(kFullMask, y, o); }
+            const float k = (float)(a.samplers * (uint32_t)kScanThreads), mean = x / k, var = fmaxf(y / k - mean * mean, 0.0f), margin = 0.02f + 3.0f * sqrtf(var / k) / mean;
+            const float e = (float)((double)(mean * (1.0f - margin)) * (double)a.n * 0.25 * a.inv_ptau);
+            if (lane == 0) s.est[j] = all && margin < 0.75f && e > 0.0f ? e : -1.0f;
+        }
+    } else {
+        // (what k_encode adds to, exchanges and reads)
+        for (uint32_t i = blockIdx.x * (uint32_t)(kScanThreads - 32) + (uint32_t)(tid - 32); i < a.J * max(a.segments, 2u * a.chunks); i += gridDim.x * (uint32_t)(kScanThreads - 32)) {
+            if (i < a.J * a.segments) a.seg[i] = 0ull;
+            if (i < 2u * a.J * a.chunks) a.chunk[i] = 0ull;
+        }
+        if (blockIdx.x == 0) {
+            const int x = tid - 32;
+            if (x < kEncMaxJobs) a.ctl->ne_count[x] = 0u;
+            if (x == 0) a.st->noblob = 0u;
+            if (x <= kMaxTau) { a.st->pw[x] = pw.P[x]; a.st->inv[x] = inv.P[x]; }
+        }
+    }
+    __syncthreads();
+    if (lane == 0 && cur < T)
+        for (uint32_t i = 1; i < (uint32_t)kRing; ++i) issue(here, i, i);
+
+    const uint32_t groups = min(kTicketGroups, gridDim.x), tg = blockIdx.x % groups;
+    uint32_t slot = 0u, parity = 0u;                           // bit i: the parity the next wait on slot i expects
+    bool failed = false;
+    while (cur < T && !failed) {
+        const uint32_t i = cur / a.J, j = cur - i * a.J, t = j * units + i;
+        uint32_t nxt = T, tk = 0u;
+        Where there = here;
+        // what follows, asked for now and needed when its first copies start.  (Eight counters, each for every eighth block: SMs differ
+        // by a quarter in the bandwidth they get, so that units cannot be shared out beforehand, and one counter for all gives 0.3
+        // tickets a nanosecond: 240 us for 65536 units.)
+        if (lane == 0) tk = atomicAdd(&a.st->ticket[tg][0], 1u);
+        const float est = s.est[j], thr = est > 0.0f ? est : __int_as_float(0x7f800000);
+        float* v1 = reinterpret_cast<float*>(a.scratch + (uint64_t)t * kUnitSlotBytes);
+        uint16_t* k1 = reinterpret_cast<uint16_t*>(v1 + kSlotEntries);
+        bool listing = true;
+        uint32_t n_list = 0u, piece = 0u, room = 0u;
+        float mx = 0.0f;
+        double mynode = 0.0;
+#pragma unroll 1
+        for (uint32_t slab = 0; slab < 4u; ++slab) {
+            if (!__all_sync(kFullMask, mbar_wait(&s.mbar[warp][slot], (parity >> slot) & 1u, a.try_limit))) { failed = true; break; }
+            parity ^= 1u << slot;
+            float* ring = s.ring[warp][slot];
+            const bool whole = here.left >= (slab + 1u) * kSlab;
+            if (!whole) {                                      // the gradient's last entries
+                for (uint32_t q = lane; q < kSlab; q += 32u) ring[q] = slab * kSlab + q < here.left ? __ldg(here.g + slab * kSlab + q) : 0.0f;
+                __syncwarp();
+            }
+            float4 v[8];
+            slab_read(ring, v, lane);
+            float f[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) f[r] = fmaxf(fmaxf(fabsf(v[r].x), fabsf(v[r].y)), fmaxf(fabsf(v[r].z), fabsf(v[r].w)));
+            const float fm = fmaxf(fmaxf(fmaxf(f[0], f[1]), fmaxf(f[2], f[3])), fmaxf(fmaxf(f[4], f[5]), fmaxf(f[6], f[7])));
+            mx = fmaxf(mx, fm);
+            if (__any_sync(kFullMask, fm >= thr) && listing) { // (uniform)
+                uint32_t m = slab_mask(v, thr, lane);
+                const uint32_t own = (uint32_t)__popc(m), incl = warp_incl_scan(own, lane), cnt = __shfl_sync(kFullMask, incl, 31);
+                if (n_list + cnt > kSlotEntries && room == 0u) {
+                    // a piece of the pool: what the unit so far promises, and a quarter more
+                    const uint32_t promise = (n_list + cnt) * 4u / (slab + 1u);
+                    room = min(kUnit, (promise * 5u / 4u + 63u) & ~31u);
+                    listing = promise <= kListMost;
+                    if (listing) {
+                        if (lane == 0) piece = pool_take(a, room * 6u);
+                        piece = __shfl_sync(kFullMask, piece, 0);
+                        listing = piece != kNoPlace;
+                    }
+                } else if (n_list + cnt > kSlotEntries + room) {
+                    listing = false;
+                }
+                if (listing) {
+                    float* v2 = reinterpret_cast<float*>(a.scratch + 16ull * piece) - kSlotEntries;
+                    uint16_t* k2 = reinterpret_cast<uint16_t*>(v2 + kSlotEntries + room) - kSlotEntries;
+                    const uint32_t key0 = (i & 3u) * kUnit + slab * kSlab + 32u * (uint32_t)lane;
+                    uint32_t pos = n_list + incl - own;
+                    for (; m != 0u; m &= m - 1u, ++pos) {
+                        const uint32_t b = (uint32_t)__ffs((int)m) - 1u;
+                        const bool in_slot = pos < kSlotEntries;
+                        (in_slot ? v1 : v2)[pos] = ring[32u * (uint32_t)lane + b];
+                        (in_slot ? k1 : k2)[pos] = (uint16_t)(key0 + b);
+                    }
+                    n_list += cnt;
+                }
+            }
+            __syncwarp();                                      // the slab has been read: its place takes the slab two further on
+            if (slab + (uint32_t)kRing == 4u) {
+                nxt = min(__shfl_sync(kFullMask, tk, 0), T) * groups + tg + gridDim.x * (uint32_t)kScanWarps;
+                there = where(min(nxt, T - 1u));
+            }
+            if (lane == 0) {
+                // (generic writes to the place only where the gradient ends: ordered before the copy that follows)
+                if (!whole) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                if (slab + (uint32_t)kRing < 4u) issue(here, slab + (uint32_t)kRing, slot);
+                else if (nxt < T) issue(there, slab + (uint32_t)kRing - 4u, slot);
+            }
+            slot = slot + 1u == (uint32_t)kRing ? 0u : slot + 1u;
+            const double u = slab_node(v);
+            if (lane == (int)slab) mynode = u;
+        }
+        if (failed) break;
+        const double node = warp_tree(mynode, 4);
+        const uint32_t um = __reduce_max_sync(kFullMask, __float_as_uint(mx));      // (non-negative floats order like their bits; a NaN shows in the sum)
+        if (lane == 0) {
+            a.partials[t] = node;
+            a.umax[t] = __uint_as_float(um);
+            *reinterpret_cast<uint4*>(a.info + t) = make_uint4(n_list, piece, room, __float_as_uint(listing ? thr : __int_as_float(0x7f800000)));
+        }
+        here = there;
+        cur = nxt;
+    }
+    if (failed && lane == 0) {                                 // (a copy never came: give up; the others' copies are waited for, bounded)
+        atomicExch(&a.ctl->error, (unsigned)kStTimeout);
+        for (int i = 0; i < kRing; ++i) mbar_wait(&s.mbar[warp][i], (parity >> i) & 1u, a.try_limit);
+    }
+    __syncthreads();
+    if (tid == 0) atomicAdd(&a.ctl->bar_count[0], 1u);         // (k_encode checks that all blocks were there)
+}
+
+// ---- k_encode ----------------------------------------------------------------------------------
+struct WorkArea {                                              // shared memory of one team: [16 warps], [4 quads] or [the block]
+    static constexpr uint32_t kWarpWords = (kWarpListMax * 27u + 31u) / 32u + 4u, kQuadWords = (kQuadListMax * 27u + 31u) / 32u + 4u,
+                              kBlockWords = (kTile * 27u + 31u) / 32u + 4u;
+    struct Warp { uint16_t key[kWarpListMax]; uint32_t blob[kWarpWords]; };
+    struct Quad { union { struct { uint16_t key[kQuadListMax]; uint32_t blob[kQuadWords]; }; Warp w[4]; }; };
+    struct Block { uint16_t key[kTile]; uint32_t blob[kBlockWords]; };
+    union { Quad q[kEncWarps / 4]; Block b; };
+};
+
+struct EncShared {
+    float    thr[kEncMaxJobs][132];
+    double   S[kEncMaxJobs];
+    uint32_t n_light, n_mid, n_heavy, next_light, next_mid, abort_flag, grab[4];
+    TeamScratch team[4];
+    uint16_t light[kEncThreads], mid[kEncThreads], heavy[kEncThreads];      // heavy: bit 15: the tile is read again
+    WorkArea area;
+};
+static_assert(2 * (sizeof(EncShared) + 1024) <= 233472, "two blocks per SM (1 KiB per block is the system's)");
+
+// The gradients' sums from the units' nodes (same tree).  The first blocks form the nodes of 512 units, a warp each, and publish them;
+// every block takes them all and forms the rest of the tree for itself.  (Blocks start in order, and those that publish wait
+// for nobody before they have: a block waits only for blocks that are resident when it is.)
+__device__ __forceinline__ void gradient_sums(const EncArgs& a, EncShared& s, int tid, int lane, int warp) {
+    const uint32_t units = 4u * a.G, C = a.J * a.chunks, R = min(gridDim.x, 32u);
+    if (blockIdx.x < R) {
+        for (uint32_t c = blockIdx.x + R * (uint32_t)warp; c < C; c += R * (uint32_t)kEncWarps) {
+            const uint32_t j = c / a.chunks, p = c - j * a.chunks;
+            double x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const uint32_t e = kChunkUnits * p + 32u * (uint32_t)i + (uint32_t)lane;
+                x[i] = e < units ? __ldcg(a.partials + (uint64_t)j * units + e) : 0.0;
+            }
+            const double node = warp_rows16_tree(x, lane);
+            if (lane == 0) st_relaxed_pair(a.chunk + 2u * c, (unsigned long long)__double_as_longlong(node), 1ull);
+        }
+    }
+    double* nodes = reinterpret_cast<double*>(&s.area);
+    static_assert(sizeof(s.area) >= kMaxChunks * sizeof(double), "the nodes fit the work area");
+    for (uint32_t c = (uint32_t)tid; c < C; c += kEncThreads) {
+        unsigned long long lo, hi;
+        uint32_t spin = 0;
+        for (;;) {
+            ld_relaxed_pair(a.chunk + 2u * c, lo, hi);
+            if (hi != 0ull) break;
+            if (++spin > a.wait_limit) { s.abort_flag = 1u; break; }
+            if (spin > 16u) __nanosleep(32);
+        }
+        nodes[c] = __longlong_as_double((long long)lo);
+    }
+    __syncthreads();
+    if ((uint32_t)warp < a.J) {
+        const double* p = nodes + (uint32_t)warp * a.chunks;
+        double S = 0.0;
+        for (uint32_t h = 0; h < (a.chunks > 512u ? 2u : 1u); ++h) {      // (at most 1024 nodes for n < 2^31)
+            double x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) { const uint32_t e = 512u * h + 32u * (uint32_t)i + (uint32_t)lane; x[i] = e < a.chunks ? p[e] : 0.0; }
+            const double y = warp_rows16_tree(x, lane);
+            S = h ? __dadd_rn(S, y) : y;
+        }
+        if (lane == 0) { s.S[warp] = S; if (blockIdx.x == 0) a.st->S[warp] = S; }
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kEncThreads, 2)
+k_encode(const EncArgs a) {
+    extern __shared__ __align__(128) unsigned char enc_smem_raw[];
+    EncShared& s = *reinterpret_cast<EncShared*>(enc_smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t T = a.J * a.G, B = gridDim.x;
+    if (tid == 0) s.abort_flag = 0u;
+    allow_next_kernel();
+    wait_for_previous_kernels();
+    __syncthreads();
+    // ---- the first batch's tiles, requested before the sums are known
+    const uint32_t owned = blockIdx.x < T ? (T - blockIdx.x + B - 1u) / B : 0u;
+    float4 um; UnitInfo in[4];
+    auto load_tile = [&](uint32_t i) {
+        if (i < owned) {
+            const uint32_t t = blockIdx.x + i * B;
+            um = __ldcg(reinterpret_cast<const float4*>(a.umax) + t);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) in[q] = load_info(a.info + 4ull * t + q);
+        }
+    };
+    load_tile((uint32_t)tid);
+    if (tid == 0) {                                            // all blocks of k_scan have finished (they have: the launch before this one)
+        uint32_t spin = 0;
+        while (ld_acquire_u32(&a.ctl->bar_count[0]) != a.scan_blocks) if (++spin > a.wait_limit) { s.abort_flag = 1u; break; }
+    }
+    if (tid == kEncThreads - 1 && ld_acquire_u32(&a.ctl->error) != 0u) s.abort_flag = 1u;
+    gradient_sums(a, s, tid, lane, warp);
+    if (s.abort_flag) {                                        // (the same in every thread; every stream of the launch reports it)
+        if (tid == 0) atomicExch(&a.ctl->error, (unsigned)kStTimeout);
+        return;
+    }
+    for (uint32_t i = (uint32_t)tid; i < a.J * 132u; i += kEncThreads) {
+        const uint32_t j = i / 132u, k = i - j * 132u;
+        if (k <= a.tau) s.thr[j][k] = boundary(s.S[j], __ldcg(a.st->pw + k), __ldcg(a.st->inv + k));
+        if (k == 131u) table_hints(s.S[j], a.base, &s.thr[j][130]);
+    }
+
+    const uint32_t warp_max = owned >= (uint32_t)kEncWarps ? kWarpListMax : 64u;      // (few tiles per block: a list is better shared out)
+    for (uint32_t first = 0; first < owned; first += kEncThreads) {
+        // ---- which of the block's tiles hold anything, and where it is
+        if (tid == 0) { s.n_light = 0u; s.n_mid = 0u; s.n_heavy = 0u; s.next_light = 0u; s.next_mid = 0u; }
+        if (first) load_tile(first + (uint32_t)tid);
+        __syncthreads();
+        if (first + (uint32_t)tid < owned) {
+            const uint32_t t = blockIdx.x + (first + (uint32_t)tid) * B, j = t / a.G;
+            const float thr_e = s.thr[j][a.tau];
+            uint32_t cnt = 0u;
+            bool again = false, any = false, slots = true;     // (a unit that does not reach the threshold counts for nothing)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float x = q == 0 ? um.x : q == 1 ? um.y : q == 2 ? um.z : um.w;
+                if (x >= thr_e) { any = true; cnt += in[q].count; again = again || !(in[q].sthr <= thr_e); slots = slots && in[q].count <= kSlotEntries; }
+            }
+            if (!(thr_e < __int_as_float(0x7f800000)) || !any) a.desc[t] = 0ull;      // nothing is kept here
+            else if (again) {
+                s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)(tid | 0x8000);
+                atomicAdd(&a.ctl->ne_count[j], 1u);
+            } else if (slots && cnt <= warp_max) s.light[atomicAdd(&s.n_light, 1u)] = (uint16_t)tid;
+            else if (cnt <= kQuadListMax) s.mid[atomicAdd(&s.n_mid, 1u)] = (uint16_t)tid;
+            else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
+        }
+        __syncthreads();
+        // (the first lane of a team records the tile's sizes)
+        auto record = [&](uint32_t t, uint32_t j, uint32_t count, uint32_t M, uint32_t words, uint32_t place) {
+            a.desc[t] = count ? tile_desc(count, M, words) : 0ull;
+            a.blob[t] = place;
+            if (count) atomicAdd(&a.seg[j * a.segments + ((t - j * a.G) >> a.seg_log2)], ((unsigned long long)count << 32) | words);
+        };
+        // (the slots of the tile's units, where the lists were, or a piece of the pool)
+        auto place_of = [&](uint32_t t, uint32_t words) -> uint32_t {
+            const uint32_t p = words <= kSlotWords ? t * (kSlotBytes / 16u) : pool_take(a, words * 4u);
+            if (p == kNoPlace) atomicAdd(&a.st->noblob, 1u);
+            return p;
+        };
+        // ---- by the whole block
+        for (uint32_t h = 0; h < s.n_heavy; ++h) {
+            const uint32_t t = blockIdx.x + (first + (s.heavy[h] & 0x7FFFu)) * B, j = t / a.G, tile = t - j * a.G;
+            uint32_t maxd, M = 0u, words = 0u, place = 0u, count;
+            if ((s.heavy[h] & 0x8000u) != 0u) {
+                count = block_tile(a, j, tile, s.thr[j], s.area.b.key, s.area.b.blob, maxd, s.team[0], tid, lane, warp);
+                M = team_width<kEncWarps>(maxd, s.team[0], warp, lane, 0);
+            } else {
+                count = team_list<kEncWarps>(a, t, s.thr[j], s.area.b.key, s.area.b.blob, M, s.team[0], warp, lane, 0);
+            }
+            if (count) {
+                team_pack<kEncWarps>(a.l, s.area.b.key, s.area.b.blob, count, M, s.team[0], warp, lane, 0, [&](uint32_t w_) {
+                    words = w_;
+                    if (tid == 0) s.team[0].word = place_of(t, w_);
+                });
+                place = s.team[0].word;
+                if (place != kNoPlace) {
+                    uint32_t* dst = reinterpret_cast<uint32_t*>(a.scratch + 16ull * place);
+                    for (uint32_t i = (uint32_t)tid; i < words; i += kEncThreads) dst[i] = bswap32(s.area.b.blob[i]);
+                }
+            }
+            if (tid == 0) record(t, j, count, M, words, place);
+            __syncthreads();
+        }
+        // ---- by four warps
+        const int quad = warp >> 2, qw = warp & 3;
+        if (qw == 0 && lane == 0) s.grab[quad] = atomicAdd(&s.next_mid, 1u);
+        team_sync<4>(quad);
+        for (;;) {
+            const uint32_t x = s.grab[quad];
+            if (x >= s.n_mid) break;
+            const uint32_t t = blockIdx.x + (first + s.mid[x]) * B, j = t / a.G;
+            WorkArea::Quad& ar = s.area.q[quad];
+            uint32_t M, words = 0u, place = 0u;
+            const uint32_t count = team_list<4>(a, t, s.thr[j], ar.key, ar.blob, M, s.team[quad], qw, lane, quad);
+            if (qw == 0 && lane == 0) s.grab[quad] = atomicAdd(&s.next_mid, 1u);
+            if (count) {
+                team_pack<4>(a.l, ar.key, ar.blob, count, M, s.team[quad], qw, lane, quad, [&](uint32_t w_) {
+                    words = w_;
+                    if (qw == 0 && lane == 0) s.team[quad].word = place_of(t, w_);
+                });
+                place = s.team[quad].word;
+                if (place != kNoPlace) {
+                    uint32_t* dst = reinterpret_cast<uint32_t*>(a.scratch + 16ull * place);
+                    for (uint32_t i = (uint32_t)(qw * 32 + lane); i < words; i += 128u) dst[i] = bswap32(ar.blob[i]);
+                }
+            }
+            if (qw == 0 && lane == 0) record(t, j, count, M, words, place);
+            team_sync<4>(quad);
+        }
+        // ---- by single warps
+        for (;;) {
+            uint32_t x = 0u;
+            if (lane == 0) x = atomicAdd(&s.next_light, 1u);
+            x = __shfl_sync(kFullMask, x, 0);
+            if (x >= s.n_light) break;
+            const uint32_t t = blockIdx.x + (first + s.light[x]) * B, j = t / a.G;
+            const float thr_e = s.thr[j][a.tau];
+            uint32_t off[5];
+            {
+                uint32_t c = 0u;
+                if (lane < 4) c = __ldcg(a.umax + 4ull * t + lane) >= thr_e ? __ldcg(&a.info[4ull * t + lane].count) : 0u;
+                const uint32_t ci = warp_incl_scan(c, lane);
+                off[0] = 0u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) off[q + 1] = __shfl_sync(kFullMask, ci, q);
+            }
+            WorkArea::Warp& ar = s.area.q[quad].w[qw];
+            uint32_t maxd, M = 0u, words = 0u;
+            const uint32_t place = t * (kSlotBytes / 16u);      // (27 bits an entry at most: the blob fits the slots)
+            const uint32_t count = warp_list(a, t, off, s.thr[j], ar.key, ar.blob, maxd, lane);
+            if (count) {
+                M = team_width<1>(maxd, s.team[quad], 0, lane, 0);
+                team_pack<1>(a.l, ar.key, ar.blob, count, M, s.team[quad], 0, lane, 0, [&](uint32_t w_) { words = w_; });
+                uint32_t* dst = reinterpret_cast<uint32_t*>(a.scratch + 16ull * place);
+                for (uint32_t i = lane; i < words; i += 32u) dst[i] = bswap32(ar.blob[i]);
+            }
+            if (lane == 0) record(t, j, count, M, words, place);
+            __syncwarp();
+        }
+        __syncthreads();
+    }
+}
+
+// ---- k_place -----------------------------------------------------------------------------------
+constexpr uint32_t kRowTiles = 8;                              // tiles whose blobs a warp copies together: neighbours in the stream
+struct PlaceShared {
+    unsigned long long seg[kMaxSegments];                      // exclusive sums over the segments of each gradient (kept entries << 32 | words)
+    unsigned long long total[kEncMaxJobs];
+    unsigned long long scan64[kEncWarps];
+    float    thr[132];
+    TeamScratch team;
+    WorkArea::Block area;
+};
+static_assert(2 * (sizeof(PlaceShared) + 1024) <= 233472, "two blocks per SM (1 KiB per block is the system's)");
+
+// kept entries and words of the tiles before `tile` in the gradient; one warp
+__device__ __forceinline__ unsigned long long tile_prefix(const EncArgs& a, const unsigned long long* seg, uint32_t j, uint32_t tile, int lane) {
+    const uint32_t sg = tile >> a.seg_log2, t0 = sg << a.seg_log2;
+    unsigned long long x = 0ull;
+    for (uint32_t i = t0 + (uint32_t)lane; i < tile; i += 32u) {
+        const unsigned long long d = __ldcg(&a.desc[(uint64_t)j * a.G + i]);
+        x += ((d & 0xFFFFFFull) << 32) | (d >> 32);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+    return seg[j * a.segments + sg] + x;
+}
+
+__global__ void __launch_bounds__(kEncThreads, 2)
+k_place(const EncArgs a) {
+    extern __shared__ __align__(128) unsigned char place_smem_raw[];
+    PlaceShared& s = *reinterpret_cast<PlaceShared*>(place_smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t B = gridDim.x, fixed_words = (kHeaderBytes + 8u * a.G) >> 2;
+    allow_next_kernel();
+    wait_for_previous_kernels();
+    if (ld_acquire_u32(&a.ctl->error) != 0u) {                 // (the same answer in every block) some wait of the launch ran out
+        if (blockIdx.x == 0 && tid < (int)a.J) enc_write_header(a, (uint32_t)tid, kStTimeout, 0ull, 0ull, 0.0);
+        return;
+    }
+    // ---- exclusive sums over the segments (all gradients' in one scan, each gradient's start taken off afterwards)
+    const uint32_t segs = a.J * a.segments;
+    {
+        constexpr uint32_t kPer = (kMaxSegments + kEncThreads - 1u) / kEncThreads;
+        unsigned long long x[kPer], sum = 0ull;
+#pragma unroll
+        for (uint32_t i = 0; i < kPer; ++i) {
+            const uint32_t e = (uint32_t)tid * kPer + i;
+            x[i] = e < segs ? __ldcg(&a.seg[e]) : 0ull;
+            sum += x[i];
+        }
+        unsigned long long incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(kFullMask, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) s.scan64[warp] = incl;
+        __syncthreads();
+        unsigned long long w = lane < kEncWarps ? s.scan64[lane] : 0ull, wi = w;
+#pragma unroll
+        for (int o = 1; o < kEncWarps; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(kFullMask, wi, o);
+            if (lane >= o) wi += u;
+        }
+        unsigned long long before = incl - sum + __shfl_sync(kFullMask, wi - w, warp);
+#pragma unroll
+        for (uint32_t i = 0; i < kPer; ++i) {
+            const uint32_t e = (uint32_t)tid * kPer + i;
+            if (e < segs) s.seg[e] = before;
+            before += x[i];
+            if (e < segs && (e + 1u) % a.segments == 0u) s.total[e / a.segments] = before;
+        }
+        __syncthreads();
+        if (a.J > 1u) {
+            unsigned long long start[kPer];
+#pragma unroll
+            for (uint32_t i = 0; i < kPer; ++i) {
+                const uint32_t e = (uint32_t)tid * kPer + i;
+                start[i] = e < segs ? s.seg[e / a.segments * a.segments] : 0ull;
+            }
+            if (tid < (int)a.J) s.total[tid] -= s.seg[(uint32_t)tid * a.segments];
+            __syncthreads();
+#pragma unroll
+            for (uint32_t i = 0; i < kPer; ++i) {
+                const uint32_t e = (uint32_t)tid * kPer + i;
+                if (e < segs) s.seg[e] -= start[i];
+            }
+            __syncthreads();
+        }
+    }
+    // ---- headers; a gradient whose sum is not finite or whose stream does not fit has nothing else
+    auto total_bytes_of = [&](uint32_t j) -> uint64_t { return ((uint64_t)fixed_words + (uint32_t)s.total[j]) << 2; };
+    auto fits = [&](uint32_t j) -> bool { return total_bytes_of(j) <= a.out_bytes; };
+    const bool noblob = __ldcg(&a.st->noblob) != 0u;
+    if (blockIdx.x == 0 && tid < (int)a.J) {
+        const double S = __ldcg(&a.st->S[tid]);
+        enc_write_header(a, (uint32_t)tid, !isfinite(S) ? kStNonfinite : !fits((uint32_t)tid) ? kStCapacity : kStOk, s.total[tid] >> 32, total_bytes_of((uint32_t)tid), S);
+    }
+    static_assert(kTicketGroups == (uint32_t)kEncMaxJobs, "reset together");
+    if (blockIdx.x == 0 && tid < kEncMaxJobs) {                // at rest again
+        a.ctl->bar_count[tid] = 0u; a.st->ticket[tid][0] = 0u;
+        for (uint32_t i = 0; i < kSampleBlocks; ++i) a.st->sample[tid][i] = 0ull;
+        if (tid == 0) a.st->pool_used = 0ull;
+    }
+    // ---- rows of eight tiles: directory entries and blobs.  When the rows are fewer than the warps, several warps share a row's words.
+    const uint32_t rows = (a.G + kRowTiles - 1u) / kRowTiles, warps = B * (uint32_t)kEncWarps;
+    const uint32_t parts = max(1u, min(8u, warps / (a.J * rows)));
+    for (uint32_t x = blockIdx.x + B * (uint32_t)warp; x < a.J * rows * parts; x += warps) {
+        const uint32_t part = x % parts, y = x / parts, j = y / rows, t0 = (y - j * rows) * kRowTiles, tile = t0 + (uint32_t)lane;
+        if (!fits(j)) continue;
+        const bool mine = (uint32_t)lane < kRowTiles && tile < a.G;
+        const unsigned long long d = mine ? __ldcg(&a.desc[(uint64_t)j * a.G + tile]) : 0ull;
+        const uint32_t place = mine ? __ldcg(&a.blob[(uint64_t)j * a.G + tile]) : 0u;
+        const uint32_t before = fixed_words + (uint32_t)tile_prefix(a, s.seg, j, t0, lane);
+        const uint32_t w = (uint32_t)(d >> 32), wi = warp_incl_scan(w, lane), we = wi - w;
+        const uint32_t all = __shfl_sync(kFullMask, wi, 31);
+        if (mine && part == 0u) *reinterpret_cast<uint2*>(a.out[j] + kHeaderBytes + 8ull * tile) = make_uint2((uint32_t)d, before + we);
+        const uint32_t p0 = (uint32_t)((uint64_t)all * part / parts), p1 = (uint32_t)((uint64_t)all * (part + 1u) / parts);
+        uint32_t* dst = reinterpret_cast<uint32_t*>(a.out[j]) + before;
+        for (uint32_t i0 = p0; i0 < p1; i0 += 128u) {
+            uint32_t v[4], ok = 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + 32u * (uint32_t)u + (uint32_t)lane;
+                // which tile is word i of?  (the last one that starts at or before it)
+                uint32_t at = 0u;
+#pragma unroll
+                for (uint32_t o = kRowTiles / 2u; o > 0u; o >>= 1) { const uint32_t e = __shfl_sync(kFullMask, we, at + o); if (e <= i) at += o; }
+                const uint32_t e = __shfl_sync(kFullMask, we, at), pl = __shfl_sync(kFullMask, place, at);
+                v[u] = 0u;
+                if (i < p1 && pl != kNoPlace) { v[u] = __ldcg(reinterpret_cast<const uint32_t*>(a.scratch + 16ull * pl) + (i - e)); ok |= 1u << u; }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if ((ok >> u) & 1u) dst[i0 + 32u * (uint32_t)u + (uint32_t)lane] = v[u];
+        }
+    }
+    // ---- tiles for whose blobs there was no room: packed here (the pool holds a sixth of the entries; only where most of them are kept)
+    if (noblob) {
+        for (uint32_t t = blockIdx.x; t < a.J * a.G; t += B) {
+            const unsigned long long d = __ldcg(&a.desc[t]);
+            const uint32_t j = t / a.G, tile = t - j * a.G;
+            if (d == 0ull || __ldcg(&a.blob[t]) != kNoPlace || !fits(j)) continue;      // (uniform)
+            __syncthreads();
+            const double S = __ldcg(&a.st->S[j]);
+            for (uint32_t k = (uint32_t)tid; k <= a.tau; k += kEncThreads) s.thr[k] = boundary(S, __ldcg(a.st->pw + k), __ldcg(a.st->inv + k));
+            if (tid == kEncThreads - 1) table_hints(S, a.base, &s.thr[130]);
+            __syncthreads();
+            uint32_t maxd;
+            const uint32_t count = block_tile(a, j, tile, s.thr, s.area.key, s.area.blob, maxd, s.team, tid, lane, warp);
+            team_pack<kEncWarps>(a.l, s.area.key, s.area.blob, count, team_width<kEncWarps>(maxd, s.team, warp, lane, 0), s.team, warp, lane, 0, [](uint32_t) {});
+            uint32_t* dst = reinterpret_cast<uint32_t*>(a.out[j]) + fixed_words + (uint32_t)tile_prefix(a, s.seg, j, tile, lane);
+            for (uint32_t i = (uint32_t)tid; i < (uint32_t)(d >> 32); i += kEncThreads) dst[i] = bswap32(s.area.blob[i]);
+            __syncthreads();
         }
     }
 }

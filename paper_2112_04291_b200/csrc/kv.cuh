@@ -28,11 +28,11 @@
 #include "common.cuh"
 #include "sum.cuh"
 #include "bits.cuh"
-#include "compress.cuh"     // tree reduction of the partials, table search, flag rule, ordering primitives
+#include "prims.cuh"
 
 namespace fsg {
 
-constexpr int      kKvThreads    = kCmpThreads;      // the shared reduction of the partials is written for this block size
+constexpr int      kKvThreads    = kBlockThreads;    // the shared reduction of the partials is written for this block size
 constexpr int      kKvWarps      = kKvThreads / 32;
 constexpr uint32_t kKvStageWords = 256;               // blobs up to this many words are packed in shared memory
 constexpr uint32_t kKvUnit       = 128;               // leaves of the sum tree formed at a time (4 per lane)
@@ -383,7 +383,7 @@ k_compress_kv(const KvArgs a_in, const __grid_constant__ PowTable pw) {
                                 [&](uint64_t head_e, uint32_t c, uint32_t) { kv_sum_chunk(ws, a, head_e, c, lane); });
         // ---- grid barrier; the last block to arrive reduces the chunk nodes (same tree, same code as the dense encoder)
         if (kv_barrier_arrive(s, a.ctl, 0, tid)) {
-            const double S = a.chunks > kCmpBigTiles ? reduce_partials<true>(a.partials, a.chunks, s.s_tree, s.s_nodes, tid, lane, warp)
+            const double S = a.chunks > 8192u ? reduce_partials<true>(a.partials, a.chunks, s.s_tree, s.s_nodes, tid, lane, warp)
                                                      : reduce_partials<false>(a.partials, a.chunks, s.s_tree, s.s_nodes, tid, lane, warp);
             __syncthreads();
             for (uint32_t i = tid; i < a.chunks; i += kKvThreads) a.partials[i] = 0.0;     // at rest again
@@ -404,12 +404,7 @@ k_compress_kv(const KvArgs a_in, const __grid_constant__ PowTable pw) {
     const bool finite = isfinite(S);
     if (tid <= (int)a.tau)
         s.thr[tid] = (finite && S != 0.0) ? fmaxf(__double2float_ru(__ddiv_rn(S, pw.P[tid])), __int_as_float(1)) : __int_as_float(0x7f800000);
-    if (tid == 0) {                                       // (estimates that only steer the table search: see make_table)
-        const unsigned long long sb = (unsigned long long)__double_as_longlong(S);
-        const float mant = __uint_as_float(0x3F800000u | (uint32_t)((sb >> 29) & 0x7FFFFFull));
-        s.thr[130] = (float)((int)((sb >> 52) & 0x7FFull) - 1023) + __log2f(mant);
-        s.thr[131] = 1.0f / __log2f((float)a.base);
-    }
+    if (tid == 0) table_hints(S, a.base, &s.thr[130]);
     __syncthreads();
     const float thr_e = s.thr[a.tau];
     const bool aborted1 = s.abort_flag != 0u;

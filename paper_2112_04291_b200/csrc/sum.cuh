@@ -1,11 +1,11 @@
-// Step 1 of Algorithm 1: sum = sum_i |v_i|, and the boundary table that follows from it.
+// Step 1 of Algorithm 1: sum = sum_i |v_i|.
 //
 // The sum is defined on the balanced binary tree over index ranges aligned to powers of two
 // (leaf = |v_i| widened to fp64, zero beyond n), every node one IEEE fp64 addition.  Any tiling
 // by aligned power-of-two ranges reproduces that tree exactly, so the result does not depend
 // on the grid: a thread reduces 4 consecutive entries, a warp 8 rows of 128 entries (1024),
 // a block of 16 warps one chunk of 2^14, and the last block to finish reduces the per-chunk
-// partials in the same tree order and derives B_k = sum / b^k.
+// partials in the same tree order.
 #pragma once
 
 #include "common.cuh"
@@ -121,24 +121,17 @@ struct SumArgs {
     const float*        grad;
     uint64_t            n;
     uint32_t            chunks;      // ceil(n / 2^14)
-    uint32_t            groups;      // look-back descriptors to clear (0: none)
-    uint32_t            tau;
     Control*            ctl;
-    float*              thr;
     double*             partials;
-    unsigned long long* desc;
     double*             sum_out;     // optional copy of the sum
 };
 
 __global__ void __launch_bounds__(kSumThreads)
-k_abs_sum(const SumArgs a, const __grid_constant__ PowTable pw) {
+k_abs_sum(const SumArgs a) {
     __shared__ double s_warp[2][kSumThreads / 32];
     __shared__ double s_tree[kSumThreads / 32];
     __shared__ bool s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-    // the look-back state of the encode kernel that follows on the same stream
-    for (uint32_t i = blockIdx.x * kSumThreads + tid; i < a.groups; i += gridDim.x * kSumThreads) a.desc[i] = 0ull;
 
     // chunks are visited from the end of the array towards its start, so that the entries the
     // encode kernel reads first are the ones most recently brought into L2
@@ -220,18 +213,8 @@ k_abs_sum(const SumArgs a, const __grid_constant__ PowTable pw) {
     }
     __syncthreads();
     const double S = s_tree[0];
-    const bool finite = isfinite(S);
-    if (tid <= (int)a.tau) {
-        // B_k = S / b^k; the compare |v| >= B_k on an fp32 |v| equals |v| >= RU32(B_k)
-        // (never below the smallest denormal: an entry must also be non-zero to be kept)
-        double Bk = __ddiv_rn(S, pw.P[tid]);
-        a.thr[tid] = finite ? fmaxf(__double2float_ru(Bk), __int_as_float(1)) : __int_as_float(0x7f800000);
-    }
     if (tid == 0) {
         a.ctl->sum = S;
-        a.ctl->skip = !finite ? 2u : (S == 0.0 ? 1u : 0u);
-        a.ctl->ticket = 0u;
-        a.ctl->error = 0u;
         a.ctl->done = 0u;
         if (a.sum_out) *a.sum_out = S;
     }
