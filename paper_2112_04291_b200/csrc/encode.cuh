@@ -35,7 +35,7 @@ constexpr int      kEncMaxJobs   = 8;                          // gradients (sim
 constexpr uint32_t kMaxResident  = 320;                        // tiles k_resident can take (its exchange words in the workspace)
 
 constexpr uint32_t kUnit         = 4u * kSlab;                 // entries of a unit, the quarter of a tile: what a warp of k_scan leaves a list of
-constexpr uint32_t kSlotEntries  = 96;                         // candidates a unit may have in its own slot of the workspace; longer lists go on in the pool
+constexpr uint32_t kSlotEntries  = 96;                         // candidates a unit may have in its own slot of the workspace; longer lists go to the pool
 constexpr uint32_t kUnitSlotBytes = kSlotEntries * 6u;
 constexpr uint32_t kSlotBytes    = 4u * kUnitSlotBytes;        // of a tile
 constexpr uint32_t kSlotWords    = kSlotBytes / 4u;
@@ -47,7 +47,7 @@ constexpr uint32_t kTicketGroups = 8;
 constexpr uint32_t kChunkUnits   = 512;                        // units under one node of the upper part of the sum tree
 constexpr uint32_t kMaxChunks    = 1552;                       // such nodes in a launch
 constexpr uint32_t kMaxSegments  = 1600;                       // segments of tiles (64 or more) whose sizes k_place scans
-constexpr uint32_t kWarpListMax  = 4u * kSlotEntries, kQuadListMax = 4096;      // candidates of a tile that one warp (all in slots), four warps take
+constexpr uint32_t kWarpListMax  = 4u * kSlotEntries, kUnitListMax = 768;      // candidates of a tile that one warp (all in slots), of a unit that one warp of four take
 
 // Encoder state in the workspace's fixed part (zero between launches, except S and the tables; k_resident's exchange words are told
 // apart by their tags).
@@ -63,7 +63,7 @@ struct EncState {
 };
 static_assert(kEncStateOffset + sizeof(EncState) <= kQueueOffset, "fits before the decoder's queue");
 
-struct alignas(16) UnitInfo { uint32_t count, piece, room; float sthr; };      // list: candidates, piece of the pool (16-byte units) and its entries, what it was made with (+inf: no list)
+struct alignas(16) UnitInfo { uint32_t count, piece, room; float sthr; };      // list: candidates, piece of the pool (16-byte units), entries it has room for (kSlotEntries: it is in the slot), what it was made with (+inf: no list)
 
 struct EncArgs {
     const float*        grad[kEncMaxJobs];
@@ -147,7 +147,7 @@ __device__ __forceinline__ uint32_t slab_mask(const float4 (&v)[8], float thr, i
 // ---- teams: one, four or sixteen warps on one tile ------------------------------------------------------
 // The kept entries' keys stand in shared memory in index order, their code bytes already in the blob (big-endian valued words); flags
 // and deltas are packed behind the codes.
-struct TeamScratch { uint32_t cnt[kEncWarps], first[kEncWarps], last[kEncWarps], maxd[kEncWarps], bits[kEncWarps], word; };
+struct TeamScratch { uint32_t cnt[kEncWarps], maxd[kEncWarps], first[4], last[4], bits[kEncWarps], word; };
 
 template <int W> __device__ __forceinline__ void team_sync(int id) {
     if constexpr (W == 1) __syncwarp();
@@ -157,69 +157,141 @@ template <int W> __device__ __forceinline__ void team_sync(int id) {
 
 __device__ __forceinline__ void put_code(uint32_t* blob, uint32_t q, uint32_t code) { reinterpret_cast<uint8_t*>(blob)[q ^ 3u] = (uint8_t)code; }
 
-// M from the threads' largest deltas; a barrier of the team (keys and codes are complete behind it)
-template <int W>
-__device__ __forceinline__ uint32_t team_width(uint32_t maxd, TeamScratch& s, int w, int lane, int id) {
-    maxd = __reduce_max_sync(kFullMask, maxd);
-    if (W > 1 && lane == 0) s.maxd[w] = maxd;
-    team_sync<W>(id);
-    if (W > 1) maxd = __reduce_max_sync(kFullMask, lane < W ? s.maxd[lane] : 0u);
-    return maxd ? 32u - (uint32_t)__clz((int)maxd) : 1u;
+// Appends bit fields to a zeroed blob from any bit position on.  Words that lie wholly in the run are stored, the first and the last
+// are shared with neighbours.
+struct BitRun {
+    uint32_t *first, *at, cur, fill;
+    __device__ __forceinline__ BitRun(uint32_t* blob, uint32_t pos) : first(blob + (pos >> 5)), at(first), cur(0u), fill(pos & 31u) {}
+    // a value of `width` (0 to 32) bits; width 0: value 0
+    __device__ __forceinline__ void put(uint32_t value, uint32_t width) {
+        const uint32_t x = value << ((32u - width) & 31u), end = fill + width;
+        cur |= x >> fill;
+        if (end >= 32u) {
+            if (at == first) atomicOr(at, cur); else *at = cur;
+            ++at;
+            cur = __funnelshift_r(0u, x, fill);
+        }
+        fill = end & 31u;
+    }
+    __device__ __forceinline__ void close() { if (cur) atomicOr(at, cur); }
+};
+
+// A thread's run of consecutive entries, taken four at a time (keys ascend: two deltas to a register without a borrow from one to the
+// other); entries beyond the run's end have delta 0.
+struct KeyRun {
+    const uint16_t* keys;                                      // 8-byte aligned
+    int left;                                                  // entries not yet taken (0 or less: none)
+    uint32_t prev;                                             // the key before them
+    __device__ __forceinline__ uint2 next4() {
+        uint2 d = make_uint2(0u, 0u);
+        if (left > 0) {
+            uint2 k = *reinterpret_cast<const uint2*>(keys);
+            if (left < 4) {                                    // (the last run's last entries)
+                const uint32_t last = keys[left - 1];
+                if (left == 1) k.x = last * 0x10001u;
+                k.y = last * 0x10001u;
+            }
+            d.x = k.x - __byte_perm(prev, k.x, 0x5410);
+            d.y = k.y - __byte_perm(k.x, k.y, 0x5432);
+            prev = k.y >> 16;
+        }
+        keys += 4;
+        left -= 4;
+        return d;
+    }
+};
+
+// The largest delta of the warp's runs (of up to 4 `quads` entries).
+__device__ __forceinline__ uint32_t runs_max(KeyRun r, uint32_t quads) {
+    uint32_t top = 0u;
+    for (uint32_t c = 0; c < quads; ++c) {
+        const uint2 d = r.next4();
+        top = __vmaxu2(top, __vmaxu2(d.x, d.y));
+    }
+    return __reduce_max_sync(kFullMask, max(top & 0xFFFFu, top >> 16));
 }
 
-// Packs flags and deltas of count > 0 entries (all written before a barrier of the team); sized(words) is called by every thread as
-// soon as the size is known.  The blob is complete when the call returns.
+// Width in bits and flag of a delta of b bits, held by lane b: flag << 16 | width.  0 bits: no entry (the only delta of 0, that of a
+// first key 0, goes by 1 bit: the same flag).
+__device__ __forceinline__ uint32_t delta_shape(uint32_t l, uint32_t M, int lane) {
+    if (lane == 0) return 0u;
+    const uint32_t flag = flag_of((uint32_t)((1ull << lane) - 1ull), l, c_inv_m[M]);
+    return (flag << 16) | (((flag + 1u) * M + (1u << l) - 1u) >> l);
+}
+__device__ __forceinline__ uint32_t bit_length(uint32_t x) { return 32u - (uint32_t)__clz((int)x); }
+
+// Bits of the lane's run.  zero_first: 1 where the run starts the group.
+__device__ __forceinline__ uint32_t run_bits(KeyRun r, uint32_t quads, uint32_t shape, uint32_t zero_first) {
+    uint32_t bits = 0u;
+    for (uint32_t c = 0; c < quads; ++c) {
+        const uint2 d = r.next4();
+        bits += __shfl_sync(kFullMask, shape, (int)max(bit_length(d.x & 0xFFFFu), zero_first)) + __shfl_sync(kFullMask, shape, (int)bit_length(d.x >> 16));
+        bits += __shfl_sync(kFullMask, shape, (int)bit_length(d.y & 0xFFFFu)) + __shfl_sync(kFullMask, shape, (int)bit_length(d.y >> 16));
+        zero_first = 0u;
+    }
+    return bits & 0xFFFFu;
+}
+
+// Flags, deltas and (where codes is set: 4-byte aligned, a byte per entry) codes of the lane's run, which starts with entry q0 of count
+// and with bit dpos of the blob.
+template <bool kCodes>
+__device__ __forceinline__ void write_runs(KeyRun r, uint32_t quads, uint32_t shape, uint32_t zero_first, uint32_t l, uint32_t* blob, uint32_t count,
+                                           uint32_t q0, uint32_t dpos, const uint8_t* codes) {
+    BitRun deltas(blob, dpos), flags(blob, 8u * count + l * q0), bytes(blob, 8u * q0);
+    for (uint32_t c = 0; c < quads; ++c) {
+        const uint32_t have = (uint32_t)max(0, min(4, r.left));
+        const uint2 d = r.next4();
+        uint32_t f = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t delta = i == 0 ? d.x & 0xFFFFu : i == 1 ? d.x >> 16 : i == 2 ? d.y & 0xFFFFu : d.y >> 16;
+            const uint32_t x = __shfl_sync(kFullMask, shape, (int)(i ? bit_length(delta) : max(bit_length(delta), zero_first)));
+            deltas.put(delta, x & 0xFFFFu);
+            f = (f << l) | (x >> 16);
+        }
+        zero_first = 0u;
+        if (have) {                                            // (a part of four only at the end of the last run)
+            flags.put(f >> (l * (4u - have)), l * have);
+            if constexpr (kCodes) bytes.put(bswap32(reinterpret_cast<const uint32_t*>(codes)[c]) >> (8u * (4u - have)), 8u * have);
+        }
+    }
+    deltas.close();
+    flags.close();
+    if constexpr (kCodes) bytes.close();
+}
+
+// Packs flags and deltas of count > 0 entries whose keys (ascending; behind a barrier) and codes (W > 1: with or without) the team has
+// written; sized(words) is called by every thread as soon as the size is known.  The blob is complete when the call returns M.  A thread
+// takes a run of consecutive entries: widths and bits are added up in registers, one scan over the threads gives each run its place.
 template <int W, typename F>
-__device__ __forceinline__ void team_pack(uint32_t l, const uint16_t* keys, uint32_t* blob, uint32_t count, uint32_t M, TeamScratch& s,
-                                          int w, int lane, int id, F sized) {
-    const uint32_t inv_m = c_inv_m[M], up = (1u << l) - 1u;
+__device__ __forceinline__ uint32_t team_pack(uint32_t l, const uint16_t* keys, uint32_t* blob, uint32_t count, TeamScratch& s, int w, int lane, int id, F sized) {
+    const uint32_t quads = (count + 128u * W - 1u) / (128u * W), q0 = 4u * quads * (uint32_t)(32 * w + lane);
+    KeyRun r;
+    r.keys = keys + q0; r.left = q0 < count ? (int)min(4u * quads, count - q0) : 0; r.prev = q0 && q0 < count ? (uint32_t)keys[q0 - 1u] : 0u;
+    uint32_t top = runs_max(r, quads);
+    if constexpr (W > 1) {
+        if (lane == 0) s.maxd[w] = top;
+        team_sync<W>(id);
+        top = __reduce_max_sync(kFullMask, lane < W ? s.maxd[lane] : 0u);
+    }
+    const uint32_t M = max(1u, bit_length(top)), shape = delta_shape(l, M, lane), zero_first = q0 == 0u ? 1u : 0u;
+    const uint32_t bits = run_bits(r, quads, shape, zero_first), incl = warp_incl_scan(bits, lane);
+    if (W > 1 && lane == 31) s.bits[w] = incl;
     // zeroes behind the codes
     if (w == 0 && lane == 0 && (count & 3u)) blob[count >> 2] &= 0xFFFFFFFFu << (32u - 8u * (count & 3u));
-    const uint32_t bound = (count * (8u + l + M) + 31u) >> 5;
+    const uint32_t bound = (count * (8u + l + M) + 31u) >> 5, delta0 = (8u + l) * count;
     for (uint32_t i = ((count + 3u) >> 2) + (uint32_t)(w * 32 + lane); i <= bound; i += 32u * W) blob[i] = 0u;
-    auto delta_of = [&](uint32_t q) -> uint32_t { return (uint32_t)keys[q] - (q ? (uint32_t)keys[q - 1u] : 0u); };
-    const uint32_t nb = (count + 31u) >> 5, b0 = nb * (uint32_t)w / W, b1 = nb * (uint32_t)(w + 1) / W;
-    const uint32_t delta0 = (8u + l) * count;
-    uint32_t dpos = delta0;
-    if (W > 1) {
-        uint32_t bits = 0u;
-        for (uint32_t q = 32u * b0 + (uint32_t)lane; q < min(count, 32u * b1); q += 32u) bits += ((flag_of(delta_of(q), l, inv_m) + 1u) * M + up) >> l;
-        bits = __reduce_add_sync(kFullMask, bits);
-        if (lane == 0) s.bits[w] = bits;
-        team_sync<W>(id);
+    team_sync<W>(id);
+    uint32_t dpos = delta0 + incl - bits, all = __shfl_sync(kFullMask, incl, 31);
+    if constexpr (W > 1) {
         const uint32_t x = lane < W ? s.bits[lane] : 0u, xi = warp_incl_scan(x, lane);
         dpos += __shfl_sync(kFullMask, xi - x, w);
-        sized((delta0 + __shfl_sync(kFullMask, xi, 31) + 31u) >> 5);
-    } else {
-        __syncwarp();
+        all = __shfl_sync(kFullMask, xi, 31);
     }
-    // deltas: a field per lane
-    for (uint32_t b = b0; b < b1; ++b) {
-        const uint32_t q = 32u * b + (uint32_t)lane;
-        uint32_t d = 0u, wd = 0u;
-        if (q < count) { d = delta_of(q); wd = ((flag_of(d, l, inv_m) + 1u) * M + up) >> l; }
-        const uint32_t wi = warp_incl_scan(wd, lane), pos = dpos + wi - wd, end = (pos & 31u) + wd;
-        if (q < count) {                                                // (wd is 1 to 20)
-            if (end <= 32u) atomicOr(&blob[pos >> 5], d << (32u - end));
-            else { atomicOr(&blob[pos >> 5], d >> (end - 32u)); atomicOr(&blob[(pos >> 5) + 1u], d << (64u - end)); }
-        }
-        dpos += __shfl_sync(kFullMask, wi, 31);
-    }
-    // flags: a word per lane, from the deltas of the entries whose flags lie in it
-    const uint32_t f0 = 8u * count, f1 = delta0;
-    for (uint32_t i = (f0 >> 5) + (uint32_t)(w * 32 + lane); i <= (f1 - 1u) >> 5; i += 32u * W) {
-        const uint32_t lo = max(32u * i, f0) - f0, q0 = lo / l, q1 = min(count, (32u * i + 32u - f0 + l - 1u) / l);
-        uint32_t word = 0u, prev = q0 ? (uint32_t)keys[q0 - 1u] : 0u;
-        int sh = (int)(32u * i + 32u) - (int)(f0 + l * q0 + l);          // where the flag's last bit lies in the word
-        for (uint32_t q = q0; q < q1; ++q, sh -= (int)l) {
-            const uint32_t k = keys[q], f = flag_of(k - prev, l, inv_m);
-            word |= sh >= 0 ? f << sh : f >> -sh;
-            prev = k;
-        }
-        if (word) atomicOr(&blob[i], word);
-    }
-    if (W == 1) sized((dpos + 31u) >> 5);
+    sized((delta0 + all + 31u) >> 5);
+    write_runs<false>(r, __any_sync(kFullMask, r.left > 0) ? quads : 0u, shape, zero_first, l, blob, count, q0, dpos, nullptr);
     team_sync<W>(id);
+    return M;
 }
 
 __device__ __forceinline__ void enc_write_header(const EncArgs& a, uint32_t j, int status, uint64_t d, uint64_t total_bytes, double S) {
@@ -238,92 +310,94 @@ __device__ __forceinline__ void enc_write_header(const EncArgs& a, uint32_t j, i
     outw[15] = a.G;
 }
 
-// A unit's list of candidates: the first kSlotEntries in its slot, the others in a piece of the pool.
-struct List {
-    const float *v1, *v2; const uint16_t *k1, *k2;
-    // batch b of 32: the slot holds three
-    __device__ __forceinline__ const float* values(uint32_t b) const { return b < kSlotEntries / 32u ? v1 + 32u * b : v2 + (32u * b - kSlotEntries); }
-    __device__ __forceinline__ const uint16_t* keys(uint32_t b) const { return b < kSlotEntries / 32u ? k1 + 32u * b : k2 + (32u * b - kSlotEntries); }
-};
+// A unit's list of candidates: in its slot, or in a piece of the pool.
+struct List { const float* v; const uint16_t* k; };
 __device__ __forceinline__ List list_of(const EncArgs& a, uint32_t u, const UnitInfo& in) {
     List x;
-    x.v1 = reinterpret_cast<const float*>(a.scratch + (uint64_t)u * kUnitSlotBytes);
-    x.k1 = reinterpret_cast<const uint16_t*>(x.v1 + kSlotEntries);
-    x.v2 = reinterpret_cast<const float*>(a.scratch + 16ull * in.piece);
-    x.k2 = reinterpret_cast<const uint16_t*>(x.v2 + in.room);
+    x.v = reinterpret_cast<const float*>(a.scratch + (in.room == kSlotEntries ? (uint64_t)u * kUnitSlotBytes : 16ull * in.piece));
+    x.k = reinterpret_cast<const uint16_t*>(x.v + in.room);
     return x;
 }
 
-// Kept keys, codes and M of a tile from its units' lists, by four or sixteen warps: warp w takes its share of unit w / (W / 4); returns the
-// number of kept entries.
+// Kept keys and codes of a tile from its units' lists, by the block: warp w takes its share of unit w / 4; returns the number of kept
+// entries.
 template <int W>
-__device__ __forceinline__ uint32_t team_list(const EncArgs& a, uint32_t t, const float* thr, uint16_t* keys, uint32_t* blob, uint32_t& M,
-                                              TeamScratch& s, int w, int lane, int id) {
+__device__ __forceinline__ uint32_t team_list(const EncArgs& a, uint32_t t, const float* thr, uint16_t* keys, uint32_t* blob, TeamScratch& s, int w, int lane, int id) {
     const float thr_e = thr[a.tau];
     const uint32_t u = 4u * t + (uint32_t)w / (W / 4), part = (uint32_t)w % (W / 4);
     const UnitInfo in = load_info(a.info + u);
     const List x = list_of(a, u, in);
     const uint32_t cnt = __ldcg(a.umax + u) >= thr_e ? in.count : 0u;
     const uint32_t nb = (cnt + 31u) >> 5, b0 = nb * part / (W / 4), b1 = nb * (part + 1u) / (W / 4);
+    const uint32_t end = min(cnt, 32u * b1);
     // how many are kept
     uint32_t n = 0u;
     for (uint32_t b = b0; b < b1; b += 4u) {
         float v[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = b + i < b1 && 32u * (b + i) + (uint32_t)lane < cnt ? __ldcg(x.values(b + i) + lane) : 0.0f;
+        for (int i = 0; i < 4; ++i) v[i] = 32u * (b + i) + (uint32_t)lane < end ? __ldcg(x.v + 32u * (b + i) + lane) : 0.0f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) n += (uint32_t)__popc(__ballot_sync(kFullMask, fabsf(v[i]) >= thr_e));
+        for (int i = 0; i < 4; ++i) n += fabsf(v[i]) >= thr_e ? 1u : 0u;
     }
+    n = __reduce_add_sync(kFullMask, n);
     if (lane == 0) s.cnt[w] = n;
+    auto value = [&](uint32_t b) -> float { return 32u * b + (uint32_t)lane < end ? __ldcg(x.v + 32u * b + lane) : 0.0f; };
+    auto key = [&](uint32_t b) -> uint32_t { return 32u * b + (uint32_t)lane < end ? __ldcg(x.k + 32u * b + lane) : 0u; };
+    float v0 = value(b0), v1 = value(b0 + 1u);
+    uint32_t k0 = key(b0), k1 = key(b0 + 1u);
     team_sync<W>(id);
     const uint32_t c = lane < W ? s.cnt[lane] : 0u, ci = warp_incl_scan(c, lane);
     uint32_t rank = __shfl_sync(kFullMask, ci - c, w);
-    const uint32_t count = __shfl_sync(kFullMask, ci, 31);
-    uint32_t maxd = 0u, prev = 0u, first = 0u;
-    bool none = true;
-    auto value = [&](uint32_t b) -> float { return b < b1 && 32u * b + (uint32_t)lane < cnt ? __ldcg(x.values(b) + lane) : 0.0f; };
-    auto key = [&](uint32_t b) -> uint32_t { return b < b1 && 32u * b + (uint32_t)lane < cnt ? __ldcg(x.keys(b) + lane) : 0u; };
-    float v0 = value(b0), v1 = value(b0 + 1u);
-    uint32_t k0 = key(b0), k1 = key(b0 + 1u);
+    const uint32_t count = __shfl_sync(kFullMask, ci, 31), below = (1u << lane) - 1u;
     for (uint32_t b = b0; b < b1; ++b) {
         const float v2 = value(b + 2u);
         const uint32_t k2 = key(b + 2u);
         const bool kept = fabsf(v0) >= thr_e;
         const uint32_t km = __ballot_sync(kFullMask, kept);
-        if (km) {
-            const uint32_t lower = km & ((1u << lane) - 1u);
-            const uint32_t pk = __shfl_sync(kFullMask, k0, lower ? 31 - __clz((int)lower) : 0);
-            if (none) { prev = first = __shfl_sync(kFullMask, k0, __ffs((int)km) - 1); none = false; }      // (the delta before the share's first key: below)
-            if (kept) {
-                const uint32_t q = rank + (uint32_t)__popc(lower);
-                maxd = max(maxd, k0 - (lower ? pk : prev));
-                keys[q] = (uint16_t)k0;
-                put_code(blob, q, code_byte_of(thr, a.tau, v0));
-            }
-            prev = __shfl_sync(kFullMask, k0, 31 - __clz((int)km));
-            rank += (uint32_t)__popc(km);
+        if (kept) {
+            const uint32_t q = rank + (uint32_t)__popc(km & below);
+            keys[q] = (uint16_t)k0;
+            put_code(blob, q, code_byte_of(thr, a.tau, v0));
         }
+        rank += (uint32_t)__popc(km);
         v0 = v1; k0 = k1; v1 = v2; k1 = k2;
     }
-    // the largest delta: within the shares, and from one share's last key to the next one's first (keys ascend)
-    maxd = __reduce_max_sync(kFullMask, maxd);
-    if (lane == 0) { s.maxd[w] = maxd; s.first[w] = first; s.last[w] = none ? 0u : prev; }
     team_sync<W>(id);
-    uint32_t last = lane < W ? s.last[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < W; o <<= 1) { const uint32_t y = __shfl_up_sync(kFullMask, last, o); if (lane >= o) last = max(last, y); }
-    uint32_t before = __shfl_up_sync(kFullMask, last, 1);
-    if (lane == 0) before = 0u;
-    maxd = 0u;
-    if (lane < W) maxd = c ? max(s.maxd[lane], s.first[lane] - before) : 0u;
-    maxd = __reduce_max_sync(kFullMask, maxd);
-    M = maxd ? 32u - (uint32_t)__clz((int)maxd) : 1u;
     return count;
 }
 
-// The same by one warp, all candidates (off[q]: those of the units before unit q) in the units' slots; maxd instead of M.
-__device__ __forceinline__ uint32_t warp_list(const EncArgs& a, uint32_t t, const uint32_t (&off)[5], const float* thr, uint16_t* keys, uint32_t* blob,
-                                              uint32_t& maxd, int lane) {
+// The same by one warp for a whole unit, without ranks among the other units: keys and code bytes in the unit's own place.
+__device__ __forceinline__ uint32_t unit_list(const List& x, uint32_t cnt, const float* thr, uint32_t tau, uint16_t* keys, uint8_t* codes, int lane) {
+    const float thr_e = thr[tau];
+    uint32_t rank = 0u;
+    const uint32_t below = (1u << lane) - 1u;
+    auto value = [&](uint32_t e) -> float { return e + (uint32_t)lane < cnt ? __ldcg(x.v + e + lane) : 0.0f; };
+    auto key = [&](uint32_t e) -> uint32_t { return e + (uint32_t)lane < cnt ? __ldcg(x.k + e + lane) : 0u; };
+    float v[4]; uint32_t k[4];
+#pragma unroll
+    for (uint32_t i = 0; i < 4u; ++i) { v[i] = value(32u * i); k[i] = key(32u * i); }
+    for (uint32_t e = 0; e < cnt; e += 128u) {
+        float nv[4]; uint32_t nk[4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) { nv[i] = value(e + 128u + 32u * i); nk[i] = key(e + 128u + 32u * i); }
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) {
+            const bool kept = fabsf(v[i]) >= thr_e;
+            const uint32_t km = __ballot_sync(kFullMask, kept);
+            if (kept) {
+                const uint32_t q = rank + (uint32_t)__popc(km & below);
+                keys[q] = (uint16_t)k[i];
+                codes[q] = (uint8_t)code_byte_of(thr, tau, v[i]);
+            }
+            rank += (uint32_t)__popc(km);
+            v[i] = nv[i]; k[i] = nk[i];
+        }
+    }
+    return rank;
+}
+
+// The same by one warp, all candidates (off[q]: those of the units before unit q) in the units' slots.
+__device__ __forceinline__ uint32_t warp_list(const EncArgs& a, uint32_t t, const uint32_t (&off)[5], const float* thr, uint16_t* keys, uint32_t* blob, int lane) {
     const float thr_e = thr[a.tau];
     const unsigned char* slots = a.scratch + (uint64_t)t * kSlotBytes;
     auto load = [&](uint32_t e, float& v, uint32_t& k) {
@@ -335,31 +409,29 @@ __device__ __forceinline__ uint32_t warp_list(const EncArgs& a, uint32_t t, cons
         v = __ldcg(reinterpret_cast<const float*>(slot) + i);
         k = __ldcg(reinterpret_cast<const uint16_t*>(slot + 4u * kSlotEntries) + i);
     };
-    uint32_t rank = 0u, prev = 0u, k0, k1, k2; float v0, v1, v2;
-    maxd = 0u;
+    uint32_t rank = 0u, k0, k1, k2; float v0, v1, v2;
+    const uint32_t below = (1u << lane) - 1u;
     load((uint32_t)lane, v0, k0);
     load(32u + (uint32_t)lane, v1, k1);
     for (uint32_t e = 0; e < off[4]; e += 32u) {
         load(e + 64u + (uint32_t)lane, v2, k2);
         const bool kept = fabsf(v0) >= thr_e;
-        const uint32_t km = __ballot_sync(kFullMask, kept), lower = km & ((1u << lane) - 1u);
-        const uint32_t pk = __shfl_sync(kFullMask, k0, lower ? 31 - __clz((int)lower) : 0);
+        const uint32_t km = __ballot_sync(kFullMask, kept);
         if (kept) {
-            const uint32_t q = rank + (uint32_t)__popc(lower);
-            maxd = max(maxd, k0 - (lower ? pk : prev));
+            const uint32_t q = rank + (uint32_t)__popc(km & below);
             keys[q] = (uint16_t)k0;
             put_code(blob, q, code_byte_of(thr, a.tau, v0));
         }
-        if (km) prev = __shfl_sync(kFullMask, k0, 31 - __clz((int)km));
         rank += (uint32_t)__popc(km);
         v0 = v1; k0 = k1; v1 = v2; k1 = k2;
     }
+    __syncwarp();
     return rank;
 }
 
-// The same from the tile itself, by the whole block: the kept keys of warp w's slab, then codes and deltas.
-__device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uint32_t tile, const float* thr, uint16_t* keys, uint32_t* blob, uint32_t& maxd,
-                                               TeamScratch& s, int tid, int lane, int warp) {
+// The same from the tile itself, by the whole block: the kept keys of warp w's slab, then the codes.
+__device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uint32_t tile, const float* thr, uint16_t* keys, uint32_t* blob, TeamScratch& s,
+                                               int tid, int lane, int warp) {
     const float* g = a.grad[j] + ((uint64_t)tile << kGroupLog2);
     const uint64_t left = a.n - ((uint64_t)tile << kGroupLog2);
     const float thr_e = thr[a.tau];
@@ -380,12 +452,7 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
     uint32_t pos = __shfl_sync(kFullMask, ci - c, warp) + incl - own;
     for (; mask != 0u; mask &= mask - 1u, ++pos) keys[pos] = (uint16_t)((uint32_t)warp * kSlab + 32u * (uint32_t)lane + (uint32_t)__ffs((int)mask) - 1u);
     __syncthreads();
-    maxd = 0u;
-    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) {
-        const uint32_t k = keys[q];
-        maxd = max(maxd, k - (q ? (uint32_t)keys[q - 1u] : 0u));
-        put_code(blob, q, code_byte_of(thr, a.tau, __ldg(g + k)));
-    }
+    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) put_code(blob, q, code_byte_of(thr, a.tau, __ldg(g + keys[q])));
     return count;
 }
 
@@ -395,7 +462,7 @@ struct ResShared {
         float    tile[kTile];
         uint32_t blob[kTile];            // 27 bits an entry at most; grows over the tile, whose values behind it are still needed
     };
-    uint16_t key[kTile];
+    alignas(16) uint16_t key[kTile];
     unsigned long long mbar[kEncWarps];
     float    thr[132];
     double   node[kEncWarps], s_tree[kEncWarps];
@@ -479,15 +546,10 @@ k_resident(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_co
         s.key[pos] = (uint16_t)((uint32_t)warp * kSlab + 32u * (uint32_t)lane + (uint32_t)__ffs((int)m) - 1u);
     __syncthreads();
     // ---- codes: those of a round replace entries of the tile whose codes have been formed (rank <= key: a code lies before its value)
-    uint32_t maxd = 0u;
     for (uint32_t q0 = 0; q0 < count; q0 += kEncThreads) {
         const uint32_t q = q0 + (uint32_t)tid;
         uint32_t code = 0u;
-        if (q < count) {
-            const uint32_t k = s.key[q];
-            maxd = max(maxd, k - (q ? (uint32_t)s.key[q - 1u] : 0u));
-            code = code_byte_of(s.thr, a.tau, s.tile[k]);
-        }
+        if (q < count) code = code_byte_of(s.thr, a.tau, s.tile[s.key[q]]);
         __syncthreads();
         if (q < count) put_code(s.blob, q, code);
     }
@@ -496,12 +558,8 @@ k_resident(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_co
         words = w;
         if (tid == 0) st_relaxed_u64(a.st->res_size + t, ((unsigned long long)gen << 32) | (count << 16) | w);
     };
-    if (count) {
-        M = team_width<kEncWarps>(maxd, s.team, warp, lane, 0);
-        team_pack<kEncWarps>(a.l, s.key, s.blob, count, M, s.team, warp, lane, 0, publish);
-    } else {
-        publish(0u);
-    }
+    if (count) M = team_pack<kEncWarps>(a.l, s.key, s.blob, count, s.team, warp, lane, 0, publish);
+    else publish(0u);
     // ---- the tile's place: the sizes of the gradient's tiles before it
     unsigned long long z = 0ull;
     if ((uint32_t)tid < tile) {
@@ -673,10 +731,10 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
         // tickets a nanosecond: 240 us for 65536 units.)
         if (lane == 0) tk = atomicAdd(&a.st->ticket[tg][0], 1u);
         const float est = s.est[j], thr = est > 0.0f ? est : __int_as_float(0x7f800000);
-        float* v1 = reinterpret_cast<float*>(a.scratch + (uint64_t)t * kUnitSlotBytes);
-        uint16_t* k1 = reinterpret_cast<uint16_t*>(v1 + kSlotEntries);
+        float* lv = reinterpret_cast<float*>(a.scratch + (uint64_t)t * kUnitSlotBytes);
+        uint16_t* lk = reinterpret_cast<uint16_t*>(lv + kSlotEntries);
         bool listing = true;
-        uint32_t n_list = 0u, piece = 0u, room = 0u;
+        uint32_t n_list = 0u, piece = 0u, room = kSlotEntries;
         float mx = 0.0f;
         double mynode = 0.0;
 #pragma unroll 1
@@ -699,29 +757,30 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
             if (__any_sync(kFullMask, fm >= thr) && listing) { // (uniform)
                 uint32_t m = slab_mask(v, thr, lane);
                 const uint32_t own = (uint32_t)__popc(m), incl = warp_incl_scan(own, lane), cnt = __shfl_sync(kFullMask, incl, 31);
-                if (n_list + cnt > kSlotEntries && room == 0u) {
-                    // a piece of the pool: what the unit so far promises, and a quarter more
+                if (n_list + cnt > room || (slab == 0u && 4u * cnt > kSlotEntries)) {
+                    // a piece of the pool instead of the slot: what the unit so far promises, and a quarter more
                     const uint32_t promise = (n_list + cnt) * 4u / (slab + 1u);
-                    room = min(kUnit, (promise * 5u / 4u + 63u) & ~31u);
-                    listing = promise <= kListMost;
+                    listing = room == kSlotEntries && promise <= kListMost;
                     if (listing) {
+                        room = min(kUnit, (promise * 5u / 4u + 63u) & ~31u);
                         if (lane == 0) piece = pool_take(a, room * 6u);
                         piece = __shfl_sync(kFullMask, piece, 0);
                         listing = piece != kNoPlace;
+                        if (listing) {
+                            float* pv = reinterpret_cast<float*>(a.scratch + 16ull * piece);
+                            uint16_t* pk = reinterpret_cast<uint16_t*>(pv + room);
+                            for (uint32_t q = lane; q < n_list; q += 32u) { pv[q] = lv[q]; pk[q] = lk[q]; }
+                            lv = pv; lk = pk;
+                        }
                     }
-                } else if (n_list + cnt > kSlotEntries + room) {
-                    listing = false;
                 }
                 if (listing) {
-                    float* v2 = reinterpret_cast<float*>(a.scratch + 16ull * piece) - kSlotEntries;
-                    uint16_t* k2 = reinterpret_cast<uint16_t*>(v2 + kSlotEntries + room) - kSlotEntries;
                     const uint32_t key0 = (i & 3u) * kUnit + slab * kSlab + 32u * (uint32_t)lane;
                     uint32_t pos = n_list + incl - own;
                     for (; m != 0u; m &= m - 1u, ++pos) {
                         const uint32_t b = (uint32_t)__ffs((int)m) - 1u;
-                        const bool in_slot = pos < kSlotEntries;
-                        (in_slot ? v1 : v2)[pos] = ring[32u * (uint32_t)lane + b];
-                        (in_slot ? k1 : k2)[pos] = (uint16_t)(key0 + b);
+                        lv[pos] = ring[32u * (uint32_t)lane + b];
+                        lk[pos] = (uint16_t)(key0 + b);
                     }
                     n_list += cnt;
                 }
@@ -762,18 +821,18 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
 
 // ---- k_encode ----------------------------------------------------------------------------------
 struct WorkArea {                                              // shared memory of one team: [16 warps], [4 quads] or [the block]
-    static constexpr uint32_t kWarpWords = (kWarpListMax * 27u + 31u) / 32u + 4u, kQuadWords = (kQuadListMax * 27u + 31u) / 32u + 4u,
+    static constexpr uint32_t kWarpWords = (kWarpListMax * 27u + 31u) / 32u + 4u, kQuadWords = (4u * kUnitListMax * 27u + 31u) / 32u + 4u,
                               kBlockWords = (kTile * 27u + 31u) / 32u + 4u;
-    struct Warp { uint16_t key[kWarpListMax]; uint32_t blob[kWarpWords]; };
-    struct Quad { union { struct { uint16_t key[kQuadListMax]; uint32_t blob[kQuadWords]; }; Warp w[4]; }; };
-    struct Block { uint16_t key[kTile]; uint32_t blob[kBlockWords]; };
+    struct Warp { alignas(16) uint16_t key[kWarpListMax]; uint32_t blob[kWarpWords]; };
+    struct Quad { union { struct { alignas(16) uint16_t key[4][kUnitListMax]; uint8_t code[4][kUnitListMax]; uint32_t blob[kQuadWords]; }; Warp w[4]; }; };
+    struct Block { alignas(16) uint16_t key[kTile]; uint32_t blob[kBlockWords]; };
     union { Quad q[kEncWarps / 4]; Block b; };
 };
 
 struct EncShared {
     float    thr[kEncMaxJobs][132];
     double   S[kEncMaxJobs];
-    uint32_t n_light, n_mid, n_heavy, next_light, next_mid, abort_flag, grab[4];
+    uint32_t n_light, n_mid, mid_entries, n_heavy, next_light, next_mid, abort_flag, grab[4];
     TeamScratch team[4];
     uint16_t light[kEncThreads], mid[kEncThreads], heavy[kEncThreads];      // heavy: bit 15: the tile is read again
     WorkArea area;
@@ -865,28 +924,32 @@ k_encode(const EncArgs a) {
         if (k == 131u) table_hints(s.S[j], a.base, &s.thr[j][130]);
     }
 
-    const uint32_t warp_max = owned >= (uint32_t)kEncWarps ? kWarpListMax : 64u;      // (few tiles per block: a list is better shared out)
+    // (few tiles per block: a list is better shared out among more warps)
+    const uint32_t warp_max = owned >= (uint32_t)kEncWarps ? kWarpListMax : 64u;
     for (uint32_t first = 0; first < owned; first += kEncThreads) {
         // ---- which of the block's tiles hold anything, and where it is
-        if (tid == 0) { s.n_light = 0u; s.n_mid = 0u; s.n_heavy = 0u; s.next_light = 0u; s.next_mid = 0u; }
+        if (tid == 0) { s.n_light = 0u; s.n_mid = 0u; s.mid_entries = 0u; s.n_heavy = 0u; s.next_light = 0u; s.next_mid = 0u; }
         if (first) load_tile(first + (uint32_t)tid);
         __syncthreads();
         if (first + (uint32_t)tid < owned) {
             const uint32_t t = blockIdx.x + (first + (uint32_t)tid) * B, j = t / a.G;
             const float thr_e = s.thr[j][a.tau];
             uint32_t cnt = 0u;
-            bool again = false, any = false, slots = true;     // (a unit that does not reach the threshold counts for nothing)
+            bool again = false, any = false, slots = true, units = true;      // (a unit that does not reach the threshold counts for nothing)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float x = q == 0 ? um.x : q == 1 ? um.y : q == 2 ? um.z : um.w;
-                if (x >= thr_e) { any = true; cnt += in[q].count; again = again || !(in[q].sthr <= thr_e); slots = slots && in[q].count <= kSlotEntries; }
+                if (x >= thr_e) { any = true; cnt += in[q].count; again = again || !(in[q].sthr <= thr_e); slots = slots && in[q].room == kSlotEntries; units = units && in[q].count <= kUnitListMax; }
             }
             if (!(thr_e < __int_as_float(0x7f800000)) || !any) a.desc[t] = 0ull;      // nothing is kept here
             else if (again) {
                 s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)(tid | 0x8000);
                 atomicAdd(&a.ctl->ne_count[j], 1u);
             } else if (slots && cnt <= warp_max) s.light[atomicAdd(&s.n_light, 1u)] = (uint16_t)tid;
-            else if (cnt <= kQuadListMax) s.mid[atomicAdd(&s.n_mid, 1u)] = (uint16_t)tid;
+            else if (units) {
+                s.mid[atomicAdd(&s.n_mid, 1u)] = (uint16_t)tid;
+                atomicAdd(&s.mid_entries, cnt);
+            }
             else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
         }
         __syncthreads();
@@ -903,17 +966,16 @@ k_encode(const EncArgs a) {
             return p;
         };
         // ---- by the whole block
-        for (uint32_t h = 0; h < s.n_heavy; ++h) {
-            const uint32_t t = blockIdx.x + (first + (s.heavy[h] & 0x7FFFu)) * B, j = t / a.G, tile = t - j * a.G;
-            uint32_t maxd, M = 0u, words = 0u, place = 0u, count;
-            if ((s.heavy[h] & 0x8000u) != 0u) {
-                count = block_tile(a, j, tile, s.thr[j], s.area.b.key, s.area.b.blob, maxd, s.team[0], tid, lane, warp);
-                M = team_width<kEncWarps>(maxd, s.team[0], warp, lane, 0);
-            } else {
-                count = team_list<kEncWarps>(a, t, s.thr[j], s.area.b.key, s.area.b.blob, M, s.team[0], warp, lane, 0);
-            }
+        // (tiles for four warps too, where those are too few to occupy the block and long enough for it)
+        const uint32_t n_mid = s.n_mid < (uint32_t)kEncWarps / 4u && s.mid_entries > 1024u * s.n_mid ? 0u : s.n_mid, n_block = s.n_heavy + s.n_mid - n_mid;
+        for (uint32_t h = 0; h < n_block; ++h) {
+            const uint32_t x = h < s.n_heavy ? s.heavy[h] : s.mid[h - s.n_heavy];
+            const uint32_t t = blockIdx.x + (first + (x & 0x7FFFu)) * B, j = t / a.G, tile = t - j * a.G;
+            uint32_t M = 0u, words = 0u, place = 0u;
+            const uint32_t count = (x & 0x8000u) != 0u ? block_tile(a, j, tile, s.thr[j], s.area.b.key, s.area.b.blob, s.team[0], tid, lane, warp)
+                                                               : team_list<kEncWarps>(a, t, s.thr[j], s.area.b.key, s.area.b.blob, s.team[0], warp, lane, 0);
             if (count) {
-                team_pack<kEncWarps>(a.l, s.area.b.key, s.area.b.blob, count, M, s.team[0], warp, lane, 0, [&](uint32_t w_) {
+                M = team_pack<kEncWarps>(a.l, s.area.b.key, s.area.b.blob, count, s.team[0], warp, lane, 0, [&](uint32_t w_) {
                     words = w_;
                     if (tid == 0) s.team[0].word = place_of(t, w_);
                 });
@@ -930,28 +992,72 @@ k_encode(const EncArgs a) {
         const int quad = warp >> 2, qw = warp & 3;
         if (qw == 0 && lane == 0) s.grab[quad] = atomicAdd(&s.next_mid, 1u);
         team_sync<4>(quad);
-        for (;;) {
-            const uint32_t x = s.grab[quad];
-            if (x >= s.n_mid) break;
-            const uint32_t t = blockIdx.x + (first + s.mid[x]) * B, j = t / a.G;
+        // (a warp per unit; three barriers a tile; the next tile's entries of the tables are asked for while this one is packed)
+        uint32_t x = s.grab[quad], t = 0u;
+        UnitInfo ui;
+        float ux = 0.0f;
+        auto next_unit = [&]() {
+            if (x >= n_mid) return;
+            t = blockIdx.x + (first + s.mid[x]) * B;
+            ui = load_info(a.info + 4ull * t + qw);
+            ux = __ldcg(a.umax + 4ull * t + qw);
+        };
+        next_unit();
+        while (x < n_mid) {
+            const uint32_t here = t, j = t / a.G;
             WorkArea::Quad& ar = s.area.q[quad];
-            uint32_t M, words = 0u, place = 0u;
-            const uint32_t count = team_list<4>(a, t, s.thr[j], ar.key, ar.blob, M, s.team[quad], qw, lane, quad);
-            if (qw == 0 && lane == 0) s.grab[quad] = atomicAdd(&s.next_mid, 1u);
-            if (count) {
-                team_pack<4>(a.l, ar.key, ar.blob, count, M, s.team[quad], qw, lane, quad, [&](uint32_t w_) {
-                    words = w_;
-                    if (qw == 0 && lane == 0) s.team[quad].word = place_of(t, w_);
-                });
-                place = s.team[quad].word;
-                if (place != kNoPlace) {
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(a.scratch + 16ull * place);
-                    for (uint32_t i = (uint32_t)(qw * 32 + lane); i < words; i += 128u) dst[i] = bswap32(ar.blob[i]);
-                }
-            }
-            if (qw == 0 && lane == 0) record(t, j, count, M, words, place);
+            TeamScratch& ts = s.team[quad];
+            const uint16_t* keys = ar.key[qw];
+            const uint32_t n = ux >= s.thr[j][a.tau] ? unit_list(list_of(a, 4u * t + (uint32_t)qw, ui), ui.count, s.thr[j], a.tau, ar.key[qw], ar.code[qw], lane) : 0u;
+            __syncwarp();
+            const uint32_t quads = (n + 127u) >> 7, q0 = 4u * quads * (uint32_t)lane;
+            KeyRun r;
+            r.keys = keys + q0; r.left = q0 < n ? (int)min(4u * quads, n - q0) : 0; r.prev = q0 < n ? (uint32_t)keys[q0 ? q0 - 1u : 0u] : 0u;
+            const uint32_t top = runs_max(r, quads);           // (within the unit)
+            if (lane == 0) { ts.cnt[qw] = n; ts.maxd[qw] = top; ts.first[qw] = n ? (uint32_t)keys[0] : 0u; ts.last[qw] = n ? (uint32_t)keys[n - 1u] : 0u; }
             team_sync<4>(quad);
+            // from one unit's last key to the next one's first; the unit's rank
+            uint32_t M = 0u, count = 0u, rank = 0u, last = 0u, before = 0u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t c = ts.cnt[q];
+                if (q == qw) { rank = count; before = last; }
+                if (c) { M = max(M, max(ts.maxd[q], ts.first[q] - last)); last = ts.last[q]; }
+                count += c;
+            }
+            if (count == 0u) {                                 // (the same in the four warps)
+                if (qw == 0 && lane == 0) { record(here, j, 0u, 0u, 0u, 0u); s.grab[quad] = atomicAdd(&s.next_mid, 1u); }
+                team_sync<4>(quad);
+                x = s.grab[quad];
+                next_unit();
+                continue;
+            }
+            M = max(1u, bit_length(M));
+            if (lane == 0) r.prev = before;
+            const uint32_t shape = delta_shape(a.l, M, lane), zero_first = rank + q0 == 0u ? 1u : 0u;
+            const uint32_t bits = run_bits(r, quads, shape, zero_first), incl = warp_incl_scan(bits, lane);
+            if (lane == 31) ts.bits[qw] = incl;
+            if (qw == 0 && lane == 0) s.grab[quad] = atomicAdd(&s.next_mid, 1u);
+            const uint32_t bound = (count * (8u + a.l + M) + 31u) >> 5, delta0 = (8u + a.l) * count;
+            for (uint32_t i = (uint32_t)(qw * 32 + lane); i <= bound; i += 128u) ar.blob[i] = 0u;
+            team_sync<4>(quad);
+            x = s.grab[quad];
+            next_unit();
+            uint32_t dpos = delta0 + incl - bits, words = delta0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { const uint32_t y = ts.bits[q]; if (q < qw) dpos += y; words += y; }
+            words = (words + 31u) >> 5;
+            if (qw == 0 && lane == 0) ts.word = place_of(here, words);
+            write_runs<true>(r, quads, shape, zero_first, a.l, ar.blob, count, rank + q0, dpos, ar.code[qw] + q0);
+            team_sync<4>(quad);
+            const uint32_t place = ts.word;
+            if (place != kNoPlace) {
+                uint32_t* dst = reinterpret_cast<uint32_t*>(a.scratch + 16ull * place);
+                for (uint32_t i = (uint32_t)(qw * 32 + lane); i < words; i += 128u) dst[i] = bswap32(ar.blob[i]);
+            }
+            if (qw == 0 && lane == 0) record(here, j, count, M, words, place);
         }
+        team_sync<4>(quad);
         // ---- by single warps
         for (;;) {
             uint32_t x = 0u;
@@ -970,12 +1076,11 @@ k_encode(const EncArgs a) {
                 for (int q = 0; q < 4; ++q) off[q + 1] = __shfl_sync(kFullMask, ci, q);
             }
             WorkArea::Warp& ar = s.area.q[quad].w[qw];
-            uint32_t maxd, M = 0u, words = 0u;
+            uint32_t M = 0u, words = 0u;
             const uint32_t place = t * (kSlotBytes / 16u);      // (27 bits an entry at most: the blob fits the slots)
-            const uint32_t count = warp_list(a, t, off, s.thr[j], ar.key, ar.blob, maxd, lane);
+            const uint32_t count = warp_list(a, t, off, s.thr[j], ar.key, ar.blob, lane);
             if (count) {
-                M = team_width<1>(maxd, s.team[quad], 0, lane, 0);
-                team_pack<1>(a.l, ar.key, ar.blob, count, M, s.team[quad], 0, lane, 0, [&](uint32_t w_) { words = w_; });
+                M = team_pack<1>(a.l, ar.key, ar.blob, count, s.team[quad], 0, lane, 0, [&](uint32_t w_) { words = w_; });
                 uint32_t* dst = reinterpret_cast<uint32_t*>(a.scratch + 16ull * place);
                 for (uint32_t i = lane; i < words; i += 32u) dst[i] = bswap32(ar.blob[i]);
             }
@@ -1090,7 +1195,7 @@ k_place(const EncArgs a) {
     }
     // ---- rows of eight tiles: directory entries and blobs.  When the rows are fewer than the warps, several warps share a row's words.
     const uint32_t rows = (a.G + kRowTiles - 1u) / kRowTiles, warps = B * (uint32_t)kEncWarps;
-    const uint32_t parts = max(1u, min(8u, warps / (a.J * rows)));
+    const uint32_t parts = max(1u, min(32u, warps / (a.J * rows)));
     for (uint32_t x = blockIdx.x + B * (uint32_t)warp; x < a.J * rows * parts; x += warps) {
         const uint32_t part = x % parts, y = x / parts, j = y / rows, t0 = (y - j * rows) * kRowTiles, tile = t0 + (uint32_t)lane;
         if (!fits(j)) continue;
@@ -1131,9 +1236,8 @@ k_place(const EncArgs a) {
             for (uint32_t k = (uint32_t)tid; k <= a.tau; k += kEncThreads) s.thr[k] = boundary(S, __ldcg(a.st->pw + k), __ldcg(a.st->inv + k));
             if (tid == kEncThreads - 1) table_hints(S, a.base, &s.thr[130]);
             __syncthreads();
-            uint32_t maxd;
-            const uint32_t count = block_tile(a, j, tile, s.thr, s.area.key, s.area.blob, maxd, s.team, tid, lane, warp);
-            team_pack<kEncWarps>(a.l, s.area.key, s.area.blob, count, team_width<kEncWarps>(maxd, s.team, warp, lane, 0), s.team, warp, lane, 0, [](uint32_t) {});
+            const uint32_t count = block_tile(a, j, tile, s.thr, s.area.key, s.area.blob, s.team, tid, lane, warp);
+            team_pack<kEncWarps>(a.l, s.area.key, s.area.blob, count, s.team, warp, lane, 0, [](uint32_t) {});
             uint32_t* dst = reinterpret_cast<uint32_t*>(a.out[j]) + fixed_words + (uint32_t)tile_prefix(a, s.seg, j, tile, lane);
             for (uint32_t i = (uint32_t)tid; i < (uint32_t)(d >> 32); i += kEncThreads) dst[i] = bswap32(s.area.blob[i]);
             __syncthreads();

@@ -153,12 +153,14 @@ __device__ __forceinline__ uint32_t flag_of(uint32_t delta, uint32_t l, uint32_t
 // table from there, so the result does not depend on how good the estimate is.
 __device__ __forceinline__ uint32_t code_byte_of(const float* thr, uint32_t tau, float val) {
     const float av = fabsf(val);
-    int guess = (int)((thr[130] - __log2f(av)) * thr[131]) + 1;
-    guess = max(0, min((int)tau, guess));
-    uint32_t L = (uint32_t)guess;
-    while (L > 0u && av >= thr[L - 1u]) --L;
-    while (L < tau && av < thr[L]) ++L;
-    L = L < 1u ? 1u : L;
+    float lg;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(av));
+    uint32_t L = (uint32_t)max(1, min((int)tau, __float2int_rd(fmaf(-lg, thr[131], thr[130] * thr[131])) + 1));
+    if (av >= thr[L - 1u] || av < thr[L]) {                    // (a few in a million)
+        while (L > 0u && av >= thr[L - 1u]) --L;
+        while (L < tau && av < thr[L]) ++L;
+        L = L < 1u ? 1u : L;
+    }
     return (val < 0.0f ? 0x80u : 0u) | (L - 1u);
 }
 
