@@ -157,18 +157,16 @@ template <int W> __device__ __forceinline__ void team_sync(int id) {
 
 __device__ __forceinline__ void put_code(uint32_t* blob, uint32_t q, uint32_t code) { reinterpret_cast<uint8_t*>(blob)[q ^ 3u] = (uint8_t)code; }
 
-// Appends bit fields to a zeroed blob from any bit position on.  Words that lie wholly in the run are stored, the first and the last
-// are shared with neighbours.
+// Appends bit fields to a zeroed blob from any bit position on (its first and last words are shared with neighbours).
 struct BitRun {
-    uint32_t *first, *at, cur, fill;
-    __device__ __forceinline__ BitRun(uint32_t* blob, uint32_t pos) : first(blob + (pos >> 5)), at(first), cur(0u), fill(pos & 31u) {}
+    uint32_t *at, cur, fill;
+    __device__ __forceinline__ BitRun(uint32_t* blob, uint32_t pos) : at(blob + (pos >> 5)), cur(0u), fill(pos & 31u) {}
     // a value of `width` (0 to 32) bits; width 0: value 0
     __device__ __forceinline__ void put(uint32_t value, uint32_t width) {
         const uint32_t x = value << ((32u - width) & 31u), end = fill + width;
         cur |= x >> fill;
         if (end >= 32u) {
-            if (at == first) atomicOr(at, cur); else *at = cur;
-            ++at;
+            atomicOr(at++, cur);
             cur = __funnelshift_r(0u, x, fill);
         }
         fill = end & 31u;
@@ -211,23 +209,29 @@ __device__ __forceinline__ uint32_t runs_max(KeyRun r, uint32_t quads) {
     return __reduce_max_sync(kFullMask, max(top & 0xFFFFu, top >> 16));
 }
 
-// Width in bits and flag of a delta of b bits, held by lane b: flag << 16 | width.  0 bits: no entry (the only delta of 0, that of a
-// first key 0, goes by 1 bit: the same flag).
+// Width in bits and flag of a delta of b bits, held by lane b - 1: flag << 16 | width.  0 bits (lane 31): no entry (the only delta of 0,
+// that of a first key 0, goes by 1 bit: the same flag).
 __device__ __forceinline__ uint32_t delta_shape(uint32_t l, uint32_t M, int lane) {
-    if (lane == 0) return 0u;
-    const uint32_t flag = flag_of((uint32_t)((1ull << lane) - 1ull), l, c_inv_m[M]);
+    if (lane == 31) return 0u;
+    const uint32_t flag = flag_of((2u << lane) - 1u, l, c_inv_m[M]);
     return (flag << 16) | (((flag + 1u) * M + (1u << l) - 1u) >> l);
 }
 __device__ __forceinline__ uint32_t bit_length(uint32_t x) { return 32u - (uint32_t)__clz((int)x); }
+// position of the highest bit; -1 (for a shuffle: lane 31) for 0
+__device__ __forceinline__ int top_bit(uint32_t x) {
+    int r;
+    asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
+}
 
-// Bits of the lane's run.  zero_first: 1 where the run starts the group.
-__device__ __forceinline__ uint32_t run_bits(KeyRun r, uint32_t quads, uint32_t shape, uint32_t zero_first) {
+// Bits of the lane's run.  least: 0 where the run starts the group, else -1.
+__device__ __forceinline__ uint32_t run_bits(KeyRun r, uint32_t quads, uint32_t shape, int least) {
     uint32_t bits = 0u;
     for (uint32_t c = 0; c < quads; ++c) {
         const uint2 d = r.next4();
-        bits += __shfl_sync(kFullMask, shape, (int)max(bit_length(d.x & 0xFFFFu), zero_first)) + __shfl_sync(kFullMask, shape, (int)bit_length(d.x >> 16));
-        bits += __shfl_sync(kFullMask, shape, (int)bit_length(d.y & 0xFFFFu)) + __shfl_sync(kFullMask, shape, (int)bit_length(d.y >> 16));
-        zero_first = 0u;
+        bits += __shfl_sync(kFullMask, shape, max(top_bit(d.x & 0xFFFFu), least)) + __shfl_sync(kFullMask, shape, top_bit(d.x >> 16));
+        bits += __shfl_sync(kFullMask, shape, top_bit(d.y & 0xFFFFu)) + __shfl_sync(kFullMask, shape, top_bit(d.y >> 16));
+        least = -1;
     }
     return bits & 0xFFFFu;
 }
@@ -235,21 +239,20 @@ __device__ __forceinline__ uint32_t run_bits(KeyRun r, uint32_t quads, uint32_t 
 // Flags, deltas and (where codes is set: 4-byte aligned, a byte per entry) codes of the lane's run, which starts with entry q0 of count
 // and with bit dpos of the blob.
 template <bool kCodes>
-__device__ __forceinline__ void write_runs(KeyRun r, uint32_t quads, uint32_t shape, uint32_t zero_first, uint32_t l, uint32_t* blob, uint32_t count,
+__device__ __forceinline__ void write_runs(KeyRun r, uint32_t quads, uint32_t shape, int least, uint32_t l, uint32_t* blob, uint32_t count,
                                            uint32_t q0, uint32_t dpos, const uint8_t* codes) {
     BitRun deltas(blob, dpos), flags(blob, 8u * count + l * q0), bytes(blob, 8u * q0);
     for (uint32_t c = 0; c < quads; ++c) {
         const uint32_t have = (uint32_t)max(0, min(4, r.left));
         const uint2 d = r.next4();
-        uint32_t f = 0u;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t delta = i == 0 ? d.x & 0xFFFFu : i == 1 ? d.x >> 16 : i == 2 ? d.y & 0xFFFFu : d.y >> 16;
-            const uint32_t x = __shfl_sync(kFullMask, shape, (int)(i ? bit_length(delta) : max(bit_length(delta), zero_first)));
-            deltas.put(delta, x & 0xFFFFu);
-            f = (f << l) | (x >> 16);
-        }
-        zero_first = 0u;
+        const uint32_t d0 = d.x & 0xFFFFu, d1 = d.x >> 16, d2 = d.y & 0xFFFFu, d3 = d.y >> 16;
+        const uint32_t x0 = __shfl_sync(kFullMask, shape, max(top_bit(d0), least)), x1 = __shfl_sync(kFullMask, shape, top_bit(d1));
+        const uint32_t x2 = __shfl_sync(kFullMask, shape, top_bit(d2)), x3 = __shfl_sync(kFullMask, shape, top_bit(d3));
+        static_assert(kGroupLog2 <= 16, "two deltas to a word");
+        deltas.put((d0 << (x1 & 0xFFFFu)) | d1, (x0 + x1) & 0xFFFFu);
+        deltas.put((d2 << (x3 & 0xFFFFu)) | d3, (x2 + x3) & 0xFFFFu);
+        const uint32_t f = ((((((x0 >> 16) << l) | (x1 >> 16)) << l) | (x2 >> 16)) << l) | (x3 >> 16);
+        least = -1;
         if (have) {                                            // (a part of four only at the end of the last run)
             flags.put(f >> (l * (4u - have)), l * have);
             if constexpr (kCodes) bytes.put(bswap32(reinterpret_cast<const uint32_t*>(codes)[c]) >> (8u * (4u - have)), 8u * have);
@@ -274,8 +277,9 @@ __device__ __forceinline__ uint32_t team_pack(uint32_t l, const uint16_t* keys, 
         team_sync<W>(id);
         top = __reduce_max_sync(kFullMask, lane < W ? s.maxd[lane] : 0u);
     }
-    const uint32_t M = max(1u, bit_length(top)), shape = delta_shape(l, M, lane), zero_first = q0 == 0u ? 1u : 0u;
-    const uint32_t bits = run_bits(r, quads, shape, zero_first), incl = warp_incl_scan(bits, lane);
+    const uint32_t M = max(1u, bit_length(top)), shape = delta_shape(l, M, lane);
+    const int least = q0 == 0u ? 0 : -1;
+    const uint32_t bits = run_bits(r, quads, shape, least), incl = warp_incl_scan(bits, lane);
     if (W > 1 && lane == 31) s.bits[w] = incl;
     // zeroes behind the codes
     if (w == 0 && lane == 0 && (count & 3u)) blob[count >> 2] &= 0xFFFFFFFFu << (32u - 8u * (count & 3u));
@@ -289,7 +293,7 @@ __device__ __forceinline__ uint32_t team_pack(uint32_t l, const uint16_t* keys, 
         all = __shfl_sync(kFullMask, xi, 31);
     }
     sized((delta0 + all + 31u) >> 5);
-    write_runs<false>(r, __any_sync(kFullMask, r.left > 0) ? quads : 0u, shape, zero_first, l, blob, count, q0, dpos, nullptr);
+    write_runs<false>(r, __any_sync(kFullMask, r.left > 0) ? quads : 0u, shape, least, l, blob, count, q0, dpos, nullptr);
     team_sync<W>(id);
     return M;
 }
@@ -324,6 +328,7 @@ __device__ __forceinline__ List list_of(const EncArgs& a, uint32_t u, const Unit
 template <int W>
 __device__ __forceinline__ uint32_t team_list(const EncArgs& a, uint32_t t, const float* thr, uint16_t* keys, uint32_t* blob, TeamScratch& s, int w, int lane, int id) {
     const float thr_e = thr[a.tau];
+    const CodeTable ct(thr, a.tau);
     const uint32_t u = 4u * t + (uint32_t)w / (W / 4), part = (uint32_t)w % (W / 4);
     const UnitInfo in = load_info(a.info + u);
     const List x = list_of(a, u, in);
@@ -357,7 +362,7 @@ __device__ __forceinline__ uint32_t team_list(const EncArgs& a, uint32_t t, cons
         if (kept) {
             const uint32_t q = rank + (uint32_t)__popc(km & below);
             keys[q] = (uint16_t)k0;
-            put_code(blob, q, code_byte_of(thr, a.tau, v0));
+            put_code(blob, q, code_byte_of(ct, v0));
         }
         rank += (uint32_t)__popc(km);
         v0 = v1; k0 = k1; v1 = v2; k1 = k2;
@@ -369,6 +374,7 @@ __device__ __forceinline__ uint32_t team_list(const EncArgs& a, uint32_t t, cons
 // The same by one warp for a whole unit, without ranks among the other units: keys and code bytes in the unit's own place.
 __device__ __forceinline__ uint32_t unit_list(const List& x, uint32_t cnt, const float* thr, uint32_t tau, uint16_t* keys, uint8_t* codes, int lane) {
     const float thr_e = thr[tau];
+    const CodeTable ct(thr, tau);
     uint32_t rank = 0u;
     const uint32_t below = (1u << lane) - 1u;
     auto value = [&](uint32_t e) -> float { return e + (uint32_t)lane < cnt ? __ldcg(x.v + e + lane) : 0.0f; };
@@ -387,7 +393,7 @@ __device__ __forceinline__ uint32_t unit_list(const List& x, uint32_t cnt, const
             if (kept) {
                 const uint32_t q = rank + (uint32_t)__popc(km & below);
                 keys[q] = (uint16_t)k[i];
-                codes[q] = (uint8_t)code_byte_of(thr, tau, v[i]);
+                codes[q] = (uint8_t)code_byte_of(ct, v[i]);
             }
             rank += (uint32_t)__popc(km);
             v[i] = nv[i]; k[i] = nk[i];
@@ -399,6 +405,7 @@ __device__ __forceinline__ uint32_t unit_list(const List& x, uint32_t cnt, const
 // The same by one warp, all candidates (off[q]: those of the units before unit q) in the units' slots.
 __device__ __forceinline__ uint32_t warp_list(const EncArgs& a, uint32_t t, const uint32_t (&off)[5], const float* thr, uint16_t* keys, uint32_t* blob, int lane) {
     const float thr_e = thr[a.tau];
+    const CodeTable ct(thr, a.tau);
     const unsigned char* slots = a.scratch + (uint64_t)t * kSlotBytes;
     auto load = [&](uint32_t e, float& v, uint32_t& k) {
         v = 0.0f; k = 0u;
@@ -420,7 +427,7 @@ __device__ __forceinline__ uint32_t warp_list(const EncArgs& a, uint32_t t, cons
         if (kept) {
             const uint32_t q = rank + (uint32_t)__popc(km & below);
             keys[q] = (uint16_t)k0;
-            put_code(blob, q, code_byte_of(thr, a.tau, v0));
+            put_code(blob, q, code_byte_of(ct, v0));
         }
         rank += (uint32_t)__popc(km);
         v0 = v1; k0 = k1; v1 = v2; k1 = k2;
@@ -435,6 +442,7 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
     const float* g = a.grad[j] + ((uint64_t)tile << kGroupLog2);
     const uint64_t left = a.n - ((uint64_t)tile << kGroupLog2);
     const float thr_e = thr[a.tau];
+    const CodeTable ct(thr, a.tau);
     // (32 loads of consecutive entries: row i of the slab's 32 rows of 32)
     uint32_t mine = 0u, mask = 0u;
 #pragma unroll 8
@@ -452,7 +460,7 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
     uint32_t pos = __shfl_sync(kFullMask, ci - c, warp) + incl - own;
     for (; mask != 0u; mask &= mask - 1u, ++pos) keys[pos] = (uint16_t)((uint32_t)warp * kSlab + 32u * (uint32_t)lane + (uint32_t)__ffs((int)mask) - 1u);
     __syncthreads();
-    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) put_code(blob, q, code_byte_of(thr, a.tau, __ldg(g + keys[q])));
+    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) put_code(blob, q, code_byte_of(ct, __ldg(g + keys[q])));
     return count;
 }
 
@@ -536,6 +544,7 @@ k_resident(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_co
     __syncthreads();
     // ---- filter; keys in order
     const float thr_e = s.thr[a.tau];
+    const CodeTable ct(s.thr, a.tau);
     uint32_t m = slab_mask(v, thr_e, lane);
     const uint32_t own = (uint32_t)__popc(m), incl = warp_incl_scan(own, lane);
     if (lane == 31) s.team.cnt[warp] = incl;
@@ -549,7 +558,7 @@ k_resident(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_co
     for (uint32_t q0 = 0; q0 < count; q0 += kEncThreads) {
         const uint32_t q = q0 + (uint32_t)tid;
         uint32_t code = 0u;
-        if (q < count) code = code_byte_of(s.thr, a.tau, s.tile[s.key[q]]);
+        if (q < count) code = code_byte_of(ct, s.tile[s.key[q]]);
         __syncthreads();
         if (q < count) put_code(s.blob, q, code);
     }
@@ -1034,8 +1043,9 @@ k_encode(const EncArgs a) {
             }
             M = max(1u, bit_length(M));
             if (lane == 0) r.prev = before;
-            const uint32_t shape = delta_shape(a.l, M, lane), zero_first = rank + q0 == 0u ? 1u : 0u;
-            const uint32_t bits = run_bits(r, quads, shape, zero_first), incl = warp_incl_scan(bits, lane);
+            const uint32_t shape = delta_shape(a.l, M, lane);
+            const int least = rank + q0 == 0u ? 0 : -1;
+            const uint32_t bits = run_bits(r, quads, shape, least), incl = warp_incl_scan(bits, lane);
             if (lane == 31) ts.bits[qw] = incl;
             if (qw == 0 && lane == 0) s.grab[quad] = atomicAdd(&s.next_mid, 1u);
             const uint32_t bound = (count * (8u + a.l + M) + 31u) >> 5, delta0 = (8u + a.l) * count;
@@ -1048,7 +1058,7 @@ k_encode(const EncArgs a) {
             for (int q = 0; q < 4; ++q) { const uint32_t y = ts.bits[q]; if (q < qw) dpos += y; words += y; }
             words = (words + 31u) >> 5;
             if (qw == 0 && lane == 0) ts.word = place_of(here, words);
-            write_runs<true>(r, quads, shape, zero_first, a.l, ar.blob, count, rank + q0, dpos, ar.code[qw] + q0);
+            write_runs<true>(r, quads, shape, least, a.l, ar.blob, count, rank + q0, dpos, ar.code[qw] + q0);
             team_sync<4>(quad);
             const uint32_t place = ts.word;
             if (place != kNoPlace) {

@@ -225,6 +225,7 @@ __device__ __forceinline__ void kv_group_pack(KvWarp& ws, const KvArgs& a, const
     if (!in_smem) __threadfence();
     __syncwarp();
     const float thr_e = thr[a.tau];
+    const CodeTable ct(thr, a.tau);
     const uint32_t inv_m = c_inv_m[M], round_up = (1u << a.l) - 1u;
     const uint32_t flag_pos0 = 8u * count;
     uint32_t prev = g << a.group_log2, rank = 0u, dpos = flag_pos0 + a.l * count;
@@ -242,7 +243,7 @@ __device__ __forceinline__ void kv_group_pack(KvWarp& ws, const KvArgs& a, const
         // several first entries and the entry may be another one's: no field is written outside [0, 32 words))
         const uint32_t q = rank + (uint32_t)__popc(b.km & ((1u << lane) - 1u));
         if (b.kept && q < count && dpos + w_incl <= 32u * words) {
-            const uint32_t code = code_byte_of(thr, a.tau, b.val);
+            const uint32_t code = code_byte_of(ct, b.val);
             const uint32_t d = w >= 32u ? b.delta : (b.delta & ((1u << w) - 1u));
             if (in_smem) {
                 put_byte_smem(blob, q, code);

@@ -151,17 +151,23 @@ __device__ __forceinline__ uint32_t flag_of(uint32_t delta, uint32_t l, uint32_t
 // to 1, and the sign: the code byte.  The search starts from an estimate of log_b(S / |v|)
 // (thr[130] = log2 S, thr[131] = 1 / log2 b, both approximate) and walks the non-increasing
 // table from there, so the result does not depend on how good the estimate is.
-__device__ __forceinline__ uint32_t code_byte_of(const float* thr, uint32_t tau, float val) {
+// (The estimate is off by one a few times in a million; the two hints are kept in registers.)
+struct CodeTable {
+    const float* thr; int tau; float h0, h1;
+    __device__ __forceinline__ CodeTable(const float* thr_, uint32_t tau_) : thr(thr_), tau((int)tau_), h0(thr_[130] * thr_[131]), h1(-thr_[131]) {}
+};
+__device__ __forceinline__ uint32_t code_byte_of(const CodeTable& t, float val) {
     const float av = fabsf(val);
     float lg;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(av));
-    uint32_t L = (uint32_t)max(1, min((int)tau, __float2int_rd(fmaf(-lg, thr[131], thr[130] * thr[131])) + 1));
-    if (av >= thr[L - 1u] || av < thr[L]) {                    // (a few in a million)
+    uint32_t L = (uint32_t)max(1, min(t.tau, __float2int_rd(fmaf(lg, t.h1, t.h0)) + 1));
+    const float* thr = t.thr;
+    if (av >= thr[L - 1u] || av < thr[L]) {
         while (L > 0u && av >= thr[L - 1u]) --L;
-        while (L < tau && av < thr[L]) ++L;
+        while (L < (uint32_t)t.tau && av < thr[L]) ++L;
         L = L < 1u ? 1u : L;
     }
-    return (val < 0.0f ? 0x80u : 0u) | (L - 1u);
+    return ((__float_as_uint(val) >> 24) & 0x80u) | (L - 1u);
 }
 
 // log2 S and 1 / log2 b only steer the table search (its result does not depend on them): single precision, and the exponent of
