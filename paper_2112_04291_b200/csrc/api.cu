@@ -14,6 +14,8 @@
 #include "bits.cuh"
 #include "prims.cuh"
 #include "encode.cuh"
+#include "groups.cuh"
+#include "place.cuh"
 #include "keys_paper.cuh"
 #include "kv.cuh"
 #include "decode.cuh"
@@ -116,22 +118,23 @@ uint32_t jobs_per_launch(uint64_t n) {
 }
 
 // The part of the workspace that depends on n, as byte offsets: per unit (a quarter of a tile of 2^14 entries) of the gradients one
-// launch can take its node of the sum tree, largest |v| and list; nodes of 512 units; per tile its descriptor and blob's place; per
-// segment of tiles its totals; the lists (a slot per unit and a pool for longer ones).  The list encoder's group entries use
+// launch can take its node of the sum tree, largest |v| and list; nodes of 512 units; per group (by default: tile) its descriptor and blob's place; per
+// segment of groups its totals; the lists (a slot per unit and a pool for longer ones).  The list encoder's group entries use
 // the descriptors' place.
 struct Layout {
     uint64_t partials, chunk, umax, info, desc, blob, seg, scratch, pool_begin, pool_bytes, end;
-    uint32_t J, tiles, chunks, seg_log2, segments;
+    uint32_t J, tiles, groups, chunks, seg_log2, segments;
 };
 Layout layout_of(uint64_t n, uint32_t group_log2) {
     Layout y;
     y.J = jobs_per_launch(n);
     y.tiles = (uint32_t)chunks_of(n);
     y.chunks = (4u * y.tiles + kChunkUnits - 1u) / kChunkUnits;
+    y.groups = (uint32_t)groups_of(n, group_log2);
     y.seg_log2 = 6u;
-    while ((uint64_t)y.J * ((y.tiles + (1ull << y.seg_log2) - 1ull) >> y.seg_log2) > kMaxSegments) ++y.seg_log2;
-    y.segments = (uint32_t)((y.tiles + (1ull << y.seg_log2) - 1ull) >> y.seg_log2);
-    const uint64_t T = (uint64_t)y.J * y.tiles, G = groups_of(n, group_log2), descs = T > G ? T : G;
+    while ((uint64_t)y.J * ((y.groups + (1ull << y.seg_log2) - 1ull) >> y.seg_log2) > kMaxSegments) ++y.seg_log2;
+    y.segments = (uint32_t)((y.groups + (1ull << y.seg_log2) - 1ull) >> y.seg_log2);
+    const uint64_t T = (uint64_t)y.J * y.tiles, descs = (uint64_t)y.J * y.groups;
     uint64_t at = kPartialsOffset;
     auto take = [&](uint64_t bytes) { const uint64_t here = at; at = (at + bytes + 255ull) & ~255ull; return here; };
     y.partials = take(32ull * T);
@@ -139,7 +142,7 @@ Layout layout_of(uint64_t n, uint32_t group_log2) {
     y.umax = take(16ull * T);
     y.info = take(4ull * sizeof(UnitInfo) * T);
     y.desc = take(8ull * descs);
-    y.blob = take(4ull * T);
+    y.blob = take(4ull * descs);
     y.seg = take(8ull * y.J * y.segments);
     // the pool: a sixth of the entries, within 2^24 (or all of a smaller gradient) and 2^27
     const uint64_t all = (uint64_t)y.J * n;
@@ -169,7 +172,9 @@ int ensure_device_setup() {
     if (cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ScanShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_encode, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EncShared)) != cudaSuccess) return FASTSGD_E_CUDA;
-    if (cudaFuncSetAttribute(k_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_place<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_place<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_compress_kv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess)
         return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_compress_kv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess)
@@ -182,7 +187,7 @@ int ensure_device_setup() {
         g_state.kv_blocks_per_sm = x < y ? x : y;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_state.res_blocks_per_sm, k_resident, kEncThreads, sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_encode, kEncThreads, sizeof(EncShared)) != cudaSuccess) return FASTSGD_E_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_place, kEncThreads, sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_place<true>, kEncThreads, sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
         g_state.enc_blocks_per_sm = x > 0 ? x : 1;
         g_state.place_blocks_per_sm = y > 0 ? y : 1;
     }
@@ -454,46 +459,8 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
     rc = ensure_device_setup();
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (params->group_log2 != (uint32_t)kGroupLog2) {
-        // Any other group size: the sum kernel, then the list encoder over the dense gradient (the fused kernel's
-        // tile is the group of 2^14).  Two launches per gradient, the gradient read three times.
-        if (params->group_log2 < 8u) return FASTSGD_E_NOT_IMPLEMENTED;
-        // sum kernel; the kept entries selected into a list in the workspace (where the default group size keeps its
-        // tiles' lists); the list encoder on that list -- or, should the list not fit, over the dense gradient itself
-        // (a warp per group: slow for large groups).  Which of the two runs is decided on the device.
-        unsigned char* wsb = static_cast<unsigned char*>(g_state.ws);
-        double* S = reinterpret_cast<double*>(wsb + kJobSumOffset);
-        unsigned long long* count_dev = reinterpret_cast<unsigned long long*>(wsb + kKvAggOffset + kKvAggBytes - 8);
-        const Layout y = layout_of(n, params->group_log2);
-        unsigned char* list = wsb + y.scratch;
-        const uint64_t capacity = ((y.end - y.scratch) / 8ull) & ~63ull;
-        for (uint32_t i = 0; i < num_grads; ++i) {
-            rc = launch_sum(grads[i], n, control_of(g_state.ws), reinterpret_cast<double*>(wsb + y.partials), S, st);
-            if (rc) return rc;
-            SelArgs sa;
-            std::memset(&sa, 0, sizeof(sa));
-            sa.grad = grads[i]; sa.n = n; sa.ctl = reinterpret_cast<Control*>(wsb);
-            sa.blk_agg = reinterpret_cast<unsigned long long*>(wsb + kKvAggOffset);
-            sa.keys = reinterpret_cast<uint32_t*>(list); sa.vals = reinterpret_cast<float*>(list + 4ull * capacity);
-            sa.count_out = count_dev; sa.capacity = capacity; sa.tau = params->tau; sa.wait_limit = g_tun.wait_limit;
-            uint64_t sgrid = (uint64_t)g_state.sm_count * 2ull;
-            const uint64_t steps = (n + 127ull) >> 7;
-            if (sgrid > (steps + kKvWarps - 1) / kKvWarps) sgrid = (steps + kKvWarps - 1) / kKvWarps;
-            if (sgrid > 511) sgrid = 511;                      // (one thread per block adds up the totals; the last slot holds the count)
-            PowTable pwc = pw;
-            void* kargs[] = {&sa, &pwc};
-            if (cudaLaunchCooperativeKernel((const void*)k_select_pairs, dim3((unsigned)sgrid), dim3(kKvThreads), kargs, 0, st) != cudaSuccess) {
-                cudaGetLastError();
-                return FASTSGD_E_CUDA;
-            }
-            g_launches.fetch_add(1, std::memory_order_relaxed);
-            rc = launch_list_encoder(false, sa.keys, sa.vals, 0, n, params, pw, outs[i], out_bytes, st, count_dev, 1u, true);
-            if (rc) return rc;
-            rc = launch_list_encoder(true, nullptr, grads[i], n, n, params, pw, outs[i], out_bytes, st, count_dev, 2u, true);
-            if (rc) return rc;
-        }
-        return FASTSGD_OK;
-    }
+    if (params->group_log2 < 8u) return FASTSGD_E_NOT_IMPLEMENTED;
+    const bool tile_groups = params->group_log2 == (uint32_t)kGroupLog2;
     const Layout y = layout_of(n, params->group_log2);
     unsigned char* wsb = static_cast<unsigned char*>(g_state.ws);
     PowTable inv = inverse_of(pw);
@@ -515,13 +482,13 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
         ea.blob = reinterpret_cast<uint32_t*>(wsb + y.blob);
         ea.seg = reinterpret_cast<unsigned long long*>(wsb + y.seg); ea.seg_log2 = y.seg_log2; ea.segments = y.segments;
         ea.scratch = wsb + y.scratch; ea.pool_begin = y.pool_begin; ea.pool_bytes = y.pool_bytes;
-        ea.base = params->base; ea.inv_ptau = inv.P[params->tau]; ea.G = y.tiles;
+        ea.base = params->base; ea.inv_ptau = inv.P[params->tau]; ea.G = y.tiles; ea.D = y.groups; ea.group_log2 = params->group_log2;
         ea.tau = params->tau; ea.l = params->flag_bits; ea.wait_limit = g_tun.wait_limit; ea.try_limit = g_tun.try_limit;
         const uint64_t tiles = (uint64_t)ea.J * ea.G;
         void* kargs[] = {&ea, &pw, &inv};
         // every tile on the GPU at once (a single block waits for nobody, so it need not be launched cooperatively)
         const uint64_t resident = (uint64_t)g_state.sm_count * (uint64_t)(g_state.res_blocks_per_sm > 0 ? g_state.res_blocks_per_sm : 0);
-        if (tiles <= resident && tiles <= kMaxResident && (!g_tun.grid_override || tiles <= g_tun.grid_override)) {
+        if (tile_groups && tiles <= resident && tiles <= kMaxResident && (!g_tun.grid_override || tiles <= g_tun.grid_override)) {
             LaunchTimer lt(1, st);
             const cudaError_t err = tiles == 1u ? launch_overlapped((const void*)k_resident, 1u, kEncThreads, sizeof(ResShared), kargs, st)
                                                 : cudaLaunchCooperativeKernel((const void*)k_resident, dim3((unsigned)tiles), dim3(kEncThreads), kargs, sizeof(ResShared), st);
@@ -542,14 +509,18 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
         ea.samplers = (uint32_t)g1 / ea.J < kSampleBlocks ? (uint32_t)g1 / ea.J : kSampleBlocks;      // (none: no estimate, every tile is read again)
         {
             LaunchTimer lt(1, st);
-            if (launch_overlapped((const void*)k_scan, (unsigned)g1, kScanThreads, sizeof(ScanShared), kargs, st) != cudaSuccess ||
-                launch_overlapped((const void*)k_encode, (unsigned)g2, kEncThreads, sizeof(EncShared), kargs, st) != cudaSuccess ||
-                launch_overlapped((const void*)k_place, (unsigned)g3, kEncThreads, sizeof(PlaceShared), kargs, st) != cudaSuccess) {
-                cudaGetLastError();
-                return FASTSGD_E_CUDA;
+            cudaError_t err = launch_overlapped((const void*)k_scan, (unsigned)g1, kScanThreads, sizeof(ScanShared), kargs, st);
+            if (tile_groups) {
+                if (err == cudaSuccess) err = launch_overlapped((const void*)k_encode, (unsigned)g2, kEncThreads, sizeof(EncShared), kargs, st);
+                if (err == cudaSuccess) err = launch_overlapped((const void*)k_place<true>, (unsigned)g3, kEncThreads, sizeof(PlaceShared), kargs, st);
+            } else {
+                if (err == cudaSuccess) err = launch_overlapped((const void*)k_filter, (unsigned)g2, kEncThreads, 0, kargs, st);
+                if (err == cudaSuccess) err = launch_overlapped((const void*)k_groups, (unsigned)g2, kEncThreads, sizeof(GroupShared), kargs, st);
+                if (err == cudaSuccess) err = launch_overlapped((const void*)k_place<false>, (unsigned)g3, kEncThreads, sizeof(PlaceShared), kargs, st);
             }
+            if (err != cudaSuccess) { cudaGetLastError(); return FASTSGD_E_CUDA; }
         }
-        g_launches.fetch_add(3, std::memory_order_relaxed);
+        g_launches.fetch_add(tile_groups ? 3 : 4, std::memory_order_relaxed);
     }
     return FASTSGD_OK;
 }

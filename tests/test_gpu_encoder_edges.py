@@ -57,3 +57,49 @@ def test_tiles_of_a_launch(workers, tiles):
 def test_tau_below_the_largest_and_no_entry_kept():
     _check([_tiles(5 * TILE + 1, (700, 3), 5)], 1.5, tau=40)
     _check([np.zeros(5 * TILE + 1, np.float32), _tiles(5 * TILE + 1, (0, 0, 1), 6)], 1.2)
+
+
+def _check_groups(v, base, group_log2, l=2, tau=128):
+    n = v.size
+    pg, po = binding.params(base, tau, l, group_log2), oracle.params(base, tau, l, group_log2)
+    binding.ensure_workspace(n, pg)
+    cap = (binding.compress_bound(n, pg) + 255) & ~255
+    buf, dev = G.Guarded(cap, fill=0x5C), G.to_dev(v)
+    rc, want = oracle.compress(v, po)
+    for rep in range(2):
+        assert binding.compress(dev, pg, buf.view) == 0
+        total, d, status = binding.stream_info(buf.view)
+        assert status == rc == 0 and total == want.size and buf.intact()
+        assert np.array_equal(buf.view[:total].cpu().numpy(), want)
+
+
+# other group sizes: a unit of 4096 entries is up to 16 groups, a group up to 256 units; kept entries around what a warp takes (512),
+# what the block takes at a time (4096), and more; tiles without, with few and with only kept entries
+@pytest.mark.parametrize("group_log2", [8, 11, 12, 13, 16, 20])
+@pytest.mark.parametrize("counts", [(0, 1), (127, 129), (511, 513, 0, 2047), (4095, 4097), (TILE, 0, TILE - 1)])
+def test_other_group_sizes(group_log2, counts):
+    _check_groups(_tiles(11 * TILE - 5, counts, 40 + counts[0]), 1.2, group_log2, l=1 + counts[0] % 5)
+
+
+def test_other_group_sizes_many_tiles():
+    for group_log2 in (10, 15, 18):
+        _check_groups(_tiles(400 * TILE + 7, (3, 0, 0, 0, 40, 900, 0, TILE), group_log2), 1.2, group_log2)
+
+
+# a sample that misses what matters (the estimate is too high where a few entries carry the sum): tiles are read again
+@pytest.mark.parametrize("group_log2", [10, 14, 17])
+def test_tiles_read_again(group_log2):
+    n = 310 * TILE + 1
+    rng = np.random.default_rng(3)
+    v = (rng.standard_normal(n) * 1e-3).astype(np.float32)
+    v[::4 * 101] += 50.0
+    v[1::3001] *= 30.0
+    _check_groups(v, 1.05, group_log2)
+    _check_groups(v, 1.1, group_log2)
+
+
+# more blobs than the workspace has room for: packed where they belong in the stream
+@pytest.mark.parametrize("group_log2", [9, 14, 16])
+def test_blobs_without_room(group_log2):
+    n = (1 << 26) + 3
+    _check_groups(np.where(np.arange(n) % 7, np.float32(1.0), np.float32(-2.0)).astype(np.float32), 1.2, group_log2, l=5)
