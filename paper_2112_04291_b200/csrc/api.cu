@@ -175,16 +175,11 @@ int ensure_device_setup() {
     if (cudaFuncSetAttribute(k_place<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_place<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
     if (cudaFuncSetAttribute(k_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupShared)) != cudaSuccess) return FASTSGD_E_CUDA;
-    if (cudaFuncSetAttribute(k_compress_kv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess)
-        return FASTSGD_E_CUDA;
-    if (cudaFuncSetAttribute(k_compress_kv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess)
-        return FASTSGD_E_CUDA;
+    if (cudaFuncSetAttribute(k_compress_kv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
     int b1 = 0, b2 = 0;
     {
         int x = 0, y = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_compress_kv<false>, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_compress_kv<true>, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
-        g_state.kv_blocks_per_sm = x < y ? x : y;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_state.kv_blocks_per_sm, k_compress_kv, kKvThreads, sizeof(KvSmem)) != cudaSuccess) return FASTSGD_E_CUDA;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_state.res_blocks_per_sm, k_resident, kEncThreads, sizeof(ResShared)) != cudaSuccess) return FASTSGD_E_CUDA;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_encode, kEncThreads, sizeof(EncShared)) != cudaSuccess) return FASTSGD_E_CUDA;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_place<true>, kEncThreads, sizeof(PlaceShared)) != cudaSuccess) return FASTSGD_E_CUDA;
@@ -390,47 +385,40 @@ int fastsgd_abs_sum(const float* grad, uint64_t n, double* sum_out, void* stream
 }
 
 namespace {
-// The list encoder (kv.cuh).  dense = false: `count` key-value pairs.  dense = true: the gradient `values` of n
-// entries itself, read as the list (i, v_i), with its sum already in the workspace.  Caller holds g_state.mu.
-int launch_list_encoder(bool dense, const uint32_t* keys, const float* values, uint64_t count, uint64_t n,
-                        const fastsgd_params* params, const PowTable& pw, void* out, uint64_t out_bytes, cudaStream_t st,
-                        const unsigned long long* count_dev = nullptr, uint32_t run_if = 0u, bool given_sum = false) {
+// The list encoder (kv.cuh).  Caller holds g_state.mu.
+int launch_list_encoder(const uint32_t* keys, const float* values, uint64_t count, uint64_t n,
+                        const fastsgd_params* params, const PowTable& pw, void* out, uint64_t out_bytes, cudaStream_t st) {
     FSG_DEVICE_STATE();
     if (g_state.kv_blocks_per_sm < 1) return FASTSGD_E_CUDA;
-    const uint64_t G = groups_of(n, params->group_log2);
     const Layout y = layout_of(n, params->group_log2);
     KvArgs ka;
     std::memset(&ka, 0, sizeof(ka));
-    ka.keys = keys; ka.vals = values; ka.count = dense ? n : count; ka.n = n;
+    ka.keys = keys; ka.vals = values; ka.count = count; ka.n = n;
     ka.out = static_cast<uint8_t*>(out); ka.out_bytes = out_bytes; ka.ctl = control_of(g_state.ws);
     ka.partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + kKvPartialsOffset);
     ka.meta = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + y.desc);
     ka.blk_agg = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + kKvAggOffset);
-    ka.base = params->base; ka.G = (uint32_t)G; ka.chunks = (uint32_t)chunks_of(n);
+    ka.base = params->base; ka.G = y.groups; ka.chunks = y.tiles;
     ka.tau = params->tau; ka.l = params->flag_bits; ka.group_log2 = params->group_log2;
-    ka.wait_limit = g_tun.wait_limit; ka.given_sum = (dense || given_sum) ? 1u : 0u;
-    ka.count_dev = count_dev; ka.run_if = run_if;
-    // a warp per 32 list entries (dense: per group) until the GPU is full; all blocks are resident: they meet at grid barriers
-    const uint64_t units = dense ? G : (count_dev ? n : count);      // (a list made on the device: its length is not known here)
-    const uint64_t per_warp = dense ? 1ull : 32ull;
-    uint64_t grid = (units + per_warp * kKvWarps - 1) / (per_warp * kKvWarps);
+    ka.wait_limit = g_tun.wait_limit;
+    // all blocks are resident (they meet at grid barriers).  A warp per kKvSlice entries until the GPU is full: a warp works off its
+    // chunks and groups one after the other, and the runs of a sparse gradient put a new one every few entries.
+    uint64_t grid = (count + kKvSlice * kKvWarps - 1) / (kKvSlice * kKvWarps);
     const uint64_t cap = (uint64_t)g_state.sm_count * (uint64_t)(g_state.kv_blocks_per_sm > 2 ? 2 : g_state.kv_blocks_per_sm);
     if (grid > cap) grid = cap;
     if (grid > kKvMaxGrid) grid = kKvMaxGrid;
     if (g_tun.grid_override && g_tun.grid_override < grid) grid = g_tun.grid_override;
     if (grid < 1) grid = 1;
     const uint64_t warps = grid * kKvWarps;
-    uint64_t slice = (units + warps - 1) / warps;
-    if (!dense) slice = (slice + 31ull) & ~31ull;
-    if (slice < per_warp) slice = per_warp;
+    uint64_t slice = ((count + warps - 1) / warps + kKvSlice - 1) / kKvSlice * kKvSlice;
+    if (slice < kKvSlice) slice = kKvSlice;
     ka.slice = (uint32_t)slice;
     PowTable pwc = pw;
     void* kargs[] = {&ka, &pwc};
     cudaError_t err;
     {
         LaunchTimer lt(1, st);
-        err = cudaLaunchCooperativeKernel(dense ? (const void*)k_compress_kv<true> : (const void*)k_compress_kv<false>,
-                                          dim3((unsigned)grid), dim3(kKvThreads), kargs, sizeof(KvSmem), st);
+        err = cudaLaunchCooperativeKernel((const void*)k_compress_kv, dim3((unsigned)grid), dim3(kKvThreads), kargs, sizeof(KvSmem), st);
     }
     if (err != cudaSuccess) { cudaGetLastError(); return FASTSGD_E_CUDA; }
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -551,7 +539,7 @@ int fastsgd_compress_kv(const uint32_t* keys, const float* values, uint64_t coun
     if (!g_state.ws || g_state.timed_out || g_state.ws_bytes < ws_bytes_for(n, params->group_log2)) return FASTSGD_E_NO_WORKSPACE;
     rc = ensure_device_setup();
     if (rc) return rc;
-    return launch_list_encoder(false, keys, values, count, n, params, pw, out, out_bytes, static_cast<cudaStream_t>(stream));
+    return launch_list_encoder(keys, values, count, n, params, pw, out, out_bytes, static_cast<cudaStream_t>(stream));
 }
 
 int fastsgd_compress(const float* grad, uint64_t n, const fastsgd_params* params,
