@@ -397,7 +397,7 @@ int launch_list_encoder(const uint32_t* keys, const float* values, uint64_t coun
     ka.out = static_cast<uint8_t*>(out); ka.out_bytes = out_bytes; ka.ctl = control_of(g_state.ws);
     ka.partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + kKvPartialsOffset);
     ka.meta = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + y.desc);
-    ka.blk_agg = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + kKvAggOffset);
+    ka.st = reinterpret_cast<EncState*>(static_cast<unsigned char*>(g_state.ws) + kEncStateOffset);
     ka.base = params->base; ka.G = y.groups; ka.chunks = y.tiles;
     ka.tau = params->tau; ka.l = params->flag_bits; ka.group_log2 = params->group_log2;
     ka.wait_limit = g_tun.wait_limit;

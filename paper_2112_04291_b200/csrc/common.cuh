@@ -39,21 +39,18 @@ struct Control {
     unsigned int       exit_count;     // blocks of the running one that have finished (self-resetting)
     unsigned int       dq[6];          // decoder work queue: -, taken, done, exited, reserved (zero between launches)
     unsigned int       pad2[24];
-    unsigned int       bar_count[8];   // k_resident: tiles of each gradient that have been summed; [0] k_scan: blocks that have finished; list encoder: arrivals at its grid barriers (zero between launches)
-    unsigned int       bar_flag[8];    // list encoder: set to bar_gen + 1 when a grid barrier opens
+    unsigned int       bar_count[8];   // k_resident: tiles of each gradient that have been summed; [0] k_scan: blocks that have finished; list encoder: arrivals at its grid barrier (zero between launches)
+    unsigned int       pad3[8];
     unsigned int       ne_count[8];    // tiles of each gradient that the last encoder launch read a second time
 };
 static_assert(sizeof(Control) == 256, "control block is 256 bytes");
 
-constexpr uint64_t kJobSumOffset   = 800;    // double: the sum of the list encoder's gradient
 constexpr uint64_t kEncStateOffset = 1024;   // EncState (encode.cuh)
 constexpr uint64_t kQueueOffset    = 32768;  // u32 queue[2^17]: decoder's grid-wide queue of groups (zero between launches)
 constexpr uint64_t kQueueBytes     = 4ull << 17;
 constexpr uint64_t kKvPartialsOffset = kQueueOffset + kQueueBytes;   // double [2^17]: chunk nodes of the key-value encoder's sum (zero between launches)
 constexpr uint64_t kKvPartialsBytes  = 8ull << 17;
-constexpr uint64_t kKvAggOffset    = kKvPartialsOffset + kKvPartialsBytes;   // u64 [512]: per-block totals of the key-value encoder
-constexpr uint64_t kKvAggBytes     = 8ull * 512ull;
-constexpr uint64_t kPartialsOffset = kKvAggOffset + kKvAggBytes;     // from here on the layout depends on n (api.cu)
+constexpr uint64_t kPartialsOffset = kKvPartialsOffset + kKvPartialsBytes;     // from here on the layout depends on n (api.cu)
 
 __host__ __device__ inline uint64_t ceil_div_u64(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 

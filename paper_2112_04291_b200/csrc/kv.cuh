@@ -10,13 +10,15 @@
 //   pass 1  sum (Algorithm 1, first step): per chunk with entries, its node of the fixed fp64 tree.  Zeros add
 //           exactly nothing, so only the units with entries are formed: a unit's 128 leaves in shared memory and
 //           its node by the usual tree, the 128 unit nodes of the chunk by the same tree one level up.  The
-//           chunk nodes go to an array that is zero between launches; the last block to arrive at the grid
-//           barrier reduces it on the top of the tree (the very code of the dense encoder), stores S and
-//           clears it again.
+//           chunk nodes go to an array that is zero between launches; behind a grid barrier every block
+//           reduces it on the top of the tree for itself.
 //   pass 2  sizes: per group with entries, the threshold filter |v| >= B_tau, the delta keys (Eq. 4), their
 //           largest (hence M) and a histogram of their bit lengths (hence the payload bits); the group's
 //           (count, M, words) is left in the workspace, the block's totals in a table of one entry per block.
-//   grid barrier; every block adds up the totals of the blocks before it: its place in the stream.
+//   every block takes the totals of all blocks (tagged words) and adds up those before it: its place in the stream.
+//
+// The launch is a chain of a dozen round trips to the L2 whatever the number of pairs.  50 M / 50000 pairs: 22.6 -> 21.0 us (2^20 / 4000: 21.6 -> 17.3) when the
+// sum no longer went through the last block to arrive and the sizes no longer through a barrier.
 //   pass 3  pack: per group again, codes || flags || deltas packed in the warp's shared memory (in place in the
 //           stream for blobs too long for it), copied out, with the group's directory entry and those of the
 //           groups without entries before it.  The owner of the last group with entries writes the header.
@@ -29,6 +31,7 @@
 #include "sum.cuh"
 #include "bits.cuh"
 #include "prims.cuh"
+#include "encode.cuh"       // exchange words of the workspace
 
 namespace fsg {
 
@@ -37,7 +40,7 @@ constexpr int      kKvWarps      = kKvThreads / 32;
 constexpr uint32_t kKvStageWords = 256;               // blobs up to this many words are packed in shared memory
 constexpr uint32_t kKvUnit       = 128;               // leaves of the sum tree formed at a time (4 per lane)
 constexpr uint64_t kKvSlice      = 16;                // list entries a warp starts with at least
-constexpr uint32_t kKvMaxGrid    = 512;               // one thread per block adds up the blocks' totals
+constexpr uint32_t kKvMaxGrid    = kMaxResident;      // one thread per block adds up the blocks' totals
 
 struct KvArgs {
     const uint32_t*     keys;        // ascending, each < n
@@ -49,7 +52,7 @@ struct KvArgs {
     Control*            ctl;
     double*             partials;    // [chunks], all zero between launches
     unsigned long long* meta;        // [G]: count | M << 24 | words << 32 of the groups with entries
-    unsigned long long* blk_agg;     // [gridDim.x]: kept entries << 32 | blob words of each block's groups
+    EncState*           st;          // res_node[2 b]: kept entries << 32 | blob words of block b's groups, and the launch's tag
     double              base;
     uint32_t            G;           // groups: ceil(n / 2^group_log2)
     uint32_t            chunks;      // ceil(n / 2^14)
@@ -61,7 +64,7 @@ struct KvArgs {
 };
 
 struct KvWarp {
-    float    unit[kKvUnit];          // leaves of the unit being formed; all zero between units
+    alignas(16) float unit[kKvUnit];  // leaves of the unit being formed; all zero between units
     double   usum[128];              // the chunk's unit nodes (2^14 / 128 of them)
     uint32_t hist[40];               // kept deltas of the group by bit length
     uint32_t stage[kKvStageWords];   // the blob being packed (big-endian valued words)
@@ -75,7 +78,7 @@ struct KvSmem {
     uint32_t wcount[kKvWarps], wwords[kKvWarps];   // pass 2: kept entries and blob words of each warp's groups
     uint32_t flag;                   // block-wide answers of thread 0
     uint32_t abort_flag;
-    double   S;
+    double   pk[132];                // b^k (a thread per entry reads them from the parameters slowly: ahead of time)
     KvWarp   w[kKvWarps];
 };
 
@@ -283,32 +286,6 @@ __device__ __forceinline__ void kv_write_header(const KvArgs& a, int status, uin
     outw[15] = a.G;
 }
 
-// Grid barrier `which` (0 or 1) of the launch, first half.  Returns true in every thread of the one block that
-// arrived last (it sets the flag itself once it has done what everybody waits for).
-__device__ __forceinline__ bool kv_barrier_arrive(KvSmem& s, Control* ctl, int which, int tid) {
-    __syncthreads();
-    if (tid == 0) {
-        s.flag = 0u;
-        if (!s.abort_flag) s.flag = atom_add_acq_rel_u32(&ctl->bar_count[which], 1u) == gridDim.x - 1u ? 1u : 0u;
-    }
-    __syncthreads();
-    return s.flag != 0u;
-}
-__device__ __forceinline__ void kv_barrier_release(Control* ctl, int which, unsigned int gen_next) {
-    ctl->bar_count[which] = 0u;
-    st_release_u32(&ctl->bar_flag[which], gen_next);
-}
-__device__ __forceinline__ void kv_barrier_wait(KvSmem& s, Control* ctl, int which, unsigned int gen_next, uint32_t limit, int tid) {
-    if (tid == 0 && !s.abort_flag) {
-        uint32_t spin = 0;
-        while (ld_acquire_u32(&ctl->bar_flag[which]) != gen_next) {
-            if (++spin > limit) { s.abort_flag = 1u; break; }
-            if (spin > 64u) __nanosleep(32);
-        }
-    }
-    __syncthreads();
-}
-
 // Calls f(head entry, group or chunk number, key of the entry before the head or 0xFFFFFFFF) for every unit of 2^shift
 // indices whose first entry lies in the warp's slice [lo, hi) of the list, in list order.
 template <typename F>
@@ -343,6 +320,7 @@ k_compress_kv(const KvArgs a, const __grid_constant__ PowTable pw) {
         s.flag = gen_next;
     }
     for (uint32_t i = lane; i < kKvUnit; i += 32u) ws.unit[i] = 0.f;
+    if (tid <= (int)a.tau) s.pk[tid] = pw.P[tid];
     __syncthreads();
     gen_next = s.flag;
 
@@ -351,32 +329,23 @@ k_compress_kv(const KvArgs a, const __grid_constant__ PowTable pw) {
     const uint64_t lo = min(a.count, gw * (uint64_t)a.slice), hi = min(a.count, lo + (uint64_t)a.slice);
 
     // ---- pass 1: the chunks whose first entry lies in the slice
-    {
-        kv_for_each_head(a, lo, hi, (uint32_t)kChunkLog2, a.chunks, lane,
-                                [&](uint64_t head_e, uint32_t c, uint32_t) { kv_sum_chunk(ws, a, head_e, c, lane); });
-        // ---- grid barrier; the last block to arrive reduces the chunk nodes (same tree, same code as the dense encoder)
-        if (kv_barrier_arrive(s, a.ctl, 0, tid)) {
-            const double S = a.chunks > 8192u ? reduce_partials<true>(a.partials, a.chunks, s.s_tree, s.s_nodes, tid, lane, warp)
-                                                     : reduce_partials<false>(a.partials, a.chunks, s.s_tree, s.s_nodes, tid, lane, warp);
-            __syncthreads();
-            for (uint32_t i = tid; i < a.chunks; i += kKvThreads) a.partials[i] = 0.0;     // at rest again
-            __syncthreads();
-            if (tid == 0) {
-                __threadfence();
-                reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(a.ctl) + kJobSumOffset)[0] = S;
-                kv_barrier_release(a.ctl, 0, gen_next);
-            }
+    kv_for_each_head(a, lo, hi, (uint32_t)kChunkLog2, a.chunks, lane, [&](uint64_t head_e, uint32_t c, uint32_t) { kv_sum_chunk(ws, a, head_e, c, lane); });
+    // ---- grid barrier; then every block reduces the chunk nodes for itself (same tree, same code)
+    __syncthreads();
+    if (tid == 0) {
+        atom_add_acq_rel_u32(&a.ctl->bar_count[0], 1u);
+        uint32_t spin = 0;
+        while (ld_acquire_u32(&a.ctl->bar_count[0]) != gridDim.x) {
+            if (++spin > a.wait_limit) { s.abort_flag = 1u; break; }
         }
-        kv_barrier_wait(s, a.ctl, 0, gen_next, a.wait_limit, tid);
     }
+    __syncthreads();
+    const double S = reduce_partials(a.partials, a.chunks, s.s_tree, s.s_nodes, tid, lane, warp);
 
     // ---- boundary table RU32(B_k), as the dense encoder forms it
-    if (tid == 0) s.S = __ldcg(reinterpret_cast<const double*>(reinterpret_cast<const unsigned char*>(a.ctl) + kJobSumOffset));
-    __syncthreads();
-    const double S = s.S;
     const bool finite = isfinite(S);
     if (tid <= (int)a.tau)
-        s.thr[tid] = (finite && S != 0.0) ? fmaxf(__double2float_ru(__ddiv_rn(S, pw.P[tid])), __int_as_float(1)) : __int_as_float(0x7f800000);
+        s.thr[tid] = (finite && S != 0.0) ? fmaxf(__double2float_ru(__ddiv_rn(S, s.pk[tid])), __int_as_float(1)) : __int_as_float(0x7f800000);
     if (tid == 0) table_hints(S, a.base, &s.thr[130]);
     __syncthreads();
     const float thr_e = s.thr[a.tau];
@@ -394,20 +363,30 @@ k_compress_kv(const KvArgs a, const __grid_constant__ PowTable pw) {
     }
     if (lane == 0) { s.wcount[warp] = my_count; s.wwords[warp] = my_words; }
     __syncthreads();
-    if (tid == 0) {
-        unsigned long long agg = 0ull;
-        for (int w = 0; w < kKvWarps; ++w) agg += ((unsigned long long)s.wcount[w] << 32) | s.wwords[w];
-        st_relaxed_u64(a.blk_agg + blockIdx.x, agg);
+    // ---- every block takes all blocks' totals: its place in the stream
+    unsigned long long mine = 0ull;
+    if (!aborted1) {
+        if (tid == 0) {
+            unsigned long long agg = 0ull;
+            for (int w = 0; w < kKvWarps; ++w) agg += ((unsigned long long)s.wcount[w] << 32) | s.wwords[w];
+            st_relaxed_pair(a.st->res_node + 2u * blockIdx.x, agg, gen_next);
+        }
+        if ((uint32_t)tid < gridDim.x) {
+            unsigned long long tag;
+            uint32_t spin = 0;
+            for (;;) {
+                ld_relaxed_pair(a.st->res_node + 2u * (uint32_t)tid, mine, tag);
+                if (tag == gen_next) break;
+                if (++spin > a.wait_limit) { s.abort_flag = 1u; break; }
+            }
+        }
     }
-    // ---- grid barrier; then every block adds up the totals of the blocks before it
-    if (kv_barrier_arrive(s, a.ctl, 1, tid)) {
-        if (tid == 0) kv_barrier_release(a.ctl, 1, gen_next);
-    }
-    kv_barrier_wait(s, a.ctl, 1, gen_next, a.wait_limit, tid);
+    __syncthreads();
     const bool aborted = s.abort_flag != 0u;
 
     if (!aborted) {
-        unsigned long long mine = (uint32_t)tid < gridDim.x ? ld_relaxed_u64(a.blk_agg + tid) : 0ull;
+        // (every block has its sum: the nodes are zero again for the next launch)
+        for (uint32_t i = blockIdx.x * kKvThreads + (uint32_t)tid; i < a.chunks; i += gridDim.x * kKvThreads) a.partials[i] = 0.0;
         unsigned long long before = (uint32_t)tid < blockIdx.x ? mine : 0ull;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -475,6 +454,7 @@ k_compress_kv(const KvArgs a, const __grid_constant__ PowTable pw) {
         if (old == gridDim.x - 1u) {
             if (ld_acquire_u32(&a.ctl->error) != 0u) kv_write_header(a, kStTimeout, 0ull, 0ull, 0.0);
             a.ctl->exit_count = 0u;
+            a.ctl->bar_count[0] = 0u;
             st_release_u32(&a.ctl->bar_gen, gen_next);
         }
     }

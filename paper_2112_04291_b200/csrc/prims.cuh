@@ -73,10 +73,7 @@ __device__ __forceinline__ unsigned int atom_add_acq_rel_u32(unsigned int* p, un
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
 }
-// Tree reduction of the per-tile partials by one block, in passes of 512
-// consecutive partials: thread t takes partial 512*p + t, the block forms that aligned node by
-// shuffles (positions = lanes, then warps); the nodes of the passes are then reduced the same
-// way.  Everything stays in registers and shared memory.
+// The node of the block's values on the tree (positions: lanes, then warps), in every thread.
 __device__ __forceinline__ double block_tree(double x, double* s_tree, int lane, int warp) {
     x = warp_tree(x);
     __syncthreads();                                   // s_tree may still be read from the last use
@@ -87,48 +84,22 @@ __device__ __forceinline__ double block_tree(double x, double* s_tree, int lane,
     return __shfl_sync(kFullMask, t, 0);
 }
 
-// BIG: with more than 8 passes a warp forms the node of a whole pass by itself (16 partials per lane,
-// all in flight at once; the same tree by the transposing shuffle pattern) and the warps take the
-// passes in turn.  (With few passes the block-wide form has the shorter chain.)
-template <bool BIG>
+// Tree reduction of up to 2^17 partials by one block, 512 to a node: a warp forms a node by itself (16 partials per lane, all in flight
+// at once, consecutive across the warp), the block the rest.  (A run of 8 per thread instead, 64 bytes apart across a warp: 5 us
+// slower with all blocks at it.)
 __device__ __forceinline__ double reduce_partials(const double* partials, uint32_t chunks, double* s_tree,
                                                   double* s_nodes, int tid, int lane, int warp) {
     const uint32_t passes = (chunks + kBlockThreads - 1) / kBlockThreads;       // <= 256 for n < 2^31
-    if (passes <= 8) {
-        // thread t folds the aligned run of R = 1, 2, 4 or 8 partials that starts at R*t (all loads in
-        // flight at once), then one tree over the threads: the same tree, one barrier pair
-        const uint32_t R = passes <= 1 ? 1u : (passes <= 2 ? 2u : (passes <= 4 ? 4u : 8u));
-        double v[8];
+    if (passes <= 1u) return block_tree((uint32_t)tid < chunks ? __ldcg(partials + tid) : 0.0, s_tree, lane, warp);
+    for (uint32_t p = (uint32_t)warp; p < passes; p += kBlockWarps) {
+        double x[16];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const uint64_t idx = (uint64_t)tid * R + k;
-            v[k] = ((uint32_t)k < R && idx < chunks) ? __ldcg(partials + idx) : 0.0;
+        for (int j = 0; j < 16; ++j) {
+            const uint64_t idx = (uint64_t)p * kBlockThreads + 32u * (uint32_t)j + (uint32_t)lane;
+            x[j] = idx < chunks ? __ldcg(partials + idx) : 0.0;
         }
-        // with R < 8 the unused slots are zero and x + 0 = x, so the full 8-leaf tree is still exact
-        const double x = __dadd_rn(__dadd_rn(__dadd_rn(v[0], v[1]), __dadd_rn(v[2], v[3])),
-                                   __dadd_rn(__dadd_rn(v[4], v[5]), __dadd_rn(v[6], v[7])));
-        return block_tree(x, s_tree, lane, warp);
-    }
-    if constexpr (BIG) {
-        for (uint32_t p = (uint32_t)warp; p < passes; p += kBlockWarps) {
-            double x[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const uint64_t idx = (uint64_t)p * kBlockThreads + 32u * (uint32_t)j + (uint32_t)lane;
-                x[j] = idx < chunks ? __ldcg(partials + idx) : 0.0;
-            }
-            const double node = warp_rows16_tree(x, lane);
-            if (lane == 0) s_nodes[p] = node;
-        }
-    } else {
-    double next = (uint32_t)tid < chunks ? __ldcg(partials + tid) : 0.0;
-    for (uint32_t p = 0; p < passes; ++p) {
-        const double x = next;
-        const uint64_t idx = (uint64_t)(p + 1) * kBlockThreads + tid;
-        next = (p + 1 < passes && idx < chunks) ? __ldcg(partials + idx) : 0.0;    // in flight during this pass
-        const double node = block_tree(x, s_tree, lane, warp);
-        if (tid == 0) s_nodes[p] = node;
-    }
+        const double node = warp_rows16_tree(x, lane);
+        if (lane == 0) s_nodes[p] = node;
     }
     __syncthreads();
     // the nodes of the passes, zero-padded to 512 positions, reduced on the same tree
