@@ -698,33 +698,32 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
             if (lane == 0) st_relaxed_u64(&a.st->sample[sj][si], ((unsigned long long)__float_as_uint(sx) << 32) | max(__float_as_uint(sy), 1u));
         }
     }
-    if (warp == 0) {
-        // every block forms the estimates by itself: lane <-> sampling block.  Margin: 2 % and three standard errors of the mean of k samples
-        static_assert(kSampleBlocks == 32u, "a lane per sampling block");
-        for (uint32_t j = 0; j < a.J; ++j) {
-            unsigned long long v = 1ull;
-            if ((uint32_t)lane < a.samplers)
-                for (uint32_t p = 0; p < kSamplePolls; ++p) if ((v = ld_relaxed_u64(&a.st->sample[j][lane])) != 0ull) break;
-            const bool all = __all_sync(kFullMask, v != 0ull);
-            float x = __uint_as_float((uint32_t)(v >> 32)), y = __uint_as_float((uint32_t)v);
-            if ((uint32_t)lane >= a.samplers) x = y = 0.0f;
+    if (warp < (int)a.J) {
+        // every block forms the estimates by itself: warp <-> gradient, lane <-> sampling block.  Margin: 2 % and three standard errors of the
+        // mean of k samples
+        static_assert(kSampleBlocks == 32u && kEncMaxJobs < kScanWarps, "a lane per sampling block, a warp per gradient");
+        unsigned long long v = 1ull;
+        if ((uint32_t)lane < a.samplers)
+            for (uint32_t p = 0; p < kSamplePolls; ++p) if ((v = ld_relaxed_u64(&a.st->sample[warp][lane])) != 0ull) break;
+        const bool all = __all_sync(kFullMask, v != 0ull);
+        float x = __uint_as_float((uint32_t)(v >> 32)), y = __uint_as_float((uint32_t)v);
+        if ((uint32_t)lane >= a.samplers) x = y = 0.0f;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) { x += __shfl_xor_sync(kFullMask, x, o); y += __shfl_xor_sync(kFullMask, y, o); }
-            const float k = (float)(a.samplers * (uint32_t)kScanThreads), mean = x / k, var = fmaxf(y / k - mean * mean, 0.0f), margin = 0.02f + 3.0f * sqrtf(var / k) / mean;
-            const float e = (float)((double)(mean * (1.0f - margin)) * (double)a.n * 0.25 * a.inv_ptau);
-            if (lane == 0) s.est[j] = all && margin < 0.75f && e > 0.0f ? e : -1.0f;
-        }
+        for (int o = 16; o > 0; o >>= 1) { x += __shfl_xor_sync(kFullMask, x, o); y += __shfl_xor_sync(kFullMask, y, o); }
+        const float k = (float)(a.samplers * (uint32_t)kScanThreads), mean = x / k, var = fmaxf(y / k - mean * mean, 0.0f), margin = 0.02f + 3.0f * sqrtf(var / k) / mean;
+        const float e = (float)((double)(mean * (1.0f - margin)) * (double)a.n * 0.25 * a.inv_ptau);
+        if (lane == 0) s.est[warp] = all && margin < 0.75f && e > 0.0f ? e : -1.0f;
     } else {
         // (what k_encode adds to, exchanges and reads)
-        for (uint32_t i = blockIdx.x * (uint32_t)(kScanThreads - 32) + (uint32_t)(tid - 32); i < a.J * max(a.segments, 2u * a.chunks); i += gridDim.x * (uint32_t)(kScanThreads - 32)) {
+        const uint32_t others = (uint32_t)kScanThreads - 32u * a.J, x = (uint32_t)tid - 32u * a.J;
+        for (uint32_t i = blockIdx.x * others + x; i < a.J * max(a.segments, 2u * a.chunks); i += gridDim.x * others) {
             if (i < a.J * a.segments) a.seg[i] = 0ull;
             if (i < 2u * a.J * a.chunks) a.chunk[i] = 0ull;
         }
         if (blockIdx.x == 0) {
-            const int x = tid - 32;
-            if (x < kEncMaxJobs) a.ctl->ne_count[x] = 0u;
-            if (x == 0) a.st->noblob = 0u;
-            if (x <= kMaxTau) { a.st->pw[x] = pw.P[x]; a.st->inv[x] = inv.P[x]; }
+            if (x < (uint32_t)kEncMaxJobs) a.ctl->ne_count[x] = 0u;
+            if (x == 0u) a.st->noblob = 0u;
+            if (x <= (uint32_t)kMaxTau) { a.st->pw[x] = pw.P[x]; a.st->inv[x] = inv.P[x]; }
         }
     }
     __syncthreads();
