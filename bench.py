@@ -2,7 +2,7 @@
 """Benchmark of the FastSGD compress + decompress-accumulate hot path on B200.
 
 One step = one pass of the whole path over one batch of synthetic gradients: every simulated
-worker's gradient is compressed (one fused kernel: abs-sum pass, grid barrier, encode pass), then every stream is
+worker's gradient is compressed (k_scan, k_encode, k_place; small ones: k_resident), then every stream is
 decompress-accumulated into one dense vector.  The metric is input GB/s = 4 n W / t.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--workload c2] [--impl reference]

@@ -104,19 +104,15 @@ typedef struct fastsgd_params {
  * If the stream does not fit, or the sum is not finite, only a 64-byte header
  * carrying the status is written.  Nothing outside out[0, out_bytes) is
  * written.
- * Group sizes: T = 2^14 is what the fused kernel is built for (its tile is the
- * group).  Any other group_log2 in 8..20 takes a general path: the sum kernel,
- * a kernel that selects the kept entries (i, v_i), |v_i| >= B_tau, into a list
- * in the workspace, and the list encoder of fastsgd_compress_kv on that list
- * (three reads of the gradient, about 1.5 times the fused kernel's time; a list
- * beyond 4.5 M pairs does not fit and the list encoder then walks the dense
- * gradient itself, a warp per group, which is slow for large groups).  The
+ * Group sizes: T = 2^14 is the encoder's tile.  Any other group_log2 in 8..20
+ * takes one launch more (the kept entries are filtered unit by unit, then
+ * packed group by group; the gradient is read once all the same).  The
  * stream is the one the definition gives for that group size (the paper's
  * Algorithm 2 has no groups: it is the case T >= n).  Below 2^8:
  * FASTSGD_E_NOT_IMPLEMENTED.  The decoder takes the same range as long as the
  * stream has at most 2^17 groups.
- * The kernel is launched cooperatively (all its thread blocks resident at
- * once, two per SM) and its blocks wait for one another with bounded waits; if
+ * Small gradients take one cooperative launch (all its thread blocks resident
+ * at once), larger ones three or four in a row; all waits are bounded; if
  * one of them runs out (it should not on a GPU the kernel has to itself) every
  * stream of that launch reports FASTSGD_ST_TIMEOUT, and the workspace must be
  * registered again before the next call: once fastsgd_stream_info or
@@ -135,8 +131,7 @@ int fastsgd_compress(const float* grad, uint64_t n, const fastsgd_params* params
  *   outs    host array of num_grads device pointers (each 16-byte aligned),
  *           every one with room for out_bytes bytes
  * Every stream is byte for byte what fastsgd_compress produces for that
- * gradient.  Up to 8 gradients share one kernel launch: thread blocks that are
- * done with one gradient start on the next while the others finish.
+ * gradient.  Up to 8 gradients share the launches.
  */
 int fastsgd_compress_batch(const float* const* grads, uint64_t n, const fastsgd_params* params,
                            void* const* outs, uint64_t out_bytes, uint32_t num_grads, void* stream);
@@ -155,8 +150,8 @@ int fastsgd_compress_batch(const float* const* grads, uint64_t n, const fastsgd_
  * (8 bytes per group) and one pass over the per-chunk sums (8 bytes per 2^14
  * indices): cost in proportion to count and to n / 2^14.  Any group_log2 in
  * 1..20.  Keys that do not ascend or reach n give an unspecified stream, never
- * an access outside the buffers.  One cooperative launch (a warp per 32 pairs;
- * two grid barriers with bounded waits, FASTSGD_ST_TIMEOUT as for
+ * an access outside the buffers.  One cooperative launch (a warp per 16 pairs;
+ * bounded waits, FASTSGD_ST_TIMEOUT as for
  * fastsgd_compress).
  */
 int fastsgd_compress_kv(const uint32_t* keys, const float* values, uint64_t count, uint64_t n,

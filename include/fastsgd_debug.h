@@ -38,20 +38,17 @@ int fastsgd_debug_set_wait_limits(uint32_t block_polls, uint32_t copy_tries, uin
 
 /* Caps the number of thread blocks of the encoders' launches (fastsgd_compress,
  * _batch, _kv) that follow; 0 restores the default (as many as are resident at
- * once).  With a cap the batch encoder does not split its blocks into two
- * teams.  The stream never depends on the grid: tests use this to show it. */
+ * once).  The stream never depends on the grid: tests use this to show it. */
 int fastsgd_debug_set_grid(uint32_t blocks);
 
 /* Byte offsets inside the registered workspace (all of them in its fixed first
- * part): [0] u32 bar_count[8], arrivals at each gradient's grid barrier;
+ * part): [0] u32 bar_count[8], arrivals (k_resident: per gradient);
  * [1] u32 ne_count[8], tiles the last encoder launch read a second time, per
- * gradient; [2] u32 error; [3] unused; [4] encoder trace, [5] its size
- * in bytes; [6] u32 decoder queue slots; [7] u32 decoder queue counters[6]. */
+ * gradient; [2] u32 error; [3] to [5] unused; [6] u32 decoder queue slots; [7] u32 decoder queue counters[6]. */
 #define FASTSGD_DEBUG_LAYOUT_FIELDS 8
 int fastsgd_debug_layout(uint64_t* offsets, uint32_t count);
 
-/* 1 if the library was built with -DFASTSGD_TRACE (the kernels then write
- * %globaltimer stamps of their phases into the trace areas), else 0 */
+/* 0: the kernels write no stamps of their phases */
 int fastsgd_debug_trace_compiled(void);
 
 #ifdef __cplusplus

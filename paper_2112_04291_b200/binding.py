@@ -371,14 +371,5 @@ def listed_tiles(jobs: int):
 
 
 def debug_trace_blocks(blocks: int = 148):
-    """Per-block stamps (ns, %globaltimer) of the last compress launch, shape (blocks, 8, 8): for
-    each block and each gradient of the launch: start, end of the sum pass, previous gradient's
-    pending tiles placed, grid barrier passed, table ready, end of the encode loop; slot 6 of
-    gradient 0 holds the end of the launch's last drain.  Only a library built with -DFASTSGD_TRACE
-    writes them (None otherwise); synchronises."""
-    ws = _workspace_keepalive
-    if ws is None or not lib().fastsgd_debug_trace_compiled():
-        return None
-    torch.cuda.synchronize()
-    off = debug_layout()["encoder_trace"]
-    return ws[off:off + 512 * blocks].cpu().numpy().view("<u8").reshape(blocks, 8, 8).astype("int64")
+    """Per-block stamps of the last compress launch: the kernels write none, None."""
+    return None

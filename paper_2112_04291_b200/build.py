@@ -36,8 +36,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         os.path.getmtime(d) > os.path.getmtime(LIB_PATH) for d in _deps())
     if force or stale:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-        trace = ["-DFASTSGD_TRACE"] if os.environ.get("FASTSGD_TRACE") == "1" else []
-        cmd = [nvcc, *NVCC_FLAGS, *trace, *(["-Xptxas", "-v"] if verbose else []), "-o", LIB_PATH, *sources()]
+        cmd = [nvcc, *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), "-o", LIB_PATH, *sources()]
         subprocess.check_call(cmd)
     return LIB_PATH
 
