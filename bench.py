@@ -844,7 +844,7 @@ def main():
                     "unit": "GB/s", "frac": kernels[dom]["achieved_gbs"] / peak, "peak_kind": f"of {peak_kind}",
                     "traffic": traffic, "traffic_kind": "counted by the kernel: 4nW + 64 KiB per tile it read a second time + streams",
                     "dram_frac": (traffic / dur / 1e9 / peak) if traffic else None,
-                    "traffic_ncu": ncu_traffic_of("k_compress_c2_4workers.md") if (default_c2 and dom == "k_compress") else None,
+                    "traffic_ncu": ncu_traffic_of("encoder_c2_4workers.md") if (default_c2 and dom == "k_compress") else None,
                     "algorithmic_bytes_per_launch": per_launch_bytes[dom]}
         if roofline["frac"] > 1.2:
             roofline["note"] = "frac counts two full reads of every gradient; the kernel skipped most tiles: dram_frac is the hardware figure"

@@ -151,8 +151,8 @@ Layout layout_of(uint64_t n, uint32_t group_log2) {
     if (pool > (1ull << 27)) pool = 1ull << 27;
     if (pool > all) pool = all;
     y.pool_begin = (uint64_t)kSlotBytes * T;
-    y.pool_bytes = 6ull * pool + 65536ull;
-    y.scratch = take(y.pool_begin + y.pool_bytes);
+    y.pool_bytes = (6ull * pool / kPools + 32768ull) & ~15ull;      // each
+    y.scratch = take(y.pool_begin + kPools * y.pool_bytes);
     y.end = at;
     return y;
 }

@@ -44,6 +44,7 @@ constexpr uint32_t kNoPlace      = 0xFFFFFFFFu;                // no room in the
 constexpr uint32_t kSampleBlocks = 32;                         // blocks that sample one gradient, four entries at 768 places each
 constexpr uint32_t kSamplePolls  = 64;                         // looks (0.7 us each) a block takes for another block's sample
 constexpr uint32_t kTicketGroups = 8;
+constexpr uint32_t kPools        = 32;
 constexpr uint32_t kChunkUnits   = 512;                        // units under one node of the upper part of the sum tree
 constexpr uint32_t kMaxChunks    = 1552;                       // such nodes in a launch
 constexpr uint32_t kMaxSegments  = 1600;                       // segments of tiles (64 or more) whose sizes k_place scans
@@ -58,7 +59,7 @@ struct EncState {
     uint32_t ticket[kTicketGroups][32];                        // k_scan: units handed out beyond each warp's first
     double   S[kEncMaxJobs];
     double   pw[132], inv[132];                                // b^k, 1 / b^k
-    unsigned long long pool_used;                              // bytes of the pool in use
+    unsigned long long pool_used[kPools][16];                  // bytes in use of each pool
     uint32_t noblob;                                           // tiles k_place has to pack
 };
 static_assert(kEncStateOffset + sizeof(EncState) <= kQueueOffset, "fits before the decoder's queue");
@@ -80,7 +81,7 @@ struct EncArgs {
     uint32_t*           blob;            // [J][G] the packed blob's place in the scratch (16-byte units)
     unsigned long long* seg;             // [J][segments] kept entries << 32 | words of the segment's tiles
     unsigned char*      scratch;         // [J G] slots, then the pool
-    uint64_t            pool_begin, pool_bytes;
+    uint64_t            pool_begin, pool_bytes;     // bytes: of one of the pools
     double              base;
     double              inv_ptau;        // 1 / b^tau (steers the estimate only)
     uint32_t            J, G;            // gradients; tiles of one
@@ -101,10 +102,17 @@ __device__ __forceinline__ UnitInfo load_info(const UnitInfo* p) {
     in.count = q.x; in.piece = q.y; in.room = q.z; in.sthr = __uint_as_float(q.w);
     return in;
 }
-// a piece of the pool (16-byte units), or kNoPlace
+// A piece of the pool (16-byte units), or kNoPlace.  The pool is 32 pools, a block's own first: atomics on one address go at 0.3 a
+// nanosecond, which was 10 us when the first slabs of 3000 units asked at once and 55 us of the 65 us scan of 2^26 entries.
 __device__ __forceinline__ uint32_t pool_take(const EncArgs& a, uint32_t bytes) {
-    const unsigned long long b = (bytes + 15u) & ~15u, at = atomicAdd(&a.st->pool_used, b);
-    return at + b <= a.pool_bytes ? (uint32_t)((a.pool_begin + at) >> 4) : kNoPlace;
+    const unsigned long long b = (bytes + 15u) & ~15u;
+#pragma unroll 1                                               // (unrolled, its code costs the kernels around it 5 to 10 %)
+    for (uint32_t i = 0; i < kPools; ++i) {
+        const uint32_t p = (blockIdx.x + i) % kPools;
+        const unsigned long long at = atomicAdd(&a.st->pool_used[p][0], b);
+        if (at + b <= a.pool_bytes) return (uint32_t)((a.pool_begin + p * a.pool_bytes + at) >> 4);
+    }
+    return kNoPlace;
 }
 
 // RU32(B_k) for one gradient: |v| >= B_k on an fp32 |v| equals |v| >= RU32(B_k); never below the smallest denormal, because an entry
@@ -843,7 +851,7 @@ struct WorkArea {                                              // shared memory 
 struct EncShared {
     float    thr[kEncMaxJobs][132];
     double   S[kEncMaxJobs];
-    uint32_t n_light, n_mid, mid_entries, n_heavy, next_light, next_mid, abort_flag, grab[4];
+    uint32_t n_light, n_mid, n_heavy, next_light, next_mid, abort_flag, grab[4];
     TeamScratch team[4];
     uint16_t light[kEncThreads], mid[kEncThreads], heavy[kEncThreads];      // heavy: bit 15: the tile is read again
     WorkArea area;
@@ -947,7 +955,7 @@ k_encode(const EncArgs a) {
     const uint32_t warp_max = owned >= (uint32_t)kEncWarps ? kWarpListMax : 64u;
     for (uint32_t first = 0; first < owned; first += kEncThreads) {
         // ---- which of the block's tiles hold anything, and where it is
-        if (tid == 0) { s.n_light = 0u; s.n_mid = 0u; s.mid_entries = 0u; s.n_heavy = 0u; s.next_light = 0u; s.next_mid = 0u; }
+        if (tid == 0) { s.n_light = 0u; s.n_mid = 0u; s.n_heavy = 0u; s.next_light = 0u; s.next_mid = 0u; }
         if (first) load_tile(first + (uint32_t)tid);
         __syncthreads();
         if (first + (uint32_t)tid < owned) {
@@ -965,10 +973,7 @@ k_encode(const EncArgs a) {
                 s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)(tid | 0x8000);
                 atomicAdd(&a.ctl->ne_count[j], 1u);
             } else if (slots && cnt <= warp_max) s.light[atomicAdd(&s.n_light, 1u)] = (uint16_t)tid;
-            else if (units) {
-                s.mid[atomicAdd(&s.n_mid, 1u)] = (uint16_t)tid;
-                atomicAdd(&s.mid_entries, cnt);
-            }
+            else if (units) s.mid[atomicAdd(&s.n_mid, 1u)] = (uint16_t)tid;
             else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
         }
         __syncthreads();
@@ -985,10 +990,8 @@ k_encode(const EncArgs a) {
             return p;
         };
         // ---- by the whole block
-        // (tiles for four warps too, where those are too few to occupy the block and long enough for it)
-        const uint32_t n_mid = s.n_mid < (uint32_t)kEncWarps / 4u && s.mid_entries > 1024u * s.n_mid ? 0u : s.n_mid, n_block = s.n_heavy + s.n_mid - n_mid;
-        for (uint32_t h = 0; h < n_block; ++h) {
-            const uint32_t x = h < s.n_heavy ? s.heavy[h] : s.mid[h - s.n_heavy];
+        for (uint32_t h = 0; h < s.n_heavy; ++h) {
+            const uint32_t x = s.heavy[h];
             const uint32_t t = blockIdx.x + (first + (x & 0x7FFFu)) * B, j = t / a.G, tile = t - j * a.G;
             uint32_t M = 0u, words = 0u, place = 0u;
             const uint32_t count = (x & 0x8000u) != 0u ? block_tile(a, j, tile, s.thr[j], s.area.b.key, s.area.b.blob, s.team[0], tid, lane, warp)
@@ -1016,13 +1019,13 @@ k_encode(const EncArgs a) {
         UnitInfo ui;
         float ux = 0.0f;
         auto next_unit = [&]() {
-            if (x >= n_mid) return;
+            if (x >= s.n_mid) return;
             t = blockIdx.x + (first + s.mid[x]) * B;
             ui = load_info(a.info + 4ull * t + qw);
             ux = __ldcg(a.umax + 4ull * t + qw);
         };
         next_unit();
-        while (x < n_mid) {
+        while (x < s.n_mid) {
             const uint32_t here = t, j = t / a.G;
             WorkArea::Quad& ar = s.area.q[quad];
             TeamScratch& ts = s.team[quad];

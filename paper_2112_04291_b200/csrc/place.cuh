@@ -105,10 +105,10 @@ k_place(const EncArgs a) {
         enc_write_header(a, (uint32_t)tid, !isfinite(S) ? kStNonfinite : !fits((uint32_t)tid) ? kStCapacity : kStOk, s.total[tid] >> 32, total_bytes_of((uint32_t)tid), S);
     }
     static_assert(kTicketGroups == (uint32_t)kEncMaxJobs, "reset together");
+    if (blockIdx.x == 0 && tid < (int)kPools) a.st->pool_used[tid][0] = 0ull;
     if (blockIdx.x == 0 && tid < kEncMaxJobs) {                // at rest again
         a.ctl->bar_count[tid] = 0u; a.st->ticket[tid][0] = 0u;
         for (uint32_t i = 0; i < kSampleBlocks; ++i) a.st->sample[tid][i] = 0ull;
-        if (tid == 0) a.st->pool_used = 0ull;
     }
     // ---- rows of eight tiles: directory entries and blobs.  When the rows are fewer than the warps, several warps share a row's words.
     const uint32_t rows = (a.D + kRowTiles - 1u) / kRowTiles, warps = B * (uint32_t)kEncWarps;
