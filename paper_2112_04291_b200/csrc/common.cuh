@@ -57,7 +57,8 @@ __host__ __device__ inline uint64_t ceil_div_u64(uint64_t a, uint64_t b) { retur
 // Programmatic dependent launch: the next kernel of the stream may be brought onto the GPU from here on (it waits below before it
 // touches memory) ...
 __device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// ... and: everything the kernels before this one in the stream have written is there.
+// ... and: everything the kernels before this one in the stream have written is there.  What they may have written (gradients, streams,
+// the workspace) is not read-only for the lifetime of such a kernel, which began before: never __ldg or __restrict__ for it.
 __device__ __forceinline__ void wait_for_previous_kernels() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 0, 0x0123); }

@@ -841,7 +841,7 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
     wait_for_previous_kernels();
     // ---- headers and the first batch of directory entries, requested together
     static_assert(16 * kDecMaxStreams <= kDecThreads, "a thread per header word");
-    if (tid < (int)(16u * W)) s.hdr[tid >> 4][tid & 15] = __ldg(reinterpret_cast<const uint32_t*>(a.stream[tid >> 4]) + (tid & 15));
+    if (tid < (int)(16u * W)) s.hdr[tid >> 4][tid & 15] = reinterpret_cast<const uint32_t*>(a.stream[tid >> 4])[tid & 15];
     const uint32_t my_w = ONE ? 0u : (uint32_t)tid % W, my_i = ONE ? (uint32_t)tid : (uint32_t)tid / W;
     uint32_t d0 = 0u, d1 = 0u, d2 = 0u;
     auto load_dir = [&](uint32_t i) {
@@ -849,8 +849,8 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
         if (my_i < per_batch && i < owned && a.bytes[my_w] >= fixed_bytes) {
             const uint32_t g = blockIdx.x + i * B;
             const uint32_t* e = reinterpret_cast<const uint32_t*>(a.stream[my_w]) + (kHeaderBytes >> 2) + 2u * g;
-            const uint2 x = __ldg(reinterpret_cast<const uint2*>(e));
-            d0 = x.x; d1 = x.y; d2 = g + 1u < a.G ? __ldg(e + 3) : 0u;
+            const uint2 x = *reinterpret_cast<const uint2*>(e);
+            d0 = x.x; d1 = x.y; d2 = g + 1u < a.G ? e[3] : 0u;
         }
     };
     load_dir(my_i);
@@ -978,8 +978,8 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
             uint32_t cm = 0u, nw = 0u, o = 0u;
             if (s.ok[tid]) {
                 const uint32_t* e = reinterpret_cast<const uint32_t*>(a.stream[tid]) + (kHeaderBytes >> 2) + 2u * g;
-                cm = __ldg(e); o = __ldg(e + 1);
-                if (!check_dir(a, g, s.total_words[tid], cm, o, g + 1u < a.G ? __ldg(e + 3) : s.total_words[tid], &nw)) { cm = 0u; nw = 0u; }
+                cm = e[0]; o = e[1];
+                if (!check_dir(a, g, s.total_words[tid], cm, o, g + 1u < a.G ? e[3] : s.total_words[tid], &nw)) { cm = 0u; nw = 0u; }
             }
             s.g_count[tid] = cm & 0xFFFFFFu; s.g_M[tid] = cm >> 24; s.g_off[tid] = o; s.g_nwords[tid] = nw;
         }

@@ -459,7 +459,7 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
 #pragma unroll 8
     for (int i = 0; i < 32; ++i) {
         const uint32_t e = (uint32_t)warp * kSlab + 32u * (uint32_t)i + (uint32_t)lane;
-        const uint32_t b = __ballot_sync(kFullMask, e < left && fabsf(__ldg(g + (e < left ? e : 0u))) >= thr_e);
+        const uint32_t b = __ballot_sync(kFullMask, e < left && fabsf(g[e < left ? e : 0u]) >= thr_e);
         if (lane == i) mask = b;                               // lane i: row i
         mine += (uint32_t)__popc(b);
     }
@@ -471,7 +471,7 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
     uint32_t pos = __shfl_sync(kFullMask, ci - c, warp) + incl - own;
     for (; mask != 0u; mask &= mask - 1u, ++pos) keys[pos] = (uint16_t)((uint32_t)warp * kSlab + 32u * (uint32_t)lane + (uint32_t)__ffs((int)mask) - 1u);
     __syncthreads();
-    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) put_code(blob, q, code_byte_of(ct, __ldg(g + keys[q])));
+    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) put_code(blob, q, code_byte_of(ct, g[keys[q]]));
     return count;
 }
 
@@ -519,7 +519,7 @@ k_resident(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_co
             bulk_load(slab, a.grad[j] + slab0, kSlab * 4u, &s.mbar[warp]);
         }
     } else {
-        for (uint32_t i = lane; i < kSlab; i += 32u) slab[i] = i < valid ? __ldg(a.grad[j] + slab0 + i) : 0.0f;
+        for (uint32_t i = lane; i < kSlab; i += 32u) slab[i] = i < valid ? a.grad[j][slab0 + i] : 0.0f;
         __syncwarp();
     }
     if (tid == 0) s.gen = ld_acquire_u32(&a.ctl->bar_gen) + 1u;      // before this block lets others go on
@@ -687,7 +687,7 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
     if (sampler) {
         const uint32_t places = (uint32_t)(a.n >> 2), count = a.samplers * (uint32_t)kScanThreads, step = places / count, at = si * (uint32_t)kScanThreads + (uint32_t)tid;
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (places) q = __ldg(reinterpret_cast<const float4*>(a.grad[sj]) + (step ? at * step + (step >> 1) : at % places));
+        if (places) q = reinterpret_cast<const float4*>(a.grad[sj])[step ? at * step + (step >> 1) : at % places];
         sx = fabsf(q.x) + fabsf(q.y) + fabsf(q.z) + fabsf(q.w);
         sy = sx * sx;
     }
@@ -763,7 +763,7 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
             float* ring = s.ring[warp][slot];
             const bool whole = here.left >= (slab + 1u) * kSlab;
             if (!whole) {                                      // the gradient's last entries
-                for (uint32_t q = lane; q < kSlab; q += 32u) ring[q] = slab * kSlab + q < here.left ? __ldg(here.g + slab * kSlab + q) : 0.0f;
+                for (uint32_t q = lane; q < kSlab; q += 32u) ring[q] = slab * kSlab + q < here.left ? here.g[slab * kSlab + q] : 0.0f;
                 __syncwarp();
             }
             float4 v[8];

@@ -21,12 +21,12 @@ __device__ __forceinline__ double abs_sum4(float4 v) {
 }
 
 // float4 at element index e (multiple of 4) of a 16-byte aligned array of n floats, zero beyond n
-__device__ __forceinline__ float4 load4_guarded(const float* __restrict__ g, uint64_t e, uint64_t n) {
-    if (e + 4 <= n) return __ldg(reinterpret_cast<const float4*>(g + e));
+__device__ __forceinline__ float4 load4_guarded(const float* g, uint64_t e, uint64_t n) {
+    if (e + 4 <= n) return *reinterpret_cast<const float4*>(g + e);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (e < n) v.x = __ldg(g + e);
-    if (e + 1 < n) v.y = __ldg(g + e + 1);
-    if (e + 2 < n) v.z = __ldg(g + e + 2);
+    if (e < n) v.x = g[e];
+    if (e + 1 < n) v.y = g[e + 1];
+    if (e + 2 < n) v.z = g[e + 2];
     return v;
 }
 

@@ -104,3 +104,17 @@ def test_workload_generators_are_seeded_and_shaped():
     w5 = workloads.make("c5", n=1 << 16, keep=0.1)
     rc, keys, codes, S = oracle.value_encode(w5.grads[0], w5.base, w5.tau)
     assert abs(keys.size / (1 << 16) - 0.1) < 0.01
+
+
+def test_kernels_that_start_early_read_no_read_only_memory():
+    """A kernel that waits for the one before it (griddepcontrol.wait) has already begun while that one writes: what it reads is
+    not read-only for its lifetime, so neither it nor what it includes may go through the non-coherent path."""
+    csrc = os.path.join(ROOT, "paper_2112_04291_b200", "csrc")
+    text = {f: re.sub(r"//[^\n]*", "", open(os.path.join(csrc, f)).read()) for f in os.listdir(csrc) if f.endswith(".cuh")}
+    early = {f for f, t in text.items() if "wait_for_previous_kernels();" in t}
+    assert {"encode.cuh", "groups.cuh", "place.cuh", "decode.cuh"} <= early
+    for f in early:
+        assert not re.search(r"__ldg\s*\(|__restrict__|\.nc\b|ld\.global\.nc", text[f]), f
+    # (of the shared helpers, the one that reads gradients)
+    helper = text["sum.cuh"][text["sum.cuh"].index("load4_guarded("):]
+    assert "__ldg" not in helper[:helper.index("\n}")] and "__restrict__" not in helper[:helper.index("\n}")]
