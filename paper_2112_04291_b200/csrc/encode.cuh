@@ -859,36 +859,56 @@ struct EncShared {
 static_assert(2 * (sizeof(EncShared) + 1024) <= 233472, "two blocks per SM (1 KiB per block is the system's)");
 
 // The gradients' sums from the units' nodes (same tree).  The first blocks form the nodes of 512 units, a warp each, and publish them;
-// every block takes them all and forms the rest of the tree for itself.  (Blocks start in order, and those that publish wait
-// for nobody before they have: a block waits only for blocks that are resident when it is.)
+// every block takes them all and forms the rest of the tree for itself.  Nobody depends on another block: one that is not given a
+// node within kNodePolls looks (0.7 us each; they come within 3 us when the GPU runs the first blocks at all) forms it from the units'
+// nodes, which the launch before this one has left.
+constexpr uint32_t kNodePolls = 256;
+// node c of the launch, by one warp
+__device__ __forceinline__ double form_node(const double* partials, uint32_t units, uint32_t chunks, uint32_t c, int lane) {
+    const uint32_t j = c / chunks, p = c - j * chunks;
+    double x[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const uint32_t e = kChunkUnits * p + 32u * (uint32_t)i + (uint32_t)lane;
+        x[i] = e < units ? __ldcg(partials + (uint64_t)j * units + e) : 0.0;
+    }
+    return warp_rows16_tree(x, lane);
+}
+// the nodes below 0, by the block (hardly ever called: kept out of the kernels' code and registers)
+__device__ __noinline__ void form_missing_nodes(const double* partials, uint32_t units, uint32_t chunks, double* nodes, uint32_t C) {
+    const int lane = threadIdx.x & 31;
+    for (uint32_t c = threadIdx.x >> 5; c < C; c += kEncWarps) {
+        if (nodes[c] != -1.0) continue;
+        const double node = form_node(partials, units, chunks, c, lane);
+        __syncwarp();
+        if (lane == 0) nodes[c] = node;
+    }
+}
 template <typename Shared>
 __device__ __forceinline__ void gradient_sums(const EncArgs& a, Shared& s, double* nodes, int tid, int lane, int warp) {
-    const uint32_t units = 4u * a.G, C = a.J * a.chunks, R = min(gridDim.x, 32u);
+    const uint32_t units = 4u * a.G, C = a.J * a.chunks, R = min(gridDim.x, 32u), polls = min(kNodePolls, a.wait_limit);
     if (blockIdx.x < R) {
         for (uint32_t c = blockIdx.x + R * (uint32_t)warp; c < C; c += R * (uint32_t)kEncWarps) {
-            const uint32_t j = c / a.chunks, p = c - j * a.chunks;
-            double x[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const uint32_t e = kChunkUnits * p + 32u * (uint32_t)i + (uint32_t)lane;
-                x[i] = e < units ? __ldcg(a.partials + (uint64_t)j * units + e) : 0.0;
-            }
-            const double node = warp_rows16_tree(x, lane);
+            const double node = form_node(a.partials, units, a.chunks, c, lane);
             if (lane == 0) st_relaxed_pair(a.chunk + 2u * c, (unsigned long long)__double_as_longlong(node), 1ull);
         }
     }
+    bool missing = false;
     for (uint32_t c = (uint32_t)tid; c < C; c += kEncThreads) {
         unsigned long long lo, hi;
         uint32_t spin = 0;
         for (;;) {
             ld_relaxed_pair(a.chunk + 2u * c, lo, hi);
             if (hi != 0ull) break;
-            if (++spin > a.wait_limit) { s.abort_flag = 1u; break; }
+            if (++spin > polls) { missing = true; break; }
             if (spin > 16u) __nanosleep(32);
         }
-        nodes[c] = __longlong_as_double((long long)lo);
+        nodes[c] = hi != 0ull ? __longlong_as_double((long long)lo) : -1.0;      // (no sum of |v| is negative)
     }
-    __syncthreads();
+    if (__syncthreads_or(missing ? 1 : 0)) {
+        form_missing_nodes(a.partials, units, a.chunks, nodes, C);
+        __syncthreads();
+    }
     if ((uint32_t)warp < a.J) {
         const double* p = nodes + (uint32_t)warp * a.chunks;
         double S = 0.0;

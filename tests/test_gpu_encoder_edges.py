@@ -103,3 +103,26 @@ def test_tiles_read_again(group_log2):
 def test_blobs_without_room(group_log2):
     n = (1 << 26) + 3
     _check_groups(np.where(np.arange(n) % 7, np.float32(1.0), np.float32(-2.0)).astype(np.float32), 1.2, group_log2, l=5)
+
+
+# blocks that are not given the sum's nodes by the blocks that form them form them for themselves: with a single look before that, no
+# launch gives up and no bit changes
+@pytest.mark.parametrize("workers,n,group_log2", [(1, 300 * TILE + 5, 14), (3, 310 * TILE - 9, 14), (1, 300 * TILE + 5, 10), (2, 700 * TILE + 1, 17)])
+def test_sum_without_help_from_other_blocks(workers, n, group_log2):
+    grads = [_tiles(n, (3, 0, 40, 900), 90 + w) for w in range(workers)]
+    pg, po = binding.params(1.2, 128, 2, group_log2), oracle.params(1.2, 128, 2, group_log2)
+    binding.ensure_workspace(n, pg)
+    bufs = [G.Guarded((binding.compress_bound(n, pg) + 255) & ~255) for _ in grads]
+    dev = [G.to_dev(v) for v in grads]
+    try:
+        binding.debug_set_wait_limits(block_polls=1)
+        for rep in range(3):
+            assert binding.compress_batch(dev, pg, [b.view for b in bufs]) == 0
+            for v, b in zip(grads, bufs):
+                rc, want = oracle.compress(v, po)
+                total, d, status = binding.stream_info(b.view)
+                assert status == rc == 0 and total == want.size and b.intact()
+                assert np.array_equal(b.view[:total].cpu().numpy(), want)
+    finally:
+        binding.debug_set_wait_limits(0, 0, 0)
+        binding.set_workspace(binding.ensure_workspace(n, pg))
