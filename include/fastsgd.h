@@ -278,7 +278,18 @@ int fastsgd_key_encode_paper(const uint32_t* keys, uint64_t d, uint32_t flag_bit
  * level); 0 for invalid arguments */
 uint64_t fastsgd_compress_bound(uint64_t n, const fastsgd_params* params);
 
-/* bytes of device scratch the two calls need for gradients of up to n entries */
+/* bytes of device scratch for gradients of up to n entries: room for the lists
+ * of as many of them as one launch takes (up to 8, 3 * 2^30 entries together);
+ * never less for a larger n.  With the default groups 54 MB for 2^20 entries,
+ * 237 MB for 25.6 M, 619 MB for 2^26, 1.29 GB from 403 M on.
+ * Any call is accepted with the part of it that it uses:
+ *   decoder, model update     2 MiB, whatever n
+ *   fastsgd_abs_sum           2 MiB + 8 bytes per 2^14 entries
+ *   fastsgd_compress_kv       2 MiB + 8 bytes per group
+ *   fastsgd_compress          3 MiB + 2432 bytes per 2^14 entries + 12 per group
+ * With less than fastsgd_workspace_bytes, fastsgd_compress_batch takes as many
+ * gradients per launch as there is room for, and gradients of which much is
+ * kept are read (and packed) a second time where their lists find no room. */
 uint64_t fastsgd_workspace_bytes(uint64_t n, const fastsgd_params* params);
 
 /* Registers caller-owned device memory (256-byte aligned) as the library's

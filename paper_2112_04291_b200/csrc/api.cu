@@ -117,17 +117,17 @@ uint32_t jobs_per_launch(uint64_t n) {
     return j < 1ull ? 1u : j > (uint64_t)kEncMaxJobs ? (uint32_t)kEncMaxJobs : (uint32_t)j;
 }
 
-// The part of the workspace that depends on n, as byte offsets: per unit (a quarter of a tile of 2^14 entries) of the gradients one
-// launch can take its node of the sum tree, largest |v| and list; nodes of 512 units; per group (by default: tile) its descriptor and blob's place; per
-// segment of groups its totals; the lists (a slot per unit and a pool for longer ones).  The list encoder's group entries use
-// the descriptors' place.
+// The part of the workspace that an encoder launch of J gradients uses, as byte offsets: per unit (a quarter of a tile of 2^14 entries)
+// its node of the sum tree, largest |v| and list; nodes of 512 units; per group (by default: tile) its descriptor and blob's place; per
+// segment of groups its totals; the lists (a slot per unit and a pool for longer ones, which takes what is left of ws_bytes).
 struct Layout {
-    uint64_t partials, chunk, umax, info, desc, blob, seg, scratch, pool_begin, pool_bytes, end;
+    uint64_t partials, chunk, umax, info, desc, blob, seg, scratch, pool_begin, pool_bytes, end;      // end: bytes needed at least
     uint32_t J, tiles, groups, chunks, seg_log2, segments;
 };
-Layout layout_of(uint64_t n, uint32_t group_log2) {
+constexpr uint64_t kLeastPool = 32768;                             // bytes of each pool at least
+Layout layout_of(uint64_t n, uint32_t group_log2, uint32_t J, uint64_t ws_bytes) {
     Layout y;
-    y.J = jobs_per_launch(n);
+    y.J = J;
     y.tiles = (uint32_t)chunks_of(n);
     y.chunks = (4u * y.tiles + kChunkUnits - 1u) / kChunkUnits;
     y.groups = (uint32_t)groups_of(n, group_log2);
@@ -144,20 +144,37 @@ Layout layout_of(uint64_t n, uint32_t group_log2) {
     y.desc = take(8ull * descs);
     y.blob = take(4ull * descs);
     y.seg = take(8ull * y.J * y.segments);
-    // the pool: a sixth of the entries, within 2^24 (or all of a smaller gradient) and 2^27
-    const uint64_t all = (uint64_t)y.J * n;
+    y.pool_begin = (uint64_t)kSlotBytes * T;
+    y.scratch = take(y.pool_begin + kPools * kLeastPool);
+    y.end = at;
+    // (never more than every entry on a list)
+    const uint64_t rest = ws_bytes > y.end ? ws_bytes - y.end : 0ull, most = 6ull * y.J * n;
+    y.pool_bytes = kLeastPool + ((rest < most ? rest : most) / kPools & ~15ull);      // each
+    return y;
+}
+
+// What fastsgd_workspace_bytes answers: enough for as many gradients of up to n entries as one launch takes, with a pool of a sixth of
+// their entries, within 2^24 (or all of smaller gradients) and 2^27.  A launch never takes more than `all` entries, whatever the length of
+// its gradients, so that every term here is at least the layout's for any shorter length and any number of gradients, and none
+// falls as n grows.
+uint64_t ws_bytes_for(uint64_t n, uint32_t group_log2) {
+    const uint64_t most = 3ull << 30, all = n < most / (uint64_t)kEncMaxJobs ? (uint64_t)kEncMaxJobs * n : most;
+    const uint64_t T = (all >> kChunkLog2) + kEncMaxJobs, descs = (all >> group_log2) + kEncMaxJobs, chunks = (4ull * T) / kChunkUnits + kEncMaxJobs;
     uint64_t pool = all / 6ull;
     if (pool < (1ull << 24)) pool = 1ull << 24;
     if (pool > (1ull << 27)) pool = 1ull << 27;
     if (pool > all) pool = all;
-    y.pool_begin = (uint64_t)kSlotBytes * T;
-    y.pool_bytes = (6ull * pool / kPools + 32768ull) & ~15ull;      // each
-    y.scratch = take(y.pool_begin + kPools * y.pool_bytes);
-    y.end = at;
-    return y;
+    const uint64_t parts = (32ull + 16ull + 4ull * sizeof(UnitInfo) + kSlotBytes) * T + 16ull * chunks + 12ull * descs + 8ull * kMaxSegments;
+    return (kPartialsOffset + parts + 8ull * 256ull + kPools * kLeastPool + 6ull * pool + 255ull) & ~255ull;
 }
 
-uint64_t ws_bytes_for(uint64_t n, uint32_t group_log2) { return layout_of(n, group_log2).end; }
+// Gradients a launch takes with the workspace at hand: as many as it has room for, of those that are there; 0: too small for one.
+uint32_t jobs_that_fit(uint64_t n, uint32_t group_log2, uint32_t num_grads, uint64_t ws_bytes) {
+    uint32_t J = jobs_per_launch(n);
+    if (J > num_grads) J = num_grads ? num_grads : 1u;
+    while (J > 0u && layout_of(n, group_log2, J, 0ull).end > ws_bytes) --J;
+    return J;
+}
 
 Control* control_of(void* ws) { return static_cast<Control*>(ws); }
 
@@ -355,7 +372,7 @@ uint64_t fastsgd_workspace_bytes(uint64_t n, const fastsgd_params* params) {
 int fastsgd_set_workspace(void* dev_ptr, uint64_t bytes, void* stream) {
     if (!dev_ptr) return FASTSGD_E_NULL;
     if (!aligned(dev_ptr, 256)) return FASTSGD_E_ALIGN;
-    if (bytes < kPartialsOffset) return FASTSGD_E_NO_WORKSPACE;   // control block, tables, trace, decoder queue
+    if (bytes < kPartialsOffset) return FASTSGD_E_NO_WORKSPACE;   // the fixed part: control block, encoder state, decoder queue, chunk sums of the list encoder
     std::lock_guard<std::mutex> lock(g_mu);
     FSG_DEVICE_STATE();
     int rc = ensure_device_setup();
@@ -377,28 +394,27 @@ int fastsgd_abs_sum(const float* grad, uint64_t n, double* sum_out, void* stream
     if (rc) return rc;
     std::lock_guard<std::mutex> lock(g_mu);
     FSG_DEVICE_STATE();
-    if (!g_state.ws || g_state.ws_bytes < ws_bytes_for(n, kGroupLog2)) return FASTSGD_E_NO_WORKSPACE;
+    if (!g_state.ws || g_state.ws_bytes < kPartialsOffset + 8ull * chunks_of(n)) return FASTSGD_E_NO_WORKSPACE;
     rc = ensure_device_setup();
     if (rc) return rc;
-    double* partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + layout_of(n, kGroupLog2).partials);
+    double* partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + kPartialsOffset);
     return launch_sum(grad, n, control_of(g_state.ws), partials, sum_out, static_cast<cudaStream_t>(stream));
 }
 
 namespace {
-// The list encoder (kv.cuh).  Caller holds g_state.mu.
+// The list encoder (kv.cuh).  Caller holds g_mu.  Of the workspace it uses the fixed part and 8 bytes per group.
 int launch_list_encoder(const uint32_t* keys, const float* values, uint64_t count, uint64_t n,
                         const fastsgd_params* params, const PowTable& pw, void* out, uint64_t out_bytes, cudaStream_t st) {
     FSG_DEVICE_STATE();
     if (g_state.kv_blocks_per_sm < 1) return FASTSGD_E_CUDA;
-    const Layout y = layout_of(n, params->group_log2);
     KvArgs ka;
     std::memset(&ka, 0, sizeof(ka));
     ka.keys = keys; ka.vals = values; ka.count = count; ka.n = n;
     ka.out = static_cast<uint8_t*>(out); ka.out_bytes = out_bytes; ka.ctl = control_of(g_state.ws);
     ka.partials = reinterpret_cast<double*>(static_cast<unsigned char*>(g_state.ws) + kKvPartialsOffset);
-    ka.meta = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + y.desc);
+    ka.meta = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(g_state.ws) + kPartialsOffset);
     ka.st = reinterpret_cast<EncState*>(static_cast<unsigned char*>(g_state.ws) + kEncStateOffset);
-    ka.base = params->base; ka.G = y.groups; ka.chunks = y.tiles;
+    ka.base = params->base; ka.G = (uint32_t)groups_of(n, params->group_log2); ka.chunks = (uint32_t)chunks_of(n);
     ka.tau = params->tau; ka.l = params->flag_bits; ka.group_log2 = params->group_log2;
     ka.wait_limit = g_tun.wait_limit;
     // all blocks are resident (they meet at grid barriers).  A warp per kKvSlice entries until the GPU is full: a warp works off its
@@ -443,13 +459,14 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
     if (bound_bytes(n, params) / 4ull >= (1ull << 31)) return FASTSGD_E_BAD_N;   // descriptor fields are 31 bits
     std::lock_guard<std::mutex> lock(g_mu);
     FSG_DEVICE_STATE();
-    if (!g_state.ws || g_state.timed_out || g_state.ws_bytes < ws_bytes_for(n, params->group_log2)) return FASTSGD_E_NO_WORKSPACE;
+    const uint32_t jobs = g_state.ws && !g_state.timed_out ? jobs_that_fit(n, params->group_log2, num_grads, g_state.ws_bytes) : 0u;
+    if (!jobs) return FASTSGD_E_NO_WORKSPACE;
     rc = ensure_device_setup();
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (params->group_log2 < 8u) return FASTSGD_E_NOT_IMPLEMENTED;
     const bool tile_groups = params->group_log2 == (uint32_t)kGroupLog2;
-    const Layout y = layout_of(n, params->group_log2);
+    const Layout y = layout_of(n, params->group_log2, jobs, g_state.ws_bytes);
     unsigned char* wsb = static_cast<unsigned char*>(g_state.ws);
     PowTable inv = inverse_of(pw);
     for (uint32_t first = 0; first < num_grads; first += y.J) {
@@ -536,7 +553,7 @@ int fastsgd_compress_kv(const uint32_t* keys, const float* values, uint64_t coun
     if (bound_bytes(n, params) / 4ull >= (1ull << 31)) return FASTSGD_E_BAD_N;
     std::lock_guard<std::mutex> lock(g_mu);
     FSG_DEVICE_STATE();
-    if (!g_state.ws || g_state.timed_out || g_state.ws_bytes < ws_bytes_for(n, params->group_log2)) return FASTSGD_E_NO_WORKSPACE;
+    if (!g_state.ws || g_state.timed_out || g_state.ws_bytes < kPartialsOffset + 8ull * G) return FASTSGD_E_NO_WORKSPACE;
     rc = ensure_device_setup();
     if (rc) return rc;
     return launch_list_encoder(keys, values, count, n, params, pw, out, out_bytes, static_cast<cudaStream_t>(stream));
@@ -575,7 +592,7 @@ int decode_launches(const void* const* streams_in, const uint64_t* bytes, uint32
     }
     std::lock_guard<std::mutex> lock(g_mu);
     FSG_DEVICE_STATE();
-    if (!g_state.ws || g_state.timed_out || g_state.ws_bytes < ws_bytes_for(n, params->group_log2)) return FASTSGD_E_NO_WORKSPACE;
+    if (!g_state.ws || g_state.timed_out) return FASTSGD_E_NO_WORKSPACE;      // (the decoder uses its fixed part alone)
     rc = ensure_device_setup();
     if (rc) return rc;
     const uint64_t G = groups_of(n, params->group_log2);

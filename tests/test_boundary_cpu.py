@@ -118,3 +118,17 @@ def test_kernels_that_start_early_read_no_read_only_memory():
     # (of the shared helpers, the one that reads gradients)
     helper = text["sum.cuh"][text["sum.cuh"].index("load4_guarded("):]
     assert "__ldg" not in helper[:helper.index("\n}")] and "__restrict__" not in helper[:helper.index("\n}")]
+
+
+@pytest.mark.parametrize("group_log2", [8, 14, 20])
+def test_workspace_size_never_falls_as_n_grows(lib, group_log2):
+    """A workspace registered for the largest n serves every smaller one (the number of gradients a launch takes changes on the way)."""
+    p = binding.params(1.1, 128, 2, group_log2)
+    ns = {int(1.09 ** i) for i in range(250)} | {3 * (1 << 30) // j + d for j in range(1, 9) for d in (-1, 0, 1)}
+    ns |= {(1 << e) + d for e in range(1, 31) for d in (-1, 0, 1)}
+    sizes = [binding.workspace_bytes(n, p) for n in sorted(n for n in ns if 1 <= n < 1 << 31)]
+    assert all(a <= b for a, b in zip(sizes, sizes[1:]))
+    # (and as many gradients of n entries as a launch takes have a slot for each of their units, within what the header states)
+    for n in sorted(n for n in ns if 1 <= n < 1 << 31):
+        jobs = max(1, min(8, 3 * (1 << 30) // n))
+        assert binding.workspace_bytes(n, p) >= jobs * 2304 * -(-n >> 14)
