@@ -454,14 +454,21 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
     const uint64_t left = a.n - ((uint64_t)tile << kGroupLog2);
     const float thr_e = thr[a.tau];
     const CodeTable ct(thr, a.tau);
-    // (32 loads of consecutive entries: row i of the slab's 32 rows of 32)
+    // (32 loads of consecutive entries: row i of the slab's 32 rows of 32; sixteen in flight, each needed by a ballot only when all of them
+    // have been asked for)
     uint32_t mine = 0u, mask = 0u;
-#pragma unroll 8
-    for (int i = 0; i < 32; ++i) {
-        const uint32_t e = (uint32_t)warp * kSlab + 32u * (uint32_t)i + (uint32_t)lane;
-        const uint32_t b = __ballot_sync(kFullMask, e < left && fabsf(g[e < left ? e : 0u]) >= thr_e);
-        if (lane == i) mask = b;                               // lane i: row i
-        mine += (uint32_t)__popc(b);
+#pragma unroll 1
+    for (int i0 = 0; i0 < 32; i0 += 16) {
+        float x[16];
+        const uint32_t e0 = (uint32_t)warp * kSlab + 32u * (uint32_t)i0 + (uint32_t)lane;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = e0 + 32u * (uint32_t)i < left ? g[e0 + 32u * (uint32_t)i] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const uint32_t b = __ballot_sync(kFullMask, fabsf(x[i]) >= thr_e);      // (thr_e > 0)
+            if (lane == i0 + i) mask = b;                      // lane i: row i
+            mine += (uint32_t)__popc(b);
+        }
     }
     if (lane == 0) s.cnt[warp] = mine;
     __syncthreads();
@@ -471,7 +478,13 @@ __device__ __forceinline__ uint32_t block_tile(const EncArgs& a, uint32_t j, uin
     uint32_t pos = __shfl_sync(kFullMask, ci - c, warp) + incl - own;
     for (; mask != 0u; mask &= mask - 1u, ++pos) keys[pos] = (uint16_t)((uint32_t)warp * kSlab + 32u * (uint32_t)lane + (uint32_t)__ffs((int)mask) - 1u);
     __syncthreads();
-    for (uint32_t q = (uint32_t)tid; q < count; q += kEncThreads) put_code(blob, q, code_byte_of(ct, g[keys[q]]));
+    for (uint32_t q = (uint32_t)tid; q < count; q += 4u * kEncThreads) {
+        float x[4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) x[i] = q + i * kEncThreads < count ? g[keys[q + i * kEncThreads]] : 0.0f;
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) if (q + i * kEncThreads < count) put_code(blob, q + i * kEncThreads, code_byte_of(ct, x[i]));
+    }
     return count;
 }
 

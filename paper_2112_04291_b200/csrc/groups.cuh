@@ -27,18 +27,23 @@ template <typename F>
 __device__ __forceinline__ uint32_t unit_again(const EncArgs& a, uint32_t j, uint32_t unit, float thr_e, int lane, F put) {
     uint32_t rank = 0u;
     const uint64_t e0 = (uint64_t)unit << kUnitLog2;
-#pragma unroll 4
-    for (uint32_t r = 0; r < kUnit / 128u; ++r) {
-        const uint32_t k = 128u * r + 4u * (uint32_t)lane;
-        const float4 q = load4_guarded(a.grad[j], e0 + k, a.n);
-        uint32_t m = reach_mask(q, thr_e);
-        const uint32_t own = (uint32_t)__popc(m), incl = warp_incl_scan(own, lane);
-        uint32_t at = rank + incl - own;
-        if (m & 1u) put(at++, k, q.x);
-        if (m & 2u) put(at++, k + 1u, q.y);
-        if (m & 4u) put(at++, k + 2u, q.z);
-        if (m & 8u) put(at++, k + 3u, q.w);
-        rank += __shfl_sync(kFullMask, incl, 31);
+#pragma unroll 1
+    for (uint32_t r0 = 0; r0 < kUnit / 128u; r0 += 4u) {
+        float4 row[4];                                         // (asked for together: the scans below wait for each in turn)
+#pragma unroll
+        for (uint32_t r = 0; r < 4u; ++r) row[r] = load4_guarded(a.grad[j], e0 + 128u * (r0 + r) + 4u * (uint32_t)lane, a.n);
+#pragma unroll
+        for (uint32_t r = 0; r < 4u; ++r) {
+            const uint32_t k = 128u * (r0 + r) + 4u * (uint32_t)lane;
+            const float4 q = row[r];
+            const uint32_t m = reach_mask(q, thr_e), own = (uint32_t)__popc(m), incl = warp_incl_scan(own, lane);
+            uint32_t at = rank + incl - own;
+            if (m & 1u) put(at++, k, q.x);
+            if (m & 2u) put(at++, k + 1u, q.y);
+            if (m & 4u) put(at++, k + 2u, q.z);
+            if (m & 8u) put(at++, k + 3u, q.w);
+            rank += __shfl_sync(kFullMask, incl, 31);
+        }
     }
     return rank;
 }
