@@ -44,7 +44,8 @@ int fastsgd_debug_set_grid(uint32_t blocks);
 /* Byte offsets inside the registered workspace (all of them in its fixed first
  * part): [0] u32 bar_count[8], arrivals (k_resident: per gradient);
  * [1] u32 ne_count[8], tiles the last encoder launch read a second time, per
- * gradient; [2] u32 error; [3] to [5] unused; [6] u32 decoder queue slots; [7] u32 decoder queue counters[6]. */
+ * gradient; [2] u32 error; [3] u32 tiles or groups the last encoder launch had no place for until its last step, which
+ * packed them anew; [4], [5] unused; [6] u32 decoder queue slots; [7] u32 decoder queue counters[6]. */
 #define FASTSGD_DEBUG_LAYOUT_FIELDS 8
 int fastsgd_debug_layout(uint64_t* offsets, uint32_t count);
 

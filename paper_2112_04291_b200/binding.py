@@ -343,7 +343,7 @@ def debug_set_grid(blocks: int = 0) -> None:
     _check(lib().fastsgd_debug_set_grid(int(blocks)), "fastsgd_debug_set_grid")
 
 
-LAYOUT_FIELDS = ("bar_count", "ne_count", "error", "decoder_trace", "encoder_trace", "encoder_trace_bytes",
+LAYOUT_FIELDS = ("bar_count", "ne_count", "error", "late_blobs", "unused_4", "unused_5",
                  "queue_slots", "queue_counters")
 
 

@@ -321,7 +321,7 @@ int fastsgd_debug_layout(uint64_t* offsets, uint32_t count) {
     if (!offsets) return FASTSGD_E_NULL;
     const uint64_t v[FASTSGD_DEBUG_LAYOUT_FIELDS] = {
         offsetof(Control, bar_count), offsetof(Control, ne_count), offsetof(Control, error),
-        0, 0, 0, kQueueOffset, offsetof(Control, dq)};
+        kEncStateOffset + offsetof(EncState, noblob), 0, 0, kQueueOffset, offsetof(Control, dq)};
     for (uint32_t i = 0; i < count && i < (uint32_t)FASTSGD_DEBUG_LAYOUT_FIELDS; ++i) offsets[i] = v[i];
     return FASTSGD_OK;
 }

@@ -60,7 +60,7 @@ struct EncState {
     double   S[kEncMaxJobs];
     double   pw[132], inv[132];                                // b^k, 1 / b^k
     unsigned long long pool_used[kPools][16];                  // bytes in use of each pool
-    uint32_t noblob;                                           // tiles k_place has to pack
+    uint32_t noblob;                                           // tiles (groups) k_place has to pack; stays until the next launch
 };
 static_assert(kEncStateOffset + sizeof(EncState) <= kQueueOffset, "fits before the decoder's queue");
 
@@ -156,7 +156,7 @@ __device__ __forceinline__ uint32_t slab_mask(const float4 (&v)[8], float thr, i
 // ---- teams: one, four or sixteen warps on one tile ------------------------------------------------------
 // The kept entries' keys stand in shared memory in index order, their code bytes already in the blob (big-endian valued words); flags
 // and deltas are packed behind the codes.
-struct TeamScratch { uint32_t cnt[kEncWarps], maxd[kEncWarps], first[4], last[4], bits[kEncWarps], word; };
+struct TeamScratch { uint32_t cnt[kEncWarps], maxd[kEncWarps], first[4], last[4], bits[kEncWarps], room[4], piece[4], word; };
 
 template <int W> __device__ __forceinline__ void team_sync(int id) {
     if constexpr (W == 1) __syncwarp();
@@ -1016,9 +1016,19 @@ k_encode(const EncArgs a) {
             a.blob[t] = place;
             if (count) atomicAdd(&a.seg[j * a.segments + ((t - j * a.G) >> a.seg_log2)], ((unsigned long long)count << 32) | words);
         };
-        // (the slots of the tile's units, where the lists were, or a piece of the pool)
-        auto place_of = [&](uint32_t t, uint32_t words) -> uint32_t {
-            const uint32_t p = words <= kSlotWords ? t * (kSlotBytes / 16u) : pool_take(a, words * 4u);
+        // Where the tile's lists were, which by now are in shared memory: the slots of its units or the largest of their pieces of the
+        // pool (a quarter of the candidates at 6 bytes holds all entries at up to 12 bits); else a new piece.  (One gradient of 2^30, a
+        // tenth kept: lists and blobs together did not fit the pool, and most tiles were packed twice: 5.9 ms, now 1.8.)
+        auto piece_of = [&](const UnitInfo& in, TeamScratch& ts, uint32_t q) {
+            ts.room[q] = in.room != kSlotEntries && in.piece != kNoPlace ? in.room : 0u;
+            ts.piece[q] = in.piece;
+        };
+        auto place_of = [&](const TeamScratch& ts, uint32_t t, uint32_t words) -> uint32_t {
+            if (words <= kSlotWords) return t * (kSlotBytes / 16u);
+            uint32_t room = 0u, p = kNoPlace;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) if (ts.room[q] > room) { room = ts.room[q]; p = ts.piece[q]; }
+            if (4u * words > 6u * room) p = pool_take(a, words * 4u);
             if (p == kNoPlace) atomicAdd(&a.st->noblob, 1u);
             return p;
         };
@@ -1027,12 +1037,13 @@ k_encode(const EncArgs a) {
             const uint32_t x = s.heavy[h];
             const uint32_t t = blockIdx.x + (first + (x & 0x7FFFu)) * B, j = t / a.G, tile = t - j * a.G;
             uint32_t M = 0u, words = 0u, place = 0u;
+            if (tid < 4) piece_of(load_info(a.info + 4ull * t + tid), s.team[0], (uint32_t)tid);
             const uint32_t count = (x & 0x8000u) != 0u ? block_tile(a, j, tile, s.thr[j], s.area.b.key, s.area.b.blob, s.team[0], tid, lane, warp)
                                                                : team_list<kEncWarps>(a, t, s.thr[j], s.area.b.key, s.area.b.blob, s.team[0], warp, lane, 0);
             if (count) {
                 M = team_pack<kEncWarps>(a.l, s.area.b.key, s.area.b.blob, count, s.team[0], warp, lane, 0, [&](uint32_t w_) {
                     words = w_;
-                    if (tid == 0) s.team[0].word = place_of(t, w_);
+                    if (tid == 0) s.team[0].word = place_of(s.team[0], t, w_);
                 });
                 place = s.team[0].word;
                 if (place != kNoPlace) {
@@ -1069,7 +1080,7 @@ k_encode(const EncArgs a) {
             KeyRun r;
             r.keys = keys + q0; r.left = q0 < n ? (int)min(4u * quads, n - q0) : 0; r.prev = q0 < n ? (uint32_t)keys[q0 ? q0 - 1u : 0u] : 0u;
             const uint32_t top = runs_max(r, quads);           // (within the unit)
-            if (lane == 0) { ts.cnt[qw] = n; ts.maxd[qw] = top; ts.first[qw] = n ? (uint32_t)keys[0] : 0u; ts.last[qw] = n ? (uint32_t)keys[n - 1u] : 0u; }
+            if (lane == 0) { piece_of(ui, ts, (uint32_t)qw); ts.cnt[qw] = n; ts.maxd[qw] = top; ts.first[qw] = n ? (uint32_t)keys[0] : 0u; ts.last[qw] = n ? (uint32_t)keys[n - 1u] : 0u; }
             team_sync<4>(quad);
             // from one unit's last key to the next one's first; the unit's rank
             uint32_t M = 0u, count = 0u, rank = 0u, last = 0u, before = 0u;
@@ -1103,7 +1114,7 @@ k_encode(const EncArgs a) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) { const uint32_t y = ts.bits[q]; if (q < qw) dpos += y; words += y; }
             words = (words + 31u) >> 5;
-            if (qw == 0 && lane == 0) ts.word = place_of(here, words);
+            if (qw == 0 && lane == 0) ts.word = place_of(ts, here, words);
             write_runs<true>(r, quads, shape, least, a.l, ar.blob, count, rank + q0, dpos, ar.code[qw] + q0);
             team_sync<4>(quad);
             const uint32_t place = ts.word;

@@ -110,3 +110,25 @@ def test_other_calls_take_the_least_workspace(workspace):
     big = torch.zeros(n, dtype=torch.float32, device=G.dev())
     assert binding.compress(big, pg, out.view) == binding.E_NO_WORKSPACE
     assert ws.intact()
+
+
+def late_blobs():
+    torch.cuda.synchronize()
+    return int(binding.workspace_u32("late_blobs", 1)[0].item())
+
+
+def test_blobs_go_where_their_lists_were(workspace):
+    # a tenth of the entries kept: a list takes 3.3 KB of the pool per unit, a blob 2.9 KB per tile and more than the tile's slots.  With room for
+    # the lists and half of the blobs beside them no tile is packed twice
+    n = 600 * TILE
+    v = np.random.default_rng(8).standard_normal(n).astype(np.float32)
+    base = workloads.base_for_keep(v, n // 10)
+    pg, po = binding.params(base), oracle.params(base)
+    ws = workspace(_least(n, 14) + 4 * 600 * 3300 + 600 * 1450)
+    out = G.Guarded((binding.compress_bound(n, pg) + 255) & ~255)
+    dev = G.to_dev(v)
+    for rep in range(2):
+        assert binding.compress(dev, pg, out.view) == 0
+        _streams_equal([out], [v], po)
+        assert binding.listed_tiles(1) == [0] and late_blobs() == 0
+    assert ws.intact()
