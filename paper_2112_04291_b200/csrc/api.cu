@@ -486,7 +486,7 @@ int compress_launches(const float* const* grads, uint64_t n, const fastsgd_param
         ea.desc = reinterpret_cast<unsigned long long*>(wsb + y.desc);
         ea.blob = reinterpret_cast<uint32_t*>(wsb + y.blob);
         ea.seg = reinterpret_cast<unsigned long long*>(wsb + y.seg); ea.seg_log2 = y.seg_log2; ea.segments = y.segments;
-        ea.scratch = wsb + y.scratch; ea.pool_begin = y.pool_begin; ea.pool_bytes = y.pool_bytes;
+        ea.scratch = wsb + y.scratch; ea.pool_begin = y.pool_begin; ea.pool_bytes = y.pool_bytes; ea.pool_units = (4u * ea.J * y.tiles + kPools - 1u) / kPools;
         ea.base = params->base; ea.inv_ptau = inv.P[params->tau]; ea.G = y.tiles; ea.D = y.groups; ea.group_log2 = params->group_log2;
         ea.tau = params->tau; ea.l = params->flag_bits; ea.wait_limit = g_tun.wait_limit; ea.try_limit = g_tun.try_limit;
         const uint64_t tiles = (uint64_t)ea.J * ea.G;

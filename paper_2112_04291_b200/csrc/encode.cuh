@@ -81,7 +81,8 @@ struct EncArgs {
     uint32_t*           blob;            // [J][G] the packed blob's place in the scratch (16-byte units)
     unsigned long long* seg;             // [J][segments] kept entries << 32 | words of the segment's tiles
     unsigned char*      scratch;         // [J G] slots, then the pool
-    uint64_t            pool_begin, pool_bytes;     // bytes: of one of the pools
+    uint64_t            pool_begin, pool_bytes;     // bytes: of one of the pools (below 2^32)
+    uint32_t            pool_units;      // units that share a pool
     double              base;
     double              inv_ptau;        // 1 / b^tau (steers the estimate only)
     uint32_t            J, G;            // gradients; tiles of one
@@ -104,15 +105,30 @@ __device__ __forceinline__ UnitInfo load_info(const UnitInfo* p) {
 }
 // A piece of the pool (16-byte units), or kNoPlace.  The pool is 32 pools, a block's own first: atomics on one address go at 0.3 a
 // nanosecond, which was 10 us when the first slabs of 3000 units asked at once and 55 us of the 65 us scan of 2^26 entries.
-__device__ __forceinline__ uint32_t pool_take(const EncArgs& a, uint32_t bytes) {
+// A piece may not reach beyond a pool's first `limit` bytes.  What a refusal adds to a counter is lost to others: pools other than the
+// block's own, and (look) that one too, are asked only after a look.  fill: how far the piece's pool is used.
+__device__ __forceinline__ uint32_t pool_take(const EncArgs& a, uint32_t bytes, uint64_t limit, bool look, uint64_t& fill) {
     const unsigned long long b = (bytes + 15u) & ~15u;
 #pragma unroll 1                                               // (unrolled, its code costs the kernels around it 5 to 10 %)
     for (uint32_t i = 0; i < kPools; ++i) {
         const uint32_t p = (blockIdx.x + i) % kPools;
+        if ((i || look) && ld_relaxed_u64(&a.st->pool_used[p][0]) + b > limit) continue;
         const unsigned long long at = atomicAdd(&a.st->pool_used[p][0], b);
-        if (at + b <= a.pool_bytes) return (uint32_t)((a.pool_begin + p * a.pool_bytes + at) >> 4);
+        fill = at + b;
+        if (at + b <= limit) return (uint32_t)((a.pool_begin + p * a.pool_bytes + at) >> 4);
     }
     return kNoPlace;
+}
+__device__ __forceinline__ uint32_t pool_take(const EncArgs& a, uint32_t bytes) { uint64_t fill; return pool_take(a, bytes, a.pool_bytes, false, fill); }
+// How far lists of `entries` candidates a unit may fill a pool: so far that the tiles that then have none find room for their blobs
+// there, unless these fit the tiles' slots.  A list takes about 8 bytes a candidate, a blob at most 2.25 (up to 18 bits an entry): with x
+// units listed of the U that share a pool, 8 e x + 2.25 e (U - x) <= pool bytes.  Eight gradients of 335 M, a tenth kept: lists
+// without a limit filled the pool, and four tiles in five were packed twice.
+__device__ __forceinline__ uint32_t lists_limit(const EncArgs& a, uint32_t entries) {
+    const uint32_t pool = (uint32_t)a.pool_bytes, blobs = entries * a.pool_units / 4u * 9u;
+    if (8u * entries <= kSlotBytes) return pool;
+    const uint32_t rest = pool > blobs ? pool - blobs : 0u;
+    return min(pool, rest + rest / 3u);
 }
 
 // RU32(B_k) for one gradient: |v| >= B_k on an fp32 |v| equals |v| >= RU32(B_k); never below the smallest denormal, because an entry
@@ -658,6 +674,8 @@ struct ScanShared {
     unsigned long long mbar[kScanWarps][kRing];
     float samp[2][kScanWarps];
     float est[kEncMaxJobs];
+    uint32_t refused;                                          // bytes of the shortest list the pools have refused one of the block's warps
+    uint32_t nearly;                                           // the pools are close to their limit
 };
 static_assert(sizeof(ScanShared) <= 232448, "shared memory of one block");
 
@@ -668,6 +686,7 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t units = 4u * a.G, T = a.J * units;
     allow_next_kernel();
+    if (tid == 0) { s.refused = 0xFFFFFFFFu; s.nearly = 0u; }
     if (lane == 0) {
         for (int i = 0; i < kRing; ++i) mbar_init(&s.mbar[warp][i], 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -795,7 +814,15 @@ k_scan(const EncArgs a, const __grid_constant__ PowTable pw, const __grid_consta
                     listing = room == kSlotEntries && promise <= kListMost;
                     if (listing) {
                         room = min(kUnit, (promise * 5u / 4u + 63u) & ~31u);
-                        if (lane == 0) piece = pool_take(a, room * 6u);
+                        piece = kNoPlace;
+                        // (32 pools in turn take 20 us: not again for as long a list)
+                        if (lane == 0 && room * 6u < *const_cast<volatile uint32_t*>(&s.refused)) {
+                            const uint32_t limit = lists_limit(a, promise);
+                            uint64_t fill = 0ull;
+                            piece = pool_take(a, room * 6u, limit, *const_cast<volatile uint32_t*>(&s.nearly) != 0u, fill);
+                            if (fill > limit - limit / 8u) s.nearly = 1u;
+                            if (piece == kNoPlace) atomicMin(&s.refused, room * 6u);
+                        }
                         piece = __shfl_sync(kFullMask, piece, 0);
                         listing = piece != kNoPlace;
                         if (listing) {

@@ -132,3 +132,21 @@ def test_blobs_go_where_their_lists_were(workspace):
         _streams_equal([out], [v], po)
         assert binding.listed_tiles(1) == [0] and late_blobs() == 0
     assert ws.intact()
+
+
+def test_lists_leave_room_for_the_blobs_of_tiles_without(workspace):
+    # a tenth of the entries kept and room for two lists in three: the other tiles are read again, and none is packed twice
+    n = 4000 * TILE
+    v = np.random.default_rng(9).standard_normal(n).astype(np.float32)
+    base = workloads.base_for_keep(v[::16], n // 160)
+    base **= (1 + np.log(16) / (128 * np.log(base)))         # (the sum of all entries, not of every sixteenth)
+    pg, po = binding.params(base), oracle.params(base)
+    ws = workspace(_least(n, 14) + 36 * MIB)
+    out = G.Guarded(4 * n)
+    dev = G.to_dev(v)
+    for rep in range(2):
+        assert binding.compress(dev, pg, out.view) == 0
+        _streams_equal([out], [v], po)
+        assert binding.listed_tiles(1)[0] > 400 and late_blobs() == 0
+    assert binding.stream_info(out.view)[1] > n // 12
+    assert ws.intact()
