@@ -30,6 +30,7 @@
 #pragma once
 
 #include <cstddef>
+#include <type_traits>
 
 #include "common.cuh"
 #include "bits.cuh"
@@ -48,6 +49,7 @@ constexpr uint32_t kDecWarpWords   = kDecWarpMax * (8u + 5u + 16u) / 32u + 4u;  
 constexpr uint32_t kDecSeveralWords = kDecWarpSeveral * (8u + 5u + 16u) / 32u + kDecMaxStreams + 4u;   // ... of several streams' together
 constexpr uint32_t kBlockStageWords = 4096;   // blobs larger than this in total are parsed from global memory
 constexpr uint32_t kBlockListMax   = 8192;    // keys of a group (all streams together) the block path lists in shared memory
+constexpr uint32_t kWideListMax    = 1u << 14;      // ... of a group wider than the tile, in the tile's place
 // From this many keys on the group's whole slice of dense_out goes through shared memory: scattered over 2048 sectors of 32 bytes
 // they touch more than half of it, and a bulk copy moves whole pages (10 % of 2^26 entries: 96 us with, 111 without the slice).
 constexpr uint32_t kTileMinKeys    = 1536;
@@ -567,6 +569,25 @@ __device__ __forceinline__ void update_slice(const DecArgs& a, const float* tile
     }
 }
 
+// K entries of stream w (those whose bit of `on` is set) straight in memory, all accesses of a step in flight together: added into
+// dense_out, or (update) their coordinates updated once with the g that the streams have left there (one stream: with its value).
+template <bool ONE, int MODE, int K>
+__device__ __forceinline__ void entries_in_memory(const DecArgs& a, const DecShared& s, uint32_t w, uint32_t lo, bool update, uint32_t on, const uint32_t (&key)[K], const uint32_t (&code)[K]) {
+    uint32_t kk[K]; float x[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) { kk[i] = lo + key[i]; x[i] = 0.0f; }
+    if (MODE == 0 || (MODE == 2 && !update)) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) if ((on >> i) & 1u) x[i] = a.dense[kk[i]];
+#pragma unroll
+        for (int i = 0; i < K; ++i) if ((on >> i) & 1u) a.dense[kk[i]] = __fadd_rn(x[i], code_value(s.val[w], code[i]));
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) if ((on >> i) & 1u) x[i] = ONE && mode_fused(MODE) ? code_value(s.val[w], code[i]) : atomicExch(a.dense + dense_at<MODE>(kk[i]), 0.0f);
+        adam_run<MODE == 3, K>(a, kk, x);
+    }
+}
+
 // One group by the whole block; s.g_* hold its directory entries.
 template <bool ONE, int MODE>
 __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t& tile_parity, int tid, int lane, int warp) {
@@ -652,6 +673,22 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
     // model update of many keys: a sweep over the slice of g
     const bool sweep_all = mode_fused(MODE) && small_group && (total >= (MODE == 2 ? kSweepMinKeys : kSweepMinPacked) || !lists) &&
                            (MODE == 3 || ((reinterpret_cast<uintptr_t>(a.theta) | reinterpret_cast<uintptr_t>(a.m) | reinterpret_cast<uintptr_t>(a.v)) & 15u) == 0u);
+    // lists of 32-bit keys in the tile's place, for groups (or passes) that do not use it otherwise
+    uint32_t* wkey = reinterpret_cast<uint32_t*>(s.u.tile);
+    const bool wide_lists = !small_group && listed <= kWideListMax && words <= kBlockStageWords;
+    const int wide_sweeps = MODE == 2 && !ONE ? 2 : 1;                  // (the update in one launch: g first, from all streams)
+    auto apply_list = [&](uint32_t w, const Blob& b, uint32_t l0, bool update) {      // neighbouring threads on neighbouring keys
+        for (uint32_t j0 = (uint32_t)tid; j0 < b.count; j0 += 4u * kDecThreads) {
+            uint32_t key[4], code[4], on = 0u;
+#pragma unroll
+            for (uint32_t i = 0; i < 4u; ++i) {
+                const uint32_t j = j0 + i * kDecThreads;
+                key[i] = 0u; code[i] = 0u;
+                if (j < b.count) { on |= 1u << i; key[i] = wkey[l0 + j]; code[i] = code_of(b, j); }
+            }
+            entries_in_memory<ONE, MODE, 4>(a, s, w, lo, update, on, key, code);
+        }
+    };
     if (lists) {
         // ---- all streams parsed side by side into the lists
         const uint32_t tn = ONE ? (uint32_t)kDecThreads : (W <= 2u ? kDecThreads / 2u : (W <= 4u ? kDecThreads / 4u : kDecThreads / 8u));
@@ -746,65 +783,111 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
                 }
             }
         }
+    } else if (MODE != 3 && wide_lists) {
+        // ---- a group wider than the tile: all streams parsed side by side into lists in the tile's place, then applied in memory one after
+        // the other.  (Before, each stream was parsed twice, the second time by threads that took runs of consecutive keys one access at a
+        // time: 442 groups of 2^15, eight streams of 200 keys, 86 us, now 40; 12.8 M entries in groups of 2^17, five streams, the update 57, now 21.)
+        const uint32_t tn = ONE ? (uint32_t)kDecThreads : (W <= 2u ? kDecThreads / 2u : (W <= 4u ? kDecThreads / 4u : kDecThreads / 8u));
+        const uint32_t mine = ONE ? 0u : (uint32_t)tid / tn;
+        uint32_t most = 0u;
+        for (uint32_t w = 0; w < W; ++w) most = max(most, s.g_count[w]);
+        const bool small = most <= 4u * tn;
+        Blob b = blob_of(mine < W ? mine : 0u);
+        if (mine >= W) b.count = 0u;
+        const uint32_t list = mine < W ? s.g_list[mine] : 0u;
+        const unsigned long long bad = parse_team<true, true>(a, s, b, span, (uint32_t)tid & (tn - 1u), tn, small, small ? 1u : (most + 8u * tn - 1u) / (8u * tn),
+                                                              lane, warp, [&](uint32_t j, int m, const auto& v) {
+            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+            for (int k = 0; k < K; ++k) if (k < m) wkey[list + j + (uint32_t)k] = v[k];
+        });
+        if (bad != ~0ull) {
+            s.bad[mine] = 1u;
+            dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+        }
+        __syncthreads();
+        for (int sweep = 0; sweep < wide_sweeps; ++sweep) {
+            for (uint32_t w = 0; w < W; ++w) {
+                if (!s.bad[w]) apply_list(w, blob_of(w), s.g_list[w], MODE == 1 || (MODE == 2 && sweep + 1 == wide_sweeps));      // (a failed stream is left out as a whole)
+                __syncthreads();                                        // this stream's updates before the next stream's
+            }
+        }
     } else {
-        // ---- more keys than the lists hold, or a group wider than the tile: stream by stream, the whole block on each
+        // ---- more keys than the lists hold: stream by stream, the whole block on each
         if (slice) { if (!wait_slice()) return; }
         if (mode_fused(MODE) && small_group) {
             for (uint32_t i = tid; i < ((span + 3u) >> 2); i += kDecThreads)
                 reinterpret_cast<float4*>(s.u.tile)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             __syncthreads();
         }
-        const bool in_tile = MODE != 1 && small_group;
-        // (fused update of a wide group: aggregation into dense_out first, then the update over all streams again)
-        const int sweeps = (mode_fused(MODE) && !small_group) ? 2 : 1;
-        for (int sweep = 0; sweep < sweeps; ++sweep) {
-            if (staged && !together) stage_copy(0u, s.g_base[0]);
-            for (uint32_t w = 0; w < W; ++w) {
-                const Blob b = blob_of(w);
-                if (staged && !together) {
-                    copies_wait();
-                    stage_swap(w, s.g_base[w]);
-                    __syncthreads();
-                    if (w + 1u < W) stage_copy(w + 1u, s.g_base[w + 1u]);
-                }
-                if (b.count == 0u) continue;                            // (uniform; the next stream's copy goes to the other half of the stage)
-                // (one stream at a time fits the list far more often than all of them: parsed once then, else once to validate and once to apply)
-                const bool fits = small_group && b.count <= kBlockListMax;
-                const bool small = b.count <= 4u * kDecThreads;
-                const uint32_t rounds = small ? 1u : (b.count + 8u * kDecThreads - 1u) / (8u * kDecThreads);
-                auto put = [&](uint32_t j, int m, const auto& v) {
-                    constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+        // (in the tile or in memory: two loops, each without the other's code)
+        auto each_stream = [&](auto in_tile_c) __attribute__((always_inline)) {
+            constexpr bool in_tile = decltype(in_tile_c)::value;
+            // (fused update of a wide group: aggregation into dense_out first, then the update over all streams again)
+            const int sweeps = small_group ? 1 : wide_sweeps;
+            for (int sweep = 0; sweep < sweeps; ++sweep) {
+                const bool update = MODE == 1 || (MODE == 2 && !small_group && sweep + 1 == sweeps);
+                if (staged && !together) stage_copy(0u, s.g_base[0]);
+                for (uint32_t w = 0; w < W; ++w) {
+                    const Blob b = blob_of(w);
+                    if (staged && !together) {
+                        copies_wait();
+                        stage_swap(w, s.g_base[w]);
+                        __syncthreads();
+                        if (w + 1u < W) stage_copy(w + 1u, s.g_base[w + 1u]);
+                    }
+                    if (b.count == 0u) continue;                        // (uniform; the next stream's copy goes to the other half of the stage)
+                    // (one stream at a time fits the list far more often than all of them: parsed once then, else once to validate and once to
+                    // apply; the tile holds the list where it holds nothing else)
+                    const bool fits = b.count <= (in_tile ? kBlockListMax : kWideListMax);
+                    const bool small = b.count <= 4u * kDecThreads;
+                    const uint32_t rounds = small ? 1u : (b.count + 8u * kDecThreads - 1u) / (8u * kDecThreads);
+                    auto put = [&](uint32_t j, int m, const auto& v) {
+                        constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
 #pragma unroll
-                    for (int k = 0; k < K; ++k) if (fits && k < m) s.u.lkey[j + (uint32_t)k] = (uint16_t)v[k];
-                };
-                const unsigned long long bad = staged ? parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put)
-                                                      : parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put);
-                if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
-                if (!__syncthreads_or(bad != ~0ull ? 1 : 0)) {          // validated in full before any of it is applied
-                    auto apply = [&](uint32_t j, uint32_t key) {
-                        if (in_tile) s.u.tile[key] = __fadd_rn(s.u.tile[key], code_value(s.val[w], code_of(b, j)));
-                        else {
-                            float* x = a.dense + dense_at<MODE>(lo + key);
-                            if (MODE == 0 || (MODE == 2 && sweep == 0)) *x = __fadd_rn(*x, code_value(s.val[w], code_of(b, j)));
-                            else {
-                                const uint32_t kk[1] = {lo + key};
-                                const float gg[1] = {atomicExch(x, 0.0f)};
-                                adam_run<MODE == 3, 1>(a, kk, gg);
+                        for (int k = 0; k < K; ++k) {
+                            if (fits && k < m) {
+                                if constexpr (in_tile) s.u.lkey[j + (uint32_t)k] = (uint16_t)v[k];
+                                else wkey[j + (uint32_t)k] = v[k];
                             }
                         }
                     };
-                    auto apply_run = [&](uint32_t j, int m, const auto& v) {
-                        constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+                    const unsigned long long bad = staged ? parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put)
+                                                          : parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put);
+                    if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+                    if (!__syncthreads_or(bad != ~0ull ? 1 : 0)) {      // validated in full before any of it is applied
+                        auto in_slice = [&](uint32_t j, uint32_t key) { s.u.tile[key] = __fadd_rn(s.u.tile[key], code_value(s.val[w], code_of(b, j))); };
+                        auto apply_run = [&](uint32_t j, int m, const auto& v) {
+                            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+                            if constexpr (in_tile) {
 #pragma unroll
-                        for (int k = 0; k < K; ++k) if (k < m) apply(j + (uint32_t)k, v[k]);
-                    };
-                    if (fits) for (uint32_t j = tid; j < b.count; j += kDecThreads) apply(j, s.u.lkey[j]);
-                    else if (staged) parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
-                    else parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+                                for (int k = 0; k < K; ++k) if (k < m) in_slice(j + (uint32_t)k, v[k]);
+                            } else {
+#pragma unroll
+                                for (int k0 = 0; k0 < K; k0 += 4) {
+                                    uint32_t key[4], code[4], on = 0u;
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) {
+                                        key[k] = v[k0 + k]; code[k] = 0u;
+                                        if (k0 + k < m) { on |= 1u << k; code[k] = code_of(b, j + (uint32_t)(k0 + k)); }
+                                    }
+                                    entries_in_memory<ONE, MODE, 4>(a, s, w, lo, update, on, key, code);
+                                }
+                            }
+                        };
+                        if (fits) {
+                            if constexpr (in_tile) { for (uint32_t j = tid; j < b.count; j += kDecThreads) in_slice(j, s.u.lkey[j]); }
+                            else apply_list(w, b, 0u, update);
+                        } else if (staged) parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+                        else parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+                    }
+                    __syncthreads();                                    // this stream's updates before the next stream's
                 }
-                __syncthreads();                                        // this stream's updates before the next stream's
             }
-        }
+        };
+        if constexpr (MODE == 1) each_stream(std::false_type{});
+        else if constexpr (MODE == 3) each_stream(std::true_type{});
+        else { if (small_group) each_stream(std::true_type{}); else each_stream(std::false_type{}); }
         if (MODE == 0 && slice) {
             store_slice();
         } else if (sweep_all) {

@@ -15,16 +15,16 @@ TILE = 16384
 HYPER = (1e-3, 0.9, 0.999, 1e-8)
 
 
-def _streams(n, counts, workers, seed, tau=128):
+def _streams(n, counts, workers, seed, tau=128, group_log2=14, l=2):
     """One stream per worker with exactly counts[g] kept keys in group g; half of the keys shared with the worker before."""
     rng = np.random.default_rng(seed)
     out, prev = [], None
-    po = oracle.params(1.3 if tau == 128 else 1.9, tau, 2, 14)
+    po = oracle.params(1.3 if tau == 128 else 1.9, tau, l, group_log2)
     for w in range(workers):
         v = np.zeros(n, np.float32)
         keys = []
         for g, c in enumerate(counts):
-            lo, span = g * TILE, min(TILE, n - g * TILE)
+            lo, span = g << group_log2, min(1 << group_log2, n - (g << group_log2))
             c = min(c, span)
             if prev is None:
                 k = rng.choice(span, c, replace=False)
@@ -37,11 +37,11 @@ def _streams(n, counts, workers, seed, tau=128):
         rc, s = oracle.compress(v, po)
         assert rc == 0 and int(np.frombuffer(s[24:32].tobytes(), np.uint64)[0]) == sum(len(k) for k in keys)
         out.append(s)
-    return out, po, binding.params(po.base, tau, 2, 14)
+    return out, po, binding.params(po.base, tau, l, group_log2)
 
 
-def _check(n, counts, workers, seed, tau=128, update=True):
-    streams, po, pg = _streams(n, counts, workers, seed, tau)
+def _check(n, counts, workers, seed, tau=128, update=True, group_log2=14, l=2):
+    streams, po, pg = _streams(n, counts, workers, seed, tau, group_log2, l)
     rng = np.random.default_rng(seed + 1)
     binding.ensure_workspace(n, pg)
     dev = [G.to_dev(np.concatenate([s, np.zeros(-s.size % 16 + 16, np.uint8)])) for s in streams]
@@ -63,11 +63,13 @@ def _check(n, counts, workers, seed, tau=128, update=True):
     packed = torch.stack(arrays, dim=1).reshape(-1)
     assert oracle.sparse_adam_update(streams, n, po, *HYPER, theta, m, v) == 0
     assert binding.sparse_adam_update_batch(dev, sizes, n, pg, binding.Adam(*HYPER), arrays[3], *arrays[:3]) == 0
-    assert binding.sparse_adam_update_packed_batch(dev, sizes, n, pg, binding.Adam(*HYPER), packed) == 0
+    if group_log2 <= 14:
+        assert binding.sparse_adam_update_packed_batch(dev, sizes, n, pg, binding.Adam(*HYPER), packed) == 0
     assert binding.decode_status() == 0
     packed = packed.reshape(n, 4)
     for i, x in enumerate((theta, m, v, np.zeros(n, np.float32))):
-        assert np.array_equal(arrays[i].cpu().numpy(), x) and np.array_equal(packed[:, i].cpu().numpy(), x), i
+        assert np.array_equal(arrays[i].cpu().numpy(), x), i
+        assert group_log2 > 14 or np.array_equal(packed[:, i].cpu().numpy(), x), i
 
 
 # one stream: warp / block (256), sweep of the update (768, packed 2048), slice of dense_out (1536), words of a blob that fit
@@ -99,3 +101,37 @@ def test_many_groups_per_block(workers):
     counts[300:330] = [1023, 1024, 1025] * 10
     counts[1000:1012] = 300
     _check(groups * TILE - 9, counts.tolist(), workers, 40 + workers, update=False)
+
+
+# groups wider than the slice of dense_out: all streams' keys in one list of up to 2^14, stream by stream, and streams beyond a list; blobs
+# in the stage (4096 words together, 2048 one at a time) or read where they are
+@pytest.mark.parametrize("group_log2", [15, 17, 20])
+@pytest.mark.parametrize("workers,count", [(1, 1), (1, 700), (1, 5000), (1, 16384), (1, 16385), (1, 30000), (2, 300), (2, 4000), (3, 5464), (8, 200), (8, 1500), (5, 2048), (8, 2100)])
+def test_wide_groups(workers, count, group_log2):
+    _check((3 << group_log2) - 5, [count, 0, max(1, count - 1)], workers, 700 + workers + count, group_log2=group_log2)
+
+
+# streams that fail in one group are left out there as a whole, the others not
+@pytest.mark.parametrize("group_log2,count", [(14, 40), (14, 90), (14, 170), (14, 400), (16, 300), (16, 6000)])
+def test_failed_streams_are_left_out(group_log2, count):
+    n, workers = (3 << group_log2) - 5, 6
+    streams, po, pg = _streams(n, [count, count + 1, count], workers, 900 + count, group_log2=group_log2)
+    sound = np.random.default_rng(5).standard_normal(n).astype(np.float32)
+    dense = torch.from_numpy(sound.copy()).to(G.dev())
+    for w in (0, 2, 3, 5):
+        assert oracle.decompress_accumulate(streams[w], n, po, sound) == 0
+    for w in (1, 4):                                       # the first deltas of group 1 become 0
+        s = streams[w] = streams[w].copy()
+        cnt, off = (int(x) for x in np.frombuffer(s[72:80].tobytes(), np.uint32))
+        cnt &= 0xFFFFFF
+        bits = np.unpackbits(s[4 * off:4 * off + 2 * cnt + 16])
+        bits[10 * cnt:10 * cnt + 40] = 0
+        s[4 * off:4 * off + 2 * cnt + 16] = np.packbits(bits)
+    status = [oracle.decompress_accumulate(s, n, po, np.zeros(n, np.float32)) for s in streams]
+    assert [bool(x) for x in status] == [False, True, False, False, True, False]
+    binding.ensure_workspace(n, pg)
+    dev = [G.to_dev(np.concatenate([s, np.zeros(-s.size % 16 + 16, np.uint8)])) for s in streams]
+    assert binding.decompress_accumulate_batch(dev, [s.size for s in streams], n, pg, dense) == 0
+    assert binding.decode_status() == status[1]
+    lo, hi = 1 << group_log2, 2 << group_log2
+    assert np.array_equal(dense.cpu().numpy()[lo:hi], sound[lo:hi])
