@@ -43,10 +43,9 @@ constexpr int      kDecWarps       = kDecThreads / 32;
 constexpr int      kDecMaxStreams  = 8;       // streams per launch
 constexpr uint32_t kDecWarpMax     = 1024;    // groups with more keys go to the whole block (one stream, many groups per block)
 constexpr uint32_t kDecWarpFew     = 256;     // the same when a block has only a few groups: its other warps would stand idle
-constexpr uint32_t kDecWarpSeveral = 248;     // the same for all streams of a launch with several together (below 255: entry numbers are bytes)
-constexpr uint32_t kWarpSlots      = 1024;    // slots of a warp's table of distinct keys
+constexpr uint32_t kTeamBytes      = 6144;    // launch with several streams: shared memory of a team, for each of its warps
+constexpr uint32_t kTeamSlotsLog2  = 10, kTeamSlots = 1u << kTeamSlotsLog2;      // ... of which slots (16 bits each) of the table of distinct keys
 constexpr uint32_t kDecWarpWords   = kDecWarpMax * (8u + 5u + 16u) / 32u + 4u;    // words of one stream's blob on the warp path (16: largest group_log2 it takes)
-constexpr uint32_t kDecSeveralWords = kDecWarpSeveral * (8u + 5u + 16u) / 32u + kDecMaxStreams + 4u;   // ... of several streams' together
 constexpr uint32_t kBlockStageWords = 4096;   // blobs larger than this in total are parsed from global memory
 constexpr uint32_t kBlockListMax   = 8192;    // keys of a group (all streams together) the block path lists in shared memory
 constexpr uint32_t kWideListMax    = 1u << 14;      // ... of a group wider than the tile, in the tile's place
@@ -187,13 +186,9 @@ struct DecWarpOne {
     uint32_t blob[kDecWarpWords];
     uint16_t key[kDecWarpMax];       // group-relative keys
 };
-struct DecWarpSeveral {
-    uint32_t blob[kDecSeveralWords];
-    uint8_t  slot[kWarpSlots];       // table of distinct keys: the entry that stands for the key; 0xFF: free
-    uint16_t key[kDecWarpSeveral];   // of all streams, stream after stream
-    uint8_t  own[kDecWarpSeveral + 8];        // the entry that stands for this entry's key
-    float    acc[kDecWarpSeveral];   // there: the key's value
-};
+// Bytes that a group of several streams takes of its team's memory beside the table: 4 for a coordinate's value and 2 for a key of each
+// entry, the blobs, two words behind them that the parse may look at, and one of flags.
+__host__ __device__ constexpr uint32_t team_bytes(uint32_t entries, uint32_t words) { return 6u * ((entries + 1u) & ~1u) + 4u * (words + 3u); }
 
 struct DecShared {
     float              val[kDecMaxStreams][132];
@@ -203,9 +198,9 @@ struct DecShared {
     uint32_t           ok[kDecMaxStreams];
     // the directory entries of the block's groups, kDecThreads (group, stream) pairs at a time
     uint32_t           e_cm[kDecThreads], e_off[kDecThreads], e_nw[kDecThreads];
-    uint32_t           gtot[kDecThreads];           // keys of each of these groups over all streams
-    uint16_t           light[kDecThreads], heavy[kDecThreads];
-    uint32_t           n_light, n_heavy, next_light;
+    uint32_t           gtot[kDecThreads];           // keys of each of these groups over all streams; several streams: from kDecThreads / 2 on their words
+    uint16_t           light[kDecThreads], heavy[kDecThreads];      // groups for a warp, and from the end on for four; for the block, and from the end on for two
+    uint32_t           n_light[3], n_heavy, next_light[3], grab[kDecWarps];
     uint32_t           scan[2][kDecWarps];
     uint32_t           got;           // answer of thread 0 to the block
     uint32_t           bad[kDecMaxStreams];
@@ -215,7 +210,7 @@ struct DecShared {
     unsigned long long tile_bar;      // mbarrier of the bulk copy that loads the tile
     union alignas(128) {               // (bulk copies need 16-byte aligned shared addresses)
         DecWarpOne     one[kDecWarps];
-        DecWarpSeveral several[kDecWarps];
+        uint8_t        team[kDecWarps][kTeamBytes];
         struct {                                 // block path
             float      tile[1u << 14];           // the group's slice of dense_out (or of g)
             uint32_t   bstage[kBlockStageWords + 4];
@@ -405,41 +400,111 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;
 
 constexpr uint32_t kNoKey = 0xFFFFu;               // (in a list of keys) an entry of a stream that failed
 
-// One group by one warp; entries eb + w of the block's table are stream w's directory entry.
-template <bool ONE, int MODE>
-__device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t eb, int lane, int warp) {
+// One group of a single stream by one warp; entry eb of the block's table is its directory entry.
+template <int MODE>
+__device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint32_t g, uint32_t eb, int lane, int warp) {
     const uint64_t lo64 = (uint64_t)g << a.group_log2;
     const uint64_t hi64 = lo64 + (1ull << a.group_log2);
     const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
-    uint32_t* blob = ONE ? s.u.one[warp].blob : s.u.several[warp].blob;
-    uint16_t* keys = ONE ? s.u.one[warp].key : s.u.several[warp].key;
+    uint32_t* blob = s.u.one[warp].blob;
+    uint16_t* keys = s.u.one[warp].key;
+    Blob b;
+    b.words = blob; b.nwords = s.e_nw[eb]; b.count = s.e_cm[eb] & 0xFFFFFFu; b.M = s.e_cm[eb] >> 24;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(a.stream[0]) + s.e_off[eb];
+    for (uint32_t i = lane; i < b.nwords; i += 32u) copy_word_async(&blob[i], src + i);
+    copies_wait();
+    __syncwarp();
+    for (uint32_t i = lane; i < b.nwords; i += 32u) blob[i] = bswap32(blob[i]);
+    __syncwarp();
+    const bool small = b.count <= 128u;
+    const unsigned long long bad = parse_team<false, true>(a, s, b, span, (uint32_t)lane, 32u, small, small ? 1u : (b.count + 255u) / 256u, lane, warp,
+                                                           [&](uint32_t j, int m, const auto& v) {
+        constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+        for (int k = 0; k < K; ++k) if (k < m) keys[j + (uint32_t)k] = (uint16_t)v[k];
+    });
+    if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+    const uint32_t c0 = __any_sync(kFullMask, bad != ~0ull) ? 0u : b.count;       // a failed group is left out as a whole
+    __syncwarp();
+    if constexpr (MODE == 0) {
+        for (uint32_t e0 = 0; e0 < c0; e0 += 256u) {
+            uint32_t kk[8]; float x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t e = e0 + 32u * i + lane;
+                kk[i] = e < c0 ? lo + keys[e] : 0xFFFFFFFFu;
+                x[i] = e < c0 ? a.dense[kk[i]] : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (kk[i] != 0xFFFFFFFFu) a.dense[kk[i]] = __fadd_rn(x[i], code_value(s.val[0], code_at<true>(b, e0 + 32u * i + lane)));
+        }
+    } else {
+        for (uint32_t e0 = 0; e0 < c0; e0 += 128u) {
+            uint32_t kk[4]; float gg[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t e = e0 + 32u * i + lane;
+                kk[i] = e < c0 ? lo + keys[e] : 0u;
+                // (a single stream: g is the decoded value; 0 + value is the value)
+                if constexpr (MODE == 1) gg[i] = e < c0 ? atomicExch(a.dense + kk[i], 0.0f) : 0.0f;
+                else gg[i] = e < c0 ? code_value(s.val[0], code_at<true>(b, e)) : 0.0f;
+            }
+            adam_run<MODE == 3, 4>(a, kk, gg);
+        }
+    }
+    __syncwarp();                                                       // (the list is rewritten by the warp's next group)
+}
+
+// Several streams: one group by a team of NW warps (1, 2 or 4); entries eb + w of the block's table are stream w's directory entry.  One
+// entry stands for every distinct key; it collects the streams' values in stream order, so that each coordinate takes one round
+// trip to memory.  keys: a key, or kSharedKey | the entry that stands for it.
+//
+// A group is a chain of about ten steps (copy, flags, deltas, table, one addition a stream, memory) of which few fill a block's 512
+// threads.  Groups of 250 to 1500 keys by the whole block took 10 us each, two at a time on an SM; by teams (32, 16 or 8 groups
+// at a time) eight streams of 47 keys a group take 51 us instead of 100 (2781 groups), of 98 keys 104 instead of 136.
+constexpr uint32_t kSharedKey = 0x8000u;
+template <int NW> __device__ __forceinline__ void dec_team_sync(int team) {
+    if constexpr (NW == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(32 * NW) : "memory");
+}
+template <int MODE, int NW>
+__device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t eb, int lane, int warp) {
+    const uint64_t lo64 = (uint64_t)g << a.group_log2;
+    const uint64_t hi64 = lo64 + (1ull << a.group_log2);
+    const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
+    const int team = warp / NW;
+    const uint32_t tl = 32u * (uint32_t)(warp % NW) + (uint32_t)lane;   // thread of the team
+    constexpr uint32_t threads = 32u * NW;
     // lane w: stream w
     uint32_t cm = 0u, off = 0u, nw = 0u;
     if (lane < (int)W) { cm = s.e_cm[eb + lane]; off = s.e_off[eb + lane]; nw = s.e_nw[eb + lane]; }
     uint32_t count = cm & 0xFFFFFFu;
-    const uint32_t M = cm >> 24;
-    uint32_t wbase = 0u, lbase = 0u, total = 0u;
-    if (!ONE) {
-        wbase = warp_incl_scan(nw, lane) - nw;
-        const uint32_t li = warp_incl_scan(count, lane);
-        lbase = li - count;
-        total = __shfl_sync(kFullMask, li, 31);
-    }
+    const uint32_t M = cm >> 24, wincl = warp_incl_scan(nw, lane), wbase = wincl - nw, lincl = warp_incl_scan(count, lane), lbase = lincl - count;
+    const uint32_t words = __shfl_sync(kFullMask, wincl, 31), total = __shfl_sync(kFullMask, lincl, 31);
+    uint8_t* mem = s.u.team[team * NW];
+    uint16_t* slot = reinterpret_cast<uint16_t*>(mem);                  // table of distinct keys: the entry that stands for the key; 0xFFFF: free
+    // (at least twice the entries, or all of the memory's share: 1.5 times)
+    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(2u * total + 63u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
+    float* acc = reinterpret_cast<float*>(slot + kTeamSlots * NW);
+    uint16_t* keys = reinterpret_cast<uint16_t*>(acc + ((total + 1u) & ~1u));
+    uint32_t* blob = reinterpret_cast<uint32_t*>(keys + ((total + 1u) & ~1u));
+    uint32_t* failed = blob + words + 2u;                               // bit w: stream w
     // ---- the streams' blobs into shared memory, all copies in flight together
     for (uint32_t w = 0; w < W; ++w) {
         const uint32_t n_w = __shfl_sync(kFullMask, nw, w), o_w = __shfl_sync(kFullMask, off, w), b_w = __shfl_sync(kFullMask, wbase, w);
         const uint32_t* src = reinterpret_cast<const uint32_t*>(a.stream[w]) + o_w;
-        for (uint32_t i = lane; i < n_w; i += 32u) copy_word_async(&blob[b_w + i], src + i);
+        for (uint32_t i = tl; i < n_w; i += threads) copy_word_async(&blob[b_w + i], src + i);
     }
-    const uint32_t words = ONE ? __shfl_sync(kFullMask, nw, 0) : __shfl_sync(kFullMask, wbase + nw, W - 1u);
-    if (!ONE) for (uint32_t i = lane; i < kWarpSlots / 4u; i += 32u) reinterpret_cast<uint32_t*>(s.u.several[warp].slot)[i] = 0xFFFFFFFFu;
+    for (uint32_t i = tl; i < slots / 2u; i += threads) reinterpret_cast<uint32_t*>(slot)[i] = 0xFFFFFFFFu;
+    if (tl == 0u) *failed = 0u;
     copies_wait();
-    __syncwarp();
-    for (uint32_t i = lane; i < words; i += 32u) blob[i] = bswap32(blob[i]);
-    __syncwarp();
-    // ---- parse: 32, 16, 8 or 4 lanes per stream
-    const uint32_t tn = ONE ? 32u : (W <= 2u ? 16u : (W <= 4u ? 8u : 4u));
-    const uint32_t mine = ONE ? 0u : (uint32_t)lane / tn;               // (beyond W - 1: a stream without keys)
+    dec_team_sync<NW>(team);
+    for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
+    dec_team_sync<NW>(team);
+    // ---- parse: the threads shared out among the streams, within a warp
+    const uint32_t tn = min(32u, (W <= 2u ? 16u : (W <= 4u ? 8u : 4u)) * NW);
+    const uint32_t mine = min(tl / tn, 31u);                            // (beyond W - 1: a stream without keys)
     Blob b;
     b.count = __shfl_sync(kFullMask, count, mine);
     b.nwords = __shfl_sync(kFullMask, nw, mine);
@@ -454,101 +519,102 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
 #pragma unroll
         for (int k = 0; k < K; ++k) if (k < m) keys[list + j + (uint32_t)k] = (uint16_t)v[k];
     });
-    const uint32_t badm = __ballot_sync(kFullMask, bad != ~0ull);
-    if (badm) {                                                         // a failed stream is left out as a whole
-        if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
-        const bool out = lane < (int)W && ((badm >> (lane * tn)) & (tn >= 32u ? 0xFFFFFFFFu : (1u << tn) - 1u)) != 0u;
-        if (!ONE && out) for (uint32_t j = 0; j < count; ++j) keys[lbase + j] = kNoKey;
-        if (out) count = 0u;
+    if (bad != ~0ull) {
+        dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+        atomicOr(failed, 1u << mine);
     }
-    __syncwarp();
-
-    if constexpr (ONE) {
-        const uint32_t c0 = __shfl_sync(kFullMask, count, 0);
-        if constexpr (MODE == 0) {
-            for (uint32_t e0 = 0; e0 < c0; e0 += 256u) {
-                uint32_t kk[8]; float x[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const uint32_t e = e0 + 32u * i + lane;
-                    kk[i] = e < c0 ? lo + keys[e] : 0xFFFFFFFFu;
-                    x[i] = e < c0 ? a.dense[kk[i]] : 0.0f;
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (kk[i] != 0xFFFFFFFFu) a.dense[kk[i]] = __fadd_rn(x[i], code_value(s.val[0], code_at<true>(b, e0 + 32u * i + lane)));
-            }
-        } else {
-            for (uint32_t e0 = 0; e0 < c0; e0 += 128u) {
-                uint32_t kk[4]; float gg[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t e = e0 + 32u * i + lane;
-                    kk[i] = e < c0 ? lo + keys[e] : 0u;
-                    // (a single stream: g is the decoded value; 0 + value is the value)
-                    if constexpr (MODE == 1) gg[i] = e < c0 ? atomicExch(a.dense + kk[i], 0.0f) : 0.0f;
-                    else gg[i] = e < c0 ? code_value(s.val[0], code_at<true>(b, e)) : 0.0f;
-                }
-                adam_run<MODE == 3, 4>(a, kk, gg);
-            }
+    dec_team_sync<NW>(team);
+    const uint32_t out = *failed;
+    if (out) {                                                          // a failed stream is left out as a whole
+        for (uint32_t w = 0; w < W; ++w) {
+            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w);
+            if ((out >> w) & 1u) for (uint32_t j = tl; j < c_w; j += threads) keys[b_w + j] = kNoKey;
         }
-    } else {
-        // Several streams: one entry stands for every distinct key (found through a small open-addressing table: a lane writes
-        // its entry into a free slot and looks who is there); it collects the streams' values in stream order.
-        DecWarpSeveral& ws = s.u.several[warp];
-        for (uint32_t e0 = 0; e0 < total; e0 += 32u) {
-            const uint32_t e = e0 + (uint32_t)lane;
-            const uint32_t key = e < total ? keys[e] : kNoKey;
-            bool open = key != kNoKey;
-            uint32_t h = (key * 0x9E3779B1u) >> 22, owner = e;
-            if (MODE == 1) open = false;                                // (g is exchanged out of dense_out: no matter how often a key comes)
+        if ((out >> lane) & 1u) count = 0u;
+        dec_team_sync<NW>(team);
+    }
+    // ---- who stands for each key (open addressing)
+    for (uint32_t e0 = 0; e0 < total; e0 += threads) {
+        const uint32_t e = e0 + tl;
+        const uint32_t key = e < total ? keys[e] : kNoKey;
+        bool open = key != kNoKey;
+        uint32_t h = (key * 0x9E3779B1u) >> (32u - slots_log2), owner = e;
+        if (MODE == 1) open = false;                                    // (g is exchanged out of dense_out: no matter how often a key comes)
+        if constexpr (NW == 1) {                                        // (a lane writes its entry into a free slot and looks who is there)
             while (__any_sync(kFullMask, open)) {
-                if (open && ws.slot[h] == 0xFFu) ws.slot[h] = (uint8_t)e;
+                if (open && slot[h] == 0xFFFFu) slot[h] = (uint16_t)e;
                 __syncwarp();
                 if (open) {
-                    const uint32_t r = ws.slot[h];
-                    if (keys[r] == key) { owner = r; open = false; }
-                    else h = (h + 1u) & (kWarpSlots - 1u);
+                    const uint32_t r = slot[h];
+                    if (r == e || keys[r] == key) { owner = r; open = false; }
+                    else h = (h + 1u) & (slots - 1u);
                 }
                 __syncwarp();
             }
-            if (key != kNoKey) {
-                ws.own[e] = (uint8_t)owner;
-                if (owner == e) {
-                    if constexpr (MODE == 0) copy_word_async(&ws.acc[e], a.dense + lo + key);
-                    else if constexpr (MODE == 1) ws.acc[e] = atomicExch(a.dense + lo + key, 0.0f);
-                    else ws.acc[e] = 0.0f;
-                }
+        } else {
+            while (open) {
+                const uint32_t r = atomicCAS(reinterpret_cast<unsigned short*>(&slot[h]), (unsigned short)0xFFFFu, (unsigned short)e);
+                if (r == 0xFFFFu) open = false;
+                else if (keys[r] == key) { owner = r; open = false; }
+                else h = (h + 1u) & (slots - 1u);
             }
+            __syncwarp();
         }
-        if constexpr (MODE == 0) copies_wait();
-        __syncwarp();
-        if constexpr (MODE != 1) {
-            for (uint32_t w = 0; w < W; ++w) {
-                const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, wbase, w);
-                const uint8_t* codes = reinterpret_cast<const uint8_t*>(blob + s_w);
-                for (uint32_t j = lane; j < c_w; j += 32u) {
-                    const uint32_t at = ws.own[b_w + j];
-                    ws.acc[at] = __fadd_rn(ws.acc[at], code_value(s.val[w], codes[j ^ 3u]));
-                }
-                __syncwarp();
-            }
-        }
-        for (uint32_t e0 = 0; e0 < total; e0 += 128u) {
-            uint32_t kk[4]; float gg[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t e = e0 + 32u * i + lane;
-                const uint32_t key = e < total ? keys[e] : kNoKey;
-                const bool on = key != kNoKey && ws.own[e] == e;
-                kk[i] = lo + key;
-                gg[i] = on ? ws.acc[e] : 0.0f;
-                if constexpr (MODE == 0) if (on) a.dense[kk[i]] = gg[i];
-            }
-            if constexpr (MODE != 0) adam_run<MODE == 3, 4>(a, kk, gg);
+        if (key != kNoKey) {
+            if (owner != e) keys[e] = (uint16_t)(kSharedKey | owner);   // (nobody looks at the key of an entry that is in no slot)
+            else if constexpr (MODE == 0) copy_word_async(&acc[e], a.dense + lo + key);
+            else if constexpr (MODE == 1) acc[e] = atomicExch(a.dense + lo + key, 0.0f);
+            else acc[e] = 0.0f;
         }
     }
-    __syncwarp();                                                       // (the lists are rewritten by the warp's next group)
+    if constexpr (MODE == 0) copies_wait();
+    dec_team_sync<NW>(team);
+    if constexpr (MODE != 1) {
+        for (uint32_t w = 0; w < W; ++w) {
+            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, wbase, w);
+            const uint8_t* codes = reinterpret_cast<const uint8_t*>(blob + s_w);
+            for (uint32_t j = tl; j < c_w; j += threads) {
+                const uint32_t k = keys[b_w + j], at = k & kSharedKey ? k & (kSharedKey - 1u) : b_w + j;
+                acc[at] = __fadd_rn(acc[at], code_value(s.val[w], codes[j ^ 3u]));
+            }
+            dec_team_sync<NW>(team);
+        }
+    }
+    for (uint32_t e0 = 0; e0 < total; e0 += 4u * threads) {
+        uint32_t kk[4]; float gg[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t e = e0 + threads * (uint32_t)i + tl;
+            const uint32_t key = e < total ? keys[e] : kNoKey;
+            const bool on = (key & kSharedKey) == 0u;                   // (a key below 2^15; not one that another entry stands for, nor kNoKey)
+            kk[i] = lo + key;
+            gg[i] = on ? acc[e] : 0.0f;
+            if constexpr (MODE == 0) if (on) a.dense[kk[i]] = gg[i];
+        }
+        if constexpr (MODE != 0) adam_run<MODE == 3, 4>(a, kk, gg);
+    }
+    dec_team_sync<NW>(team);                                            // (the memory is rewritten for the team's next group)
+}
+
+// entry x of the list of groups for one (list 0), two or four (2) warps
+__device__ __forceinline__ uint16_t& team_list_entry(DecShared& s, uint32_t list, uint32_t x) {
+    return list == 0u ? s.light[x] : list == 1u ? s.heavy[kDecThreads - 1u - x] : s.light[kDecThreads - 1u - x];
+}
+
+// The block's groups for teams of NW warps, one after the other to whichever team is free.
+template <int MODE, int NW>
+__device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint32_t W, uint32_t first, int lane, int warp) {
+    constexpr uint32_t kList = NW == 1 ? 0u : NW == 2 ? 1u : 2u;
+    const uint32_t n = s.n_light[kList];
+    const int team = warp / NW;
+    for (;;) {
+        if (warp % NW == 0 && lane == 0) s.grab[team] = atomicAdd(&s.next_light[kList], 1u);
+        dec_team_sync<NW>(team);
+        const uint32_t x = s.grab[team];
+        if (x >= n) break;
+        const uint32_t i = team_list_entry(s, kList, x);
+        team_group<MODE, NW>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
+    }
 }
 
 // index of coordinate k's aggregated gradient (or entry of dense_out) as a float
@@ -963,11 +1029,15 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
     unsigned int* q_taken = a.q_ctl + 1, *q_done = a.q_ctl + 2, *q_exited = a.q_ctl + 3, *q_reserved = a.q_ctl + 4;
     const bool queue = a.G > B;
     const uint32_t warp_max = owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew;
+    // Several streams: teams take groups of fewer keys than the slice (the update: the sweep) is for; with few groups to a block larger
+    // teams, so that its warps have work.
+    const uint32_t team_max = MODE == 2 ? kSweepMinKeys : kTileMinKeys, least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
     for (uint32_t first = 0; first < owned; first += per_batch) {
         if (first > 0u) { __syncthreads(); d0 = d1 = d2 = 0u; load_dir(first + my_i); }
         // ---- classify the batch's groups
         s.gtot[tid] = 0u;
-        if (tid == 0) { s.n_light = 0u; s.n_heavy = 0u; s.next_light = 0u; }
+        if (tid < 3) { s.n_light[tid] = 0u; s.next_light[tid] = 0u; }
+        if (tid == 0) s.n_heavy = 0u;
         __syncthreads();
         const uint32_t in_batch = min(per_batch, owned - first);
         if (my_i < in_batch) {
@@ -977,13 +1047,20 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
             const uint32_t cm = sound ? d0 : 0u;
             s.e_cm[tid] = cm; s.e_off[tid] = d1; s.e_nw[tid] = nw;
             if (ONE) s.gtot[tid] = cm & 0xFFFFFFu;
-            else if (cm) atomicAdd(&s.gtot[my_i], cm & 0xFFFFFFu);
+            else if (cm) { atomicAdd(&s.gtot[my_i], cm & 0xFFFFFFu); atomicAdd(&s.gtot[kDecThreads / 2 + my_i], nw); }
         }
         __syncthreads();
         if (tid < (int)in_batch) {
             const uint32_t tot = s.gtot[tid];
             if (tot != 0u) {
-                if (ONE ? tot <= warp_max && a.group_log2 <= 16u : tot <= kDecWarpSeveral && a.group_log2 <= 15u) s.light[atomicAdd(&s.n_light, 1u)] = (uint16_t)tid;
+                uint32_t list = 3u;
+                if (ONE) { if (tot <= warp_max && a.group_log2 <= 16u) list = 0u; }
+                else if (a.group_log2 <= 15u && tot < team_max) {
+                    const uint32_t bytes = team_bytes(tot, s.gtot[kDecThreads / 2 + tid]), room = kTeamBytes - 2u * kTeamSlots;
+                    list = bytes <= room ? 0u : bytes <= 2u * room ? 1u : bytes <= 4u * room ? 2u : 3u;
+                    if (list < least_team && tot > 64u) list = least_team;
+                }
+                if (list < 3u) team_list_entry(s, list, atomicAdd(&s.n_light[list], 1u)) = (uint16_t)tid;
                 else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
             }
         }
@@ -1016,15 +1093,21 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
             if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             __syncthreads();
         }
-        // ---- groups for single warps
-        const uint32_t n_light = s.n_light;
-        for (;;) {
-            uint32_t x = 0u;
-            if (lane == 0) x = atomicAdd(&s.next_light, 1u);
-            x = __shfl_sync(kFullMask, x, 0);
-            if (x >= n_light) break;
-            const uint32_t i = s.light[x];
-            warp_group<ONE, MODE>(a, s, W, blockIdx.x + (first + i) * B, i * W, lane, warp);
+        // ---- groups for teams of warps
+        if constexpr (ONE) {
+            const uint32_t n_light = s.n_light[0];
+            for (;;) {
+                uint32_t x = 0u;
+                if (lane == 0) x = atomicAdd(&s.next_light[0], 1u);
+                x = __shfl_sync(kFullMask, x, 0);
+                if (x >= n_light) break;
+                const uint32_t i = s.light[x];
+                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, lane, warp);
+            }
+        } else {
+            if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp); __syncthreads(); }
+            if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, lane, warp); __syncthreads(); }
+            team_groups<MODE, 1>(a, s, W, first, lane, warp);
         }
     }
 

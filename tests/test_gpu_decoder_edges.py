@@ -135,3 +135,21 @@ def test_failed_streams_are_left_out(group_log2, count):
     assert binding.decode_status() == status[1]
     lo, hi = 1 << group_log2, 2 << group_log2
     assert np.array_equal(dense.cpu().numpy()[lo:hi], sound[lo:hi])
+
+
+# groups of several streams for teams of one, two and four warps (at most 6 bytes an entry and the blobs in 4, 8 and 16 KiB; less than 1536
+# keys, the update 768) and beyond, next to each other in one block; many groups to a block, few, and one
+@pytest.mark.parametrize("groups,workers,l,group_log2", [(2700, 8, 2, 14), (740, 2, 2, 14), (740, 3, 1, 14), (740, 4, 5, 14), (740, 8, 2, 14),
+                                                         (740, 8, 5, 10), (740, 5, 3, 11), (290, 2, 5, 14), (290, 8, 1, 14)])
+def test_teams_of_warps(groups, workers, l, group_log2):
+    rng = np.random.default_rng(workers + l)
+    totals = rng.choice([0, 8, 60, 64, 65, 230, 248, 256, 380, 470, 480, 490, 500, 512, 540, 767, 768, 769, 940, 960, 1000, 1500, 1535, 1536, 1600], groups)
+    if groups > 1000:
+        totals[rng.random(groups) < 0.7] = 0
+    counts = np.minimum(-(-totals // workers), 1 << group_log2)
+    _check((groups << group_log2) - 9, counts.tolist(), workers, 500 + workers, group_log2=group_log2, l=l, update=groups == 740)
+
+
+@pytest.mark.parametrize("workers,count", [(2, 200), (3, 110), (8, 30), (8, 100), (8, 190), (8, 300)])
+def test_teams_on_groups_of_two_tiles(workers, count):
+    _check((40 << 15) - 9, [count, count + 1] * 20, workers, 600 + count, group_log2=15)
