@@ -186,6 +186,8 @@ struct DecWarpOne {
     uint32_t blob[kDecWarpWords];
     uint16_t key[kDecWarpMax];       // group-relative keys
 };
+constexpr uint32_t kTeamFew        = 249;     // groups of fewer keys go to a warp where groups differ much
+constexpr uint32_t kTeamShared     = 200;     // from this many keys on two warps (four) are quicker than one (eight streams of 16 keys: 18 us, by two 21)
 // Bytes that a group of several streams takes of its team's memory beside the table: 4 for a coordinate's value and 2 for a key of each
 // entry, the blobs, two words behind them that the parse may look at, and one of flags.
 __host__ __device__ constexpr uint32_t team_bytes(uint32_t entries, uint32_t words) { return 6u * ((entries + 1u) & ~1u) + 4u * (words + 3u); }
@@ -484,8 +486,8 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     const uint32_t words = __shfl_sync(kFullMask, wincl, 31), total = __shfl_sync(kFullMask, lincl, 31);
     uint8_t* mem = s.u.team[team * NW];
     uint16_t* slot = reinterpret_cast<uint16_t*>(mem);                  // table of distinct keys: the entry that stands for the key; 0xFFFF: free
-    // (at least twice the entries, or all of the memory's share: 1.5 times)
-    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(2u * total + 63u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
+    // (four times the entries as far as the memory's share goes; never less than 1.5 times)
+    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
     float* acc = reinterpret_cast<float*>(slot + kTeamSlots * NW);
     uint16_t* keys = reinterpret_cast<uint16_t*>(acc + ((total + 1u) & ~1u));
     uint32_t* blob = reinterpret_cast<uint32_t*>(keys + ((total + 1u) & ~1u));
@@ -497,14 +499,14 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
         for (uint32_t i = tl; i < n_w; i += threads) copy_word_async(&blob[b_w + i], src + i);
     }
     for (uint32_t i = tl; i < slots / 2u; i += threads) reinterpret_cast<uint32_t*>(slot)[i] = 0xFFFFFFFFu;
-    if (tl == 0u) *failed = 0u;
+    if (NW > 1 && tl == 0u) *failed = 0u;
     copies_wait();
     dec_team_sync<NW>(team);
     for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
     dec_team_sync<NW>(team);
     // ---- parse: the threads shared out among the streams, within a warp
-    const uint32_t tn = min(32u, (W <= 2u ? 16u : (W <= 4u ? 8u : 4u)) * NW);
-    const uint32_t mine = min(tl / tn, 31u);                            // (beyond W - 1: a stream without keys)
+    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), tn = 1u << tn_log2;
+    const uint32_t mine = tl >> tn_log2;                            // (beyond W - 1: a stream without keys)
     Blob b;
     b.count = __shfl_sync(kFullMask, count, mine);
     b.nwords = __shfl_sync(kFullMask, nw, mine);
@@ -521,10 +523,16 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     });
     if (bad != ~0ull) {
         dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
-        atomicOr(failed, 1u << mine);
+        if (NW > 1) atomicOr(failed, 1u << mine);
     }
-    dec_team_sync<NW>(team);
-    const uint32_t out = *failed;
+    uint32_t out;
+    if constexpr (NW == 1) {
+        out = __any_sync(kFullMask, bad != ~0ull) ? __reduce_or_sync(kFullMask, bad != ~0ull ? 1u << mine : 0u) : 0u;
+        __syncwarp();
+    } else {
+        dec_team_sync<NW>(team);
+        out = *failed;
+    }
     if (out) {                                                          // a failed stream is left out as a whole
         for (uint32_t w = 0; w < W; ++w) {
             const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w);
@@ -608,9 +616,10 @@ __device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint
     const uint32_t n = s.n_light[kList];
     const int team = warp / NW;
     for (;;) {
-        if (warp % NW == 0 && lane == 0) s.grab[team] = atomicAdd(&s.next_light[kList], 1u);
-        dec_team_sync<NW>(team);
-        const uint32_t x = s.grab[team];
+        uint32_t x = 0u;
+        if (warp % NW == 0 && lane == 0) { x = atomicAdd(&s.next_light[kList], 1u); if (NW > 1) s.grab[team] = x; }
+        if constexpr (NW == 1) x = __shfl_sync(kFullMask, x, 0);
+        else { dec_team_sync<NW>(team); x = s.grab[team]; }
         if (x >= n) break;
         const uint32_t i = team_list_entry(s, kList, x);
         team_group<MODE, NW>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
@@ -1029,9 +1038,10 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
     unsigned int* q_taken = a.q_ctl + 1, *q_done = a.q_ctl + 2, *q_exited = a.q_ctl + 3, *q_reserved = a.q_ctl + 4;
     const bool queue = a.G > B;
     const uint32_t warp_max = owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew;
-    // Several streams: teams take groups of fewer keys than the slice (the update: the sweep) is for; with few groups to a block larger
-    // teams, so that its warps have work.
-    const uint32_t team_max = MODE == 2 ? kSweepMinKeys : kTileMinKeys, least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
+    // Several streams, keys of a group on average (what the headers say: it steers who decodes a group, nothing else)
+    uint64_t all_keys = 0ull;
+    if constexpr (!ONE) for (uint32_t w = 0; w < W; ++w) all_keys += s.hdr[w][6];
+    const uint32_t mean = all_keys < 65535ull * a.G ? (uint32_t)(all_keys / a.G) : 65535u;
     for (uint32_t first = 0; first < owned; first += per_batch) {
         if (first > 0u) { __syncthreads(); d0 = d1 = d2 = 0u; load_dir(first + my_i); }
         // ---- classify the batch's groups
@@ -1050,6 +1060,19 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
             else if (cm) { atomicAdd(&s.gtot[my_i], cm & 0xFFFFFFu); atomicAdd(&s.gtot[kDecThreads / 2 + my_i], nw); }
         }
         __syncthreads();
+        // Where most groups have about as many keys, they all go to teams, up to as many keys as the slice (the update: the sweep) is for; with
+        // few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a block with one
+        // group, those of many keys are for whole blocks, which share them through the queue below: teams of several sizes work one after
+        // the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
+        uint32_t team_max = kTeamFew, least_team = 0u;
+        if constexpr (!ONE) {
+            const uint32_t x = tid < (int)in_batch ? s.gtot[tid] : 0u;
+            const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= mean && x <= 2u * mean);
+            if (in_batch > 1u && 4u * alike >= 3u * in_batch) {
+                team_max = MODE == 2 ? kSweepMinKeys : kTileMinKeys;
+                if (mean >= kTeamShared) least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
+            }
+        }
         if (tid < (int)in_batch) {
             const uint32_t tot = s.gtot[tid];
             if (tot != 0u) {
@@ -1058,7 +1081,7 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
                 else if (a.group_log2 <= 15u && tot < team_max) {
                     const uint32_t bytes = team_bytes(tot, s.gtot[kDecThreads / 2 + tid]), room = kTeamBytes - 2u * kTeamSlots;
                     list = bytes <= room ? 0u : bytes <= 2u * room ? 1u : bytes <= 4u * room ? 2u : 3u;
-                    if (list < least_team && tot > 64u) list = least_team;
+                    list = max(list, least_team);
                 }
                 if (list < 3u) team_list_entry(s, list, atomicAdd(&s.n_light[list], 1u)) = (uint16_t)tid;
                 else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
