@@ -202,7 +202,7 @@ struct DecShared {
     uint32_t           e_cm[kDecThreads], e_off[kDecThreads], e_nw[kDecThreads];
     uint32_t           gtot[kDecThreads];           // keys of each of these groups over all streams; several streams: from kDecThreads / 2 on their words
     uint16_t           light[kDecThreads], heavy[kDecThreads];      // groups for a warp, and from the end on for four; for the block, and from the end on for two
-    uint32_t           n_light[3], n_heavy, next_light[3], grab[kDecWarps];
+    uint32_t           n_light[3], n_heavy, next_light[3], grab[kDecWarps], mean;
     uint32_t           scan[2][kDecWarps];
     uint32_t           got;           // answer of thread 0 to the block
     uint32_t           bad[kDecMaxStreams];
@@ -1024,6 +1024,12 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
         if (st != kStOk && blockIdx.x == 0) dec_fail(a, 0u, 0u, st);
     }
     __syncthreads();
+    // several streams: keys of a group on average (what the headers say: it steers who decodes a group, nothing else)
+    if (!ONE && tid == kDecThreads - 1) {
+        float keys = 0.0f;
+        for (uint32_t w = 0; w < W; ++w) keys += (float)s.hdr[w][6];
+        s.mean = (uint32_t)fminf(__fdividef(keys, (float)a.G), 65535.0f);
+    }
     // phases 3-4 as a table per stream: value[L] = (float)(sum / b^L).  The division is a multiplication by the reciprocal
     // (within 2^-51 of the quotient) whenever everything within 2^-50 of the product rounds to the same float.
     for (uint32_t idx = tid; idx < W * 132u; idx += kDecThreads) {
@@ -1038,10 +1044,6 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
     unsigned int* q_taken = a.q_ctl + 1, *q_done = a.q_ctl + 2, *q_exited = a.q_ctl + 3, *q_reserved = a.q_ctl + 4;
     const bool queue = a.G > B;
     const uint32_t warp_max = owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew;
-    // Several streams, keys of a group on average (what the headers say: it steers who decodes a group, nothing else)
-    uint64_t all_keys = 0ull;
-    if constexpr (!ONE) for (uint32_t w = 0; w < W; ++w) all_keys += s.hdr[w][6];
-    const uint32_t mean = all_keys < 65535ull * a.G ? (uint32_t)(all_keys / a.G) : 65535u;
     for (uint32_t first = 0; first < owned; first += per_batch) {
         if (first > 0u) { __syncthreads(); d0 = d1 = d2 = 0u; load_dir(first + my_i); }
         // ---- classify the batch's groups
@@ -1067,10 +1069,10 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
         uint32_t team_max = kTeamFew, least_team = 0u;
         if constexpr (!ONE) {
             const uint32_t x = tid < (int)in_batch ? s.gtot[tid] : 0u;
-            const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= mean && x <= 2u * mean);
+            const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= s.mean && x <= 2u * s.mean);
             if (in_batch > 1u && 4u * alike >= 3u * in_batch) {
                 team_max = MODE == 2 ? kSweepMinKeys : kTileMinKeys;
-                if (mean >= kTeamShared) least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
+                if (s.mean >= kTeamShared) least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
             }
         }
         if (tid < (int)in_batch) {
