@@ -30,7 +30,6 @@
 #pragma once
 
 #include <cstddef>
-#include <type_traits>
 
 #include "common.cuh"
 #include "bits.cuh"
@@ -663,7 +662,147 @@ __device__ __forceinline__ void entries_in_memory(const DecArgs& a, const DecSha
     }
 }
 
-// One group by the whole block; s.g_* hold its directory entries.
+// A group's blobs for the block: all streams' together in the stage, or (together = false) one in each half of it, or (staged = false) where
+// they are in memory.
+struct Stage {
+    uint32_t words, listed; bool together, staged;                     // (listed: entries of the lists, each padded to a multiple of 8)
+    __device__ __forceinline__ Stage(const DecShared& s, uint32_t W) : words(0u), listed(0u), staged(true) {
+        for (uint32_t w = 0; w < W; ++w) { words += s.g_nwords[w]; listed += (s.g_count[w] + 7u) & ~7u; }
+        together = words <= kBlockStageWords;
+        for (uint32_t w = 0; w < W; ++w) staged = staged && (together || s.g_nwords[w] <= kBlockStageWords / 2u);
+    }
+    __device__ __forceinline__ void copy(const DecArgs& a, DecShared& s, uint32_t w, uint32_t at, int tid) const {
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(a.stream[w]) + s.g_off[w];
+        for (uint32_t i = tid; i < s.g_nwords[w]; i += kDecThreads) copy_word_async(&s.u.bstage[at + i], src + i);
+    }
+    __device__ __forceinline__ void swap(DecShared& s, uint32_t w, uint32_t at, int tid) const {      // (every thread the words it has copied itself)
+        for (uint32_t i = tid; i < s.g_nwords[w]; i += kDecThreads) s.u.bstage[at + i] = bswap32(s.u.bstage[at + i]);
+    }
+    __device__ __forceinline__ Blob blob(const DecArgs& a, const DecShared& s, uint32_t w) const {
+        Blob b;
+        b.words = staged ? s.u.bstage + s.g_base[w] : reinterpret_cast<const uint32_t*>(a.stream[w]) + s.g_off[w];
+        b.nwords = s.g_nwords[w]; b.count = s.g_count[w]; b.M = s.g_M[w];
+        return b;
+    }
+};
+
+// One group wider than the tile by the whole block, in memory.  (A function of its own, so that its registers do not weigh on the groups of
+// the default size: inlined, these took 3 % longer.)
+template <bool ONE, int MODE>
+__device__ __noinline__ void block_wide(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t lo64 = (uint64_t)g << a.group_log2;
+    const uint64_t hi64 = lo64 + (1ull << a.group_log2);
+    const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
+    const Stage st(s, W);
+    {
+        uint32_t used = 0u, list = 0u;
+        for (uint32_t w = 0; w < W; ++w) {
+            if (tid == 0) { s.g_base[w] = st.together ? used : (w & 1u) * (kBlockStageWords / 2u + 2u); s.g_list[w] = list; s.bad[w] = 0u; }
+            if (st.together) st.copy(a, s, w, used, tid);
+            used += s.g_nwords[w]; list += (s.g_count[w] + 7u) & ~7u;
+        }
+        if (st.together) {
+            copies_wait();
+            used = 0u;
+            for (uint32_t w = 0; w < W; ++w) { st.swap(s, w, used, tid); used += s.g_nwords[w]; }
+        }
+    }
+    __syncthreads();
+    uint32_t* wkey = reinterpret_cast<uint32_t*>(s.u.tile);             // a list of 32-bit keys
+    const int sweeps = MODE == 2 && !ONE ? 2 : 1;                       // (the update in one launch: g first, from all streams)
+    auto code_of = [&](const Blob& b, uint32_t j) -> uint32_t { return st.staged ? code_at<true>(b, j) : code_at<false>(b, j); };
+    auto apply_list = [&](uint32_t w, const Blob& b, uint32_t l0, bool update) {      // neighbouring threads on neighbouring keys
+        for (uint32_t j0 = (uint32_t)tid; j0 < b.count; j0 += 4u * kDecThreads) {
+            uint32_t key[4], code[4], on = 0u;
+#pragma unroll
+            for (uint32_t i = 0; i < 4u; ++i) {
+                const uint32_t j = j0 + i * kDecThreads;
+                key[i] = 0u; code[i] = 0u;
+                if (j < b.count) { on |= 1u << i; key[i] = wkey[l0 + j]; code[i] = code_of(b, j); }
+            }
+            entries_in_memory<ONE, MODE, 4>(a, s, w, lo, update, on, key, code);
+        }
+    };
+    if (st.listed <= kWideListMax && st.together) {
+        // ---- all streams parsed side by side into lists, then applied one after the other.  (Before, each stream was parsed twice, the second
+        // time by threads that took runs of consecutive keys one access at a time: 442 groups of 2^15, eight streams of 200 keys, 87 us, now
+        // 38; 12.8 M entries in groups of 2^17, five streams, the update 60, now 21.)
+        const uint32_t tn = ONE ? (uint32_t)kDecThreads : (W <= 2u ? kDecThreads / 2u : (W <= 4u ? kDecThreads / 4u : kDecThreads / 8u));
+        const uint32_t mine = ONE ? 0u : (uint32_t)tid / tn;
+        uint32_t most = 0u;
+        for (uint32_t w = 0; w < W; ++w) most = max(most, s.g_count[w]);
+        const bool small = most <= 4u * tn;
+        Blob b = st.blob(a, s, mine < W ? mine : 0u);
+        if (mine >= W) b.count = 0u;
+        const uint32_t list = mine < W ? s.g_list[mine] : 0u;
+        const unsigned long long bad = parse_team<true, true>(a, s, b, span, (uint32_t)tid & (tn - 1u), tn, small, small ? 1u : (most + 8u * tn - 1u) / (8u * tn),
+                                                              lane, warp, [&](uint32_t j, int m, const auto& v) {
+            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+            for (int k = 0; k < K; ++k) if (k < m) wkey[list + j + (uint32_t)k] = v[k];
+        });
+        if (bad != ~0ull) {
+            s.bad[mine] = 1u;
+            dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+        }
+        __syncthreads();
+        for (int sweep = 0; sweep < sweeps; ++sweep) {
+            for (uint32_t w = 0; w < W; ++w) {
+                if (!s.bad[w]) apply_list(w, st.blob(a, s, w), s.g_list[w], MODE == 1 || (MODE == 2 && sweep + 1 == sweeps));      // (a failed stream is left out as a whole)
+                __syncthreads();                                        // this stream's updates before the next stream's
+            }
+        }
+    } else {
+        // ---- stream by stream; one that has more keys than the list holds is parsed once to validate and once to apply
+        for (int sweep = 0; sweep < sweeps; ++sweep) {
+            const bool update = MODE == 1 || (MODE == 2 && sweep + 1 == sweeps);
+            if (st.staged && !st.together) st.copy(a, s, 0u, s.g_base[0], tid);
+            for (uint32_t w = 0; w < W; ++w) {
+                const Blob b = st.blob(a, s, w);
+                if (st.staged && !st.together) {
+                    copies_wait();
+                    st.swap(s, w, s.g_base[w], tid);
+                    __syncthreads();
+                    if (w + 1u < W) st.copy(a, s, w + 1u, s.g_base[w + 1u], tid);
+                }
+                if (b.count == 0u) continue;                            // (uniform; the next stream's copy goes to the other half of the stage)
+                const bool fits = b.count <= kWideListMax, small = b.count <= 4u * kDecThreads;
+                const uint32_t rounds = small ? 1u : (b.count + 8u * kDecThreads - 1u) / (8u * kDecThreads);
+                auto put = [&](uint32_t j, int m, const auto& v) {
+                    constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+                    for (int k = 0; k < K; ++k) if (fits && k < m) wkey[j + (uint32_t)k] = v[k];
+                };
+                const unsigned long long bad = st.staged ? parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put)
+                                                         : parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put);
+                if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+                if (!__syncthreads_or(bad != ~0ull ? 1 : 0)) {          // validated in full before any of it is applied
+                    auto apply_run = [&](uint32_t j, int m, const auto& v) {
+                        constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+                        for (int k0 = 0; k0 < K; k0 += 4) {
+                            uint32_t key[4], code[4], on = 0u;
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                key[k] = v[k0 + k]; code[k] = 0u;
+                                if (k0 + k < m) { on |= 1u << k; code[k] = code_of(b, j + (uint32_t)(k0 + k)); }
+                            }
+                            entries_in_memory<ONE, MODE, 4>(a, s, w, lo, update, on, key, code);
+                        }
+                    };
+                    if (fits) apply_list(w, b, 0u, update);
+                    else if (st.staged) parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+                    else parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+                }
+                __syncthreads();                                        // this stream's updates before the next stream's
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// One group of up to 2^14 indices by the whole block; s.g_* hold its directory entries.
 template <bool ONE, int MODE>
 __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t& tile_parity, int tid, int lane, int warp) {
     const uint64_t lo64 = (uint64_t)g << a.group_log2;
@@ -672,11 +811,10 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
     uint32_t total = 0u, words = 0u;
     uint32_t listed = 0u;                                               // entries of the lists (each padded to a multiple of 8)
     for (uint32_t w = 0; w < W; ++w) { total += s.g_count[w]; words += s.g_nwords[w]; listed += (s.g_count[w] + 7u) & ~7u; }
-    const bool small_group = a.group_log2 <= 14u;
-    const bool lists = small_group && listed <= kBlockListMax && words <= kBlockStageWords;      // (else: stream by stream)
+    const bool lists = listed <= kBlockListMax && words <= kBlockStageWords;      // (else: stream by stream)
     const bool bulk_ok = ((reinterpret_cast<uintptr_t>(a.dense) & 15u) == 0u) && ((span & 3u) == 0u);
     // aggregation of many keys: the slice of dense_out goes through shared memory as a whole
-    const bool slice = MODE == 0 && small_group && (total >= kTileMinKeys || !lists);
+    const bool slice = MODE == 0 && (total >= kTileMinKeys || !lists);
     if (tid == 0) {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the last write-back has read the tile
         if (slice && bulk_ok) {
@@ -746,24 +884,8 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
     };
 
     // model update of many keys: a sweep over the slice of g
-    const bool sweep_all = mode_fused(MODE) && small_group && (total >= (MODE == 2 ? kSweepMinKeys : kSweepMinPacked) || !lists) &&
+    const bool sweep_all = mode_fused(MODE) && (total >= (MODE == 2 ? kSweepMinKeys : kSweepMinPacked) || !lists) &&
                            (MODE == 3 || ((reinterpret_cast<uintptr_t>(a.theta) | reinterpret_cast<uintptr_t>(a.m) | reinterpret_cast<uintptr_t>(a.v)) & 15u) == 0u);
-    // lists of 32-bit keys in the tile's place, for groups (or passes) that do not use it otherwise
-    uint32_t* wkey = reinterpret_cast<uint32_t*>(s.u.tile);
-    const bool wide_lists = !small_group && listed <= kWideListMax && words <= kBlockStageWords;
-    const int wide_sweeps = MODE == 2 && !ONE ? 2 : 1;                  // (the update in one launch: g first, from all streams)
-    auto apply_list = [&](uint32_t w, const Blob& b, uint32_t l0, bool update) {      // neighbouring threads on neighbouring keys
-        for (uint32_t j0 = (uint32_t)tid; j0 < b.count; j0 += 4u * kDecThreads) {
-            uint32_t key[4], code[4], on = 0u;
-#pragma unroll
-            for (uint32_t i = 0; i < 4u; ++i) {
-                const uint32_t j = j0 + i * kDecThreads;
-                key[i] = 0u; code[i] = 0u;
-                if (j < b.count) { on |= 1u << i; key[i] = wkey[l0 + j]; code[i] = code_of(b, j); }
-            }
-            entries_in_memory<ONE, MODE, 4>(a, s, w, lo, update, on, key, code);
-        }
-    };
     if (lists) {
         // ---- all streams parsed side by side into the lists
         const uint32_t tn = ONE ? (uint32_t)kDecThreads : (W <= 2u ? kDecThreads / 2u : (W <= 4u ? kDecThreads / 4u : kDecThreads / 8u));
@@ -858,117 +980,62 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
                 }
             }
         }
-    } else if (MODE != 3 && wide_lists) {
-        // ---- a group wider than the tile: all streams parsed side by side into lists in the tile's place, then applied in memory one after
-        // the other.  (Before, each stream was parsed twice, the second time by threads that took runs of consecutive keys one access at a
-        // time: 442 groups of 2^15, eight streams of 200 keys, 86 us, now 40; 12.8 M entries in groups of 2^17, five streams, the update 57, now 21.)
-        const uint32_t tn = ONE ? (uint32_t)kDecThreads : (W <= 2u ? kDecThreads / 2u : (W <= 4u ? kDecThreads / 4u : kDecThreads / 8u));
-        const uint32_t mine = ONE ? 0u : (uint32_t)tid / tn;
-        uint32_t most = 0u;
-        for (uint32_t w = 0; w < W; ++w) most = max(most, s.g_count[w]);
-        const bool small = most <= 4u * tn;
-        Blob b = blob_of(mine < W ? mine : 0u);
-        if (mine >= W) b.count = 0u;
-        const uint32_t list = mine < W ? s.g_list[mine] : 0u;
-        const unsigned long long bad = parse_team<true, true>(a, s, b, span, (uint32_t)tid & (tn - 1u), tn, small, small ? 1u : (most + 8u * tn - 1u) / (8u * tn),
-                                                              lane, warp, [&](uint32_t j, int m, const auto& v) {
-            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
-#pragma unroll
-            for (int k = 0; k < K; ++k) if (k < m) wkey[list + j + (uint32_t)k] = v[k];
-        });
-        if (bad != ~0ull) {
-            s.bad[mine] = 1u;
-            dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
-        }
-        __syncthreads();
-        for (int sweep = 0; sweep < wide_sweeps; ++sweep) {
-            for (uint32_t w = 0; w < W; ++w) {
-                if (!s.bad[w]) apply_list(w, blob_of(w), s.g_list[w], MODE == 1 || (MODE == 2 && sweep + 1 == wide_sweeps));      // (a failed stream is left out as a whole)
-                __syncthreads();                                        // this stream's updates before the next stream's
-            }
-        }
     } else {
         // ---- more keys than the lists hold: stream by stream, the whole block on each
         if (slice) { if (!wait_slice()) return; }
-        if (mode_fused(MODE) && small_group) {
+        if constexpr (mode_fused(MODE)) {
             for (uint32_t i = tid; i < ((span + 3u) >> 2); i += kDecThreads)
                 reinterpret_cast<float4*>(s.u.tile)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             __syncthreads();
         }
-        // (in the tile or in memory: two loops, each without the other's code)
-        auto each_stream = [&](auto in_tile_c) __attribute__((always_inline)) {
-            constexpr bool in_tile = decltype(in_tile_c)::value;
-            // (fused update of a wide group: aggregation into dense_out first, then the update over all streams again)
-            const int sweeps = small_group ? 1 : wide_sweeps;
-            for (int sweep = 0; sweep < sweeps; ++sweep) {
-                const bool update = MODE == 1 || (MODE == 2 && !small_group && sweep + 1 == sweeps);
-                if (staged && !together) stage_copy(0u, s.g_base[0]);
-                for (uint32_t w = 0; w < W; ++w) {
-                    const Blob b = blob_of(w);
-                    if (staged && !together) {
-                        copies_wait();
-                        stage_swap(w, s.g_base[w]);
-                        __syncthreads();
-                        if (w + 1u < W) stage_copy(w + 1u, s.g_base[w + 1u]);
-                    }
-                    if (b.count == 0u) continue;                        // (uniform; the next stream's copy goes to the other half of the stage)
-                    // (one stream at a time fits the list far more often than all of them: parsed once then, else once to validate and once to
-                    // apply; the tile holds the list where it holds nothing else)
-                    const bool fits = b.count <= (in_tile ? kBlockListMax : kWideListMax);
-                    const bool small = b.count <= 4u * kDecThreads;
-                    const uint32_t rounds = small ? 1u : (b.count + 8u * kDecThreads - 1u) / (8u * kDecThreads);
-                    auto put = [&](uint32_t j, int m, const auto& v) {
-                        constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
-#pragma unroll
-                        for (int k = 0; k < K; ++k) {
-                            if (fits && k < m) {
-                                if constexpr (in_tile) s.u.lkey[j + (uint32_t)k] = (uint16_t)v[k];
-                                else wkey[j + (uint32_t)k] = v[k];
-                            }
-                        }
-                    };
-                    const unsigned long long bad = staged ? parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put)
-                                                          : parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put);
-                    if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
-                    if (!__syncthreads_or(bad != ~0ull ? 1 : 0)) {      // validated in full before any of it is applied
-                        auto in_slice = [&](uint32_t j, uint32_t key) { s.u.tile[key] = __fadd_rn(s.u.tile[key], code_value(s.val[w], code_of(b, j))); };
-                        auto apply_run = [&](uint32_t j, int m, const auto& v) {
-                            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
-                            if constexpr (in_tile) {
-#pragma unroll
-                                for (int k = 0; k < K; ++k) if (k < m) in_slice(j + (uint32_t)k, v[k]);
-                            } else {
-#pragma unroll
-                                for (int k0 = 0; k0 < K; k0 += 4) {
-                                    uint32_t key[4], code[4], on = 0u;
-#pragma unroll
-                                    for (int k = 0; k < 4; ++k) {
-                                        key[k] = v[k0 + k]; code[k] = 0u;
-                                        if (k0 + k < m) { on |= 1u << k; code[k] = code_of(b, j + (uint32_t)(k0 + k)); }
-                                    }
-                                    entries_in_memory<ONE, MODE, 4>(a, s, w, lo, update, on, key, code);
-                                }
-                            }
-                        };
-                        if (fits) {
-                            if constexpr (in_tile) { for (uint32_t j = tid; j < b.count; j += kDecThreads) in_slice(j, s.u.lkey[j]); }
-                            else apply_list(w, b, 0u, update);
-                        } else if (staged) parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
-                        else parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
-                    }
-                    __syncthreads();                                    // this stream's updates before the next stream's
-                }
+        if (staged && !together) stage_copy(0u, s.g_base[0]);
+        for (uint32_t w = 0; w < W; ++w) {
+            const Blob b = blob_of(w);
+            if (staged && !together) {
+                copies_wait();
+                stage_swap(w, s.g_base[w]);
+                __syncthreads();
+                if (w + 1u < W) stage_copy(w + 1u, s.g_base[w + 1u]);
             }
-        };
-        if constexpr (MODE == 1) each_stream(std::false_type{});
-        else if constexpr (MODE == 3) each_stream(std::true_type{});
-        else { if (small_group) each_stream(std::true_type{}); else each_stream(std::false_type{}); }
+            if (b.count == 0u) continue;                            // (uniform; the next stream's copy goes to the other half of the stage)
+            // (one stream at a time fits the list far more often than all of them: parsed once then, else once to validate and once to apply)
+            const bool fits = b.count <= kBlockListMax;
+            const bool small = b.count <= 4u * kDecThreads;
+            const uint32_t rounds = small ? 1u : (b.count + 8u * kDecThreads - 1u) / (8u * kDecThreads);
+            auto put = [&](uint32_t j, int m, const auto& v) {
+                constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+                for (int k = 0; k < K; ++k) if (fits && k < m) s.u.lkey[j + (uint32_t)k] = (uint16_t)v[k];
+            };
+            const unsigned long long bad = staged ? parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put)
+                                                  : parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, put);
+            if (bad != ~0ull) dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+            if (!__syncthreads_or(bad != ~0ull ? 1 : 0)) {          // validated in full before any of it is applied
+                auto apply = [&](uint32_t j, uint32_t key) {
+                    if constexpr (MODE != 1) s.u.tile[key] = __fadd_rn(s.u.tile[key], code_value(s.val[w], code_of(b, j)));
+                    else {
+                        const uint32_t kk[1] = {lo + key};
+                        const float gg[1] = {atomicExch(a.dense + lo + key, 0.0f)};
+                        adam_run<false, 1>(a, kk, gg);
+                    }
+                };
+                auto apply_run = [&](uint32_t j, int m, const auto& v) {
+                    constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+                    for (int k = 0; k < K; ++k) if (k < m) apply(j + (uint32_t)k, v[k]);
+                };
+                if (fits) for (uint32_t j = tid; j < b.count; j += kDecThreads) apply(j, s.u.lkey[j]);
+                else if (staged) parse_team<true, true>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+                else parse_team<true, false>(a, s, b, span, (uint32_t)tid, (uint32_t)kDecThreads, small, rounds, lane, warp, apply_run);
+            }
+            __syncthreads();                                        // this stream's updates before the next stream's
+        }
         if (MODE == 0 && slice) {
             store_slice();
         } else if (sweep_all) {
             if constexpr (MODE == 2) adam_sweep(a, s.u.tile, lo, span, tid, kDecThreads);
             else if constexpr (MODE == 3) update_slice<MODE>(a, s.u.tile, lo, span, tid);
-        } else if (mode_fused(MODE) && small_group) {
+        } else if constexpr (mode_fused(MODE)) {
             update_slice<MODE>(a, s.u.tile, lo, span, tid);
         }
     }
@@ -978,7 +1045,7 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
 // ONE: the launch holds a single stream (its own instantiation, so that the code of the many-stream paths does not weigh on it).
 template <bool ONE, int MODE = 0>
 __global__ void __launch_bounds__(kDecThreads, 2)
-k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const __grid_constant__ PowTable inv) {
+k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ PowTable pw, const __grid_constant__ PowTable inv) {
     extern __shared__ __align__(128) unsigned char dec_smem_raw[];
     DecShared& s = *reinterpret_cast<DecShared*>(dec_smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1112,7 +1179,8 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
                 s.g_count[tid] = cm & 0xFFFFFFu; s.g_M[tid] = cm >> 24; s.g_off[tid] = s.e_off[e]; s.g_nwords[tid] = s.e_nw[e];
             }
             __syncthreads();
-            block_group<ONE, MODE>(a, s, W, blockIdx.x + (first + i) * B, tile_parity, tid, lane, warp);
+            if (MODE != 3 && a.group_log2 > 14u) block_wide<ONE, MODE>(a, s, W, blockIdx.x + (first + i) * B);
+            else block_group<ONE, MODE>(a, s, W, blockIdx.x + (first + i) * B, tile_parity, tid, lane, warp);
         }
         if (keep > 0u) {                                  // (the tile becomes the warps' memory)
             if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -1177,7 +1245,8 @@ k_decode_accumulate(const DecArgs a, const __grid_constant__ PowTable pw, const 
             s.g_count[tid] = cm & 0xFFFFFFu; s.g_M[tid] = cm >> 24; s.g_off[tid] = o; s.g_nwords[tid] = nw;
         }
         __syncthreads();
-        block_group<ONE, MODE>(a, s, W, g, tile_parity, tid, lane, warp);
+        if (MODE != 3 && a.group_log2 > 14u) block_wide<ONE, MODE>(a, s, W, g);
+        else block_group<ONE, MODE>(a, s, W, g, tile_parity, tid, lane, warp);
     }
     if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // write-backs complete before the block leaves
     // the last block to leave clears the counters for the next launch.  The slots were cleared as they were taken; a
