@@ -86,7 +86,7 @@ def test_other_group_sizes_many_tiles():
         _check_groups(_tiles(400 * TILE + 7, (3, 0, 0, 0, 40, 900, 0, TILE), group_log2), 1.2, group_log2)
 
 
-# a sample that misses what matters (the estimate is too high where a few entries carry the sum): tiles are read again
+# a few entries carry the sum: a wide margin below the estimate
 @pytest.mark.parametrize("group_log2", [10, 14, 17])
 def test_tiles_read_again(group_log2):
     n = 310 * TILE + 1
@@ -98,7 +98,7 @@ def test_tiles_read_again(group_log2):
     _check_groups(v, 1.1, group_log2)
 
 
-# more blobs than the workspace has room for: packed where they belong in the stream
+# every entry kept: units without lists, the longest blobs (what has no room in the workspace: test_gpu_workspace.py)
 @pytest.mark.parametrize("group_log2", [9, 14, 16])
 def test_blobs_without_room(group_log2):
     n = (1 << 26) + 3
@@ -126,3 +126,27 @@ def test_sum_without_help_from_other_blocks(workers, n, group_log2):
     finally:
         binding.debug_set_wait_limits(0, 0, 0)
         binding.set_workspace(binding.ensure_workspace(n, pg))
+
+
+# an estimate that is too high: the entries that the sample looks at (four at each of 32 * 768 regular places) are four times the
+# others, the kept ones lie elsewhere, in every third unit of 4096.  Exactly the tiles (other group sizes: units) that hold kept
+# entries are read again, and none of them where the same values stand in another order
+@pytest.mark.parametrize("group_log2", [9, 14, 16])
+def test_estimate_above_the_threshold(group_log2):
+    n = 310 * TILE + 1
+    rng = np.random.default_rng(4)
+    v = (0.5 * rng.choice([-1.0, 1.0], n)).astype(np.float32)
+    step = (n >> 2) // (32 * 768)
+    at = 4 * (np.arange(32 * 768) * step + step // 2)
+    for i in range(4):
+        v[at + i] = 2.0
+    keys = rng.choice(n - 1, 3000, replace=False)
+    keys = keys[((keys >> 12) % 3 == 0) & (keys % 7 != 0)]
+    keys = keys[~np.isin(keys >> 2, at >> 2)]
+    v[keys] = -3.0
+    base = float((np.abs(v, dtype=np.float64).sum() / 2.5) ** (1 / 128))
+    again = np.unique(keys >> (14 if group_log2 == 14 else 12)).size
+    _check_groups(v, base, group_log2)
+    assert binding.listed_tiles(1) == [again] and again > 100
+    _check_groups(rng.permutation(v), base, group_log2)
+    assert binding.listed_tiles(1) == [0]
