@@ -203,7 +203,7 @@ def run_sweep(args):
             assert status == 0 and binding.decode_status() == 0
             listed = binding.listed_tiles(1)
             ms_c, ms_d, ms_b = med(comp), med(dec), med(both)
-            alg_c, alg_d = 8.0 * n + total, total + 8.0 * d
+            alg_c, alg_d = 4.0 * n + total, total + 8.0 * d
             tr_c, tr_d = traffic_model(n, [total], [d], listed)
             row = {"log2n": log2n, "keep": keep, "kept": d, "stream_bytes": total,
                    "compress_ms": ms_c, "decompress_ms": ms_d, "combined_ms": ms_b,
@@ -345,14 +345,40 @@ def ncu_traffic_of(profile_md: str):
 
 
 def traffic_model(n, stream_bytes, kept, listed):
-    """DRAM bytes the two kernels have to move, counted rather than assumed: the sum pass reads every gradient
-    once (4 n each); the encode pass reads again only the tiles the kernel listed (it leaves their number per
-    gradient in the workspace), 64 KiB each; the streams are written once and read once; every kept entry is a
-    read-modify-write of one 32-byte sector of the accumulator (never more than the whole accumulator)."""
+    """DRAM bytes the two kernels cannot do without, a lower bound: every gradient is read once (4 n each), the tiles
+    the encoder reads again (it leaves their number per gradient in the workspace), 64 KiB each; the streams are
+    written once and read once; every kept entry is a read-modify-write of one 32-byte sector of the accumulator
+    (never more than the whole accumulator).  Not counted: the candidate lists and the blobs' way through the
+    workspace, which stay in L2 unless much is kept."""
     W = len(stream_bytes)
     comp = sum(4.0 * n + min(4.0 * n, 4.0 * TILE * listed[w]) + stream_bytes[w] for w in range(W))
     dec = float(sum(stream_bytes)) + min(64.0 * float(sum(kept)), 8.0 * n)
     return comp, dec
+
+
+def short_line(line):
+    """The result as one line that a log's tail holds: numbers to five digits, of the details the medians."""
+    def num(x):
+        return float("%.5g" % x) if isinstance(x, float) else x
+
+    def pick(d, *keys):
+        return {k: num(d[k]) for k in keys if d and d.get(k) is not None}
+
+    out = {k: num(v) for k, v in line.items() if not isinstance(v, (dict, list))}
+    out["config"] = dict(line["config"], workload=line["config"]["workload"].split(":")[0], l2=line["config"]["l2"].split(";")[0])
+    out["config"].pop("dense_zero_fill", None)
+    out["clocks"] = line["clocks"]
+    for key, names in (("ms_per_step_each", ("median", "min")), ("compress", ("ms", "input_gbs", "frac_of_hbm_peak")),
+                       ("decompress", ("ms", "input_gbs")), ("sparse_adam_update", ("ms", "packed_state_ms")),
+                       ("e2e", ("value", "unit", "steps", "h2d_bytes_per_step", "d2h_bytes_per_step")),
+                       ("sustained", ("ms_per_step", "value")), ("cpu_baseline", ("value", "unit", "cores", "kind")),
+                       ("roofline", ("bound", "kernel", "achieved", "peak", "unit", "frac", "peak_kind", "traffic", "dram_frac"))):
+        if line.get(key):
+            out[key] = pick(line[key], *names)
+    if line.get("configs"):                                            # us per call: compress, decompress, both
+        out["configs_us"] = {k: [num(1e3 * (v.get(leg) or {}).get("median", (v.get(leg) or {}).get("mean", 0.0)))
+                                 for leg in ("compress_ms", "decompress_ms", "combined_ms")] for k, v in line["configs"].items()}
+    return out
 
 
 def series_stats(ts):
@@ -465,7 +491,7 @@ def measure_config(torch, binding, dev, wl, grads, peak, reps, flush, outs=None,
 
         tc, tb = series_rot(comp_run, comp_run2), series_rot(both_run, both_run2)
         del grads2
-    alg_c = 8.0 * n * W + float(sum(stream_bytes))
+    alg_c = 4.0 * n * W + float(sum(stream_bytes))
     alg_d = float(sum(stream_bytes)) + 8.0 * float(sum(kept))
     tr_c, tr_d = traffic_model(n, stream_bytes, kept, listed)
     mc, md, mb = statistics.median(tc), statistics.median(td), statistics.median(tb)
@@ -488,8 +514,6 @@ def measure_config(torch, binding, dev, wl, grads, peak, reps, flush, outs=None,
         entry["frac_flushed"] = (alg_c + alg_d) / statistics.median(tb_flushed) / 1e6 / peak
     else:
         entry["protocol"] = "256 MiB written before every launch"
-    if entry["frac"] > 1.2:
-        entry["note"] = "frac counts two full reads of every gradient; the kernel skipped most tiles: dram_frac is the hardware figure"
     if in_bytes < L2_BYTES:
         tw = series(both_run, False)
         entry["combined_ms_l2_warm"] = series_stats(tw)
@@ -810,13 +834,13 @@ def main():
 
     peak, peak_kind = measured_peak()
     in_bytes = 4.0 * n * W
-    alg_comp = 8.0 * n * W + float(sum(stream_bytes))              # two reads of the gradient + stream written
+    alg_comp = 4.0 * n * W + float(sum(stream_bytes))              # gradient read + stream written
     alg_dec = float(sum(stream_bytes)) + 8.0 * float(sum(kept))    # stream read + read-modify-write of kept entries
     value = in_bytes * world / (ms_step * 1e-3) / 1e9
 
     per_launch_bytes = {
         "k_abs_sum": 4.0 * n + 8.0 * ((n + 16383) // 16384),
-        "k_compress": (8.0 * n * W + float(sum(stream_bytes))) / max(1, (W + 7) // 8),
+        "k_compress": (4.0 * n * W + float(sum(stream_bytes))) / max(1, (W + 7) // 8),
         "k_decode_accumulate": (float(sum(stream_bytes)) + 8.0 * float(sum(kept))) / max(1, (W + 7) // 8),
     }
     kernels = {}
@@ -842,12 +866,10 @@ def main():
         dur = kernels[dom]["avg_us"] * 1e-6
         roofline = {"bound": "hbm", "kernel": dom, "achieved": kernels[dom]["achieved_gbs"], "peak": peak,
                     "unit": "GB/s", "frac": kernels[dom]["achieved_gbs"] / peak, "peak_kind": f"of {peak_kind}",
-                    "traffic": traffic, "traffic_kind": "counted by the kernel: 4nW + 64 KiB per tile it read a second time + streams",
+                    "traffic": traffic, "traffic_kind": "lower bound: 4nW + 64 KiB per tile read a second time + streams (candidate lists and blobs not counted)",
                     "dram_frac": (traffic / dur / 1e9 / peak) if traffic else None,
                     "traffic_ncu": ncu_traffic_of("encoder_c2_4workers.md") if (default_c2 and dom == "k_compress") else None,
                     "algorithmic_bytes_per_launch": per_launch_bytes[dom]}
-        if roofline["frac"] > 1.2:
-            roofline["note"] = "frac counts two full reads of every gradient; the kernel skipped most tiles: dram_frac is the hardware figure"
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -973,7 +995,8 @@ def main():
             line["configs_error"] = repr(exc)
 
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)         # everything
+        print(json.dumps(short_line(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
