@@ -49,9 +49,6 @@ int fastsgd_debug_set_grid(uint32_t blocks);
 #define FASTSGD_DEBUG_LAYOUT_FIELDS 8
 int fastsgd_debug_layout(uint64_t* offsets, uint32_t count);
 
-/* 0: the kernels write no stamps of their phases */
-int fastsgd_debug_trace_compiled(void);
-
 #ifdef __cplusplus
 }
 #endif

@@ -30,7 +30,7 @@ EXPORTS = [
     "fastsgd_strerror", "fastsgd_version", "fastsgd_kernel_timing_enable", "fastsgd_kernel_timing_read", "fastsgd_abs_sum_noalloc",
     "fastsgd_sparse_adam_update_batch", "fastsgd_sparse_adam_update_packed_batch", "fastsgd_key_encode_paper", "fastsgd_key_encode_paper_bound",
     "fastsgd_compress_kv",
-    "fastsgd_debug_set_wait_limits", "fastsgd_debug_layout", "fastsgd_debug_trace_compiled", "fastsgd_debug_set_grid",
+    "fastsgd_debug_set_wait_limits", "fastsgd_debug_layout", "fastsgd_debug_set_grid",
 ]
 
 
@@ -121,8 +121,6 @@ def lib():
         L.fastsgd_debug_set_grid.argtypes = [C.c_uint32]
         L.fastsgd_debug_layout.restype = C.c_int
         L.fastsgd_debug_layout.argtypes = [u64p, C.c_uint32]
-        L.fastsgd_debug_trace_compiled.restype = C.c_int
-        L.fastsgd_debug_trace_compiled.argtypes = []
         _lib = L
     return _lib
 
@@ -368,8 +366,3 @@ def listed_tiles(jobs: int):
     (the others held nothing to keep, or were still in shared memory).  Synchronises."""
     torch.cuda.synchronize()
     return [int(x) for x in workspace_u32("ne_count", 8)[:jobs].cpu().tolist()]
-
-
-def debug_trace_blocks(blocks: int = 148):
-    """Per-block stamps of the last compress launch: the kernels write none, None."""
-    return None

@@ -29,9 +29,7 @@ def _deps():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compiles the library if it is missing or older than its sources.  With FASTSGD_TRACE=1 in the
-    environment the kernels are built with their %globaltimer phase stamps (a profiling build: force it,
-    and force a plain build afterwards)."""
+    """Compiles the library if it is missing or older than its sources."""
     stale = (not os.path.exists(LIB_PATH)) or any(
         os.path.getmtime(d) > os.path.getmtime(LIB_PATH) for d in _deps())
     if force or stale:

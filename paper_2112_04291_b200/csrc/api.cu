@@ -326,8 +326,6 @@ int fastsgd_debug_layout(uint64_t* offsets, uint32_t count) {
     return FASTSGD_OK;
 }
 
-int fastsgd_debug_trace_compiled(void) { return 0; }
-
 const char* fastsgd_strerror(int code) {
     switch (code) {
         case FASTSGD_OK: return "ok";

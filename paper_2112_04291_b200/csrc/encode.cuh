@@ -39,7 +39,7 @@ constexpr uint32_t kSlotEntries  = 96;                         // candidates a u
 constexpr uint32_t kUnitSlotBytes = kSlotEntries * 6u;
 constexpr uint32_t kSlotBytes    = 4u * kUnitSlotBytes;        // of a tile
 constexpr uint32_t kSlotWords    = kSlotBytes / 4u;
-constexpr uint32_t kListMost     = 2048;                       // units that promise more candidates are not listed (a list costs 6 bytes an entry, reading again 4)
+constexpr uint32_t kListMost     = 2048;                       // units that promise more candidates are not listed: from half of the entries on, a list (8 bytes a candidate with its spare room, written and read) is more traffic than the unit's 16 KB once more
 constexpr uint32_t kNoPlace      = 0xFFFFFFFFu;                // no room in the pool
 constexpr uint32_t kSampleBlocks = 32;                         // blocks that sample one gradient, four entries at 768 places each
 constexpr uint32_t kSamplePolls  = 64;                         // looks (0.7 us each) a block takes for another block's sample

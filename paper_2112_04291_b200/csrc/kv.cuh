@@ -15,13 +15,14 @@
 //   pass 2  sizes: per group with entries, the threshold filter |v| >= B_tau, the delta keys (Eq. 4), their
 //           largest (hence M) and a histogram of their bit lengths (hence the payload bits); the group's
 //           (count, M, words) is left in the workspace, the block's totals in a table of one entry per block.
-//   every block takes the totals of all blocks (tagged words) and adds up those before it: its place in the stream.
-//
-// The launch is a chain of a dozen round trips to the L2 whatever the number of pairs.  50 M / 50000 pairs: 22.6 -> 21.0 us (2^20 / 4000: 21.6 -> 17.3) when the
-// sum no longer went through the last block to arrive and the sizes no longer through a barrier.
+//           Every block takes the totals of all blocks (tagged words) and adds up those before it: its place in the stream.
 //   pass 3  pack: per group again, codes || flags || deltas packed in the warp's shared memory (in place in the
 //           stream for blobs too long for it), copied out, with the group's directory entry and those of the
-//           groups without entries before it.  The owner of the last group with entries writes the header.
+//           groups without entries before it.  Block 0 writes the
+//           directory entries behind the last group with entries, and the header.
+//
+// What bounds it: a chain of a dozen round trips to the L2 whatever the number of pairs (50 M / 50000 pairs: 22 us; 2^20 / 4000: 21.2 us when
+// the sum went through the last block to arrive and the sizes through a barrier, now 19.5).
 //
 // Every wait is bounded; when one runs out the block marks the stream FASTSGD_ST_TIMEOUT and leaves.
 // Keys that do not ascend or reach n give an unspecified stream, never an access outside the buffers.
