@@ -19,7 +19,7 @@
 //
 // What bounds it.  With few groups per block, the latency of the chain launch - directory - blob - parse - entries of
 // dense_out (about 3 + 5 us); with many scattered keys, DRAM transactions: a bare kernel that only reads and writes 2.7 M
-// floats at ascending random places of a 1 GiB array takes 108 to 125 us, the decoder 130.  So what counts is warps in
+// floats at ascending random places of a 1 GiB array takes 100 us, the decoder 122.  So what counts is warps in
 // flight and few instructions per key: 512 threads per block and two blocks per SM at 64 registers are 32 warps (256 threads
 // with longer register-resident runs, 16 warps, took 149 us there); parsing side by side with independent fetches instead of a
 // bit reader per thread halved the parse; the table of distinct keys (warps) and the slice (blocks) give each coordinate one
@@ -84,6 +84,13 @@ struct DecArgs {
 // (dense_out holds the aggregated gradient, left there by mode-0 launches over the same streams); 2 both in one launch
 // (dense_out: all zero, and left so); 3 both in one launch on the packed state (theta, m, v, g per coordinate).
 __host__ __device__ constexpr bool mode_fused(int mode) { return mode == 2 || mode == 3; }
+
+// Scattered entries: loads that bring 64 bytes of a line from memory, not all 128.
+__device__ __forceinline__ float load_entry(const float* p) {
+    float x;
+    asm volatile("ld.global.L2::64B.f32 %0, [%1];" : "=f"(x) : "l"(p) : "memory");
+    return x;
+}
 
 // One Adam step (the experimental set-up's equations, no bias correction; one IEEE fp32 operation at a time) on up to K
 // coordinates kk[i] with aggregated gradient g[i]; nothing happens where g[i] == 0 (kk[i] is then not looked at).  All loads
@@ -401,9 +408,9 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;
 
 constexpr uint32_t kNoKey = 0xFFFFu;               // (in a list of keys) an entry of a stream that failed
 
-// One group of a single stream by one warp; entry eb of the block's table is its directory entry.
+// One group of a single stream by one warp; entry eb of the block's table is its directory entry; many: of more than the block has warps.
 template <int MODE>
-__device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint32_t g, uint32_t eb, int lane, int warp) {
+__device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint32_t g, uint32_t eb, bool many, int lane, int warp) {
     const uint64_t lo64 = (uint64_t)g << a.group_log2;
     const uint64_t hi64 = lo64 + (1ull << a.group_log2);
     const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
@@ -428,18 +435,28 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
     const uint32_t c0 = __any_sync(kFullMask, bad != ~0ull) ? 0u : b.count;       // a failed group is left out as a whole
     __syncwarp();
     if constexpr (MODE == 0) {
-        for (uint32_t e0 = 0; e0 < c0; e0 += 256u) {
-            uint32_t kk[8]; float x[8];
+        auto add = [&](auto flight) {                          // so many entries in flight a lane
+            constexpr int K = (int)(sizeof(flight) / sizeof(uint32_t));
+#pragma unroll 1
+            for (uint32_t e0 = 0; e0 < c0; e0 += 32u * K) {
+                uint32_t kk[K]; float x[K];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const uint32_t e = e0 + 32u * i + lane;
-                kk[i] = e < c0 ? lo + keys[e] : 0xFFFFFFFFu;
-                x[i] = e < c0 ? a.dense[kk[i]] : 0.0f;
+                for (int i = 0; i < K; ++i) {
+                    const uint32_t e = e0 + 32u * i + lane;
+                    kk[i] = 0xFFFFFFFFu; x[i] = 0.0f;
+                    if (e < c0) { kk[i] = lo + keys[e]; x[i] = load_entry(a.dense + kk[i]); }
+                }
+#pragma unroll
+                for (int i = 0; i < K; ++i)
+                    if (kk[i] != 0xFFFFFFFFu) a.dense[kk[i]] = __fadd_rn(x[i], code_value(s.val[0], code_at<true>(b, e0 + 32u * i + lane)));
             }
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (kk[i] != 0xFFFFFFFFu) a.dense[kk[i]] = __fadd_rn(x[i], code_value(s.val[0], code_at<true>(b, e0 + 32u * i + lane)));
-        }
+        };
+        // Where every warp has several groups, memory is the bound, and more in flight only make it switch between reading and writing more
+        // often (a bare kernel that updates 2.7 M floats at ascending random places of 1 GiB, a group a warp: eight a lane 113 us, four 107,
+        // two 101, and 8 us more with whole lines fetched; 268 M entries, 1 % kept: 131.5, now 122); else it is the latency.
+        struct Two { uint32_t x[2]; };
+        struct Eight { uint32_t x[8]; };
+        if (many) add(Two()); else add(Eight());
     } else {
         for (uint32_t e0 = 0; e0 < c0; e0 += 128u) {
             uint32_t kk[4]; float gg[4];
@@ -1195,7 +1212,7 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                 x = __shfl_sync(kFullMask, x, 0);
                 if (x >= n_light) break;
                 const uint32_t i = s.light[x];
-                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, lane, warp);
+                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, owned > (uint32_t)kDecWarps, lane, warp);
             }
         } else {
             if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp); __syncthreads(); }
