@@ -91,17 +91,26 @@ __device__ __forceinline__ float load_entry(const float* p) {
     asm volatile("ld.global.L2::64B.f32 %0, [%1];" : "=f"(x) : "l"(p) : "memory");
     return x;
 }
+__device__ __forceinline__ float4 load_entry(const float4* p) {
+    float4 x;
+    asm volatile("ld.global.L2::64B.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "l"(p) : "memory");
+    return x;
+}
 
 // One Adam step (the experimental set-up's equations, no bias correction; one IEEE fp32 operation at a time) on up to K
 // coordinates kk[i] with aggregated gradient g[i]; nothing happens where g[i] == 0 (kk[i] is then not looked at).  All loads
-// are issued before the first of them is needed.  PACKED: one 16-byte entry (theta, m, v, g) per coordinate.
-template <bool PACKED, int K>
+// are issued before the first of them is needed.  PACKED: one 16-byte entry (theta, m, v, g) per coordinate.  ASCENDING: neighbouring threads
+// have neighbouring coordinates (what shares a line is asked for together).
+template <bool PACKED, int K, bool ASCENDING = false>
 __device__ __forceinline__ void adam_run(const DecArgs& a, const uint32_t (&kk)[K], const float (&g)[K]) {
     if constexpr (PACKED) {
         float4* state = reinterpret_cast<float4*>(a.dense);
         float4 st[K];
 #pragma unroll
-        for (int k = 0; k < K; ++k) st[k] = g[k] != 0.0f ? state[kk[k]] : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < K; ++k) {
+            st[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (g[k] != 0.0f) st[k] = ASCENDING ? load_entry(state + kk[k]) : state[kk[k]];
+        }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             if (g[k] != 0.0f) {
@@ -116,9 +125,9 @@ __device__ __forceinline__ void adam_run(const DecArgs& a, const uint32_t (&kk)[
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const bool on = g[k] != 0.0f;
-            pm[k] = on ? a.m[kk[k]] : 0.0f;
-            pv[k] = on ? a.v[kk[k]] : 0.0f;
-            pt[k] = on ? a.theta[kk[k]] : 0.0f;
+            pm[k] = !on ? 0.0f : ASCENDING ? load_entry(a.m + kk[k]) : a.m[kk[k]];
+            pv[k] = !on ? 0.0f : ASCENDING ? load_entry(a.v + kk[k]) : a.v[kk[k]];
+            pt[k] = !on ? 0.0f : ASCENDING ? load_entry(a.theta + kk[k]) : a.theta[kk[k]];
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -197,6 +206,12 @@ constexpr uint32_t kTeamShared     = 200;     // from this many keys on two warp
 // Bytes that a group of several streams takes of its team's memory beside the table: 4 for a coordinate's value and 2 for a key of each
 // entry, the blobs, two words behind them that the parse may look at, and one of flags.
 __host__ __device__ constexpr uint32_t team_bytes(uint32_t entries, uint32_t words) { return 6u * ((entries + 1u) & ~1u) + 4u * (words + 3u); }
+
+// The same for a team of four warps: a bit and the share of a 16-bit count for each index of the group, 8 for each entry (a sum, a key, a place in
+// a list), the blobs, two words behind them that the parse may look at, and five more.
+__host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t words, uint32_t group_log2) {
+    return 6u * ((1u << group_log2) / 32u) + 8u * ((entries + 1u) & ~1u) + 4u * (words + 2u + 5u);
+}
 
 struct DecShared {
     float              val[kDecMaxStreams][132];
@@ -406,6 +421,11 @@ __device__ __forceinline__ void copy_word_async(void* dst_smem, const void* src)
 }
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// the same for a scattered entry: 64 bytes of its line from memory, not all 128
+__device__ __forceinline__ void copy_entry_async(void* dst_smem, const void* src) {
+    asm volatile("cp.async.ca.shared.global.L2::64B [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(__cvta_generic_to_global(src)) : "memory");
+}
+
 constexpr uint32_t kNoKey = 0xFFFFu;               // (in a list of keys) an entry of a stream that failed
 
 // One group of a single stream by one warp; entry eb of the block's table is its directory entry; many: of more than the block has warps.
@@ -474,7 +494,7 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
     __syncwarp();                                                       // (the list is rewritten by the warp's next group)
 }
 
-// Several streams: one group by a team of NW warps (1, 2 or 4); entries eb + w of the block's table are stream w's directory entry.  One
+// Several streams: one group by a team of NW warps (1 or 2); entries eb + w of the block's table are stream w's directory entry.  One
 // entry stands for every distinct key; it collects the streams' values in stream order, so that each coordinate takes one round
 // trip to memory.  keys: a key, or kSharedKey | the entry that stands for it.
 //
@@ -503,7 +523,7 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     uint8_t* mem = s.u.team[team * NW];
     uint16_t* slot = reinterpret_cast<uint16_t*>(mem);                  // table of distinct keys: the entry that stands for the key; 0xFFFF: free
     // (four times the entries as far as the memory's share goes; never less than 1.5 times)
-    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
+    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : 1u)), slots = 1u << slots_log2;
     float* acc = reinterpret_cast<float*>(slot + kTeamSlots * NW);
     uint16_t* keys = reinterpret_cast<uint16_t*>(acc + ((total + 1u) & ~1u));
     uint32_t* blob = reinterpret_cast<uint32_t*>(keys + ((total + 1u) & ~1u));
@@ -521,7 +541,7 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
     dec_team_sync<NW>(team);
     // ---- parse: the threads shared out among the streams, within a warp
-    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), tn = 1u << tn_log2;
+    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + (NW == 1 ? 0u : 1u)), tn = 1u << tn_log2;
     const uint32_t mine = tl >> tn_log2;                            // (beyond W - 1: a stream without keys)
     Blob b;
     b.count = __shfl_sync(kFullMask, count, mine);
@@ -620,6 +640,157 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     dec_team_sync<NW>(team);                                            // (the memory is rewritten for the team's next group)
 }
 
+// The same by a team of four warps, for groups of many keys: a bit for every index of the group and counts of the bits before each word give
+// every distinct key its rank, and the sums go to memory in the order of the coordinates, so that what shares a line is asked for together.
+// (With the table, coordinates came in the streams' order, and it was a third of the instructions: eight streams of 671 K keys over 67 M, the update on the packed
+// state 285 us, now 221.  Of few keys a group the bits cost more than the table: 29 keys of each of four streams 12.9 us, so 14.4.)
+template <int MODE>
+__device__ __forceinline__ void ranked_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t eb, int lane, int warp) {
+    const uint64_t lo64 = (uint64_t)g << a.group_log2;
+    const uint64_t hi64 = lo64 + (1ull << a.group_log2);
+    const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
+    constexpr uint32_t threads = 128u;
+    const int team = warp / 4;
+    const uint32_t tl = 32u * (uint32_t)(warp % 4) + (uint32_t)lane;    // thread of the team
+    // lane w: stream w
+    uint32_t cm = 0u, off = 0u, nw = 0u;
+    if (lane < (int)W) { cm = s.e_cm[eb + lane]; off = s.e_off[eb + lane]; nw = s.e_nw[eb + lane]; }
+    uint32_t count = cm & 0xFFFFFFu;
+    const uint32_t M = cm >> 24, wincl = warp_incl_scan(nw, lane), wbase = wincl - nw, lincl = warp_incl_scan(count, lane), lbase = lincl - count;
+    const uint32_t words = __shfl_sync(kFullMask, wincl, 31), total = __shfl_sync(kFullMask, lincl, 31), even = (total + 1u) & ~1u;
+    const uint32_t map_words = (1u << a.group_log2) / 32u;
+    uint32_t* bits = reinterpret_cast<uint32_t*>(s.u.team[team * 4]);
+    uint16_t* before = reinterpret_cast<uint16_t*>(bits + map_words);   // bits set in the words before
+    float* acc = reinterpret_cast<float*>(before + map_words);          // per rank: the sum
+    uint16_t* key_of = reinterpret_cast<uint16_t*>(acc + even);         // ... and the key
+    uint16_t* list = key_of + even;                                     // the streams' keys, then their ranks
+    uint32_t* blob = reinterpret_cast<uint32_t*>(list + even);
+    uint32_t* failed = blob + words + 2u;                               // bit w: stream w
+    uint32_t* sums = failed + 1;                                        // bits set in the words of each warp
+    // ---- the streams' blobs into shared memory, all copies in flight together
+    for (uint32_t w = 0; w < W; ++w) {
+        const uint32_t n_w = __shfl_sync(kFullMask, nw, w), o_w = __shfl_sync(kFullMask, off, w), b_w = __shfl_sync(kFullMask, wbase, w);
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(a.stream[w]) + o_w;
+        for (uint32_t i = tl; i < n_w; i += threads) copy_word_async(&blob[b_w + i], src + i);
+    }
+    auto clear = [&]() { for (uint32_t i = tl; i < map_words / 4u; i += threads) reinterpret_cast<uint4*>(bits)[i] = make_uint4(0u, 0u, 0u, 0u); };
+    clear();
+    if (tl == 0u) *failed = 0u;
+    copies_wait();
+    dec_team_sync<4>(team);
+    for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
+    dec_team_sync<4>(team);
+    // ---- parse: the threads shared out among the streams, within a warp
+    auto mark = [&](uint32_t k) { if (k < span) atomicOr(&bits[k >> 5], 1u << (k & 31u)); };      // (beyond: the stream fails)
+    {
+        const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + 2u), tn = 1u << tn_log2;
+        const uint32_t mine = tl >> tn_log2;                            // (beyond W - 1: a stream without keys)
+        Blob b;
+        b.count = __shfl_sync(kFullMask, count, mine);
+        b.nwords = __shfl_sync(kFullMask, nw, mine);
+        b.M = __shfl_sync(kFullMask, M, mine);
+        b.words = blob + __shfl_sync(kFullMask, wbase, mine);
+        uint16_t* keys = list + __shfl_sync(kFullMask, lbase, mine);
+        const uint32_t most = __reduce_max_sync(kFullMask, b.count);
+        const bool small = most <= 4u * tn;
+        const unsigned long long bad = parse_team<false, true>(a, s, b, span, (uint32_t)lane & (tn - 1u), tn, small, small ? 1u : (most + 8u * tn - 1u) / (8u * tn),
+                                                               lane, warp, [&](uint32_t j, int m, const auto& v) {
+            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
+#pragma unroll
+            for (int k = 0; k < K; ++k) if (k < m) { keys[j + (uint32_t)k] = (uint16_t)v[k]; mark(v[k]); }
+        });
+        if (bad != ~0ull) {
+            dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
+            atomicOr(failed, 1u << mine);
+        }
+    }
+    dec_team_sync<4>(team);
+    const uint32_t out = *failed;                                       // a failed stream is left out as a whole
+    if (out) {                                                          // the others' keys again
+        clear();
+        if ((out >> lane) & 1u) count = 0u;
+        dec_team_sync<4>(team);
+        for (uint32_t w = 0; w < W; ++w) {
+            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, cm & 0xFFFFFFu, w);
+            for (uint32_t j = tl; j < c_w; j += threads) {
+                if ((out >> w) & 1u) list[b_w + j] = kNoKey; else mark(list[b_w + j]);
+            }
+        }
+        dec_team_sync<4>(team);
+    }
+    // ---- counts of the bits before each word
+    uint32_t distinct;
+    {
+        const uint32_t per = max(1u, map_words / 512u), w0 = tl * per;      // in fours of words
+        const uint4* fours = reinterpret_cast<const uint4*>(bits);
+        const bool any = 4u * w0 < map_words;
+        uint32_t c = 0u;
+        if (any) for (uint32_t i = 0; i < per; ++i) { const uint4 q = fours[w0 + i]; c += (uint32_t)(__popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w)); }
+        const uint32_t incl = warp_incl_scan(c, lane);
+        uint32_t at = incl - c;
+        if (lane == 31) sums[tl >> 5] = incl;
+        dec_team_sync<4>(team);
+        distinct = 0u;
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) { if (i == (tl >> 5)) at += distinct; distinct += sums[i]; }
+        if (any) for (uint32_t i = 0; i < per; ++i) {
+            const uint4 q = fours[w0 + i];
+            const uint32_t x = at + (uint32_t)__popc(q.x), y = x + (uint32_t)__popc(q.y), z = y + (uint32_t)__popc(q.z);
+            reinterpret_cast<uint2*>(before)[w0 + i] = make_uint2(at | (x << 16), y | (z << 16));
+            at = z + (uint32_t)__popc(q.w);
+        }
+    }
+    dec_team_sync<4>(team);
+    // ---- ranks, and what their sums start from (a key of several streams: the same every time)
+    for (uint32_t e0 = tl; e0 < total; e0 += 4u * threads) {
+        uint32_t k[4], word[4], r[4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) k[i] = e0 + threads * i < total ? (uint32_t)list[e0 + threads * i] : (uint32_t)kNoKey;
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) { word[i] = 0u; r[i] = 0u; if (k[i] != kNoKey) { word[i] = bits[k[i] >> 5]; r[i] = before[k[i] >> 5]; } }
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) {
+            if (k[i] == kNoKey) continue;
+            r[i] += (uint32_t)__popc(word[i] & ((1u << (k[i] & 31u)) - 1u));
+            list[e0 + threads * i] = (uint16_t)r[i];
+            key_of[r[i]] = (uint16_t)k[i];
+            if constexpr (MODE == 0) copy_entry_async(&acc[r[i]], a.dense + lo + k[i]);
+            else acc[r[i]] = 0.0f;
+        }
+    }
+    if constexpr (MODE == 0) copies_wait();
+    dec_team_sync<4>(team);
+    if constexpr (MODE != 1) {
+        for (uint32_t w = 0; w < W; ++w) {
+            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, wbase, w);
+            if (c_w == 0u) continue;
+            const uint8_t* codes = reinterpret_cast<const uint8_t*>(blob + s_w);
+            for (uint32_t j = tl; j < c_w; j += threads) {
+                const uint32_t r = list[b_w + j];
+                acc[r] = __fadd_rn(acc[r], code_value(s.val[w], codes[j ^ 3u]));
+            }
+            dec_team_sync<4>(team);
+        }
+    }
+    for (uint32_t r0 = 0; r0 < distinct; r0 += 4u * threads) {
+        uint32_t kk[4]; float gg[4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) {
+            const uint32_t r = r0 + threads * i + tl;
+            const bool on = r < distinct;
+            kk[i] = on ? lo + key_of[r] : 0u;
+            gg[i] = 0.0f;
+            if (on) {
+                if constexpr (MODE == 0) a.dense[kk[i]] = acc[r];
+                else if constexpr (MODE == 1) { gg[i] = a.dense[kk[i]]; a.dense[kk[i]] = 0.0f; }
+                else gg[i] = acc[r];
+            }
+        }
+        if constexpr (MODE != 0) adam_run<MODE == 3, 4, true>(a, kk, gg);
+    }
+    dec_team_sync<4>(team);                                       // (the memory is rewritten for the team's next group)
+}
+
 // entry x of the list of groups for one (list 0), two or four (2) warps
 __device__ __forceinline__ uint16_t& team_list_entry(DecShared& s, uint32_t list, uint32_t x) {
     return list == 0u ? s.light[x] : list == 1u ? s.heavy[kDecThreads - 1u - x] : s.light[kDecThreads - 1u - x];
@@ -638,7 +809,8 @@ __device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint
         else { dec_team_sync<NW>(team); x = s.grab[team]; }
         if (x >= n) break;
         const uint32_t i = team_list_entry(s, kList, x);
-        team_group<MODE, NW>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
+        if constexpr (NW == 4) ranked_group<MODE>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
+        else team_group<MODE, NW>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
     }
 }
 
@@ -1166,8 +1338,10 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                 if (ONE) { if (tot <= warp_max && a.group_log2 <= 16u) list = 0u; }
                 else if (a.group_log2 <= 15u && tot < team_max) {
                     const uint32_t bytes = team_bytes(tot, s.gtot[kDecThreads / 2 + tid]), room = kTeamBytes - 2u * kTeamSlots;
-                    list = bytes <= room ? 0u : bytes <= 2u * room ? 1u : bytes <= 4u * room ? 2u : 3u;
+                    const uint32_t ranked = ranked_bytes(tot, s.gtot[kDecThreads / 2 + tid], a.group_log2);
+                    list = bytes <= room ? 0u : bytes <= 2u * room ? 1u : 2u;
                     list = max(list, least_team);
+                    if (list == 2u && ranked > 4u * kTeamBytes) list = 3u;
                 }
                 if (list < 3u) team_list_entry(s, list, atomicAdd(&s.n_light[list], 1u)) = (uint16_t)tid;
                 else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;

@@ -153,3 +153,50 @@ def test_teams_of_warps(groups, workers, l, group_log2):
 @pytest.mark.parametrize("workers,count", [(2, 200), (3, 110), (8, 30), (8, 100), (8, 190), (8, 300)])
 def test_teams_on_groups_of_two_tiles(workers, count):
     _check((40 << 15) - 9, [count, count + 1] * 20, workers, 600 + count, group_log2=15)
+
+
+# teams of four warps (ranks by a bit for every index): keys at the edges of the bits' words and of the groups, streams that fail in one group
+@pytest.mark.parametrize("workers,count,group_log2", [(6, 170, 14), (3, 500, 14), (8, 130, 15), (7, 200, 11)])
+def test_teams_of_four_warps(workers, count, group_log2):
+    groups, size = 620, 1 << group_log2
+    n = groups * size - 3
+    rng = np.random.default_rng(count)
+    po, pg = oracle.params(1.3, 128, 2, group_log2), binding.params(1.3, 128, 2, group_log2)
+    edges = np.array([0, 31, 32, 63, 127, 128, size // 2, size - 33, size - 32, size - 4])
+    streams = []
+    for w in range(workers):
+        v = np.zeros(n, np.float32)
+        for g in range(groups):
+            k = np.unique(np.concatenate([rng.choice(edges, 6, replace=False), rng.integers(0, size - 4, count)]))
+            v[g * size + k] = (rng.uniform(0.5, 2.0, k.size) * rng.choice([-1.0, 1.0], k.size)).astype(np.float32)
+        rc, s = oracle.compress(v, po)
+        assert rc == 0
+        streams.append(s)
+    bad, group = (1, 2), 300
+    lo, hi = group * size, (group + 1) * size
+    dense0 = rng.standard_normal(n).astype(np.float32)
+    want, sound = dense0.copy(), dense0.copy()
+    for w, s in enumerate(streams):
+        assert oracle.decompress_accumulate(s, n, po, want) == 0
+        assert w in bad or oracle.decompress_accumulate(s, n, po, sound) == 0
+    binding.ensure_workspace(n, pg)
+
+    def decode():
+        dense = torch.from_numpy(dense0.copy()).to(G.dev())
+        dev = [G.to_dev(np.concatenate([s, np.zeros(-s.size % 16 + 16, np.uint8)])) for s in streams]
+        assert binding.decompress_accumulate_batch(dev, [s.size for s in streams], n, pg, dense) == 0
+        return dense.cpu().numpy(), binding.decode_status()
+
+    got, status = decode()
+    assert status == 0 and np.array_equal(got, want)
+    for w in bad:                                          # the first deltas of one group become 0
+        s = streams[w] = streams[w].copy()
+        cnt, off = (int(x) for x in np.frombuffer(s[64 + 8 * group:72 + 8 * group].tobytes(), np.uint32))
+        cnt &= 0xFFFFFF
+        bits = np.unpackbits(s[4 * off:4 * off + 2 * cnt + 16])
+        bits[10 * cnt:10 * cnt + 40] = 0
+        s[4 * off:4 * off + 2 * cnt + 16] = np.packbits(bits)
+    want[lo:hi] = sound[lo:hi]
+    got, status = decode()
+    assert status == oracle.decompress_accumulate(streams[bad[0]], n, po, np.zeros(n, np.float32)) != 0
+    assert np.array_equal(got, want)
