@@ -49,8 +49,15 @@ constexpr uint32_t kBlockStageWords = 4096;   // blobs larger than this in total
 constexpr uint32_t kBlockListMax   = 8192;    // keys of a group (all streams together) the block path lists in shared memory
 constexpr uint32_t kWideListMax    = 1u << 14;      // ... of a group wider than the tile, in the tile's place
 // From this many keys on the group's whole slice of dense_out goes through shared memory: scattered over 2048 sectors of 32 bytes
-// they touch more than half of it, and a bulk copy moves whole pages (10 % of 2^26 entries: 96 us with, 111 without the slice).
-constexpr uint32_t kTileMinKeys    = 1536;
+// they touch a third of it, and a bulk copy moves whole pages (7.5 % of 2^26 entries, one stream: 96 us with, 111 without the slice).
+constexpr uint32_t kTileMinKeys    = 768;
+// Several streams whose groups have about as many keys: from this many a group on ranks by bits (four warps) instead of the table of keys, up to as
+// many as aggregation has the slice for.  Eight streams over 2^25 entries, us by table and by ranks (slice), at keys a group:
+//   aggregation  180: 22, 27; 290: 27, 31; 420: 38, 37; 650: 59, 56; 850: 75, 68 (78); 980: 77 by ranks (78); 1310: 94 by ranks (78)
+//   update       180: 64, 63; 290: 97, 84; 420: 131, 102; 650: 183, 126; 1310: 182 over the slice of g, 164; 1770: 186, 174
+//   packed       180: 25, 28; 290: 34, 35; 420: 51, 50; 650: 85, 76; 850: 112, 90; 1770: 196 over the slice, 139
+__host__ __device__ constexpr uint32_t ranked_mean(int mode) { return mode == 2 ? 256u : 400u; }
+constexpr uint32_t kSliceMean      = 1000;
 // From this many keys on the model update goes over the slice of g, four neighbouring coordinates at a time, instead of key by key
 // (eight streams, 5 % of 2^24 entries: 292 -> 125 us); on the packed state, where a key is one access anyway, later (235 -> 132 us).
 constexpr uint32_t kSweepMinKeys   = 768;
@@ -488,7 +495,7 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
                 if constexpr (MODE == 1) gg[i] = e < c0 ? atomicExch(a.dense + kk[i], 0.0f) : 0.0f;
                 else gg[i] = e < c0 ? code_value(s.val[0], code_at<true>(b, e)) : 0.0f;
             }
-            adam_run<MODE == 3, 4>(a, kk, gg);
+            adam_run<MODE == 3, 4, true>(a, kk, gg);
         }
     }
     __syncwarp();                                                       // (the list is rewritten by the warp's next group)
@@ -643,7 +650,7 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
 // The same by a team of four warps, for groups of many keys: a bit for every index of the group and counts of the bits before each word give
 // every distinct key its rank, and the sums go to memory in the order of the coordinates, so that what shares a line is asked for together.
 // (With the table, coordinates came in the streams' order, and it was a third of the instructions: eight streams of 671 K keys over 67 M, the update on the packed
-// state 285 us, now 221.  Of few keys a group the bits cost more than the table: 29 keys of each of four streams 12.9 us, so 14.4.)
+// state 285 us, now 216.  Of few keys a group the bits cost more than the table: 29 keys of each of four streams 12.9 us, so 14.4.)
 template <int MODE>
 __device__ __forceinline__ void ranked_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t eb, int lane, int warp) {
     const uint64_t lo64 = (uint64_t)g << a.group_log2;
@@ -1318,8 +1325,8 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
             else if (cm) { atomicAdd(&s.gtot[my_i], cm & 0xFFFFFFu); atomicAdd(&s.gtot[kDecThreads / 2 + my_i], nw); }
         }
         __syncthreads();
-        // Where most groups have about as many keys, they all go to teams, up to as many keys as the slice (the update: the sweep) is for; with
-        // few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a block with one
+        // Where most groups have about as many keys, they all go to teams (of the same size: ranked_mean), up to as many keys as the
+        // slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a block with one
         // group, those of many keys are for whole blocks, which share them through the queue below: teams of several sizes work one after
         // the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
         uint32_t team_max = kTeamFew, least_team = 0u;
@@ -1327,8 +1334,9 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
             const uint32_t x = tid < (int)in_batch ? s.gtot[tid] : 0u;
             const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= s.mean && x <= 2u * s.mean);
             if (in_batch > 1u && 4u * alike >= 3u * in_batch) {
-                team_max = MODE == 2 ? kSweepMinKeys : kTileMinKeys;
-                if (s.mean >= kTeamShared) least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
+                team_max = MODE == 0 && s.mean >= kSliceMean ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
+                if (s.mean >= ranked_mean(MODE)) least_team = 2u;
+                else if (s.mean >= kTeamShared) least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
             }
         }
         if (tid < (int)in_batch) {
