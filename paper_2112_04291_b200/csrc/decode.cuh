@@ -58,6 +58,7 @@ constexpr uint32_t kTileMinKeys    = 768;
 //   packed       180: 25, 28; 290: 34, 35; 420: 51, 50; 650: 85, 76; 850: 112, 90; 1770: 196 over the slice, 139
 __host__ __device__ constexpr uint32_t ranked_mean(int mode) { return mode == 2 ? 256u : 400u; }
 constexpr uint32_t kSliceMean      = 1000;
+constexpr uint32_t kFewGroups      = 4;       // groups of a block that teams of four take side by side
 // From this many keys on the model update goes over the slice of g, four neighbouring coordinates at a time, instead of key by key
 // (eight streams, 5 % of 2^24 entries: 292 -> 125 us); on the packed state, where a key is one access anyway, later (235 -> 132 us).
 constexpr uint32_t kSweepMinKeys   = 768;
@@ -501,7 +502,7 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
     __syncwarp();                                                       // (the list is rewritten by the warp's next group)
 }
 
-// Several streams: one group by a team of NW warps (1 or 2); entries eb + w of the block's table are stream w's directory entry.  One
+// Several streams: one group by a team of NW warps (1, 2 or 4); entries eb + w of the block's table are stream w's directory entry.  One
 // entry stands for every distinct key; it collects the streams' values in stream order, so that each coordinate takes one round
 // trip to memory.  keys: a key, or kSharedKey | the entry that stands for it.
 //
@@ -530,7 +531,7 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     uint8_t* mem = s.u.team[team * NW];
     uint16_t* slot = reinterpret_cast<uint16_t*>(mem);                  // table of distinct keys: the entry that stands for the key; 0xFFFF: free
     // (four times the entries as far as the memory's share goes; never less than 1.5 times)
-    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : 1u)), slots = 1u << slots_log2;
+    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
     float* acc = reinterpret_cast<float*>(slot + kTeamSlots * NW);
     uint16_t* keys = reinterpret_cast<uint16_t*>(acc + ((total + 1u) & ~1u));
     uint32_t* blob = reinterpret_cast<uint32_t*>(keys + ((total + 1u) & ~1u));
@@ -548,7 +549,7 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
     dec_team_sync<NW>(team);
     // ---- parse: the threads shared out among the streams, within a warp
-    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + (NW == 1 ? 0u : 1u)), tn = 1u << tn_log2;
+    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), tn = 1u << tn_log2;
     const uint32_t mine = tl >> tn_log2;                            // (beyond W - 1: a stream without keys)
     Blob b;
     b.count = __shfl_sync(kFullMask, count, mine);
@@ -803,9 +804,10 @@ __device__ __forceinline__ uint16_t& team_list_entry(DecShared& s, uint32_t list
     return list == 0u ? s.light[x] : list == 1u ? s.heavy[kDecThreads - 1u - x] : s.light[kDecThreads - 1u - x];
 }
 
-// The block's groups for teams of NW warps, one after the other to whichever team is free.
+// The block's groups for teams of NW warps, one after the other to whichever team is free.  table: aggregation by a table of keys in teams of four
+// too: a block's few groups stand side by side then, and what counts is the shorter chain (550 groups of 790 keys, four streams: 19.6 us, by ranks 20.8).
 template <int MODE, int NW>
-__device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint32_t W, uint32_t first, int lane, int warp) {
+__device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint32_t W, uint32_t first, bool table, int lane, int warp) {
     constexpr uint32_t kList = NW == 1 ? 0u : NW == 2 ? 1u : 2u;
     const uint32_t n = s.n_light[kList];
     const int team = warp / NW;
@@ -816,8 +818,9 @@ __device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint
         else { dec_team_sync<NW>(team); x = s.grab[team]; }
         if (x >= n) break;
         const uint32_t i = team_list_entry(s, kList, x);
-        if constexpr (NW == 4) ranked_group<MODE>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
-        else team_group<MODE, NW>(a, s, W, blockIdx.x + (first + i) * gridDim.x, i * W, lane, warp);
+        const uint32_t g = blockIdx.x + (first + i) * gridDim.x;
+        if (NW == 4 && !(MODE == 0 && table)) ranked_group<MODE>(a, s, W, g, i * W, lane, warp);
+        else if constexpr (NW < 4 || MODE == 0) team_group<MODE, NW>(a, s, W, g, i * W, lane, warp);
     }
 }
 
@@ -1336,7 +1339,7 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
             if (in_batch > 1u && 4u * alike >= 3u * in_batch) {
                 team_max = MODE == 0 && s.mean >= kSliceMean ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
                 if (s.mean >= ranked_mean(MODE)) least_team = 2u;
-                else if (s.mean >= kTeamShared) least_team = owned <= 4u ? 2u : owned <= 8u ? 1u : 0u;
+                else if (s.mean >= kTeamShared) least_team = owned <= kFewGroups ? 2u : owned <= 8u ? 1u : 0u;
             }
         }
         if (tid < (int)in_batch) {
@@ -1349,7 +1352,7 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                     const uint32_t ranked = ranked_bytes(tot, s.gtot[kDecThreads / 2 + tid], a.group_log2);
                     list = bytes <= room ? 0u : bytes <= 2u * room ? 1u : 2u;
                     list = max(list, least_team);
-                    if (list == 2u && ranked > 4u * kTeamBytes) list = 3u;
+                    if (list == 2u && (ranked > 4u * kTeamBytes || bytes > 4u * room)) list = 3u;
                 }
                 if (list < 3u) team_list_entry(s, list, atomicAdd(&s.n_light[list], 1u)) = (uint16_t)tid;
                 else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
@@ -1397,9 +1400,9 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                 warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, owned > (uint32_t)kDecWarps, lane, warp);
             }
         } else {
-            if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp); __syncthreads(); }
-            if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, lane, warp); __syncthreads(); }
-            team_groups<MODE, 1>(a, s, W, first, lane, warp);
+            if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, owned <= kFewGroups, lane, warp); __syncthreads(); }
+            if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, owned <= kFewGroups, lane, warp); __syncthreads(); }
+            team_groups<MODE, 1>(a, s, W, first, owned <= kFewGroups, lane, warp);
         }
     }
 
