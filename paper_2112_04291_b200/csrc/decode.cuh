@@ -22,7 +22,7 @@
 // floats at ascending random places of a 1 GiB array takes 100 us, the decoder 122.  So what counts is warps in
 // flight and few instructions per key: 512 threads per block and two blocks per SM at 64 registers are 32 warps (256 threads
 // with longer register-resident runs, 16 warps, took 149 us there); parsing side by side with independent fetches instead of a
-// bit reader per thread halved the parse; the table of distinct keys (warps) and the slice (blocks) give each coordinate one
+// bit reader per thread halved the parse; the table of distinct keys or their ranks (teams) and the slice (blocks) give each coordinate one
 // round trip to memory however many streams hold it (one per stream before).  Measured before and after: four
 // streams of 128 K keys over 25.6 M entries 28.8 -> 23.5 us, eight streams of 33 K keys over 33.5 M 26.7 -> 16.8, one stream of
 // 1.3 M over 67 M 97.8 -> 59.5; model update of the first 68.6 -> 41.0, of eight streams of 671 K keys over 67 M on the
@@ -59,7 +59,7 @@ constexpr uint32_t kTileMinKeys    = 768;
 __host__ __device__ constexpr uint32_t ranked_mean(int mode) { return mode == 2 ? 256u : 400u; }
 constexpr uint32_t kSliceMean      = 1000;
 constexpr uint32_t kFewGroups      = 4;       // groups of a block that teams of four take side by side
-// From this many keys on the model update goes over the slice of g, four neighbouring coordinates at a time, instead of key by key
+// From this many keys on the model update by a block goes over the slice of g, four neighbouring coordinates at a time, instead of key by key
 // (eight streams, 5 % of 2^24 entries: 292 -> 125 us); on the packed state, where a key is one access anyway, later (235 -> 132 us).
 constexpr uint32_t kSweepMinKeys   = 768;
 constexpr uint32_t kSweepMinPacked = 2048;
