@@ -41,6 +41,19 @@ int fastsgd_debug_set_wait_limits(uint32_t block_polls, uint32_t copy_tries, uin
  * once).  The stream never depends on the grid: tests use this to show it. */
 int fastsgd_debug_set_grid(uint32_t blocks);
 
+/* Who decodes one group, by the rules of the decoder's launch (a pure function: no GPU is used):
+ *   mode        0 aggregation, 1 update as a pass of its own, 2 update in one launch, 3 the same on the packed state
+ *   streams     1..8, of the launch
+ *   n           entries of the gradient
+ *   owned       groups of the thread block that holds the group
+ *   alike_mean  keys of a group on average where most groups of the block have about as many; else 0
+ *   keys, words keys of the group over all streams, 32-bit words of its blobs
+ *   bulk        dense_out (mode 2: theta, m and v) is 16-byte aligned
+ * Returns 0, 1, 2: one, two, four warps (several streams: by a table of keys); 3: four warps by ranks; 4: the block, entry by
+ * entry (the update: or over its slice of g); 5: the block over the group's slice of dense_out; 6: the block, a group wider than that slice;
+ * 7: one warp with two entries a lane in flight; -1: bad arguments. */
+int fastsgd_debug_decoder_route(uint32_t mode, uint32_t streams, uint64_t n, uint32_t group_log2, uint32_t owned, uint32_t alike_mean, uint32_t keys, uint32_t words, int bulk);
+
 /* Byte offsets inside the registered workspace (all of them in its fixed first
  * part): [0] u32 bar_count[8], arrivals (k_resident: per gradient);
  * [1] u32 ne_count[8], tiles the last encoder launch read a second time, per

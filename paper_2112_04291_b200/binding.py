@@ -31,6 +31,7 @@ EXPORTS = [
     "fastsgd_sparse_adam_update_batch", "fastsgd_sparse_adam_update_packed_batch", "fastsgd_key_encode_paper", "fastsgd_key_encode_paper_bound",
     "fastsgd_compress_kv",
     "fastsgd_debug_set_wait_limits", "fastsgd_debug_layout", "fastsgd_debug_set_grid",
+    "fastsgd_debug_decoder_route",
 ]
 
 
@@ -119,6 +120,8 @@ def lib():
         L.fastsgd_debug_set_wait_limits.argtypes = [C.c_uint32, C.c_uint32, C.c_uint32]
         L.fastsgd_debug_set_grid.restype = C.c_int
         L.fastsgd_debug_set_grid.argtypes = [C.c_uint32]
+        L.fastsgd_debug_decoder_route.restype = C.c_int
+        L.fastsgd_debug_decoder_route.argtypes = [C.c_uint32, C.c_uint32, u64] + [C.c_uint32] * 5 + [C.c_int]
         L.fastsgd_debug_layout.restype = C.c_int
         L.fastsgd_debug_layout.argtypes = [u64p, C.c_uint32]
         _lib = L
@@ -339,6 +342,17 @@ def debug_set_wait_limits(block_polls: int = 0, copy_tries: int = 0, queue_polls
 def debug_set_grid(blocks: int = 0) -> None:
     """fastsgd_debug_set_grid: cap the encoders' thread blocks (0: default).  Test aid."""
     _check(lib().fastsgd_debug_set_grid(int(blocks)), "fastsgd_debug_set_grid")
+
+
+ROUTES = ("warp", "two warps", "four warps", "four warps by ranks", "block", "block over the slice", "wide block", "warp, two in flight")
+
+
+def debug_decoder_route(mode: int, streams: int, n: int, group_log2: int, owned: int, alike_mean: int, keys: int, words: int, bulk: bool = True) -> str:
+    """fastsgd_debug_decoder_route: who decodes a group (one of ROUTES).  Test aid; needs no GPU."""
+    r = lib().fastsgd_debug_decoder_route(mode, streams, n, group_log2, owned, alike_mean, keys, words, int(bulk))
+    if r < 0:
+        raise ValueError("bad arguments")
+    return ROUTES[r]
 
 
 LAYOUT_FIELDS = ("bar_count", "ne_count", "error", "late_blobs", "unused_4", "unused_5",

@@ -221,6 +221,40 @@ __host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t w
     return 6u * ((1u << group_log2) / 32u) + 8u * ((entries + 1u) & ~1u) + 4u * (words + 2u + 5u);
 }
 
+// Who decodes the groups of several streams (mode as below): those of fewer than `below` keys teams of at least `least` (0, 1, 2: one, two, four
+// warps), the others the block.  table: teams of four by the table of keys, not by ranks.
+// Where most of a block's groups have about as many keys (alike), they all go to teams (of the same size: ranked_mean), up to as many keys as the
+// slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a
+// block with one group, those of many keys are for whole blocks, which share them through a queue: teams of several sizes work one after
+// the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
+// Aggregation by the table in teams of four too where a block's few groups stand side by side: what counts then is the shorter chain (550 groups
+// of 790 keys, four streams: 19.6 us, by ranks 20.8).
+struct TeamRule { uint32_t below, least; bool table; };
+__host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, uint32_t owned, bool alike, uint32_t mean) {
+    const bool few = owned <= kFewGroups;
+    TeamRule r{kTeamFew, 0u, mode == 0 && few};
+    if (alike) {
+        r.below = mode == 0 && mean >= kSliceMean ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
+        r.least = mean >= ranked_mean(mode) ? 2u : mean < kTeamShared ? 0u : few ? 2u : owned <= 8u ? 1u : 0u;
+    }
+    if (group_log2 > 15u) r.below = 0u;
+    return r;
+}
+// ... and a group of so many keys, with blobs of so many words: 0, 1, 2 as above, or 3, the block
+__host__ __device__ constexpr uint32_t team_for(const TeamRule& r, uint32_t group_log2, uint32_t keys, uint32_t words) {
+    if (keys >= r.below) return 3u;
+    const uint32_t bytes = team_bytes(keys, words), room = kTeamBytes - 2u * kTeamSlots;
+    const uint32_t fits = bytes <= room ? 0u : bytes <= 2u * room ? 1u : 2u, team = fits < r.least ? r.least : fits;
+    if (team == 2u && (ranked_bytes(keys, words, group_log2) > 4u * kTeamBytes || bytes > 4u * room)) return 3u;
+    return team;
+}
+// One stream: the most keys of a group that one warp decodes.
+__host__ __device__ constexpr uint32_t warp_max(uint32_t owned) { return owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew; }
+// ... and whether it keeps two entries a lane in flight when it adds them up, not eight
+__host__ __device__ constexpr bool two_in_flight(uint32_t owned) { return owned > (uint32_t)kDecWarps; }
+// Aggregation by the block: over the group's whole slice of dense_out from this many keys on.
+__host__ __device__ constexpr uint32_t slice_min() { return kTileMinKeys; }
+
 struct DecShared {
     float              val[kDecMaxStreams][132];
     uint32_t           hdr[kDecMaxStreams][16];
@@ -436,9 +470,9 @@ __device__ __forceinline__ void copy_entry_async(void* dst_smem, const void* src
 
 constexpr uint32_t kNoKey = 0xFFFFu;               // (in a list of keys) an entry of a stream that failed
 
-// One group of a single stream by one warp; entry eb of the block's table is its directory entry; many: of more than the block has warps.
+// One group of a single stream by one warp; entry eb of the block's table is its directory entry; two: as in two_in_flight.
 template <int MODE>
-__device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint32_t g, uint32_t eb, bool many, int lane, int warp) {
+__device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint32_t g, uint32_t eb, bool two, int lane, int warp) {
     const uint64_t lo64 = (uint64_t)g << a.group_log2;
     const uint64_t hi64 = lo64 + (1ull << a.group_log2);
     const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
@@ -484,7 +518,7 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
         // two 101, and 8 us more with whole lines fetched; 268 M entries, 1 % kept: 131.5, now 122); else it is the latency.
         struct Two { uint32_t x[2]; };
         struct Eight { uint32_t x[8]; };
-        if (many) add(Two()); else add(Eight());
+        if (two) add(Two()); else add(Eight());
     } else {
         for (uint32_t e0 = 0; e0 < c0; e0 += 128u) {
             uint32_t kk[4]; float gg[4];
@@ -804,10 +838,9 @@ __device__ __forceinline__ uint16_t& team_list_entry(DecShared& s, uint32_t list
     return list == 0u ? s.light[x] : list == 1u ? s.heavy[kDecThreads - 1u - x] : s.light[kDecThreads - 1u - x];
 }
 
-// The block's groups for teams of NW warps, one after the other to whichever team is free.  table: aggregation by a table of keys in teams of four
-// too: a block's few groups stand side by side then, and what counts is the shorter chain (550 groups of 790 keys, four streams: 19.6 us, by ranks 20.8).
+// The block's groups for teams of NW warps, one after the other to whichever team is free.  table (teams of four, aggregation): as in TeamRule.
 template <int MODE, int NW>
-__device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint32_t W, uint32_t first, bool table, int lane, int warp) {
+__device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint32_t W, uint32_t first, int lane, int warp, bool table = false) {
     constexpr uint32_t kList = NW == 1 ? 0u : NW == 2 ? 1u : 2u;
     const uint32_t n = s.n_light[kList];
     const int team = warp / NW;
@@ -819,8 +852,8 @@ __device__ __forceinline__ void team_groups(const DecArgs& a, DecShared& s, uint
         if (x >= n) break;
         const uint32_t i = team_list_entry(s, kList, x);
         const uint32_t g = blockIdx.x + (first + i) * gridDim.x;
-        if (NW == 4 && !(MODE == 0 && table)) ranked_group<MODE>(a, s, W, g, i * W, lane, warp);
-        else if constexpr (NW < 4 || MODE == 0) team_group<MODE, NW>(a, s, W, g, i * W, lane, warp);
+        if (NW < 4 || (MODE == 0 && table)) team_group<MODE, NW>(a, s, W, g, i * W, lane, warp);
+        else ranked_group<MODE>(a, s, W, g, i * W, lane, warp);
     }
 }
 
@@ -1013,7 +1046,7 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
     const bool lists = listed <= kBlockListMax && words <= kBlockStageWords;      // (else: stream by stream)
     const bool bulk_ok = ((reinterpret_cast<uintptr_t>(a.dense) & 15u) == 0u) && ((span & 3u) == 0u);
     // aggregation of many keys: the slice of dense_out goes through shared memory as a whole
-    const bool slice = MODE == 0 && (total >= kTileMinKeys || !lists);
+    const bool slice = MODE == 0 && (total >= slice_min() || !lists);
     if (tid == 0) {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the last write-back has read the tile
         if (slice && bulk_ok) {
@@ -1309,7 +1342,6 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
 
     unsigned int* q_taken = a.q_ctl + 1, *q_done = a.q_ctl + 2, *q_exited = a.q_ctl + 3, *q_reserved = a.q_ctl + 4;
     const bool queue = a.G > B;
-    const uint32_t warp_max = owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew;
     for (uint32_t first = 0; first < owned; first += per_batch) {
         if (first > 0u) { __syncthreads(); d0 = d1 = d2 = 0u; load_dir(first + my_i); }
         // ---- classify the batch's groups
@@ -1328,32 +1360,18 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
             else if (cm) { atomicAdd(&s.gtot[my_i], cm & 0xFFFFFFu); atomicAdd(&s.gtot[kDecThreads / 2 + my_i], nw); }
         }
         __syncthreads();
-        // Where most groups have about as many keys, they all go to teams (of the same size: ranked_mean), up to as many keys as the
-        // slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a block with one
-        // group, those of many keys are for whole blocks, which share them through the queue below: teams of several sizes work one after
-        // the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
-        uint32_t team_max = kTeamFew, least_team = 0u;
+        TeamRule rule{};
         if constexpr (!ONE) {
             const uint32_t x = tid < (int)in_batch ? s.gtot[tid] : 0u;
             const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= s.mean && x <= 2u * s.mean);
-            if (in_batch > 1u && 4u * alike >= 3u * in_batch) {
-                team_max = MODE == 0 && s.mean >= kSliceMean ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
-                if (s.mean >= ranked_mean(MODE)) least_team = 2u;
-                else if (s.mean >= kTeamShared) least_team = owned <= kFewGroups ? 2u : owned <= 8u ? 1u : 0u;
-            }
+            rule = team_rule(MODE, a.group_log2, owned, in_batch > 1u && 4u * alike >= 3u * in_batch, s.mean);
         }
         if (tid < (int)in_batch) {
             const uint32_t tot = s.gtot[tid];
             if (tot != 0u) {
                 uint32_t list = 3u;
-                if (ONE) { if (tot <= warp_max && a.group_log2 <= 16u) list = 0u; }
-                else if (a.group_log2 <= 15u && tot < team_max) {
-                    const uint32_t bytes = team_bytes(tot, s.gtot[kDecThreads / 2 + tid]), room = kTeamBytes - 2u * kTeamSlots;
-                    const uint32_t ranked = ranked_bytes(tot, s.gtot[kDecThreads / 2 + tid], a.group_log2);
-                    list = bytes <= room ? 0u : bytes <= 2u * room ? 1u : 2u;
-                    list = max(list, least_team);
-                    if (list == 2u && (ranked > 4u * kTeamBytes || bytes > 4u * room)) list = 3u;
-                }
+                if (ONE) { if (tot <= warp_max(owned) && a.group_log2 <= 16u) list = 0u; }
+                else list = team_for(rule, a.group_log2, tot, s.gtot[kDecThreads / 2 + tid]);
                 if (list < 3u) team_list_entry(s, list, atomicAdd(&s.n_light[list], 1u)) = (uint16_t)tid;
                 else s.heavy[atomicAdd(&s.n_heavy, 1u)] = (uint16_t)tid;
             }
@@ -1397,12 +1415,12 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                 x = __shfl_sync(kFullMask, x, 0);
                 if (x >= n_light) break;
                 const uint32_t i = s.light[x];
-                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, owned > (uint32_t)kDecWarps, lane, warp);
+                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, two_in_flight(owned), lane, warp);
             }
         } else {
-            if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, owned <= kFewGroups, lane, warp); __syncthreads(); }
-            if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, owned <= kFewGroups, lane, warp); __syncthreads(); }
-            team_groups<MODE, 1>(a, s, W, first, owned <= kFewGroups, lane, warp);
+            if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp, MODE == 0 && owned <= kFewGroups); __syncthreads(); }
+            if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, lane, warp); __syncthreads(); }
+            team_groups<MODE, 1>(a, s, W, first, lane, warp);
         }
     }
 

@@ -1,0 +1,34 @@
+"""Who decodes a group: the rules of the decoder's launch, asked without a GPU."""
+import pytest
+
+from paper_2112_04291_b200 import binding, build
+
+N = 1 << 26                        # entries, more than the L2 holds
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+
+
+def _route(mode=0, streams=8, n=N, group_log2=14, owned=13, mean=0, keys=None, words=None, bulk=True):
+    keys = mean if keys is None else keys
+    return binding.debug_decoder_route(mode, streams, n, group_log2, owned, mean, keys, -(-keys * 15 // 32) if words is None else words, bulk)
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
+def test_groups_of_few_keys_go_to_a_warp_and_unlike_large_ones_to_the_block(mode):
+    assert _route(mode, keys=248) == "warp" and _route(mode, keys=249) == "block"
+    assert _route(mode, streams=1, n=1 << 24, keys=1024) == "warp" and _route(mode, streams=1, n=1 << 24, owned=7, keys=257) == "block"
+    assert _route(mode, group_log2=16, keys=10) == "wide block" and _route(mode, streams=1, group_log2=17, keys=10) == "wide block"
+
+
+@pytest.mark.parametrize("mode,line", [(0, 400), (1, 400), (2, 256), (3, 400)])
+def test_ranks_from_a_mean_on(mode, line):
+    assert _route(mode, mean=line) == "four warps by ranks" and _route(mode, mean=line - 1) == "warp"
+    assert _route(mode, mean=line, owned=4) == ("four warps" if mode == 0 else "four warps by ranks")
+    assert _route(mode, mean=line - 1, owned=8) == "two warps"
+
+
+def test_aggregation_over_the_slice_from_a_mean_on():
+    assert _route(mean=999) == "four warps by ranks" and _route(mean=1000) == "block over the slice"
