@@ -227,6 +227,8 @@ __host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t w
 // slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a
 // block with one group, those of many keys are for whole blocks, which share them through a queue: teams of several sizes work one after
 // the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
+// (Groups wider than the slice have no slice: eight streams over 2^25 entries in groups of 2^15, 1050, 1500, 1750 keys a group: by teams 51, 70, 80 us, by
+// blocks 70, 85, 95.)
 // Aggregation by the table in teams of four too where a block's few groups stand side by side: what counts then is the shorter chain (550 groups
 // of 790 keys, four streams: 19.6 us, by ranks 20.8).
 struct TeamRule { uint32_t below, least; bool table; };
@@ -234,7 +236,7 @@ __host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, 
     const bool few = owned <= kFewGroups;
     TeamRule r{kTeamFew, 0u, mode == 0 && few};
     if (alike) {
-        r.below = mode == 0 && mean >= kSliceMean ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
+        r.below = mode == 0 && mean >= kSliceMean && group_log2 <= 14u ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
         r.least = mean >= ranked_mean(mode) ? 2u : mean < kTeamShared ? 0u : few ? 2u : owned <= 8u ? 1u : 0u;
     }
     if (group_log2 > 15u) r.below = 0u;

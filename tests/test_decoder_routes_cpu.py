@@ -32,3 +32,9 @@ def test_ranks_from_a_mean_on(mode, line):
 
 def test_aggregation_over_the_slice_from_a_mean_on():
     assert _route(mean=999) == "four warps by ranks" and _route(mean=1000) == "block over the slice"
+
+
+def test_groups_wider_than_the_slice_stay_with_teams():
+    for mean in (1000, 1500, 1800):
+        assert _route(group_log2=15, mean=mean, words=mean // 2) == "four warps by ranks", mean
+    assert _route(group_log2=15, mean=1000, owned=4) == "four warps"
