@@ -319,15 +319,15 @@ int fastsgd_debug_set_grid(uint32_t blocks) {
 
 int fastsgd_debug_decoder_route(uint32_t mode, uint32_t streams, uint64_t n, uint32_t group_log2, uint32_t owned, uint32_t alike_mean, uint32_t keys, uint32_t words, int bulk) {
     if (mode > 3u || streams < 1u || streams > (uint32_t)kDecMaxStreams) return -1;
-    (void)n; (void)bulk;
+    (void)n;
     if (streams == 1u) {
         if (keys <= warp_max(owned) && group_log2 <= 16u) return mode == 0u && two_in_flight(owned) ? 7 : 0;
     } else {
-        const TeamRule rule = team_rule((int)mode, group_log2, owned, alike_mean != 0u, alike_mean);
+        const TeamRule rule = team_rule((int)mode, group_log2, owned, alike_mean != 0u, alike_mean, bulk != 0);
         const uint32_t team = team_for(rule, group_log2, keys, words);
         if (team < 3u) return team == 2u && !rule.table ? 3 : (int)team;
     }
-    return group_log2 > 14u ? 6 : mode == 0u && keys >= slice_min() ? 5 : 4;
+    return group_log2 > 14u ? 6 : mode == 0u && keys >= slice_min(bulk != 0) ? 5 : 4;
 }
 
 int fastsgd_debug_layout(uint64_t* offsets, uint32_t count) {

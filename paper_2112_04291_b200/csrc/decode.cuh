@@ -51,6 +51,9 @@ constexpr uint32_t kWideListMax    = 1u << 14;      // ... of a group wider than
 // From this many keys on the group's whole slice of dense_out goes through shared memory: scattered over 2048 sectors of 32 bytes
 // they touch a third of it, and a bulk copy moves whole pages (7.5 % of 2^26 entries, one stream: 96 us with, 111 without the slice).
 constexpr uint32_t kTileMinKeys    = 768;
+// ... where no bulk copy moves it, but words (dense_out not 16-byte aligned, or the ragged last group; 2^25 entries, one stream, 800, 1100, 1450 keys a
+// group: entry by entry 57, 59, 65 us, over the slice 89, 88, 89)
+constexpr uint32_t kTileMinWords   = 1536;
 // Several streams whose groups have about as many keys: from this many a group on ranks by bits (four warps) instead of the table of keys, up to as
 // many as aggregation has the slice for.  Eight streams over 2^25 entries, us by table and by ranks (slice), at keys a group:
 //   aggregation  180: 22, 27; 290: 27, 31; 420: 38, 37; 650: 59, 56; 850: 75, 68 (78); 980: 77 by ranks (78); 1310: 94 by ranks (78)
@@ -227,16 +230,18 @@ __host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t w
 // slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a
 // block with one group, those of many keys are for whole blocks, which share them through a queue: teams of several sizes work one after
 // the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
+// bulk: dense_out is aligned for copies of the slice (else, eight streams over 2^25 entries, 1100, 1450, 1800 keys a group: by teams 83, 98, 111 us, by
+// blocks 119, 120, 121).
 // (Groups wider than the slice have no slice: eight streams over 2^25 entries in groups of 2^15, 1050, 1500, 1750 keys a group: by teams 51, 70, 80 us, by
 // blocks 70, 85, 95.)
 // Aggregation by the table in teams of four too where a block's few groups stand side by side: what counts then is the shorter chain (550 groups
 // of 790 keys, four streams: 19.6 us, by ranks 20.8).
 struct TeamRule { uint32_t below, least; bool table; };
-__host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, uint32_t owned, bool alike, uint32_t mean) {
+__host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, uint32_t owned, bool alike, uint32_t mean, bool bulk) {
     const bool few = owned <= kFewGroups;
     TeamRule r{kTeamFew, 0u, mode == 0 && few};
     if (alike) {
-        r.below = mode == 0 && mean >= kSliceMean && group_log2 <= 14u ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
+        r.below = mode == 0 && mean >= kSliceMean && group_log2 <= 14u && bulk ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
         r.least = mean >= ranked_mean(mode) ? 2u : mean < kTeamShared ? 0u : few ? 2u : owned <= 8u ? 1u : 0u;
     }
     if (group_log2 > 15u) r.below = 0u;
@@ -255,7 +260,7 @@ __host__ __device__ constexpr uint32_t warp_max(uint32_t owned) { return owned >
 // ... and whether it keeps two entries a lane in flight when it adds them up, not eight
 __host__ __device__ constexpr bool two_in_flight(uint32_t owned) { return owned > (uint32_t)kDecWarps; }
 // Aggregation by the block: over the group's whole slice of dense_out from this many keys on.
-__host__ __device__ constexpr uint32_t slice_min() { return kTileMinKeys; }
+__host__ __device__ constexpr uint32_t slice_min(bool bulk) { return bulk ? kTileMinKeys : kTileMinWords; }
 
 struct DecShared {
     float              val[kDecMaxStreams][132];
@@ -1048,7 +1053,7 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
     const bool lists = listed <= kBlockListMax && words <= kBlockStageWords;      // (else: stream by stream)
     const bool bulk_ok = ((reinterpret_cast<uintptr_t>(a.dense) & 15u) == 0u) && ((span & 3u) == 0u);
     // aggregation of many keys: the slice of dense_out goes through shared memory as a whole
-    const bool slice = MODE == 0 && (total >= slice_min() || !lists);
+    const bool slice = MODE == 0 && (total >= slice_min(bulk_ok) || !lists);
     if (tid == 0) {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the last write-back has read the tile
         if (slice && bulk_ok) {
@@ -1366,7 +1371,7 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
         if constexpr (!ONE) {
             const uint32_t x = tid < (int)in_batch ? s.gtot[tid] : 0u;
             const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= s.mean && x <= 2u * s.mean);
-            rule = team_rule(MODE, a.group_log2, owned, in_batch > 1u && 4u * alike >= 3u * in_batch, s.mean);
+            rule = team_rule(MODE, a.group_log2, owned, in_batch > 1u && 4u * alike >= 3u * in_batch, s.mean, (reinterpret_cast<uintptr_t>(a.dense) & 15u) == 0u);
         }
         if (tid < (int)in_batch) {
             const uint32_t tot = s.gtot[tid];

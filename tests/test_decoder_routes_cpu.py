@@ -38,3 +38,11 @@ def test_groups_wider_than_the_slice_stay_with_teams():
     for mean in (1000, 1500, 1800):
         assert _route(group_log2=15, mean=mean, words=mean // 2) == "four warps by ranks", mean
     assert _route(group_log2=15, mean=1000, owned=4) == "four warps"
+
+
+def test_no_slice_early_where_it_moves_in_words():
+    for mean in (1000, 1500, 2000):
+        assert _route(mean=mean, bulk=False) == "four warps by ranks", mean
+    for streams in (1, 3):
+        assert _route(streams=streams, owned=7, keys=1535, bulk=False) == "block"
+        assert _route(streams=streams, owned=7, keys=1536, bulk=False) == _route(streams=streams, owned=7, keys=768) == "block over the slice"
