@@ -319,7 +319,6 @@ int fastsgd_debug_set_grid(uint32_t blocks) {
 
 int fastsgd_debug_decoder_route(uint32_t mode, uint32_t streams, uint64_t n, uint32_t group_log2, uint32_t owned, uint32_t alike_mean, uint32_t keys, uint32_t words, int bulk) {
     if (mode > 3u || streams < 1u || streams > (uint32_t)kDecMaxStreams) return -1;
-    (void)n;
     if (streams == 1u) {
         if (keys <= warp_max(owned) && group_log2 <= 16u) return mode == 0u && two_in_flight(owned) ? 7 : 0;
     } else {
@@ -327,7 +326,7 @@ int fastsgd_debug_decoder_route(uint32_t mode, uint32_t streams, uint64_t n, uin
         const uint32_t team = team_for(rule, group_log2, keys, words);
         if (team < 3u) return team == 2u && !rule.table ? 3 : (int)team;
     }
-    return group_log2 > 14u ? 6 : mode == 0u && keys >= slice_min(bulk != 0) ? 5 : 4;
+    return group_log2 > 14u ? 6 : mode == 0u && keys >= slice_min(bulk != 0, streams == 1u, n) ? 5 : 4;
 }
 
 int fastsgd_debug_layout(uint64_t* offsets, uint32_t count) {

@@ -259,8 +259,13 @@ __host__ __device__ constexpr uint32_t team_for(const TeamRule& r, uint32_t grou
 __host__ __device__ constexpr uint32_t warp_max(uint32_t owned) { return owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew; }
 // ... and whether it keeps two entries a lane in flight when it adds them up, not eight
 __host__ __device__ constexpr bool two_in_flight(uint32_t owned) { return owned > (uint32_t)kDecWarps; }
-// Aggregation by the block: over the group's whole slice of dense_out from this many keys on.
-__host__ __device__ constexpr uint32_t slice_min(bool bulk) { return bulk ? kTileMinKeys : kTileMinWords; }
+// Aggregation by the block: over the group's whole slice of dense_out from this many keys on.  One stream (a warp takes up to 1024 keys where the block
+// has 8 groups): what fits the L2 is read there entry by entry, and the slice's 64 KiB both ways are 8 bytes an entry of the vector at 5 TB/s.  us entry by entry
+// and over the slice at 800, 1000, 1250 keys a group: 12 M entries 18.6, 19.4, 20.5 and 23.6, 22.2, 23.2; 16.8 M 29.4, 31.9, 33.7 and 31.6, 31.2,
+// 31.3; 25 M 44.4, 46.3, 47.4 and 42.5, 42.0, 42.3; 36 M 61, 66, 67 and 60, 62, 57.
+__host__ __device__ constexpr uint32_t slice_min(bool bulk, bool one, uint64_t n) {
+    return !bulk ? kTileMinWords : !one || n > 20000000u ? kTileMinKeys : n > 15000000u ? 900u : kTileMinWords;
+}
 
 struct DecShared {
     float              val[kDecMaxStreams][132];
@@ -1053,7 +1058,7 @@ __device__ __forceinline__ void block_group(const DecArgs& a, DecShared& s, uint
     const bool lists = listed <= kBlockListMax && words <= kBlockStageWords;      // (else: stream by stream)
     const bool bulk_ok = ((reinterpret_cast<uintptr_t>(a.dense) & 15u) == 0u) && ((span & 3u) == 0u);
     // aggregation of many keys: the slice of dense_out goes through shared memory as a whole
-    const bool slice = MODE == 0 && (total >= slice_min(bulk_ok) || !lists);
+    const bool slice = MODE == 0 && (total >= slice_min(bulk_ok, ONE, a.n) || !lists);
     if (tid == 0) {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the last write-back has read the tile
         if (slice && bulk_ok) {

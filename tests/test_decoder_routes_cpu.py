@@ -46,3 +46,10 @@ def test_no_slice_early_where_it_moves_in_words():
     for streams in (1, 3):
         assert _route(streams=streams, owned=7, keys=1535, bulk=False) == "block"
         assert _route(streams=streams, owned=7, keys=1536, bulk=False) == _route(streams=streams, owned=7, keys=768) == "block over the slice"
+
+
+def test_one_stream_over_a_vector_that_the_l2_holds():
+    for n, line in ((8_000_000, 1536), (15_000_000, 1536), (15_000_001, 900), (20_000_000, 900), (20_000_001, 768)):
+        assert _route(streams=1, n=n, owned=7, keys=line - 1) == "block", n
+        assert _route(streams=1, n=n, owned=7, keys=line) == "block over the slice", n
+        assert _route(streams=2, n=n, owned=7, keys=768) == "block over the slice", n

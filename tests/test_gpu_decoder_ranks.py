@@ -157,3 +157,15 @@ def test_means_near_the_lines(owned, workers, count):
     assert oracle.sparse_adam_update(streams, n, po, *HYPER, *want) == 0
     for p in (False, True):
         assert _check_update(streams, n, pg, model, want, p) == 0
+
+
+# one stream: entries by the block or over the slice
+@pytest.mark.parametrize("n,group_log2,count,routes", [(1160 << 14, 14, 960, ("block over the slice",)), (13_000_001, 14, 1100, ("block",))])
+def test_one_stream_of_many_groups(n, group_log2, count, routes):
+    streams, po, pg = _streams(n, group_log2, 1, count, count)
+    assert _routes(streams, n, group_log2, 0) == set(routes)
+    binding.ensure_workspace(n, pg)
+    dense0 = np.random.default_rng(count).standard_normal(n).astype(np.float32)
+    want = dense0.copy()
+    assert oracle.decompress_accumulate(streams[0], n, po, want) == 0
+    assert _check_decode(streams, n, po, pg, want, dense0) == 0
