@@ -252,7 +252,7 @@ __host__ __device__ constexpr uint32_t team_for(const TeamRule& r, uint32_t grou
     if (keys >= r.below) return 3u;
     const uint32_t bytes = team_bytes(keys, words), room = kTeamBytes - 2u * kTeamSlots;
     const uint32_t fits = bytes <= room ? 0u : bytes <= 2u * room ? 1u : 2u, team = fits < r.least ? r.least : fits;
-    if (team == 2u && (ranked_bytes(keys, words, group_log2) > 4u * kTeamBytes || bytes > 4u * room)) return 3u;
+    if (team == 2u && (r.table ? bytes > 4u * room : ranked_bytes(keys, words, group_log2) > 4u * kTeamBytes)) return 3u;
     return team;
 }
 // One stream: the most keys of a group that one warp decodes.

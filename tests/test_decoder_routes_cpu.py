@@ -53,3 +53,16 @@ def test_one_stream_over_a_vector_that_the_l2_holds():
         assert _route(streams=1, n=n, owned=7, keys=line - 1) == "block", n
         assert _route(streams=1, n=n, owned=7, keys=line) == "block over the slice", n
         assert _route(streams=2, n=n, owned=7, keys=768) == "block over the slice", n
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
+def test_teams_of_four_take_what_their_memory_holds(mode):
+    # a team's memory: 4 x 6144 bytes.  Ranks: 6 bytes a word of the bit map, 8 an entry, the blobs and 7 words; the table: 8 KiB, 6 bytes an
+    # entry (even numbers of entries in both), the blobs and 3 words
+    for group_log2, words in ((14, 1000), (11, 900), (8, 700)):
+        most = (24576 - 6 * (1 << group_log2) // 32 - 4 * (words + 7)) // 16 * 2
+        by_ranks = dict(mode=mode, group_log2=group_log2, mean=999 if mode == 0 else 1200, words=words)
+        assert _route(keys=most, **by_ranks) == "four warps by ranks" and _route(keys=most + 1, **by_ranks).startswith("block")
+    if mode == 0:
+        most = (24576 - 8192 - 4 * (1000 + 3)) // 12 * 2
+        assert _route(owned=4, mean=999, keys=most, words=1000) == "four warps" and _route(owned=4, mean=999, keys=most + 1, words=1000).startswith("block")
