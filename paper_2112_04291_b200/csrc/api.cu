@@ -322,7 +322,7 @@ int fastsgd_debug_decoder_route(uint32_t mode, uint32_t streams, uint64_t n, uin
     if (streams == 1u) {
         if (keys <= warp_max(owned) && group_log2 <= 16u) return mode == 0u && two_in_flight(owned) ? 7 : 0;
     } else {
-        const TeamRule rule = team_rule((int)mode, group_log2, owned, alike_mean != 0u, alike_mean, bulk != 0);
+        const TeamRule rule = team_rule((int)mode, group_log2, owned, alike_mean != 0u, alike_mean, bulk != 0, streams);
         const uint32_t team = team_for(rule, group_log2, keys, words);
         if (team < 3u) return team == 2u && !rule.table ? 3 : (int)team;
     }

@@ -230,18 +230,22 @@ __host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t w
 // slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a
 // block with one group, those of many keys are for whole blocks, which share them through a queue: teams of several sizes work one after
 // the other, and nobody helps a block that has many (four streams of 25.6 M: 33 to 42 us, so 24).
-// bulk: dense_out is aligned for copies of the slice (else, eight streams over 2^25 entries, 1100, 1450, 1800 keys a group: by teams 83, 98, 111 us, by
+// bulk: dense_out (the update: theta, m and v) is 16-byte aligned, as the slice wants it (else, eight streams over 2^25 entries, 1100, 1450, 1800 keys a group: by teams 83, 98, 111 us, by
 // blocks 119, 120, 121).
+// The update goes over the slice of g (sweep_all) from a mean on that grows with the streams, whose lists the block adds up one after the other (2^25 entries;
+// us by ranks and over the slice at 1200, 1600, 2000 keys a group: two streams 157, 172, 181 and 164, 165, 167; four 155, 166, 176 and 168, 170,
+// 174; eight 161, 172, 182 and 182, 184, 188, 2050 keys 212 and 189).
 // (Groups wider than the slice have no slice: eight streams over 2^25 entries in groups of 2^15, 1050, 1500, 1750 keys a group: by teams 51, 70, 80 us, by
 // blocks 70, 85, 95.)
 // Aggregation by the table in teams of four too where a block's few groups stand side by side: what counts then is the shorter chain (550 groups
 // of 790 keys, four streams: 19.6 us, by ranks 20.8).
 struct TeamRule { uint32_t below, least; bool table; };
-__host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, uint32_t owned, bool alike, uint32_t mean, bool bulk) {
+__host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, uint32_t owned, bool alike, uint32_t mean, bool bulk, uint32_t W) {
     const bool few = owned <= kFewGroups;
     TeamRule r{kTeamFew, 0u, mode == 0 && few};
     if (alike) {
-        r.below = mode == 0 && mean >= kSliceMean && group_log2 <= 14u && bulk ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
+        const uint32_t slice = mode == 0 ? kSliceMean : mode == 2 ? (W < 5u ? 1000u + 200u * W : 2000u) : 0xFFFFFFFFu;
+        r.below = mean >= slice && group_log2 <= 14u && bulk ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
         r.least = mean >= ranked_mean(mode) ? 2u : mean < kTeamShared ? 0u : few ? 2u : owned <= 8u ? 1u : 0u;
     }
     if (group_log2 > 15u) r.below = 0u;
@@ -1376,7 +1380,9 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
         if constexpr (!ONE) {
             const uint32_t x = tid < (int)in_batch ? s.gtot[tid] : 0u;
             const uint32_t alike = (uint32_t)__syncthreads_count(x != 0u && 2u * x >= s.mean && x <= 2u * s.mean);
-            rule = team_rule(MODE, a.group_log2, owned, in_batch > 1u && 4u * alike >= 3u * in_batch, s.mean, (reinterpret_cast<uintptr_t>(a.dense) & 15u) == 0u);
+            const uintptr_t at = MODE == 2 ? reinterpret_cast<uintptr_t>(a.theta) | reinterpret_cast<uintptr_t>(a.m) | reinterpret_cast<uintptr_t>(a.v)
+                                           : reinterpret_cast<uintptr_t>(a.dense);
+            rule = team_rule(MODE, a.group_log2, owned, in_batch > 1u && 4u * alike >= 3u * in_batch, s.mean, (at & 15u) == 0u, W);
         }
         if (tid < (int)in_batch) {
             const uint32_t tot = s.gtot[tid];

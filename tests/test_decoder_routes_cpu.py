@@ -66,3 +66,10 @@ def test_teams_of_four_take_what_their_memory_holds(mode):
     if mode == 0:
         most = (24576 - 8192 - 4 * (1000 + 3)) // 12 * 2
         assert _route(owned=4, mean=999, keys=most, words=1000) == "four warps" and _route(owned=4, mean=999, keys=most + 1, words=1000).startswith("block")
+
+
+def test_update_over_the_slice_of_g_from_a_mean_on():
+    for streams, line in ((2, 1400), (3, 1600), (4, 1800), (5, 2000), (8, 2000)):
+        assert _route(2, streams, mean=line - 1, words=900) == "four warps by ranks" and _route(2, streams, mean=line, words=900) == "block", streams
+        assert _route(2, streams, mean=line, words=900, bulk=False) == _route(3, streams, mean=line, words=900) == "four warps by ranks", streams
+    assert _route(2, 2, group_log2=15, mean=1500, words=900) == "four warps by ranks"

@@ -142,7 +142,7 @@ def test_ranks(owned, workers, count, group_log2, modes, shift):
 
 # about as many keys a group as where another way of decoding begins: more groups to a block than teams of four take side by side, and as many
 @pytest.mark.parametrize("owned", [3, 6])
-@pytest.mark.parametrize("workers,count", [(8, 27), (4, 64), (8, 45), (3, 140), (5, 199), (2, 580)])
+@pytest.mark.parametrize("workers,count", [(8, 27), (4, 64), (8, 45), (3, 140), (5, 199), (2, 580), (2, 900)])
 def test_means_near_the_lines(owned, workers, count):
     n = owned * _blocks() * 2048 - 5
     streams, po, pg = _streams(n, 11, workers, count, count)
