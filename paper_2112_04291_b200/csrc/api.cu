@@ -320,7 +320,7 @@ int fastsgd_debug_set_grid(uint32_t blocks) {
 int fastsgd_debug_decoder_route(uint32_t mode, uint32_t streams, uint64_t n, uint32_t group_log2, uint32_t owned, uint32_t alike_mean, uint32_t keys, uint32_t words, int bulk) {
     if (mode > 3u || streams < 1u || streams > (uint32_t)kDecMaxStreams) return -1;
     if (streams == 1u) {
-        if (keys <= warp_max(owned) && group_log2 <= 16u) return mode == 0u && two_in_flight(owned) ? 7 : 0;
+        if (keys <= warp_max(owned) && group_log2 <= 16u) return mode == 0u && two_in_flight(owned, n) && sparse_group(keys, 1u << group_log2) ? 7 : 0;
     } else {
         const TeamRule rule = team_rule((int)mode, group_log2, owned, alike_mean != 0u, alike_mean, bulk != 0, streams);
         const uint32_t team = team_for(rule, group_log2, keys, words);

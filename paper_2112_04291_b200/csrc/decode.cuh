@@ -66,6 +66,7 @@ constexpr uint32_t kFewGroups      = 4;       // groups of a block that teams of
 // (eight streams, 5 % of 2^24 entries: 292 -> 125 us); on the packed state, where a key is one access anyway, later (235 -> 132 us).
 constexpr uint32_t kSweepMinKeys   = 768;
 constexpr uint32_t kSweepMinPacked = 2048;
+constexpr uint64_t kL2Entries      = 1u << 25;      // entries of dense_out that fill the L2
 constexpr uint32_t kDecSpinLimit   = 1u << 20;
 
 struct DecArgs {
@@ -261,8 +262,13 @@ __host__ __device__ constexpr uint32_t team_for(const TeamRule& r, uint32_t grou
 }
 // One stream: the most keys of a group that one warp decodes.
 __host__ __device__ constexpr uint32_t warp_max(uint32_t owned) { return owned >= (uint32_t)kDecWarps / 2u ? kDecWarpMax : kDecWarpFew; }
-// ... and whether it keeps two entries a lane in flight when it adds them up, not eight
-__host__ __device__ constexpr bool two_in_flight(uint32_t owned) { return owned > (uint32_t)kDecWarps; }
+// ... and whether it keeps two entries a lane in flight when it adds them up, not eight.  Where every warp has several groups, entries are further apart than
+// a line and dense_out is more than the L2 holds, memory is the bound, and more in flight only make it switch between reading and writing
+// more often (a bare kernel that updates 2.7 M floats at ascending random places of 1 GiB, a group a warp: eight a lane 113 us, four 107, two 101, and 8 us
+// more with whole lines fetched; 268 M entries, 1 % kept: 131.5, now 121).  Else it is the latency.  us with two and with eight at keys a group: groups of
+// 2^14, 140 M entries 400: 120, 121; 600: 153, 150; 900: 185, 183; of 2^12, 20 M entries 900: 52.5, 47.1; of 2^10, 6 M 400: 17.4, 15.8.
+__host__ __device__ constexpr bool two_in_flight(uint32_t owned, uint64_t n) { return owned > (uint32_t)kDecWarps && n > kL2Entries; }
+__host__ __device__ constexpr bool sparse_group(uint32_t keys, uint32_t span) { return 32u * keys < span; }
 // Aggregation by the block: over the group's whole slice of dense_out from this many keys on.  One stream (a warp takes up to 1024 keys where the block
 // has 8 groups): what fits the L2 is read there entry by entry, and the slice's 64 KiB both ways are 8 bytes an entry of the vector at 5 TB/s.  us entry by entry
 // and over the slice at 800, 1000, 1250 keys a group: 12 M entries 18.6, 19.4, 20.5 and 23.6, 22.2, 23.2; 16.8 M 29.4, 31.9, 33.7 and 31.6, 31.2,
@@ -529,12 +535,9 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
                     if (kk[i] != 0xFFFFFFFFu) a.dense[kk[i]] = __fadd_rn(x[i], code_value(s.val[0], code_at<true>(b, e0 + 32u * i + lane)));
             }
         };
-        // Where every warp has several groups, memory is the bound, and more in flight only make it switch between reading and writing more
-        // often (a bare kernel that updates 2.7 M floats at ascending random places of 1 GiB, a group a warp: eight a lane 113 us, four 107,
-        // two 101, and 8 us more with whole lines fetched; 268 M entries, 1 % kept: 131.5, now 122); else it is the latency.
         struct Two { uint32_t x[2]; };
         struct Eight { uint32_t x[8]; };
-        if (two) add(Two()); else add(Eight());
+        if (two && sparse_group(c0, span)) add(Two()); else add(Eight());
     } else {
         for (uint32_t e0 = 0; e0 < c0; e0 += 128u) {
             uint32_t kk[4]; float gg[4];
@@ -1433,7 +1436,7 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                 x = __shfl_sync(kFullMask, x, 0);
                 if (x >= n_light) break;
                 const uint32_t i = s.light[x];
-                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, two_in_flight(owned), lane, warp);
+                warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, two_in_flight(owned, a.n), lane, warp);
             }
         } else {
             if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp, MODE == 0 && owned <= kFewGroups); __syncthreads(); }

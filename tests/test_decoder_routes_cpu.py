@@ -73,3 +73,12 @@ def test_update_over_the_slice_of_g_from_a_mean_on():
         assert _route(2, streams, mean=line - 1, words=900) == "four warps by ranks" and _route(2, streams, mean=line, words=900) == "block", streams
         assert _route(2, streams, mean=line, words=900, bulk=False) == _route(3, streams, mean=line, words=900) == "four warps by ranks", streams
     assert _route(2, 2, group_log2=15, mean=1500, words=900) == "four warps by ranks"
+
+
+def test_two_entries_a_lane_in_flight_only_where_memory_is_the_bound():
+    two = "warp, two in flight"
+    assert _route(streams=1, n=1 << 28, owned=55, keys=164) == two
+    assert _route(streams=1, n=1 << 28, owned=55, keys=511) == two and _route(streams=1, n=1 << 28, owned=55, keys=512) == "warp"
+    assert _route(streams=1, n=(1 << 25) + 1, group_log2=12, owned=28, keys=100) == two
+    assert _route(streams=1, n=1 << 25, group_log2=12, owned=28, keys=100) == "warp"
+    assert _route(streams=1, n=1 << 26, owned=16, keys=100) == "warp"

@@ -160,8 +160,11 @@ def test_means_near_the_lines(owned, workers, count):
         assert _check_update(streams, n, pg, model, want, p) == 0
 
 
-# one stream: entries by the block or over the slice
-@pytest.mark.parametrize("n,group_log2,count,routes", [(1160 << 14, 14, 960, ("block over the slice",)), (13_000_001, 14, 1100, ("block",))])
+# one stream: entries by the block or over the slice; by warps with two entries in flight or eight
+@pytest.mark.parametrize("n,group_log2,count,routes", [(1160 << 14, 14, 960, ("block over the slice",)),
+                                                        (13_000_001, 14, 1100, ("block",)),
+                                                        (45_000_001, 13, 150, ("warp, two in flight",)),
+                                                        (45_000_001, 13, 250, ("warp", "warp, two in flight"))])
 def test_one_stream_of_many_groups(n, group_log2, count, routes):
     streams, po, pg = _streams(n, group_log2, 1, count, count)
     assert _routes(streams, n, group_log2, 0) == set(routes)
