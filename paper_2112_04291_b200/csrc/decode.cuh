@@ -226,7 +226,8 @@ __host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t w
 }
 
 // Who decodes the groups of several streams (mode as below): those of fewer than `below` keys teams of at least `least` (0, 1, 2: one, two, four
-// warps), the others the block.  table: teams of four by the table of keys, not by ranks.
+// warps), the others the block.  table: teams of four by the table of keys, not by ranks.  two: there are teams of two (not in the update in one launch: four
+// streams of 230 keys a group over 20 M and 33 M entries 55 and 82 us, by ranks 49 and 71).
 // Where most of a block's groups have about as many keys (alike), they all go to teams (of the same size: ranked_mean), up to as many keys as the
 // slice is for (kSliceMean); with few groups to a block to larger teams, so that its warps have work.  Else (layers of different scales) and in a
 // block with one group, those of many keys are for whole blocks, which share them through a queue: teams of several sizes work one after
@@ -240,14 +241,14 @@ __host__ __device__ constexpr uint32_t ranked_bytes(uint32_t entries, uint32_t w
 // blocks 70, 85, 95.)
 // Aggregation by the table in teams of four too where a block's few groups stand side by side: what counts then is the shorter chain (550 groups
 // of 790 keys, four streams: 19.6 us, by ranks 20.8).
-struct TeamRule { uint32_t below, least; bool table; };
+struct TeamRule { uint32_t below, least; bool table, two; };
 __host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, uint32_t owned, bool alike, uint32_t mean, bool bulk, uint32_t W) {
     const bool few = owned <= kFewGroups;
-    TeamRule r{kTeamFew, 0u, mode == 0 && few};
+    TeamRule r{kTeamFew, 0u, mode == 0 && few, mode != 2};
     if (alike) {
         const uint32_t slice = mode == 0 ? kSliceMean : mode == 2 ? (W < 5u ? 1000u + 200u * W : 2000u) : 0xFFFFFFFFu;
         r.below = mean >= slice && group_log2 <= 14u && bulk ? kTeamFew : 0xFFFFFFFFu;      // (as many as the memory of four warps holds)
-        r.least = mean >= ranked_mean(mode) ? 2u : mean < kTeamShared ? 0u : few ? 2u : owned <= 8u ? 1u : 0u;
+        r.least = mean >= ranked_mean(mode) ? 2u : mean < kTeamShared ? 0u : few ? 2u : owned <= 8u ? (r.two ? 1u : 2u) : 0u;
     }
     if (group_log2 > 15u) r.below = 0u;
     return r;
@@ -256,7 +257,7 @@ __host__ __device__ constexpr TeamRule team_rule(int mode, uint32_t group_log2, 
 __host__ __device__ constexpr uint32_t team_for(const TeamRule& r, uint32_t group_log2, uint32_t keys, uint32_t words) {
     if (keys >= r.below) return 3u;
     const uint32_t bytes = team_bytes(keys, words), room = kTeamBytes - 2u * kTeamSlots;
-    const uint32_t fits = bytes <= room ? 0u : bytes <= 2u * room ? 1u : 2u, team = fits < r.least ? r.least : fits;
+    const uint32_t fits = bytes <= room ? 0u : bytes <= 2u * room && r.two ? 1u : 2u, team = fits < r.least ? r.least : fits;
     if (team == 2u && (r.table ? bytes > 4u * room : ranked_bytes(keys, words, group_log2) > 4u * kTeamBytes)) return 3u;
     return team;
 }
@@ -1439,9 +1440,16 @@ k_decode_accumulate(const __grid_constant__ DecArgs a, const __grid_constant__ P
                 warp_group<MODE>(a, s, blockIdx.x + (first + i) * B, i, two_in_flight(owned, a.n), lane, warp);
             }
         } else {
-            if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp, MODE == 0 && owned <= kFewGroups); __syncthreads(); }
-            if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, lane, warp); __syncthreads(); }
-            team_groups<MODE, 1>(a, s, W, first, lane, warp);
+            // (The update in one launch takes the single warps' first: the compiler then spills less; four streams of 25.6 M entries 51.4 us, so 50.4, of
+            // 5 M 16.8 and 16.4.  The others are quicker with the long ones in front: packed 216 us, else 220.)
+            if constexpr (MODE == 2) {
+                team_groups<MODE, 1>(a, s, W, first, lane, warp);
+                if (s.n_light[2]) { __syncthreads(); team_groups<MODE, 4>(a, s, W, first, lane, warp); }
+            } else {
+                if (s.n_light[2]) { team_groups<MODE, 4>(a, s, W, first, lane, warp, MODE == 0 && owned <= kFewGroups); __syncthreads(); }
+                if (s.n_light[1]) { team_groups<MODE, 2>(a, s, W, first, lane, warp); __syncthreads(); }
+                team_groups<MODE, 1>(a, s, W, first, lane, warp);
+            }
         }
     }
 

@@ -27,7 +27,7 @@ def test_groups_of_few_keys_go_to_a_warp_and_unlike_large_ones_to_the_block(mode
 def test_ranks_from_a_mean_on(mode, line):
     assert _route(mode, mean=line) == "four warps by ranks" and _route(mode, mean=line - 1) == "warp"
     assert _route(mode, mean=line, owned=4) == ("four warps" if mode == 0 else "four warps by ranks")
-    assert _route(mode, mean=line - 1, owned=8) == "two warps"
+    assert _route(mode, mean=line - 1, owned=8) == ("two warps" if mode != 2 else "four warps by ranks")
 
 
 def test_aggregation_over_the_slice_from_a_mean_on():
@@ -82,3 +82,9 @@ def test_two_entries_a_lane_in_flight_only_where_memory_is_the_bound():
     assert _route(streams=1, n=(1 << 25) + 1, group_log2=12, owned=28, keys=100) == two
     assert _route(streams=1, n=1 << 25, group_log2=12, owned=28, keys=100) == "warp"
     assert _route(streams=1, n=1 << 26, owned=16, keys=100) == "warp"
+
+
+def test_no_teams_of_two_in_the_update_in_one_launch():
+    for owned, mean in ((8, 200), (8, 255), (13, 150)):
+        assert _route(2, owned=owned, mean=mean, keys=2 * mean, words=900 if owned == 13 else 100) == "four warps by ranks", owned
+        assert _route(3, owned=owned, mean=mean, keys=2 * mean, words=900 if owned == 13 else 100) == "two warps", owned

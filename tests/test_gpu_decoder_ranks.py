@@ -102,6 +102,7 @@ def _check_update(streams, n, pg, model, want, packed):
     (5, 10, 66, 11, (0, 1), 0),               # ten streams: eight of 560 keys, and two
     (5, 3, 400, 15, (0,), 0),                 # 1200 of 2^15: no slice to go over
     (5, 4, 330, 13, (0,), 2),                 # 1320, where the slice is not aligned
+    (6, 8, 22, 11, (2,), 0),                  # 215, the update
     (5, 8, 300, 11, (3,), 0),                 # 2200: as many as the memory holds
 ])
 def test_ranks(owned, workers, count, group_log2, modes, shift):
