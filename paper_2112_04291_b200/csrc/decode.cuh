@@ -556,68 +556,59 @@ __device__ __forceinline__ void warp_group(const DecArgs& a, DecShared& s, uint3
     __syncwarp();                                                       // (the list is rewritten by the warp's next group)
 }
 
-// Several streams: one group by a team of NW warps (1, 2 or 4); entries eb + w of the block's table are stream w's directory entry.  One
-// entry stands for every distinct key; it collects the streams' values in stream order, so that each coordinate takes one round
-// trip to memory.  keys: a key, or kSharedKey | the entry that stands for it.
-//
-// A group is a chain of about ten steps (copy, flags, deltas, table, one addition a stream, memory) of which few fill a block's 512
-// threads.  Groups of 250 to 1500 keys by the whole block took 10 us each, two at a time on an SM; by teams (32, 16 or 8 groups
-// at a time) eight streams of 47 keys a group take 51 us instead of 100 (2781 groups), of 98 keys 104 instead of 136.
-constexpr uint32_t kSharedKey = 0x8000u;
 template <int NW> __device__ __forceinline__ void dec_team_sync(int team) {
     if constexpr (NW == 1) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(32 * NW) : "memory");
 }
-template <int MODE, int NW>
-__device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t eb, int lane, int warp) {
-    const uint64_t lo64 = (uint64_t)g << a.group_log2;
-    const uint64_t hi64 = lo64 + (1ull << a.group_log2);
-    const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
+// Lane w: stream w's directory entry in the block's table (entries eb + w), and where its blob and its list begin among the group's.
+struct TeamEntries {
+    uint32_t count, M, off, nw, wbase, lbase, words, total;
+    __device__ __forceinline__ TeamEntries(const DecShared& s, uint32_t W, uint32_t eb, int lane) {
+        uint32_t cm = 0u;
+        off = nw = 0u;
+        if (lane < (int)W) { cm = s.e_cm[eb + lane]; off = s.e_off[eb + lane]; nw = s.e_nw[eb + lane]; }
+        count = cm & 0xFFFFFFu; M = cm >> 24;
+        const uint32_t wincl = warp_incl_scan(nw, lane), lincl = warp_incl_scan(count, lane);
+        wbase = wincl - nw; lbase = lincl - count;
+        words = __shfl_sync(kFullMask, wincl, 31); total = __shfl_sync(kFullMask, lincl, 31);
+    }
+};
+
+// The streams' blobs into shared memory and parsed into lists of keys, side by side, by a team of NW warps (tl: thread of the team).  prepare(): what
+// else is to be done before the first barrier, while the copies are in flight; each(k): every key as it is found.  Returns the streams that failed (bit w).
+template <int NW, typename P, typename E>
+__device__ __forceinline__ uint32_t team_lists(const DecArgs& a, DecShared& s, const TeamEntries& q, uint32_t W, uint32_t g, uint32_t span, uint32_t* blob,
+                                               uint16_t* lists, uint32_t tl, int lane, int warp, P prepare, E each) {
+    constexpr uint32_t threads = 32u * NW, nw_log2 = NW == 1 ? 0u : NW == 2 ? 1u : 2u;
     const int team = warp / NW;
-    const uint32_t tl = 32u * (uint32_t)(warp % NW) + (uint32_t)lane;   // thread of the team
-    constexpr uint32_t threads = 32u * NW;
-    // lane w: stream w
-    uint32_t cm = 0u, off = 0u, nw = 0u;
-    if (lane < (int)W) { cm = s.e_cm[eb + lane]; off = s.e_off[eb + lane]; nw = s.e_nw[eb + lane]; }
-    uint32_t count = cm & 0xFFFFFFu;
-    const uint32_t M = cm >> 24, wincl = warp_incl_scan(nw, lane), wbase = wincl - nw, lincl = warp_incl_scan(count, lane), lbase = lincl - count;
-    const uint32_t words = __shfl_sync(kFullMask, wincl, 31), total = __shfl_sync(kFullMask, lincl, 31);
-    uint8_t* mem = s.u.team[team * NW];
-    uint16_t* slot = reinterpret_cast<uint16_t*>(mem);                  // table of distinct keys: the entry that stands for the key; 0xFFFF: free
-    // (four times the entries as far as the memory's share goes; never less than 1.5 times)
-    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
-    float* acc = reinterpret_cast<float*>(slot + kTeamSlots * NW);
-    uint16_t* keys = reinterpret_cast<uint16_t*>(acc + ((total + 1u) & ~1u));
-    uint32_t* blob = reinterpret_cast<uint32_t*>(keys + ((total + 1u) & ~1u));
-    uint32_t* failed = blob + words + 2u;                               // bit w: stream w
-    // ---- the streams' blobs into shared memory, all copies in flight together
-    for (uint32_t w = 0; w < W; ++w) {
-        const uint32_t n_w = __shfl_sync(kFullMask, nw, w), o_w = __shfl_sync(kFullMask, off, w), b_w = __shfl_sync(kFullMask, wbase, w);
+    uint32_t* failed = blob + q.words + 2u;                             // bit w: stream w
+    for (uint32_t w = 0; w < W; ++w) {                                  // all copies in flight together
+        const uint32_t n_w = __shfl_sync(kFullMask, q.nw, w), o_w = __shfl_sync(kFullMask, q.off, w), b_w = __shfl_sync(kFullMask, q.wbase, w);
         const uint32_t* src = reinterpret_cast<const uint32_t*>(a.stream[w]) + o_w;
         for (uint32_t i = tl; i < n_w; i += threads) copy_word_async(&blob[b_w + i], src + i);
     }
-    for (uint32_t i = tl; i < slots / 2u; i += threads) reinterpret_cast<uint32_t*>(slot)[i] = 0xFFFFFFFFu;
+    prepare();
     if (NW > 1 && tl == 0u) *failed = 0u;
     copies_wait();
     dec_team_sync<NW>(team);
-    for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
+    for (uint32_t i = tl; i < q.words; i += threads) blob[i] = bswap32(blob[i]);
     dec_team_sync<NW>(team);
     // ---- parse: the threads shared out among the streams, within a warp
-    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), tn = 1u << tn_log2;
-    const uint32_t mine = tl >> tn_log2;                            // (beyond W - 1: a stream without keys)
+    const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + nw_log2), tn = 1u << tn_log2;
+    const uint32_t mine = tl >> tn_log2;                                // (beyond W - 1: a stream without keys)
     Blob b;
-    b.count = __shfl_sync(kFullMask, count, mine);
-    b.nwords = __shfl_sync(kFullMask, nw, mine);
-    b.M = __shfl_sync(kFullMask, M, mine);
-    b.words = blob + __shfl_sync(kFullMask, wbase, mine);
-    const uint32_t list = __shfl_sync(kFullMask, lbase, mine);
+    b.count = __shfl_sync(kFullMask, q.count, mine);
+    b.nwords = __shfl_sync(kFullMask, q.nw, mine);
+    b.M = __shfl_sync(kFullMask, q.M, mine);
+    b.words = blob + __shfl_sync(kFullMask, q.wbase, mine);
+    uint16_t* keys = lists + __shfl_sync(kFullMask, q.lbase, mine);
     const uint32_t most = __reduce_max_sync(kFullMask, b.count);
     const bool small = most <= 4u * tn;
     const unsigned long long bad = parse_team<false, true>(a, s, b, span, (uint32_t)lane & (tn - 1u), tn, small, small ? 1u : (most + 8u * tn - 1u) / (8u * tn),
                                                            lane, warp, [&](uint32_t j, int m, const auto& v) {
         constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
 #pragma unroll
-        for (int k = 0; k < K; ++k) if (k < m) keys[list + j + (uint32_t)k] = (uint16_t)v[k];
+        for (int k = 0; k < K; ++k) if (k < m) { keys[j + (uint32_t)k] = (uint16_t)v[k]; each(v[k]); }
     });
     if (bad != ~0ull) {
         dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
@@ -631,9 +622,40 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
         dec_team_sync<NW>(team);
         out = *failed;
     }
+    return out;
+}
+
+// Several streams: one group by a team of NW warps (1, 2 or 4); entries eb + w of the block's table are stream w's directory entry.  One
+// entry stands for every distinct key; it collects the streams' values in stream order, so that each coordinate takes one round
+// trip to memory.  keys: a key, or kSharedKey | the entry that stands for it.
+//
+// A group is a chain of about ten steps (copy, flags, deltas, table, one addition a stream, memory) of which few fill a block's 512
+// threads.  Groups of 250 to 1500 keys by the whole block took 10 us each, two at a time on an SM; by teams (32, 16 or 8 groups
+// at a time) eight streams of 47 keys a group take 51 us instead of 100 (2781 groups), of 98 keys 104 instead of 136.
+constexpr uint32_t kSharedKey = 0x8000u;
+template <int MODE, int NW>
+__device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint32_t W, uint32_t g, uint32_t eb, int lane, int warp) {
+    const uint64_t lo64 = (uint64_t)g << a.group_log2;
+    const uint64_t hi64 = lo64 + (1ull << a.group_log2);
+    const uint32_t lo = (uint32_t)lo64, span = (uint32_t)((hi64 < a.n ? hi64 : a.n) - lo64);
+    const int team = warp / NW;
+    const uint32_t tl = 32u * (uint32_t)(warp % NW) + (uint32_t)lane;   // thread of the team
+    constexpr uint32_t threads = 32u * NW;
+    const TeamEntries q(s, W, eb, lane);
+    const uint32_t total = q.total;
+    uint32_t count = q.count;
+    uint8_t* mem = s.u.team[team * NW];
+    uint16_t* slot = reinterpret_cast<uint16_t*>(mem);                  // table of distinct keys: the entry that stands for the key; 0xFFFF: free
+    // (four times the entries as far as the memory's share goes; never less than 1.5 times)
+    const uint32_t slots_log2 = min(32u - (uint32_t)__clz((int)(4u * total + 31u)), kTeamSlotsLog2 + (NW == 1 ? 0u : NW == 2 ? 1u : 2u)), slots = 1u << slots_log2;
+    float* acc = reinterpret_cast<float*>(slot + kTeamSlots * NW);
+    uint16_t* keys = reinterpret_cast<uint16_t*>(acc + ((total + 1u) & ~1u));
+    uint32_t* blob = reinterpret_cast<uint32_t*>(keys + ((total + 1u) & ~1u));
+    const uint32_t out = team_lists<NW>(a, s, q, W, g, span, blob, keys, tl, lane, warp,
+        [&]() { for (uint32_t i = tl; i < slots / 2u; i += threads) reinterpret_cast<uint32_t*>(slot)[i] = 0xFFFFFFFFu; }, [](uint32_t) {});
     if (out) {                                                          // a failed stream is left out as a whole
         for (uint32_t w = 0; w < W; ++w) {
-            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w);
+            const uint32_t b_w = __shfl_sync(kFullMask, q.lbase, w), c_w = __shfl_sync(kFullMask, count, w);
             if ((out >> w) & 1u) for (uint32_t j = tl; j < c_w; j += threads) keys[b_w + j] = kNoKey;
         }
         if ((out >> lane) & 1u) count = 0u;
@@ -677,7 +699,7 @@ __device__ __forceinline__ void team_group(const DecArgs& a, DecShared& s, uint3
     dec_team_sync<NW>(team);
     if constexpr (MODE != 1) {
         for (uint32_t w = 0; w < W; ++w) {
-            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, wbase, w);
+            const uint32_t b_w = __shfl_sync(kFullMask, q.lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, q.wbase, w);
             const uint8_t* codes = reinterpret_cast<const uint8_t*>(blob + s_w);
             for (uint32_t j = tl; j < c_w; j += threads) {
                 const uint32_t k = keys[b_w + j], at = k & kSharedKey ? k & (kSharedKey - 1u) : b_w + j;
@@ -714,12 +736,9 @@ __device__ __forceinline__ void ranked_group(const DecArgs& a, DecShared& s, uin
     constexpr uint32_t threads = 128u;
     const int team = warp / 4;
     const uint32_t tl = 32u * (uint32_t)(warp % 4) + (uint32_t)lane;    // thread of the team
-    // lane w: stream w
-    uint32_t cm = 0u, off = 0u, nw = 0u;
-    if (lane < (int)W) { cm = s.e_cm[eb + lane]; off = s.e_off[eb + lane]; nw = s.e_nw[eb + lane]; }
-    uint32_t count = cm & 0xFFFFFFu;
-    const uint32_t M = cm >> 24, wincl = warp_incl_scan(nw, lane), wbase = wincl - nw, lincl = warp_incl_scan(count, lane), lbase = lincl - count;
-    const uint32_t words = __shfl_sync(kFullMask, wincl, 31), total = __shfl_sync(kFullMask, lincl, 31), even = (total + 1u) & ~1u;
+    const TeamEntries q(s, W, eb, lane);
+    const uint32_t total = q.total, even = (total + 1u) & ~1u;
+    uint32_t count = q.count;
     const uint32_t map_words = (1u << a.group_log2) / 32u;
     uint32_t* bits = reinterpret_cast<uint32_t*>(s.u.team[team * 4]);
     uint16_t* before = reinterpret_cast<uint16_t*>(bits + map_words);   // bits set in the words before
@@ -727,53 +746,16 @@ __device__ __forceinline__ void ranked_group(const DecArgs& a, DecShared& s, uin
     uint16_t* key_of = reinterpret_cast<uint16_t*>(acc + even);         // ... and the key
     uint16_t* list = key_of + even;                                     // the streams' keys, then their ranks
     uint32_t* blob = reinterpret_cast<uint32_t*>(list + even);
-    uint32_t* failed = blob + words + 2u;                               // bit w: stream w
-    uint32_t* sums = failed + 1;                                        // bits set in the words of each warp
-    // ---- the streams' blobs into shared memory, all copies in flight together
-    for (uint32_t w = 0; w < W; ++w) {
-        const uint32_t n_w = __shfl_sync(kFullMask, nw, w), o_w = __shfl_sync(kFullMask, off, w), b_w = __shfl_sync(kFullMask, wbase, w);
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(a.stream[w]) + o_w;
-        for (uint32_t i = tl; i < n_w; i += threads) copy_word_async(&blob[b_w + i], src + i);
-    }
+    uint32_t* sums = blob + q.words + 3u;                               // (behind the failed streams' bits) bits set in the words of each warp
     auto clear = [&]() { for (uint32_t i = tl; i < map_words / 4u; i += threads) reinterpret_cast<uint4*>(bits)[i] = make_uint4(0u, 0u, 0u, 0u); };
-    clear();
-    if (tl == 0u) *failed = 0u;
-    copies_wait();
-    dec_team_sync<4>(team);
-    for (uint32_t i = tl; i < words; i += threads) blob[i] = bswap32(blob[i]);
-    dec_team_sync<4>(team);
-    // ---- parse: the threads shared out among the streams, within a warp
     auto mark = [&](uint32_t k) { if (k < span) atomicOr(&bits[k >> 5], 1u << (k & 31u)); };      // (beyond: the stream fails)
-    {
-        const uint32_t tn_log2 = min(5u, (W <= 2u ? 4u : (W <= 4u ? 3u : 2u)) + 2u), tn = 1u << tn_log2;
-        const uint32_t mine = tl >> tn_log2;                            // (beyond W - 1: a stream without keys)
-        Blob b;
-        b.count = __shfl_sync(kFullMask, count, mine);
-        b.nwords = __shfl_sync(kFullMask, nw, mine);
-        b.M = __shfl_sync(kFullMask, M, mine);
-        b.words = blob + __shfl_sync(kFullMask, wbase, mine);
-        uint16_t* keys = list + __shfl_sync(kFullMask, lbase, mine);
-        const uint32_t most = __reduce_max_sync(kFullMask, b.count);
-        const bool small = most <= 4u * tn;
-        const unsigned long long bad = parse_team<false, true>(a, s, b, span, (uint32_t)lane & (tn - 1u), tn, small, small ? 1u : (most + 8u * tn - 1u) / (8u * tn),
-                                                               lane, warp, [&](uint32_t j, int m, const auto& v) {
-            constexpr int K = (int)(sizeof(v) / sizeof(v[0]));
-#pragma unroll
-            for (int k = 0; k < K; ++k) if (k < m) { keys[j + (uint32_t)k] = (uint16_t)v[k]; mark(v[k]); }
-        });
-        if (bad != ~0ull) {
-            dec_fail(a, g, (uint32_t)(bad >> 8), (int)(bad & 0xFFull));
-            atomicOr(failed, 1u << mine);
-        }
-    }
-    dec_team_sync<4>(team);
-    const uint32_t out = *failed;                                       // a failed stream is left out as a whole
-    if (out) {                                                          // the others' keys again
+    const uint32_t out = team_lists<4>(a, s, q, W, g, span, blob, list, tl, lane, warp, clear, mark);
+    if (out) {                                                          // a failed stream is left out as a whole: the others' keys again
         clear();
         if ((out >> lane) & 1u) count = 0u;
         dec_team_sync<4>(team);
         for (uint32_t w = 0; w < W; ++w) {
-            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, cm & 0xFFFFFFu, w);
+            const uint32_t b_w = __shfl_sync(kFullMask, q.lbase, w), c_w = __shfl_sync(kFullMask, q.count, w);
             for (uint32_t j = tl; j < c_w; j += threads) {
                 if ((out >> w) & 1u) list[b_w + j] = kNoKey; else mark(list[b_w + j]);
             }
@@ -824,7 +806,7 @@ __device__ __forceinline__ void ranked_group(const DecArgs& a, DecShared& s, uin
     dec_team_sync<4>(team);
     if constexpr (MODE != 1) {
         for (uint32_t w = 0; w < W; ++w) {
-            const uint32_t b_w = __shfl_sync(kFullMask, lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, wbase, w);
+            const uint32_t b_w = __shfl_sync(kFullMask, q.lbase, w), c_w = __shfl_sync(kFullMask, count, w), s_w = __shfl_sync(kFullMask, q.wbase, w);
             if (c_w == 0u) continue;
             const uint8_t* codes = reinterpret_cast<const uint8_t*>(blob + s_w);
             for (uint32_t j = tl; j < c_w; j += threads) {
