@@ -10,23 +10,24 @@
 // per stream.
 //
 // Work split.  A block owns groups blockIdx.x, blockIdx.x + gridDim.x, ... and reads their
-// directory entries first, one entry per thread.  Groups with up to kDecWarpMax keys over all streams
-// are decoded by one warp each, larger ones by the whole block.  Either way the streams are parsed side
-// by side (the warp's lanes or the block's threads are shared out among them, a thread owns a run of
+// directory entries first, one entry per thread.  One stream: groups of up to kDecWarpMax keys (kDecWarpFew
+// where a block has few groups) are decoded by one warp each, larger ones by the whole block.  Several streams: groups go to
+// teams of one, two or four warps or to the block (team_rule).  Either way the streams are parsed side
+// by side (the team's lanes or the block's threads are shared out among them, a thread owns a run of
 // consecutive keys), into lists of keys in shared memory; a stream's group is validated in full
 // before any of it is applied; then the lists are applied with neighbouring threads on neighbouring keys
 // and all of a batch's memory accesses in flight together.
 //
 // What bounds it.  With few groups per block, the latency of the chain launch - directory - blob - parse - entries of
 // dense_out (about 3 + 5 us); with many scattered keys, DRAM transactions: a bare kernel that only reads and writes 2.7 M
-// floats at ascending random places of a 1 GiB array takes 100 us, the decoder 122.  So what counts is warps in
+// floats at ascending random places of a 1 GiB array takes 100 us, the decoder 121.  So what counts is warps in
 // flight and few instructions per key: 512 threads per block and two blocks per SM at 64 registers are 32 warps (256 threads
 // with longer register-resident runs, 16 warps, took 149 us there); parsing side by side with independent fetches instead of a
 // bit reader per thread halved the parse; the table of distinct keys or their ranks (teams) and the slice (blocks) give each coordinate one
 // round trip to memory however many streams hold it (one per stream before).  Measured before and after: four
-// streams of 128 K keys over 25.6 M entries 28.8 -> 23.5 us, eight streams of 33 K keys over 33.5 M 26.7 -> 16.8, one stream of
-// 1.3 M over 67 M 97.8 -> 59.5; model update of the first 68.6 -> 41.0, of eight streams of 671 K keys over 67 M on the
-// packed state 510 -> 307.
+// streams of 128 K keys over 25.6 M entries 28.8 -> 25.0 us, eight streams of 33 K keys over 33.5 M 26.7 -> 16.8, one stream of
+// 1.3 M over 67 M 97.8 -> 59.5; model update of the first 68.6 -> 50.5, of eight streams of 671 K keys over 67 M on the
+// packed state 510 -> 216.
 #pragma once
 
 #include <cstddef>
@@ -55,9 +56,10 @@ constexpr uint32_t kTileMinKeys    = 768;
 // group: entry by entry 57, 59, 65 us, over the slice 89, 88, 89)
 constexpr uint32_t kTileMinWords   = 1536;
 // Several streams whose groups have about as many keys: from this many a group on ranks by bits (four warps) instead of the table of keys, up to as
-// many as aggregation has the slice for.  Eight streams over 2^25 entries, us by table and by ranks (slice), at keys a group:
+// many as the slice is for (team_rule).  Eight streams over 2^25 entries, us by table and by ranks (slice), at keys a group:
 //   aggregation  180: 22, 27; 290: 27, 31; 420: 38, 37; 650: 59, 56; 850: 75, 68 (78); 980: 77 by ranks (78); 1310: 94 by ranks (78)
 //   update       180: 64, 63; 290: 97, 84; 420: 131, 102; 650: 183, 126; 1310: 182 over the slice of g, 164; 1770: 186, 174
+//   (two streams over as many entries: aggregation 450: 45, 43; 930: 70, 59; update 450: 124, 99; 700: 164, 127; packed 450: 61, 54; 930: 114, 90)
 //   packed       180: 25, 28; 290: 34, 35; 420: 51, 50; 650: 85, 76; 850: 112, 90; 1770: 196 over the slice, 139
 __host__ __device__ constexpr uint32_t ranked_mean(int mode) { return mode == 2 ? 256u : 400u; }
 constexpr uint32_t kSliceMean      = 1000;

@@ -72,7 +72,7 @@ def _check(n, counts, workers, seed, tau=128, update=True, group_log2=14, l=2):
         assert group_log2 > 14 or np.array_equal(packed[:, i].cpu().numpy(), x), i
 
 
-# one stream: warp / block (256), sweep of the update (768, packed 2048), slice of dense_out (1536), words of a blob that fit
+# one stream: warp / block (256), sweep of the update (768, packed 2048), slice of dense_out (1536 on so few entries), words of a blob that fit
 # the stage (4096 words at 8 + 2 + up to 8 bits a key), keys that fit the lists (8192); the last group is ragged
 @pytest.mark.parametrize("count", [1, 32, 33, 255, 256, 257, 767, 768, 1535, 1536, 2047, 2048, 2049, 4096, 4097, 8184, 8192, 8193, TILE])
 def test_one_stream(count):
@@ -137,8 +137,8 @@ def test_failed_streams_are_left_out(group_log2, count):
     assert np.array_equal(dense.cpu().numpy()[lo:hi], sound[lo:hi])
 
 
-# groups of several streams for teams of one, two and four warps (at most 6 bytes an entry and the blobs in 4, 8 and 16 KiB; less than 1536
-# keys, the update 768) and beyond, next to each other in one block; many groups to a block, few, and one
+# groups of several streams for teams of one, two and four warps (at most 6 bytes an entry and the blobs in 4, 8 and 16 KiB; by ranks what 24 KiB
+# hold; groups as unlike as these 249 keys at most) and beyond, next to each other in one block; many groups to a block, few, and one
 @pytest.mark.parametrize("groups,workers,l,group_log2", [(2700, 8, 2, 14), (740, 2, 2, 14), (740, 3, 1, 14), (740, 4, 5, 14), (740, 8, 2, 14),
                                                          (740, 8, 5, 10), (740, 5, 3, 11), (290, 2, 5, 14), (290, 8, 1, 14)])
 def test_teams_of_warps(groups, workers, l, group_log2):
@@ -155,7 +155,8 @@ def test_teams_on_groups_of_two_tiles(workers, count):
     _check((40 << 15) - 9, [count, count + 1] * 20, workers, 600 + count, group_log2=15)
 
 
-# teams of four warps (ranks by a bit for every index): keys at the edges of the bits' words and of the groups, streams that fail in one group
+# alike groups of more than 1000 keys over all streams, a few to a block: over the slice of dense_out, those of 2^15 by teams of four warps; keys at the
+# edges of 32 and of the groups, streams that fail in one group (ranks: test_gpu_decoder_ranks.py)
 @pytest.mark.parametrize("workers,count,group_log2", [(6, 170, 14), (3, 500, 14), (8, 130, 15), (7, 200, 11)])
 def test_teams_of_four_warps(workers, count, group_log2):
     groups, size = 620, 1 << group_log2
